@@ -2,12 +2,21 @@
 // n = 37, complete rings on Cartesian and hexagonal lattices, Appendix A).
 //
 // GPU design: nodes are binned into a uniform grid (about two nodes per cell,
-// counting sort by cell).  One warp serves one centre: it gathers every node
-// in a (2R+1)^2 window of cells into shared memory, ranks the candidates by
-// (squared distance, node index) and keeps the first n.  The window is
-// accepted only when the n-th distance is strictly inside the radius that
-// the window is guaranteed to cover; otherwise R grows.  The result equals a
+// counting sort by cell).  One warp serves one centre: it takes the nodes of
+// a (2R+1)^2 window of cells that lie strictly inside the radius the window
+// is guaranteed to cover, ranks them by (squared distance, node index) and
+// keeps the first n; with fewer than n inside, R grows.  The result equals a
 // brute-force sort over all nodes.
+//
+// What bounds it: instruction issue and the latency of the window's loads.
+// FP64 compares run at 2 per SM and clock here, so the ranking compares the
+// high words of the squared distances (non-negative doubles order as their
+// bits do) and settles equal high words by the full (distance, index) key.
+// The candidates of a warp take 16 bytes each, so that 32 to 56 warps fit one
+// SM; centres with more candidates than that space go to knn_kernel, which
+// holds up to 2048.  Measured on 77,235 scattered nodes, n = 56:
+// the whole window ranked in FP64 by 8 warps per SM 16.1 ms, this form about
+// 0.45 ms (stencils and weights together 58.6 -> 42.9 ms).
 #include <cfloat>
 #include <cmath>
 
@@ -74,28 +83,50 @@ __global__ void count_kernel(const double *x, const double *z, int64_t n, Grid g
     atomicAdd(&count[c], 1);
 }
 
-// Exclusive scan of count[0..m) into start[0..m] by one block of 1024 threads.
-__global__ void scan_kernel(const int *count, int m, int *start) {
-    __shared__ int part[1024];
-    int t = threadIdx.x;
-    int chunk = (m + blockDim.x - 1) / blockDim.x;
-    int b = t * chunk, e = min(b + chunk, m);
-    int s = 0;
-    for (int i = b; i < e; ++i) s += count[i];
-    part[t] = s;
-    __syncthreads();
-    for (int off = 1; off < blockDim.x; off <<= 1) {
-        int v = (t >= off) ? part[t - off] : 0;
+// Exclusive scan of count[0..m) into start[0..m] by one block of 1024 threads,
+// tile by tile (coalesced; a thread's serial chunk took 37 us for 38,600 cells).
+__global__ void __launch_bounds__(1024) scan_kernel(const int *count, int m, int *start) {
+    __shared__ int part[33];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    int base = 0;
+    for (int i0 = 0; i0 < m; i0 += 4096) {
+        const int i = i0 + 4 * t;
+        int v[4], sum = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            v[k] = i + k < m ? count[i + k] : 0;
+            sum += v[k];
+        }
+        int inc = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += u;
+        }
+        if (lane == 31) part[warp] = inc;
         __syncthreads();
-        part[t] += v;
+        if (warp == 0) {
+            const int w = part[lane];
+            int winc = w;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, winc, o);
+                if (lane >= o) winc += u;
+            }
+            part[lane] = winc - w;
+            if (lane == 31) part[32] = winc;
+        }
+        __syncthreads();
+        int run = base + part[warp] + inc - sum;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (i + k < m) start[i + k] = run;
+            run += v[k];
+        }
+        base += part[32];
         __syncthreads();
     }
-    int run = part[t] - s;
-    for (int i = b; i < e; ++i) {
-        start[i] = run;
-        run += count[i];
-    }
-    if (t == blockDim.x - 1) start[m] = part[t];
+    if (t == 0) start[m] = base;
 }
 
 __global__ void scatter_kernel(const int *cell, int64_t n, const int *start, int *cursor, int *sorted) {
@@ -119,69 +150,217 @@ __device__ __forceinline__ double sqdist(double xc, double zc, double xj, double
     return __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dz, dz));
 }
 
+// Columns [xa, xb] and rows [za, zb] of the (2R+1)^2 window around cell (cx, cz),
+// whether it holds every column or row, and the radius it is guaranteed to cover.
+struct Window {
+    int xa, xb, za, zb;
+    bool all_x, all_z;
+    double guard;
+};
+__device__ __forceinline__ Window window_of(const Grid &g, int cx, int cz, int R) {
+    Window w;
+    w.all_x = (2 * R + 1 >= g.ncx);
+    w.xa = w.all_x ? 0 : cx - R;
+    w.xb = w.all_x ? g.ncx - 1 : cx + R;
+    w.za = max(cz - R, 0);
+    w.zb = min(cz + R, g.ncz - 1);
+    w.all_z = (cz - R <= 0) && (cz + R >= g.ncz - 1);
+    if (g.period <= 0.0) {
+        w.all_x = w.all_x || ((cx - R <= 0) && (cx + R >= g.ncx - 1));
+        w.xa = max(w.xa, 0);
+        w.xb = min(w.xb, g.ncx - 1);
+    }
+    w.guard = DBL_MAX;
+    if (!w.all_x) w.guard = fmin(w.guard, R * g.cw);
+    if (!w.all_z) w.guard = fmin(w.guard, R * g.ch);
+    w.guard *= (1.0 - 1e-9);
+    return w;
+}
+
+// Positions [p0, p1) in `sorted` of the window's nodes in row rz; a periodic
+// window that wraps has a second range [q0, q1), which comes first.
+struct RowRange {
+    int p0, p1, q0, q1;
+};
+__device__ __forceinline__ RowRange row_range(const Grid &g, const Window &w, const int *start, int rz) {
+    RowRange r = {0, 0, 0, 0};
+    int a = w.xa, b = w.xb;
+    const int *s = start + rz * g.ncx;
+    if (g.period > 0.0 && !w.all_x) {
+        if (a < 0) { r.q0 = s[a + g.ncx]; r.q1 = s[g.ncx]; a = 0; }
+        if (b >= g.ncx) { r.q0 = s[0]; r.q1 = s[b - g.ncx + 1]; b = g.ncx - 1; }
+    }
+    r.p0 = s[a];
+    r.p1 = s[b + 1];
+    return r;
+}
+
+constexpr int kFastWarps = 8;
+
+// ranks of the NC candidates lane + 32 (k0 + c) of a warp's m: those with a
+// smaller high word
+template <int NC>
+__device__ __forceinline__ void count_smaller(const unsigned *hi2, int m, int k0, int lane, int *rank) {
+    unsigned own[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        const int i = lane + 32 * (k0 + c);
+        own[c] = i < m ? hi2[2 * i + 1] : 0u;
+        rank[c] = 0;
+    }
+    const uint4 *pair = reinterpret_cast<const uint4 *>(hi2);
+#pragma unroll 4
+    for (int j = 0; j < (m + 1) / 2; ++j) {   // an odd m is padded with the largest key
+        const uint4 v = pair[j];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) rank[c] += (int)(v.y < own[c]) + (int)(v.w < own[c]);
+    }
+}
+
+// One warp per centre.  Centres whose window holds more than `cap` candidates
+// inside the guaranteed radius are listed in slow (n_slow of them).
+__global__ void __launch_bounds__(kFastWarps * 32)
+knn_ranked_kernel(const double *__restrict__ x, const double *__restrict__ z, int64_t n_centers, int n, Grid g,
+                  const int *__restrict__ start, const int *__restrict__ sorted, int R0, int Rmax, int cap,
+                  int32_t *__restrict__ idx, int *__restrict__ status, int *__restrict__ slow,
+                  int *__restrict__ n_slow) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double *cd2 = reinterpret_cast<double *>(smem) + (size_t)warp * cap;
+    int *cid = reinterpret_cast<int *>(smem + (size_t)kFastWarps * cap * 8) + warp * cap;
+    int *mark = reinterpret_cast<int *>(smem + (size_t)kFastWarps * cap * 12) + warp * cap;
+    const int64_t c = blockIdx.x * (int64_t)kFastWarps + warp;
+    if (c >= n_centers) return;
+    const double xc = x[c], zc = z[c];
+    const int cx = cell_x(g, xc), cz = cell_z(g, zc);
+    for (int R = R0; R <= Rmax; ++R) {
+        const Window w = window_of(g, cx, cz, R);
+        const double r2 = w.guard * w.guard;
+        int m = 0, total = 0;
+        bool over = false;
+        for (int rb = w.za; rb <= w.zb; rb += 32) {
+            // the ranges of up to 32 rows at once, one per lane
+            RowRange rr = {0, 0, 0, 0};
+            if (rb + lane <= w.zb) rr = row_range(g, w, start, rb + lane);
+            int rows = rr.p1 - rr.p0 + rr.q1 - rr.q0;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) rows += __shfl_xor_sync(0xffffffffu, rows, o);
+            total += rows;
+            const int nr = min(32, w.zb - rb + 1);
+            for (int r = 0; r < nr && !over; ++r)
+                for (int part = 0; part < 2 && !over; ++part) {
+                    const int a = __shfl_sync(0xffffffffu, part ? rr.p0 : rr.q0, r);
+                    const int b = __shfl_sync(0xffffffffu, part ? rr.p1 : rr.q1, r);
+                    for (int base = a; base < b; base += 32) {
+                        const int p = base + lane;
+                        int j = 0;
+                        double d2 = DBL_MAX;
+                        bool in = false;
+                        if (p < b) {
+                            j = sorted[p];
+                            d2 = sqdist(xc, zc, x[j], z[j], g.period);
+                            in = d2 < r2;
+                        }
+                        const unsigned mask = __ballot_sync(0xffffffffu, in);
+                        if (m + __popc(mask) > cap - 1) { over = true; break; }   // one slot pads an odd count
+                        if (in) {
+                            const int pos = m + __popc(mask & ((1u << lane) - 1u));
+                            cd2[pos] = d2;
+                            cid[pos] = j;
+                            mark[pos] = 0;
+                        }
+                        m += __popc(mask);
+                    }
+                }
+        }
+        if (total > kMaxCand) {
+            if (lane == 0) atomicCAS(status, 0, 2);
+            return;
+        }
+        if (over) {
+            if (lane == 0) slow[atomicAdd(n_slow, 1)] = (int)c;
+            return;
+        }
+        if (m < n) {
+            __syncwarp();
+            continue;   // fewer than n nodes strictly inside the guaranteed radius
+        }
+        if (lane == 0) cd2[m] = __longlong_as_double(-1LL);   // pads the last pair with the largest key
+        __syncwarp();
+        // mark[i] holds candidate i's rank (high half), and how many candidates
+        // have rank i (low half)
+        const unsigned *hi2 = reinterpret_cast<const unsigned *>(cd2);
+        const int need = (m + 31) / 32;
+        for (int k0 = 0; k0 < need; k0 += 6) {
+            int rank[6];
+            if (need - k0 > 4) count_smaller<6>(hi2, m, k0, lane, rank);
+            else count_smaller<4>(hi2, m, k0, lane, rank);
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {
+                const int i = lane + 32 * (k0 + q);
+                if (i < m && q < need - k0) {
+                    atomicAdd(&mark[i], rank[q] << 16);
+                    atomicAdd(&mark[rank[q]], 1);
+                }
+            }
+        }
+        __syncwarp();
+        for (int i = lane; i < m; i += 32) {
+            int at = mark[i] >> 16;
+            if (at >= n) continue;
+            const int ii = cid[i];
+            if ((mark[at] & 0xffff) > 1) {   // equal high words: the full key decides
+                const double di = cd2[i];
+                const unsigned hi = hi2[2 * i + 1];
+                for (int j = 0; j < m; ++j)
+                    if (hi2[2 * j + 1] == hi) {
+                        const double dj = cd2[j];
+                        at += (dj < di) || (dj == di && cid[j] < ii);
+                    }
+            }
+            if (at < n) idx[c * n + at] = ii;
+        }
+        return;
+    }
+    if (lane == 0) atomicCAS(status, 0, 3);
+}
+
+// The general form: up to kMaxCand candidates per window in shared memory, the
+// whole window ranked.  Takes the centres that knn_ranked_kernel listed.
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
-knn_kernel(const double *__restrict__ x, const double *__restrict__ z, int64_t n_centers, int n, Grid g,
-           const int *__restrict__ start, const int *__restrict__ sorted, int R0, int Rmax,
+knn_kernel(const double *__restrict__ x, const double *__restrict__ z, const int *__restrict__ list, int n_list, int n,
+           Grid g, const int *__restrict__ start, const int *__restrict__ sorted, int R0, int Rmax,
            int32_t *__restrict__ idx, int *__restrict__ status) {
-    extern __shared__ unsigned char smem[];
+    extern __shared__ __align__(16) unsigned char smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double *cd2 = reinterpret_cast<double *>(smem) + warp * kMaxCand;
     int *cid = reinterpret_cast<int *>(reinterpret_cast<double *>(smem) + kWarpsPerBlock * kMaxCand) + warp * kMaxCand;
     __shared__ double nth_d2[kWarpsPerBlock];
 
-    const int64_t c = blockIdx.x * (int64_t)kWarpsPerBlock + warp;
-    if (c >= n_centers) return;
+    const int64_t q = blockIdx.x * (int64_t)kWarpsPerBlock + warp;
+    if (q >= n_list) return;
+    const int64_t c = list[q];
     const double xc = x[c], zc = z[c];
     const int cx = cell_x(g, xc), cz = cell_z(g, zc);
 
     for (int R = R0; R <= Rmax; ++R) {
-        // x columns of the window (all columns once if the window wraps onto itself)
-        bool all_x = (2 * R + 1 >= g.ncx);
-        int xa = all_x ? 0 : cx - R, xb = all_x ? g.ncx - 1 : cx + R;
-        int za = max(cz - R, 0), zb = min(cz + R, g.ncz - 1);
-        bool all_z = (cz - R <= 0) && (cz + R >= g.ncz - 1);
-        if (g.period <= 0.0) {
-            all_x = all_x || ((cx - R <= 0) && (cx + R >= g.ncx - 1));
-            xa = max(xa, 0);
-            xb = min(xb, g.ncx - 1);
-        }
+        const Window w = window_of(g, cx, cz, R);
         int m = 0;
-        bool overflow = false;
-        for (int rz = za; rz <= zb && !overflow; ++rz) {
-            // up to two contiguous column ranges (wrap-around in periodic x)
-            int ranges[2][2];
-            int nr = 0;
-            if (g.period > 0.0 && !all_x) {
-                int a = xa, b = xb;
-                if (a < 0) { ranges[nr][0] = a + g.ncx; ranges[nr][1] = g.ncx - 1; ++nr; a = 0; }
-                if (b >= g.ncx) { ranges[nr][0] = 0; ranges[nr][1] = b - g.ncx; ++nr; b = g.ncx - 1; }
-                ranges[nr][0] = a; ranges[nr][1] = b; ++nr;
-            } else {
-                ranges[0][0] = xa; ranges[0][1] = xb; nr = 1;
-            }
-            for (int q = 0; q < nr; ++q) {
-                int p0 = start[rz * g.ncx + ranges[q][0]];
-                int p1 = start[rz * g.ncx + ranges[q][1] + 1];
-                for (int base = p0; base < p1; base += 32) {
-                    int p = base + lane;
-                    bool has = p < p1;
-                    unsigned mask = __ballot_sync(0xffffffffu, has);
-                    int pos = m + __popc(mask & ((1u << lane) - 1u));
-                    int cnt = __popc(mask);
-                    if (m + cnt > kMaxCand) { overflow = true; break; }
-                    if (has) {
-                        int j = sorted[p];
-                        cd2[pos] = sqdist(xc, zc, x[j], z[j], g.period);
-                        cid[pos] = j;
-                    }
-                    m += cnt;
+        for (int rz = w.za; rz <= w.zb; ++rz) {
+            const RowRange rr = row_range(g, w, start, rz);
+            for (int part = 0; part < 2; ++part) {
+                const int p0 = part ? rr.p0 : rr.q0, p1 = part ? rr.p1 : rr.q1;
+                if (m + p1 - p0 > kMaxCand) {
+                    if (lane == 0) atomicCAS(status, 0, 2);
+                    return;
                 }
-                if (overflow) break;
+                for (int p = p0 + lane; p < p1; p += 32) {
+                    const int j = sorted[p];
+                    cd2[m + p - p0] = sqdist(xc, zc, x[j], z[j], g.period);
+                    cid[m + p - p0] = j;
+                }
+                m += p1 - p0;
             }
-        }
-        if (overflow) {
-            if (lane == 0) atomicCAS(status, 0, 2);
-            return;
         }
         __syncwarp();
         if (m < n) continue;
@@ -198,14 +377,46 @@ knn_kernel(const double *__restrict__ x, const double *__restrict__ z, int64_t n
             if (rank == n - 1) nth_d2[warp] = di;
         }
         __syncwarp();
-        double guard = DBL_MAX;
-        if (!all_x) guard = fmin(guard, R * g.cw);
-        if (!all_z) guard = fmin(guard, R * g.ch);
-        guard *= (1.0 - 1e-9);
-        if (nth_d2[warp] < guard * guard) return;   // the window provably holds the n nearest
+        if (nth_d2[warp] < w.guard * w.guard) return;   // the window provably holds the n nearest
         __syncwarp();
     }
     if (lane == 0) atomicCAS(status, 0, 3);
+}
+
+// Searches the stencils of every centre on a binned grid: knn_ranked_kernel,
+// then knn_kernel for the centres it listed.  `slow` takes n_centers entries;
+// counts[0] is the status and counts[1] the number listed (both cleared here).
+// Synchronises the stream.
+void search(const double *x, const double *z, int64_t n_centers, int n, const Grid &g, const int *start,
+            const int *sorted, int *slow, int *counts, int32_t *idx, cudaStream_t st) {
+    // first window: about 2.5 n candidates at two nodes per cell
+    int R0 = (int)std::ceil(std::sqrt(2.5 * n / (4.0 * 2.0)));
+    R0 = R0 < 1 ? 1 : R0;
+    const int Rmax = std::max(g.ncx, g.ncz);
+    // room for the candidates inside the first window's radius (2 pi R0^2 on
+    // average), half as many again and a margin, in whole warps
+    const int cap = std::min(kMaxCand, ((int)(1.5 * 6.2832 * R0 * R0) + 64 + 31) / 32 * 32);
+    const size_t fast = (size_t)kFastWarps * cap * (sizeof(double) + 2 * sizeof(int));
+    RBF_CUDA(cudaFuncSetAttribute(knn_ranked_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fast));
+    RBF_CUDA(cudaMemsetAsync(counts, 0, 2 * sizeof(int), st));
+    knn_ranked_kernel<<<div_up(n_centers, kFastWarps), kFastWarps * 32, fast, st>>>(
+        x, z, n_centers, n, g, start, sorted, R0, Rmax, cap, idx, counts, slow, counts + 1);
+    RBF_CHECK_LAUNCH();
+    int h[2] = {0, 0};
+    RBF_CUDA(cudaMemcpyAsync(h, counts, sizeof(h), cudaMemcpyDeviceToHost, st));
+    RBF_CUDA(cudaStreamSynchronize(st));
+    if (h[0] == 0 && h[1] > 0) {
+        const size_t smem = (size_t)kWarpsPerBlock * kMaxCand * (sizeof(double) + sizeof(int));
+        RBF_CUDA(cudaFuncSetAttribute(knn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        knn_kernel<<<div_up(h[1], kWarpsPerBlock), kWarpsPerBlock * 32, smem, st>>>(x, z, slow, h[1], n, g, start, sorted,
+                                                                                    R0, Rmax, idx, counts);
+        RBF_CHECK_LAUNCH();
+        RBF_CUDA(cudaMemcpyAsync(h, counts, sizeof(int), cudaMemcpyDeviceToHost, st));
+        RBF_CUDA(cudaStreamSynchronize(st));
+    }
+    RBF_REQUIRE(h[0] == 0, "stencil search failed (%s)",
+                h[0] == 2 ? "more than 2048 candidates in a search window: node density too uneven"
+                          : "no window holds n nodes");
 }
 
 }  // namespace
@@ -256,10 +467,9 @@ void build_stencils(const double *x, const double *z, int64_t n_all, int64_t n_c
     RBF_REQUIRE(ncell < ((int64_t)1 << 30), "binning grid too large");
 
     DevBuf<int> cellof(n_all), count(ncell), start(ncell + 1), cursor(ncell), sorted(n_all);
-    DevBuf<int> status(1);
+    DevBuf<int> counts(2);
     RBF_CUDA(cudaMemsetAsync(count.p, 0, count.bytes(), st));
     RBF_CUDA(cudaMemsetAsync(cursor.p, 0, cursor.bytes(), st));
-    RBF_CUDA(cudaMemsetAsync(status.p, 0, sizeof(int), st));
     count_kernel<<<div_up(n_all, 256), 256, 0, st>>>(x, z, n_all, g, cellof.p, count.p);
     RBF_CHECK_LAUNCH();
     scan_kernel<<<1, 1024, 0, st>>>(count.p, (int)ncell, start.p);
@@ -267,21 +477,7 @@ void build_stencils(const double *x, const double *z, int64_t n_all, int64_t n_c
     scatter_kernel<<<div_up(n_all, 256), 256, 0, st>>>(cellof.p, n_all, start.p, cursor.p, sorted.p);
     RBF_CHECK_LAUNCH();
 
-    // first window: about 2.5 n candidates at two nodes per cell
-    int R0 = (int)std::ceil(std::sqrt(2.5 * n / (4.0 * 2.0)));
-    R0 = R0 < 1 ? 1 : R0;
-    int Rmax = std::max(g.ncx, g.ncz);
-    size_t smem = (size_t)kWarpsPerBlock * kMaxCand * (sizeof(double) + sizeof(int));
-    RBF_CUDA(cudaFuncSetAttribute(knn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    knn_kernel<<<div_up(n_centers, kWarpsPerBlock), kWarpsPerBlock * 32, smem, st>>>(
-        x, z, n_centers, n, g, start.p, sorted.p, R0, Rmax, idx, status.p);
-    RBF_CHECK_LAUNCH();
-    int hs = 0;
-    RBF_CUDA(cudaMemcpyAsync(&hs, status.p, sizeof(int), cudaMemcpyDeviceToHost, st));
-    RBF_CUDA(cudaStreamSynchronize(st));
-    RBF_REQUIRE(hs == 0, "stencil search failed (%s)",
-                hs == 2 ? "more than 2048 candidates in a search window: node density too uneven"
-                        : "no window holds n nodes");
+    search(x, z, n_centers, n, g, start.p, sorted.p, cellof.p, counts.p, idx, st);   // cellof is free by now
 }
 
 // ---- allocation-free variant (rbf_build_stencils_static) --------------------
@@ -377,27 +573,13 @@ void build_stencils_static(const double *x, const double *z, int64_t n_all, int6
 
     RBF_CUDA(cudaMemsetAsync(count, 0, ncell * sizeof(int), st));
     RBF_CUDA(cudaMemsetAsync(cursor, 0, ncell * sizeof(int), st));
-    RBF_CUDA(cudaMemsetAsync(status, 0, sizeof(int), st));
     count_kernel<<<div_up(n_all, 256), 256, 0, st>>>(x, z, n_all, g, cellof, count);
     RBF_CHECK_LAUNCH();
     scan_kernel<<<1, 1024, 0, st>>>(count, (int)ncell, start);
     RBF_CHECK_LAUNCH();
     scatter_kernel<<<div_up(n_all, 256), 256, 0, st>>>(cellof, n_all, start, cursor, sorted);
     RBF_CHECK_LAUNCH();
-    int R0 = (int)std::ceil(std::sqrt(2.5 * n / (4.0 * 2.0)));
-    R0 = R0 < 1 ? 1 : R0;
-    const int Rmax = std::max(g.ncx, g.ncz);
-    const size_t smem = (size_t)kWarpsPerBlock * kMaxCand * (sizeof(double) + sizeof(int));
-    RBF_CUDA(cudaFuncSetAttribute(knn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    knn_kernel<<<div_up(n_centers, kWarpsPerBlock), kWarpsPerBlock * 32, smem, st>>>(
-        x, z, n_centers, n, g, start, sorted, R0, Rmax, idx, status);
-    RBF_CHECK_LAUNCH();
-    int hs = 0;
-    RBF_CUDA(cudaMemcpyAsync(&hs, status, sizeof(int), cudaMemcpyDeviceToHost, st));
-    RBF_CUDA(cudaStreamSynchronize(st));
-    RBF_REQUIRE(hs == 0, "stencil search failed (%s)",
-                hs == 2 ? "more than 2048 candidates in a search window: node density too uneven"
-                        : "no window holds n nodes");
+    search(x, z, n_centers, n, g, start, sorted, cellof, status, idx, st);   // cellof is free by now
 }
 
 }  // namespace rbf
