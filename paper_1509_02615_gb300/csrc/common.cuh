@@ -113,12 +113,12 @@ __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol
 // captured graph it becomes the kernel node's priority, which graphs
 // instantiated with cudaGraphInstantiateFlagUseNodePriority honour).
 template <typename... KArgs, typename... Args>
-void launch_kernel_prio(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t s, bool pdl, int prio,
+void launch_kernel_full(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool pdl, int prio,
                         Args &&...args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute at[2];
     int na = 0;
@@ -135,6 +135,19 @@ void launch_kernel_prio(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStr
     cfg.attrs = na ? at : nullptr;
     cfg.numAttrs = na;
     RBF_CUDA(cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...));
+}
+
+template <typename... KArgs, typename... Args>
+void launch_kernel_prio(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t s, bool pdl, int prio,
+                        Args &&...args) {
+    launch_kernel_full(kernel, grid, block, 0, s, pdl, prio, std::forward<Args>(args)...);
+}
+
+// with dynamic shared memory
+template <typename... KArgs, typename... Args>
+void launch_kernel_smem(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool pdl,
+                        Args &&...args) {
+    launch_kernel_full(kernel, grid, block, smem, s, pdl, 0, std::forward<Args>(args)...);
 }
 
 template <typename... KArgs, typename... Args>

@@ -12,10 +12,11 @@
 // thousand nodes, latency-bound, not a tensor-core sized GEMM):
 //   mlp_infer_kernel  fused gather + forward, one thread per node, weights in
 //                     shared memory as BF16
-//   mlp_train_kernel  fused gather + forward + backward for 128 samples per
-//                     block; per-block weight gradients (H^T dH products over
-//                     the block's samples) are added to FP32 gradients
-//   mlp_adam_kernel   Adam on FP32 master weights, refreshes the BF16 copy
+//   mlp_train_kernel  fused gather + forward + backward for 31 samples per
+//                     block; the block's weight gradients (H^T dH products
+//                     over its samples) go to its own FP32 partials
+//   mlp_reduce_kernel sums the partials in block order, then Adam on the FP32
+//                     master weights and the refresh of the BF16 copy
 #include <cuda_bf16.h>
 
 #include <cmath>
@@ -28,7 +29,10 @@
 namespace rbf {
 
 constexpr int kWidth = 64;
-constexpr int kTrainBlock = 128;
+constexpr int kTrainRows = 32;               // rows of a training block: 31 samples and the all-zero row
+constexpr int kTrainSamples = kTrainRows - 1;
+constexpr int kTrainThreads = 320;           // 10 warps: two passes over the 592 tiles of dW1 (n = 37)
+constexpr int kMaxInputs = 240;              // widest input layer (stencils of up to 60 nodes)
 constexpr int kScaleWarps = 2048;   // warps of the scale-sum launch (256 blocks of 256 threads)
 constexpr float kClip = 4.f;   // |y| <= 4 (in output-scale units) when the correction is applied
 
@@ -229,229 +233,351 @@ struct TrainArgs {
     float *Lp;            // [blocks]: this block's loss
 };
 
-// Fused gather + forward + backward for one block of 128 samples; the block's
+// Shared memory of the training kernel, in floats: features, activations and
+// their gradients are stored [unit][row] with kRS floats per unit, weights as
+// FP32 values of their BF16 copies.
+constexpr int kRS = kTrainRows + 4;   // row stride: 16-byte vectors of eight units hit distinct banks
+struct TrainSmem {
+    int X, W1, W2, W2t, W3, b, H1, H2, P, dH2, dH1, Y, end;
+};
+__host__ __device__ inline TrainSmem train_layout(int n_in) {
+    TrainSmem L;
+    L.X = 0;
+    L.W1 = L.X + n_in * kRS;
+    L.W2 = L.W1 + n_in * kWidth;
+    L.W2t = L.W2 + kWidth * kWidth;       // [j][m], stride kWidth + 4
+    L.W3 = L.W2t + kWidth * (kWidth + 4);
+    L.b = L.W3 + kWidth * 4;              // b1, b2, b3
+    L.H1 = L.b + 2 * kWidth + 4;
+    L.H2 = L.H1 + kWidth * kRS;
+    L.P = L.H2 + kWidth * kRS;            // two partial products
+    L.dH2 = L.P + 2 * kWidth * kRS;
+    L.dH1 = L.dH2 + kWidth * kRS;
+    L.Y = L.dH1 + kWidth * kRS;           // [row][4]: outputs, then their gradients
+    L.end = L.Y + kTrainRows * 4;
+    return L;
+}
+
+__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+
+// eight BF16 values as FP32
+__device__ __forceinline__ void put8(float *dst, const uint4 &v) {
+    const unsigned u[4] = {v.x, v.y, v.z, v.w};
+    float f[8];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        f[2 * q] = __uint_as_float(u[q] << 16);
+        f[2 * q + 1] = __uint_as_float(u[q] & 0xffff0000u);
+    }
+    *reinterpret_cast<float4 *>(dst) = make_float4(f[0], f[1], f[2], f[3]);
+    *reinterpret_cast<float4 *>(dst + 4) = make_float4(f[4], f[5], f[6], f[7]);
+}
+
+// P[half][c][row] = sum over half of k of A[k][row] B[k][c] for 32 rows and 64
+// columns: 128 threads per half of k, 4 rows x 4 columns each.
+__device__ __forceinline__ void rows_times(const float *A, const float *B, int bs, int K, float *P) {
+    if (threadIdx.x >= 256) return;
+    const int half = threadIdx.x >> 7, t = threadIdx.x & 127, lane = t & 31, w = t >> 5;
+    const int r0 = 4 * ((lane >> 3) + 4 * (w & 1)), c0 = 4 * ((lane & 7) + 8 * (w >> 1));
+    const int k0 = half ? K / 2 : 0, k1 = half ? K : K / 2;
+    float acc[4][4];   // [column][row]
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) acc[c][r] = 0.f;
+#pragma unroll 4
+    for (int k = k0; k < k1; ++k) {
+        const float4 x = ld4(A + k * kRS + r0), v = ld4(B + k * bs + c0);
+        const float xr[4] = {x.x, x.y, x.z, x.w}, vc[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) acc[c][r] += xr[r] * vc[c];
+    }
+    float *out = P + half * kWidth * kRS;
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+        *reinterpret_cast<float4 *>(out + (c0 + c) * kRS + r0) = make_float4(acc[c][0], acc[c][1], acc[c][2], acc[c][3]);
+}
+
+// G[a][b] = sum over the 32 rows of A[a][row] B[b][row] for a < na and 64
+// columns b (a weight gradient): 4 x 4 outputs per thread, interleaved so that
+// the vectors a warp reads lie in distinct banks.
+__device__ __forceinline__ void outer_sum(const float *A, int na, const float *B, float *G) {
+    const int ga = (na + 3) / 4;
+    for (int e = threadIdx.x; e < ga * 16; e += blockDim.x) {
+        const int tb = e & 15, ta = e >> 4;
+        float acc[4][4];
+        int ai[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            ai[i] = min(ta + i * ga, na - 1);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+        }
+#pragma unroll 2
+        for (int r = 0; r < kTrainRows; r += 4) {
+            float4 bv[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) bv[j] = ld4(B + (tb + 16 * j) * kRS + r);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float4 av = ld4(A + ai[i] * kRS + r);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    acc[i][j] += av.x * bv[j].x;
+                    acc[i][j] += av.y * bv[j].y;
+                    acc[i][j] += av.z * bv[j].z;
+                    acc[i][j] += av.w * bv[j].w;
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (ta + i * ga < na)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) G[(int64_t)(ta + i * ga) * kWidth + tb + 16 * j] = acc[i][j];
+    }
+}
+
+__device__ __forceinline__ float row_sum(const float *v) {
+    float s = 0.f;
+#pragma unroll
+    for (int r = 0; r < kTrainRows; r += 4) {
+        const float4 x = ld4(v + r);
+        s += (x.x + x.y) + (x.z + x.w);
+    }
+    return s;
+}
+
+// Fused gather + forward + backward for one block of 31 samples; the block's
 // weight gradients (X^T dH1, H1^T dH2, H2^T dY and bias sums) and loss go to
 // its own partials, which mlp_reduce_kernel sums over the blocks in block
-// order (so training is deterministic).
-__global__ void __launch_bounds__(kTrainBlock) mlp_train_kernel(TrainArgs a, Offs m_off) {
-    extern __shared__ unsigned char sm[];
+// order (so training is deterministic).  Row 31 is the all-zero feature row:
+// its output is f(0), which enters every y with the opposite sign, so its
+// output gradient is minus the sum of the others'.
+//
+// What bounds it: FP32 FMA issue (1.0 M products per block, 8 k cycles at the
+// full rate) behind the latency of the gather.  31 samples per block give one
+// block per SM at the default batch of 4096 (133 blocks); every product runs
+// from shared memory with 16 FMAs per two 16-byte loads.  One thread per
+// sample with the activations in registers (32 blocks of 128 threads) took
+// 207 us per launch and 217 us per iteration with its two follow-up kernels
+// at 4096 samples, n = 37; this form 21 us per iteration, reduction and Adam
+// included.
+__global__ void __launch_bounds__(kTrainThreads) mlp_train_kernel(TrainArgs a, Offs m_off) {
+    extern __shared__ __align__(16) float sf[];
+    __shared__ int64_t s_state[kTrainRows];   // first record of each row's state
+    __shared__ int64_t s_target[kTrainRows];  // its target record
+    __shared__ int s_node[kTrainRows];
     float *const gp = a.Gp + blockIdx.x * a.n_params;
-    const int n_in = 4 * (a.n - 1) + 4;
-    const int xs = n_in + 1;                 // padded row strides (bank spread)
-    const int hs = kWidth + 1;
-    const Net net = load_net(sm, a.Pb, a.P, n_in, m_off);
-    __shared__ float z1[kWidth], z2[kWidth], y0[4], dz[4], dz2[kWidth], dz1[kWidth];
-    zero_branch(net, z1, z2, y0);
-    float *X = reinterpret_cast<float *>(sm + ((net_bytes(n_in) + 15) & ~size_t(15)));
-    float *H1 = X + kTrainBlock * xs;
-    float *H2 = H1 + kTrainBlock * hs;
-    float *DY = H2 + kTrainBlock * hs;
-    __shared__ float red[kTrainBlock];
-    const int t = threadIdx.x;
-    const int s = blockIdx.x * kTrainBlock + t;
-    const bool live = s < a.B;
-    int64_t k = 0, i = 0;
-    if (live) {
-        if (a.samples) {
-            k = a.samples[2 * (int64_t)s];
-            i = a.samples[2 * (int64_t)s + 1];
-        } else {
-            const unsigned long long h = splitmix64(a.seed ^ splitmix64((unsigned long long)a.iter * 0x100000001ull + s));
-            k = (int64_t)(h % (unsigned long long)a.n_states);
-            i = (int64_t)((h >> 32) % (unsigned long long)a.n_prog);
+    const int n_in = 4 * (a.n - 1) + 4, slots = a.n - 1;
+    const TrainSmem L = train_layout(n_in);
+    float *X = sf + L.X, *H1 = sf + L.H1, *H2 = sf + L.H2, *P = sf + L.P, *dH2 = sf + L.dH2, *dH1 = sf + L.dH1,
+          *Y = sf + L.Y;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    // samples and features do not depend on the preceding kernel
+    if (t < kTrainRows) {
+        const int s = blockIdx.x * kTrainSamples + t;
+        int64_t k = 0, i = -1;
+        if (t < kTrainSamples && s < a.B) {
+            if (a.samples) {
+                k = a.samples[2 * (int64_t)s];
+                i = a.samples[2 * (int64_t)s + 1];
+            } else {
+                const unsigned long long h = splitmix64(a.seed ^ splitmix64((unsigned long long)a.iter * 0x100000001ull + s));
+                k = (int64_t)(h % (unsigned long long)a.n_states);
+                i = (int64_t)((h >> 32) % (unsigned long long)a.n_prog);
+            }
         }
+        s_state[t] = state_of(k, a.n_snap) * a.n_all;
+        s_target[t] = k * a.n_prog + i;
+        s_node[t] = (int)i;
     }
-    // features
-    const float *Uk = a.S + state_of(k, a.n_snap) * a.n_all * 4;
-    const Rec<float> own = load_rec(Uk, i);
-    const float is0 = 1.f / a.scales[0], is1 = 1.f / a.scales[1], is2 = 1.f / a.scales[2], is3 = 1.f / a.scales[3];
-    const int slots = a.n - 1;
-    float *x = X + t * xs;
-    float h[kWidth];
-#pragma unroll
-    for (int j = 0; j < kWidth; ++j) h[j] = net.b1[j];
-    for (int q = 1; q < a.n; ++q) {
-        const Rec<float> r = load_rec(Uk, a.idx[i * a.n + q]);
-        const float f0 = live ? (r.u - own.u) * is0 : 0.f, f1 = live ? (r.w - own.w) * is1 : 0.f;
-        const float f2 = live ? (r.t - own.t) * is2 : 0.f, f3 = live ? (r.p - own.p) * is3 : 0.f;
-        x[q - 1] = f0;
-        x[slots + q - 1] = f1;
-        x[2 * slots + q - 1] = f2;
-        x[3 * slots + q - 1] = f3;
-        layer1_row(h, net.W1, q - 1, f0);
-        layer1_row(h, net.W1, slots + q - 1, f1);
-        layer1_row(h, net.W1, 2 * slots + q - 1, f2);
-        layer1_row(h, net.W1, 3 * slots + q - 1, f3);
-    }
+    __syncthreads();
     {
-        // the node's own values
-        const float o0 = live ? own.u / a.scales[8] : 0.f, o1 = live ? own.w / a.scales[9] : 0.f;
-        const float o2 = live ? own.t / a.scales[10] : 0.f, o3 = live ? own.p / a.scales[11] : 0.f;
-        x[4 * slots + 0] = o0;
-        x[4 * slots + 1] = o1;
-        x[4 * slots + 2] = o2;
-        x[4 * slots + 3] = o3;
-        layer1_row(h, net.W1, 4 * slots + 0, o0);
-        layer1_row(h, net.W1, 4 * slots + 1, o1);
-        layer1_row(h, net.W1, 4 * slots + 2, o2);
-        layer1_row(h, net.W1, 4 * slots + 3, o3);
-    }
-#pragma unroll
-    for (int j = 0; j < kWidth; ++j) {
-        h[j] = tanhf(h[j]);
-        H1[t * hs + j] = h[j];
-    }
-    float h2[kWidth];
-    layer2(h, net.W2, net.b2, h2);
-#pragma unroll
-    for (int j = 0; j < kWidth; ++j) H2[t * hs + j] = h2[j];
-    float y[4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) y[c] = net.b3[c] - y0[c];
-#pragma unroll
-    for (int m = 0; m < kWidth; ++m)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) y[c] += h2[m] * bf(net.W3[m * 4 + c]);
-    float lsum = 0.f;
-    const float inv = 1.f / (4.f * (float)a.B);
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        float d = 0.f;
-        if (live) {
-            const float tgt = a.Tg[(k * a.n_prog + i) * 4 + c] / a.scales[4 + c];
-            const float r = y[c] - tgt;
-            lsum += r * r * inv;
-            d = 2.f * r * inv;
+        // a warp takes one slot of the 32 rows at a time (the last one: the node's own values)
+        const int i = s_node[lane];
+        const float *Uk = a.S + s_state[lane] * 4;
+        Rec<float> own = {0.f, 0.f, 0.f, 0.f};
+        if (i >= 0) own = load_rec(Uk, i);
+        const float is0 = 1.f / a.scales[0], is1 = 1.f / a.scales[1], is2 = 1.f / a.scales[2], is3 = 1.f / a.scales[3];
+#pragma unroll 4
+        for (int q = warp; q <= slots; q += kTrainThreads / 32) {
+            float f0 = 0.f, f1 = 0.f, f2 = 0.f, f3 = 0.f;
+            if (i >= 0) {
+                if (q < slots) {
+                    const Rec<float> r = load_rec(Uk, __ldg(a.idx + (int64_t)i * a.n + q + 1));
+                    f0 = (r.u - own.u) * is0;
+                    f1 = (r.w - own.w) * is1;
+                    f2 = (r.t - own.t) * is2;
+                    f3 = (r.p - own.p) * is3;
+                } else {
+                    f0 = own.u / a.scales[8];
+                    f1 = own.w / a.scales[9];
+                    f2 = own.t / a.scales[10];
+                    f3 = own.p / a.scales[11];
+                }
+            }
+            const int c = q < slots ? q : 4 * slots, step = q < slots ? slots : 1;
+            X[c * kRS + lane] = f0;
+            X[(c + step) * kRS + lane] = f1;
+            X[(c + 2 * step) * kRS + lane] = f2;
+            X[(c + 3 * step) * kRS + lane] = f3;
         }
-        DY[t * 4 + c] = d;
     }
-    red[t] = lsum;
-    __syncthreads();
-    for (int w = kTrainBlock / 2; w > 0; w >>= 1) {
-        if (t < w) red[t] += red[t + w];
-        __syncthreads();
+    grid_dep_wait();     // the weights come from the preceding iteration's kernel
+    grid_dep_launch();
+    // BF16 weights, eight per load (every block of Pb starts at a multiple of 64 values)
+    const uint4 *w1 = reinterpret_cast<const uint4 *>(a.Pb + m_off.oW1), *w2 = reinterpret_cast<const uint4 *>(a.Pb + m_off.oW2);
+#pragma unroll 4
+    for (int e = t; e < n_in * kWidth / 8; e += kTrainThreads) put8(sf + L.W1 + 8 * e, __ldcg(w1 + e));
+#pragma unroll 2
+    for (int e = t; e < kWidth * kWidth / 8; e += kTrainThreads) {
+        float *v = sf + L.W2 + 8 * e;
+        put8(v, __ldcg(w2 + e));
+        const int m = e / (kWidth / 8), j = e % (kWidth / 8) * 8;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) sf[L.W2t + (j + q) * (kWidth + 4) + m] = v[q];
     }
-    if (t == 0) a.Lp[blockIdx.x] = red[0];
-    // the f(0) branch enters y with the opposite sign: its output gradient is
-    // dz = -sum dY over the block, propagated back through z2 and z1
-    if (t < 4) {
-        float acc = 0.f;
-        for (int q = 0; q < kTrainBlock; ++q) acc += DY[q * 4 + t];
-        dz[t] = -acc;
-    }
-    __syncthreads();
+    for (int e = t; e < kWidth * 4; e += kTrainThreads) sf[L.W3 + e] = bf(a.Pb[m_off.oW3 + e]);
     if (t < kWidth) {
-        float g = 0.f;
-        for (int c = 0; c < 4; ++c) g += bf(net.W3[t * 4 + c]) * dz[c];
-        dz2[t] = g * (1.f - z2[t] * z2[t]);
+        sf[L.b + t] = a.P[m_off.ob1 + t];
+        sf[L.b + kWidth + t] = a.P[m_off.ob2 + t];
+    }
+    if (t < 4) sf[L.b + 2 * kWidth + t] = a.P[m_off.ob3 + t];
+    __syncthreads();
+    // forward
+    rows_times(X, sf + L.W1, kWidth, n_in, P);
+    __syncthreads();
+    for (int e = t; e < kWidth * kTrainRows; e += kTrainThreads) {
+        const int j = e / kTrainRows, at = j * kRS + e % kTrainRows;
+        H1[at] = tanhf(sf[L.b + j] + (P[at] + P[kWidth * kRS + at]));
     }
     __syncthreads();
-    if (t < kWidth) {
-        float g = 0.f;
-        for (int j = 0; j < kWidth; ++j) g += bf(net.W2[t * kWidth + j]) * dz2[j];
-        dz1[t] = g * (1.f - z1[t] * z1[t]);
+    rows_times(H1, sf + L.W2, kWidth, kWidth, P);
+    __syncthreads();
+    for (int e = t; e < kWidth * kTrainRows; e += kTrainThreads) {
+        const int j = e / kTrainRows, at = j * kRS + e % kTrainRows;
+        H2[at] = tanhf(sf[L.b + kWidth + j] + (P[at] + P[kWidth * kRS + at]));
     }
     __syncthreads();
-    // dW3 = H2^T dY + z2 dz^T, db3 = sum dY + dz
-    for (int o = t; o < kWidth * 4 + 4; o += kTrainBlock) {
-        float acc = 0.f;
-        if (o < kWidth * 4) {
-            const int m = o >> 2, c = o & 3;
-            for (int q = 0; q < kTrainBlock; ++q) acc += H2[q * hs + m] * DY[q * 4 + c];
-            gp[m_off.oW3 + o] = acc + z2[m] * dz[c];
-        } else {
-            const int c = o - kWidth * 4;
-            for (int q = 0; q < kTrainBlock; ++q) acc += DY[q * 4 + c];
-            gp[m_off.ob3 + c] = acc + dz[c];
+    if (t < 4 * kTrainRows) {
+        const int r = t % kTrainRows, c = t / kTrainRows;
+        float y0 = 0.f, y1 = 0.f, y2 = 0.f, y3 = 0.f;
+#pragma unroll 4
+        for (int m = 0; m < kWidth; m += 4) {
+            y0 += H2[m * kRS + r] * sf[L.W3 + m * 4 + c];
+            y1 += H2[(m + 1) * kRS + r] * sf[L.W3 + m * 4 + 4 + c];
+            y2 += H2[(m + 2) * kRS + r] * sf[L.W3 + m * 4 + 8 + c];
+            y3 += H2[(m + 3) * kRS + r] * sf[L.W3 + m * 4 + 12 + c];
         }
+        Y[r * 4 + c] = sf[L.b + 2 * kWidth + c] + ((y0 + y1) + (y2 + y3));
     }
     __syncthreads();
-    // dH2 = (dY W3^T) o (1 - h2^2), written over this thread's H2 row
+    if (warp == 0) {
+        // loss and output gradients, one row per lane; row 31 holds f(0)
+        const bool live = s_node[lane] >= 0;
+        const float inv = 1.f / (4.f * (float)a.B);
+        const float4 y = ld4(Y + lane * 4);
+        const float yr[4] = {y.x, y.y, y.z, y.w};
+        float loss = 0.f, d[4];
 #pragma unroll
-    for (int m = 0; m < kWidth; ++m) {
-        float g = 0.f;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) g += DY[t * 4 + c] * bf(net.W3[m * 4 + c]);
-        H2[t * hs + m] = g * (1.f - h2[m] * h2[m]);
-    }
-    __syncthreads();
-    // dW2 = H1^T dH2 + z1 dz2^T, db2 = sum dH2 + dz2
-    for (int o = t; o < kWidth * kWidth + kWidth; o += kTrainBlock) {
-        float acc = 0.f;
-        if (o < kWidth * kWidth) {
-            const int m = o / kWidth, j = o % kWidth;
-            for (int q = 0; q < kTrainBlock; ++q) acc += H1[q * hs + m] * H2[q * hs + j];
-            gp[m_off.oW2 + o] = acc + z1[m] * dz2[j];
-        } else {
-            const int j = o - kWidth * kWidth;
-            for (int q = 0; q < kTrainBlock; ++q) acc += H2[q * hs + j];
-            gp[m_off.ob2 + j] = acc + dz2[j];
+        for (int c = 0; c < 4; ++c) {
+            const float f0 = __shfl_sync(0xffffffffu, yr[c], kTrainRows - 1);
+            d[c] = 0.f;
+            if (live) {
+                const float r = yr[c] - f0 - a.Tg[s_target[lane] * 4 + c] / a.scales[4 + c];
+                loss += r * r * inv;
+                d[c] = 2.f * r * inv;
+            }
+            float sum = d[c];
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            if (lane == kTrainRows - 1) d[c] = -sum;
+            if (lane == c) gp[m_off.ob3 + c] = sum - sum;   // the rows' gradients cancel: db3 = 0 (or NaN)
         }
+        *reinterpret_cast<float4 *>(Y + lane * 4) = make_float4(d[0], d[1], d[2], d[3]);
+        for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+        if (lane == 0) a.Lp[blockIdx.x] = loss;
     }
     __syncthreads();
-    // dH1 = (dH2 W2^T) o (1 - h1^2), written over this thread's H1 row
-    for (int m = 0; m < kWidth; ++m) {
-        float g = 0.f;
-        const __nv_bfloat162 *w = reinterpret_cast<const __nv_bfloat162 *>(net.W2 + m * kWidth);
-#pragma unroll
-        for (int j = 0; j < kWidth / 2; ++j) {
-            const float2 v = __bfloat1622float2(w[j]);
-            g += H2[t * hs + 2 * j] * v.x + H2[t * hs + 2 * j + 1] * v.y;
+    // dW3 = H2^T dY; dH2 = (dY W3^T) o (1 - h2^2)
+    for (int e = t; e < kWidth * 4; e += kTrainThreads) {
+        const int m = e >> 2, c = e & 3;
+        float s0 = 0.f, s1 = 0.f;
+#pragma unroll 8
+        for (int r = 0; r < kTrainRows; r += 2) {
+            s0 += H2[m * kRS + r] * Y[r * 4 + c];
+            s1 += H2[m * kRS + r + 1] * Y[r * 4 + 4 + c];
         }
-        const float hm = H1[t * hs + m];
-        // each thread rewrites only its own row, after every thread has read
-        // all rows of H1 in the dW2 product above
-        h[m] = g * (1.f - hm * hm);
+        gp[m_off.oW3 + e] = s0 + s1;
+    }
+    for (int e = t; e < kWidth * kTrainRows; e += kTrainThreads) {
+        const int m = e / kTrainRows, r = e % kTrainRows;
+        const float4 dy = ld4(Y + r * 4), w = ld4(sf + L.W3 + m * 4);
+        const float h = H2[m * kRS + r];
+        dH2[m * kRS + r] = (dy.x * w.x + dy.y * w.y + dy.z * w.z + dy.w * w.w) * (1.f - h * h);
     }
     __syncthreads();
-#pragma unroll
-    for (int m = 0; m < kWidth; ++m) H1[t * hs + m] = h[m];
+    // dW2 = H1^T dH2, db2 = sum dH2; dH1 = (dH2 W2^T) o (1 - h1^2)
+    outer_sum(H1, kWidth, dH2, gp + m_off.oW2);
+    rows_times(dH2, sf + L.W2t, kWidth + 4, kWidth, P);
+    if (t >= kTrainThreads - kWidth) gp[m_off.ob2 + t - (kTrainThreads - kWidth)] = row_sum(dH2 + (t - (kTrainThreads - kWidth)) * kRS);
+    __syncthreads();
+    for (int e = t; e < kWidth * kTrainRows; e += kTrainThreads) {
+        const int m = e / kTrainRows, at = m * kRS + e % kTrainRows;
+        const float h = H1[at];
+        dH1[at] = (P[at] + P[kWidth * kRS + at]) * (1.f - h * h);
+    }
     __syncthreads();
     // dW1 = X^T dH1, db1 = sum dH1
-    for (int o = t; o < n_in * kWidth + kWidth; o += kTrainBlock) {
-        float acc = 0.f;
-        if (o < n_in * kWidth) {
-            const int r = o / kWidth, j = o % kWidth;
-            for (int q = 0; q < kTrainBlock; ++q) acc += X[q * xs + r] * H1[q * hs + j];
-            gp[m_off.oW1 + o] = acc;
+    outer_sum(X, n_in, dH1, gp + m_off.oW1);
+    if (t >= kTrainThreads - kWidth) gp[m_off.ob1 + t - (kTrainThreads - kWidth)] = row_sum(dH1 + (t - (kTrainThreads - kWidth)) * kRS);
+}
+
+// G = sum over the blocks of their gradient partials and the iteration's loss
+// = sum of the blocks' losses, in a fixed order: 8 threads per parameter take
+// every eighth block, and their sums are added in thread order.  ADAM: the
+// step of the FP32 master weights and the refresh of the BF16 copy in the same
+// launch (G is then not kept).
+template <bool ADAM>
+__global__ void __launch_bounds__(256) mlp_reduce_kernel(const float *Gp, const float *Lp, int nb, int64_t n_params,
+                                                         float *G, float *loss, float *P, __nv_bfloat16 *Pb, float *M,
+                                                         float *V, float lr, float b1t, float b2t) {
+    __shared__ float part[8][32];
+    const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
+    const int64_t p = blockIdx.x * (int64_t)32 + lane;
+    grid_dep_wait();
+    grid_dep_launch();
+    float g = 0.f;
+    if (p < n_params) {
+#pragma unroll 8
+        for (int b = grp; b < nb; b += 8) g += __ldcg(Gp + b * n_params + p);
+    }
+    part[grp][lane] = g;
+    __syncthreads();
+    if (grp == 0 && p < n_params) {
+        g = 0.f;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) g += part[q][lane];
+        if (ADAM) {
+            const float m = 0.9f * M[p] + 0.1f * g;
+            const float v = 0.999f * V[p] + 0.001f * g * g;
+            M[p] = m;
+            V[p] = v;
+            const float w = P[p] - lr * (m / (1.f - b1t)) / (sqrtf(v / (1.f - b2t)) + 1e-8f);
+            P[p] = w;
+            Pb[p] = __float2bfloat16_rn(w);
         } else {
-            const int j = o - n_in * kWidth;
-            for (int q = 0; q < kTrainBlock; ++q) acc += H1[q * hs + j];
-            gp[m_off.ob1 + j] = acc + dz1[j];
+            G[p] = g;
         }
     }
-}
-
-// G = sum over the blocks of their gradient partials, and the iteration's
-// loss = sum of the blocks' losses, both in block order.
-__global__ void mlp_reduce_kernel(const float *Gp, const float *Lp, int nb, int64_t n_params, float *G,
-                                  float *loss) {
-    const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (p < n_params) {
-        float g = 0.f;
-        for (int b = 0; b < nb; ++b) g += Gp[b * n_params + p];
-        G[p] = g;
-    }
-    if (p == 0) {
+    if (blockIdx.x == 0 && grp == 1) {
         float l = 0.f;
-        for (int b = 0; b < nb; ++b) l += Lp[b];
-        *loss = l;
+        for (int b = lane; b < nb; b += 32) l += Lp[b];
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (lane == 0) *loss = l;
     }
-}
-
-__global__ void mlp_adam_kernel(float *P, __nv_bfloat16 *Pb, float *G, float *M, float *V, int64_t n, float lr,
-                                float b1t, float b2t) {
-    const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    const float g = G[p];
-    const float m = 0.9f * M[p] + 0.1f * g;
-    const float v = 0.999f * V[p] + 0.001f * g * g;
-    M[p] = m;
-    V[p] = v;
-    const float w = P[p] - lr * (m / (1.f - b1t)) / (sqrtf(v / (1.f - b2t)) + 1e-8f);
-    P[p] = w;
-    Pb[p] = __float2bfloat16_rn(w);
-    G[p] = 0.f;
 }
 
 __global__ void to_bf16(const float *P, __nv_bfloat16 *Pb, int64_t n) {
@@ -523,9 +649,7 @@ __global__ void target_kernel(const float *next, const float *stepped, float *tg
     if (e < n_prog * 4) tg[e] = (next[e] - stepped[e]) * inv_dt;
 }
 
-size_t train_smem(int n_in) {
-    return ((net_bytes(n_in) + 15) & ~size_t(15)) + (size_t)kTrainBlock * ((n_in + 1) + 2 * (kWidth + 1) + 4) * 4;
-}
+size_t train_smem(int n_in) { return (size_t)train_layout(n_in).end * sizeof(float); }
 
 void mlp_launch_infer(Mlp &m, Problem &pb, const void *U, void *delta, cudaStream_t s) {
     const size_t smem = net_bytes(m.n_in);
@@ -539,8 +663,13 @@ void mlp_launch_infer(Mlp &m, Problem &pb, const void *U, void *delta, cudaStrea
     RBF_CHECK_LAUNCH();
 }
 
+struct AdamStep {
+    float lr = 0.f, b1t = 0.f, b2t = 0.f;   // step size, powers of the decay rates
+};
+
 void mlp_launch_train(Mlp &m, Problem &pb, const float *S, const float *Tg, int64_t n_runs, int64_t n_snap,
-                      const int64_t *samples, int B, unsigned long long seed, long long iter, float *loss) {
+                      const int64_t *samples, int B, unsigned long long seed, long long iter, float *loss,
+                      const AdamStep *adam) {
     TrainArgs a{};
     a.S = S;
     a.Tg = Tg;
@@ -557,16 +686,19 @@ void mlp_launch_train(Mlp &m, Problem &pb, const float *S, const float *Tg, int6
     a.Pb = m.Pb.p;
     a.P = m.P.p;
     a.scales = m.scales.p;
-    const int nb = div_up(B, kTrainBlock);
+    const int nb = div_up(B, kTrainSamples);
     if (m.Gp.n < (size_t)nb * m.n_params) m.Gp.alloc((size_t)nb * m.n_params);
     if (m.Lp.n < (size_t)nb) m.Lp.alloc(nb);
     a.Gp = m.Gp.p;
     a.n_params = m.n_params;
     a.Lp = m.Lp.p;
-    mlp_train_kernel<<<nb, kTrainBlock, train_smem(m.n_in), m.st>>>(a, offs_of(m));
-    RBF_CHECK_LAUNCH();
-    mlp_reduce_kernel<<<div_up(m.n_params, 256), 256, 0, m.st>>>(m.Gp.p, m.Lp.p, nb, m.n_params, m.Gr.p, loss);
-    RBF_CHECK_LAUNCH();
+    // programmatic dependent launches: the next iteration's gather overlaps
+    // this one's reduction
+    launch_kernel_smem(mlp_train_kernel, dim3(nb), dim3(kTrainThreads), train_smem(m.n_in), m.st, true, a, offs_of(m));
+    const AdamStep s = adam ? *adam : AdamStep{};
+    launch_kernel(adam ? mlp_reduce_kernel<true> : mlp_reduce_kernel<false>, dim3(div_up(m.n_params, 32)), dim3(256), m.st,
+                  true, (const float *)m.Gp.p, (const float *)m.Lp.p, nb, m.n_params, m.Gr.p, loss, m.P.p, m.Pb.p,
+                  m.M.p, m.V.p, s.lr, s.b1t, s.b2t);
 }
 
 }  // namespace
@@ -578,7 +710,7 @@ void mlp_init(Mlp &m, Problem &pb, void *stream) {
     m.n = pb.n;
     m.slots = pb.n - 1;
     m.n_in = 4 * m.slots + 4;
-    RBF_REQUIRE(train_smem(m.n_in) <= 227 * 1024, "stencil of %d nodes too large for the training kernel", pb.n);
+    RBF_REQUIRE(m.n_in <= kMaxInputs, "stencil of %d nodes too large for the training kernel", pb.n);
     m.oW1 = 0;
     m.ob1 = m.oW1 + (int64_t)m.n_in * kWidth;
     m.oW2 = m.ob1 + kWidth;
@@ -715,7 +847,8 @@ int rbf_mlp_grad(rbf_mlp *h, const float *states, const float *targets, int64_t 
         rbf::DevBuf<float> loss(1);
         RBF_CUDA(cudaMemsetAsync(loss.p, 0, sizeof(float), m.st));
         RBF_CUDA(cudaMemsetAsync(m.Gr.p, 0, m.Gr.bytes(), m.st));
-        rbf::mlp_launch_train(m, h->coarse->impl, states, targets, n_runs, n_snap, samples, batch, 0, 0, loss.p);
+        rbf::mlp_launch_train(m, h->coarse->impl, states, targets, n_runs, n_snap, samples, batch, 0, 0, loss.p,
+                              nullptr);
         if (grad_host) RBF_CUDA(cudaMemcpyAsync(grad_host, m.Gr.p, m.Gr.bytes(), cudaMemcpyDeviceToHost, m.st));
         if (loss_host) RBF_CUDA(cudaMemcpyAsync(loss_host, loss.p, sizeof(float), cudaMemcpyDeviceToHost, m.st));
         RBF_CUDA(cudaMemsetAsync(m.Gr.p, 0, m.Gr.bytes(), m.st));
@@ -732,15 +865,14 @@ int rbf_mlp_train(rbf_mlp *h, const float *states, const float *targets, int64_t
         m.loss.alloc(std::max<int64_t>(iters, 1));
         RBF_CUDA(cudaMemsetAsync(m.loss.p, 0, m.loss.bytes(), m.st));
         for (int64_t it = 0; it < iters; ++it) {
-            rbf::mlp_launch_train(m, h->coarse->impl, states, targets, n_runs, n_snap, nullptr, batch, seed, it,
-                                  m.loss.p + it);
             m.t += 1;
             // cosine decay of the step size over the run
-            const float lr_t = lr * 0.5f * (1.f + std::cos(3.14159265358979f * (float)it / (float)iters));
-            rbf::mlp_adam_kernel<<<rbf::div_up(m.n_params, 256), 256, 0, m.st>>>(
-                m.P.p, m.Pb.p, m.Gr.p, m.M.p, m.V.p, m.n_params, lr_t, std::pow(0.9f, (float)m.t),
-                std::pow(0.999f, (float)m.t));
-            RBF_CHECK_LAUNCH();
+            rbf::AdamStep step;
+            step.lr = lr * 0.5f * (1.f + std::cos(3.14159265358979f * (float)it / (float)iters));
+            step.b1t = std::pow(0.9f, (float)m.t);
+            step.b2t = std::pow(0.999f, (float)m.t);
+            rbf::mlp_launch_train(m, h->coarse->impl, states, targets, n_runs, n_snap, nullptr, batch, seed, it,
+                                  m.loss.p + it, &step);
         }
         if (loss_host) RBF_CUDA(cudaMemcpyAsync(loss_host, m.loss.p, iters * sizeof(float), cudaMemcpyDeviceToHost, m.st));
         RBF_CUDA(cudaStreamSynchronize(m.st));
