@@ -94,8 +94,8 @@ void choose_threads(Problem &pb, int requested) {
                     "threads_per_node must be 0, 1, 2, 4 or 8");
         pb.G = requested;
         pack_operators(pb);
-        // registers hold the operands when they fit (per-node storage only)
-        pb.pf = (pb.kind == kNS && pb.SLQ <= 3 && !pb.lat.enabled) ? 3 : 0;
+        // registers hold the operands when they fit (FP32, per-node storage only)
+        pb.pf = (pb.kind == kNS && pb.precision == 32 && pb.SLQ <= 3 && !pb.lat.enabled) ? 3 : 0;
     }
 }
 

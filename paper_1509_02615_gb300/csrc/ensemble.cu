@@ -16,6 +16,7 @@
 #include <cstring>
 #include <numeric>
 
+#include "fixdot.cuh"
 #include "problem.cuh"
 #include "records.cuh"
 
@@ -26,7 +27,8 @@ namespace {
 template <class T>
 struct BlockDesc {
     const int32_t *pidx;
-    const T *wx, *wz, *wd, *wh;
+    const T *wx, *wz, *wd, *wh;   // FP64: fixed-point pairs (fixdot.cuh)
+    const short4 *wexp, *lexp;    // FP64: row exponents of the member's nodes, of its classes
     const T *pibar;
     const unsigned char *flags;
     const int32_t *lcls, *loff;   // member's lattice storage (null: per-node rows only)
@@ -59,22 +61,46 @@ struct VecE<float> {
     __device__ static int at(const int4 &v, int k) { return k == 0 ? v.x : k == 1 ? v.y : k == 2 ? v.z : v.w; }
     __device__ static int4 shift(const int4 &v, int d) { return make_int4(v.x + d, v.y + d, v.z + d, v.w + d); }
 };
-template <>
-struct VecE<double> {
-    static constexpr int V = 2;
-    using W = double2;
-    using I = int2;
-    __device__ static double at(const double2 &v, int k) { return k == 0 ? v.x : v.y; }
-    __device__ static int at(const int2 &v, int k) { return k == 0 ? v.x : v.y; }
-    __device__ static int2 shift(const int2 &v, int d) { return make_int2(v.x + d, v.y + d); }
-};
+
+// Tendencies of Eqs. (uEq)-(piEq) of member node i from its record c and its
+// sums, and the RK4 update; the node's G lanes split the four fields.
+template <class T, int G>
+__device__ __forceinline__ void finish_node(const BlockDesc<T> &d, const EnsArgs<T> &a, int64_t i, int g, const Rec<T> &c,
+                                            T ux, T uz, T ud, T wx_, T wz_, T wd_, T tx, T tz, T td, T px, T pz, T ph) {
+    const unsigned char fl = d.flags[i];
+    const T cpth = a.cp * (a.theta_bar + c.t);
+    T k[4];
+    k[0] = -c.u * ux - c.w * uz - cpth * px + ud;
+    k[1] = -c.u * wx_ - c.w * wz_ - cpth * pz + a.g_over_tb * c.t + wd_;
+    k[2] = -c.u * tx - c.w * tz + td;
+    k[3] = -c.u * px - c.w * (a.dpibar + pz) - a.rd_cv * (d.pibar[i] + c.p) * (ux + wz_) + ph;
+    if (fl & 1) k[1] = 0;
+    if (fl & 2) k[0] = 0;
+    const T an = (T)(a.cA * d.dt), bs = (T)(a.cB * d.dt);
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+        if (f % G != g) continue;
+        const T kf = k[f];
+        const int64_t e = (d.rec0 + i) * 4 + f;
+        const T un = a.Un[e];
+        if (a.stage == 0) {
+            a.K[e] = bs * kf;
+            a.Uout[e] = un + an * kf;
+        } else if (a.stage < 3) {
+            a.K[e] += bs * kf;
+            a.Uout[e] = un + an * kf;
+        } else {
+            a.Uout[e] = un + (a.K[e] + bs * kf);
+        }
+    }
+}
 
 // The stage kernel of Eqs. (uEq)-(piEq) with the RK4 update, for a block of
 // one ensemble member (same arithmetic and operand order as the single-problem
 // stage kernel with streamed operands).  LAT: members with lattice storage
 // take a class node's operands from the member's class table.
 template <class T, int G, bool DIFF, bool LAT>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) ens_stage_kernel(const BlockDesc<T> *__restrict__ descs, EnsArgs<T> a) {
+__global__ void __launch_bounds__(256, 4) ens_stage_kernel(const BlockDesc<T> *__restrict__ descs, EnsArgs<T> a) {
     using VT = VecE<T>;
     using W = typename VT::W;
     using I = typename VT::I;
@@ -140,41 +166,68 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) ens_stage_kernel(
     }
     if (!live) return;
     const Rec<T> c = DIFF ? fi : load_rec(U, i);
-    const unsigned char fl = d.flags[i];
-    const T cpth = a.cp * (a.theta_bar + c.t);
-    T k[4];
-    k[0] = -c.u * ux - c.w * uz - cpth * px + ud;
-    k[1] = -c.u * wx_ - c.w * wz_ - cpth * pz + a.g_over_tb * c.t + wd_;
-    k[2] = -c.u * tx - c.w * tz + td;
-    k[3] = -c.u * px - c.w * (a.dpibar + pz) - a.rd_cv * (d.pibar[i] + c.p) * (ux + wz_) + ph;
-    if (fl & 1) k[1] = 0;
-    if (fl & 2) k[0] = 0;
-    const T an = (T)(a.cA * d.dt), bs = (T)(a.cB * d.dt);
-#pragma unroll
-    for (int f = 0; f < 4; ++f) {
-        if (f % G != g) continue;
-        const T kf = k[f];
-        const int64_t e = (d.rec0 + i) * 4 + f;
-        const T un = a.Un[e];
-        if (a.stage == 0) {
-            a.K[e] = bs * kf;
-            a.Uout[e] = un + an * kf;
-        } else if (a.stage < 3) {
-            a.K[e] += bs * kf;
-            a.Uout[e] = un + an * kf;
-        } else {
-            a.Uout[e] = un + (a.K[e] + bs * kf);
-        }
+    finish_node<T, G>(d, a, i, g, c, ux, uz, ud, wx_, wz_, wd_, tx, tz, td, px, pz, ph);
+}
+
+// The FP64 form: sums in fixed point (fixdot.cuh), two threads per lane, as the
+// single-problem stage kernel has them, in blocks of kFixThreads threads.
+template <int G, bool LAT>
+__global__ void __launch_bounds__(kFixThreads, 7) ens_stage_fixed_kernel(const BlockDesc<double> *__restrict__ descs,
+                                                                         EnsArgs<double> a) {
+    __shared__ FixRing ring;
+    const BlockDesc<double> d = descs[blockIdx.x];
+    const int pair = threadIdx.x >> 1, h = threadIdx.x & 1, g = pair % G;
+    int64_t i = d.node0 + pair / G;
+    const bool live = i < d.n_prog;
+    if (!live) i = d.n_prog - 1;
+    FixStream s;
+    s.SLQ = d.SLQ;
+    s.step = d.n_prog * G;   // in vectors
+    s.ops = s.step * d.SLQ;
+    s.w = reinterpret_cast<const int4 *>(d.wx) + i * G + g;
+    s.idx = reinterpret_cast<const int2 *>(d.pidx) + i * G + g;
+    s.shift = 0;
+    short4 ew;
+    const int cl = (LAT && d.lcls) ? __ldg(d.lcls + i) : -1;
+    if (LAT && cl >= 0) {
+        s.step = G;
+        s.ops = (int64_t)d.n_cls * d.SLQ * G;
+        s.w = reinterpret_cast<const int4 *>(d.lw) + (int64_t)cl * d.SLQ * G + g;
+        s.idx = reinterpret_cast<const int2 *>(d.loff) + (int64_t)cl * d.SLQ * G + g;
+        s.shift = (int)i;
+        ew = __ldg(d.lexp + cl);
+    } else {
+        ew = __ldg(d.wexp + i);
     }
+    FixFetch<LAT> fetch;
+    fetch.start(s, &ring[0][0][0], kFixThreads / 2);
+    fetch.copy(0);
+    fetch.copy(1);
+    grid_dep_wait();
+    grid_dep_launch();
+    const double *U = a.Uin + d.rec0 * 4;   // member-local record indices from here on
+    FixHalf f;
+    fix_sums<G, LAT>(U, s, ring, fetch, f);
+    const HalfSums sums = fix_finish<G>(f, ew, h);
+    const Rec<double> c = load_rec(U, i);
+    const double2 k = fix_tendency(sums, {a.cp, a.g_over_tb, a.theta_bar, a.dpibar, a.rd_cv}, h,
+                                   make_double4(c.u, c.w, c.t, c.p), d.pibar[i], d.flags[i]);
+    if (!live || g != 0) return;
+    const int64_t e = 2 * (d.rec0 + i) + h;   // the half record of both fields
+    fix_rk4_update(a.stage, a.cA * d.dt, a.cB * d.dt, k, reinterpret_cast<const double2 *>(a.Un) + e,
+                   reinterpret_cast<double2 *>(a.K) + e, reinterpret_cast<double2 *>(a.Uout) + e);
 }
 
 const double kA[4] = {0.5, 0.5, 1.0, 0.0};
 const double kB[4] = {1.0 / 6.0, 1.0 / 3.0, 1.0 / 3.0, 1.0 / 6.0};
 
+// threads of a stage block
+int block_threads(const Problem &pb) { return pb.precision == 64 ? kFixThreads : 256; }
+
 template <class T>
 void fill_descs(Problem &pb) {
     EnsembleState &E = *pb.ens;
-    const int C = 256 / pb.G;
+    const int C = block_threads(pb) / (pb.precision == 64 ? 2 * pb.G : pb.G);   // nodes per block
     std::vector<BlockDesc<T>> h;
     E.blocks_before.assign(1, 0);
     for (int oi : E.order) {
@@ -188,12 +241,14 @@ void fill_descs(Problem &pb) {
             d.wz = pw + total;
             d.wd = pw + 2 * total;
             d.wh = pw + 3 * total;
+            d.wexp = m.wexp.p;
             d.pibar = (const T *)m.pibar.p;
             d.flags = m.flags.p;
             if (m.lat.enabled) {
                 d.lcls = m.lat.cls.p;
                 d.loff = m.lat.loff.p;
                 d.lw = (const T *)m.lat.lw.p;
+                d.lexp = m.lat.lexp.p;
                 d.n_cls = m.lat.n_cls;
             }
             d.n_prog = m.n_prog;
@@ -212,13 +267,15 @@ void fill_descs(Problem &pb) {
 
 template <class T, int G>
 void launch_ens(Problem &pb, const EnsArgs<T> &a, int64_t nblocks, cudaStream_t s, bool pdl) {
-    constexpr bool kDiff = sizeof(T) == 4;
-    if (pb.lat.enabled)
-        launch_kernel(ens_stage_kernel<T, G, kDiff, true>, dim3((unsigned)nblocks), dim3(256), s, pdl,
-                      (const BlockDesc<T> *)pb.ens->descs.p, a);
-    else
-        launch_kernel(ens_stage_kernel<T, G, kDiff, false>, dim3((unsigned)nblocks), dim3(256), s, pdl,
-                      (const BlockDesc<T> *)pb.ens->descs.p, a);
+    const BlockDesc<T> *descs = (const BlockDesc<T> *)pb.ens->descs.p;
+    const dim3 grid((unsigned)nblocks), blk(block_threads(pb));
+    if constexpr (sizeof(T) == 8) {
+        if (pb.lat.enabled) launch_kernel(ens_stage_fixed_kernel<G, true>, grid, blk, s, pdl, descs, a);
+        else launch_kernel(ens_stage_fixed_kernel<G, false>, grid, blk, s, pdl, descs, a);
+    } else {
+        if (pb.lat.enabled) launch_kernel(ens_stage_kernel<T, G, true, true>, grid, blk, s, pdl, descs, a);
+        else launch_kernel(ens_stage_kernel<T, G, true, false>, grid, blk, s, pdl, descs, a);
+    }
 }
 
 template <class T>

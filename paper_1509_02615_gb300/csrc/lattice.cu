@@ -18,6 +18,7 @@
 #include <cstring>
 #include <unordered_map>
 
+#include "fixdot.cuh"
 #include "problem.cuh"
 
 namespace rbf {
@@ -159,8 +160,30 @@ void pack_lattice(Problem &pb, const std::vector<double> &comb, int nops) {
     L.loff.alloc(std::max<size_t>(off.size(), 1));
     RBF_CUDA(cudaMemcpyAsync(L.loff.p, off.data(), off.size() * 4, cudaMemcpyHostToDevice, pb.st));
     L.lw.alloc(std::max<size_t>(w.size(), 1) * pb.tsize());
+    std::vector<int2> fixed;
+    std::vector<short4> ex;
     if (pb.precision == 64) {
-        RBF_CUDA(cudaMemcpyAsync(L.lw.p, w.data(), w.size() * 8, cudaMemcpyHostToDevice, pb.st));
+        // fixed point, as pack_fixed_kernel forms it for the class's first member
+        fixed.resize(w.size());
+        ex.resize(std::max<int32_t>(L.n_cls, 1));
+        for (int32_t c = 0; c < L.n_cls; ++c) {
+            short e4[4];
+            for (int p = 0; p < 4; ++p) {
+                const size_t at = ((size_t)p * L.n_cls + c) * per;
+                double top = 0.0, sum = 0.0;
+                for (int t = 0; t < per; ++t) {
+                    top = std::max(top, std::fabs(w[at + t]));
+                    sum += std::fabs(w[at + t]);
+                }
+                const int e = fix_exponent(top, sum);
+                for (int t = 0; t < per; ++t) fixed[at + t] = fix_weight(w[at + t], e);
+                e4[p] = (short)e;
+            }
+            ex[c] = make_short4(e4[0], e4[1], e4[2], e4[3]);
+        }
+        L.lexp.alloc(ex.size());
+        RBF_CUDA(cudaMemcpyAsync(L.lexp.p, ex.data(), L.lexp.bytes(), cudaMemcpyHostToDevice, pb.st));
+        RBF_CUDA(cudaMemcpyAsync(L.lw.p, fixed.data(), fixed.size() * sizeof(int2), cudaMemcpyHostToDevice, pb.st));
     } else {
         std::vector<float> wf(w.begin(), w.end());
         RBF_CUDA(cudaMemcpyAsync(L.lw.p, wf.data(), wf.size() * 4, cudaMemcpyHostToDevice, pb.st));

@@ -12,7 +12,8 @@
 // FP32 mode uses the difference form sum_j w_ij (f_j - f_i) (every operator
 // here annihilates constants: the p_0 = 1 constraint row of Eq. (weights)),
 // which drops the centre slot and keeps cancellation errors relative to the
-// local variation.  FP64 mode keeps the plain product sum_j w_ij f_j.
+// local variation.  FP64 mode forms the plain product sum_j w_ij f_j, in fixed
+// point on the integer units (fixdot.cuh).
 //
 // Each stage kernel evaluates all 12 stencil sums of a node (d/dx, d/dz of
 // the four fields, the dissipation mu Lap + hyperviscosity on u, w, theta',
@@ -22,6 +23,7 @@
 #include <cmath>
 #include <cstring>
 
+#include "fixdot.cuh"
 #include "problem.cuh"
 #include "records.cuh"
 
@@ -37,7 +39,8 @@ struct NSArgs {
     T *K;             // [n_prog][4] RK4 accumulator
     T *dUdt;          // [n_prog][4] tendency (stage < 0)
     const int32_t *pidx;
-    const T *wx, *wz, *wd, *wh;
+    const T *wx, *wz, *wd, *wh;   // FP64: fixed-point pairs (fixdot.cuh), not doubles
+    const short4 *wexp;           // FP64: row exponents of each node, or of each class
     const T *pibar;
     const unsigned char *flags;
     // split stage launches: each of the two launches takes its nodes from
@@ -49,6 +52,7 @@ struct NSArgs {
     // of every slot, [4][n_cls][SLQ][G][V] (null: per-node storage only)
     const int32_t *lcls, *loff;
     const T *lw;
+    const short4 *lexp;
     int n_cls;
     int64_t n_prog, n_all;
     int SLQ;          // operand vectors per lane
@@ -57,7 +61,7 @@ struct NSArgs {
     T cp, g_over_tb, theta_bar, dpibar, rd_cv;
 };
 
-// 16-byte operand vectors: 4 FP32 or 2 FP64 slots, with matching index vectors.
+// 16-byte operand vectors of 4 FP32 slots, with matching index vectors.
 template <class T>
 struct Vec;
 template <>
@@ -69,17 +73,45 @@ struct Vec<float> {
     __device__ static int at(const int4 &v, int k) { return k == 0 ? v.x : k == 1 ? v.y : k == 2 ? v.z : v.w; }
     __device__ static int4 shift(const int4 &v, int d) { return make_int4(v.x + d, v.y + d, v.z + d, v.w + d); }
 };
-template <>
-struct Vec<double> {
-    static constexpr int V = 2;
-    using W = double2;
-    using I = int2;
-    __device__ static double at(const double2 &v, int k) { return k == 0 ? v.x : v.y; }
-    __device__ static int at(const int2 &v, int k) { return k == 0 ? v.x : v.y; }
-    __device__ static int2 shift(const int2 &v, int d) { return make_int2(v.x + d, v.y + d); }
-};
 
 constexpr int kPrefetchVec = 3;   // operand vectors per lane held in registers (prefetch variant)
+
+// Tendencies of Eqs. (uEq)-(piEq) of node i from its record c and its sums,
+// and the RK4 update (or the bare tendency when stage < 0); the node's G lanes
+// split the four fields between them.
+template <class T, int G>
+__device__ __forceinline__ void finish_node(const NSArgs<T> &a, int64_t i, int g, const Rec<T> &c, T ux, T uz, T ud, T wx_,
+                                            T wz_, T wd_, T tx, T tz, T td, T px, T pz, T ph) {
+    const unsigned char fl = a.flags[i];
+    const T cpth = a.cp * (a.theta_bar + c.t);
+    T k[4];
+    k[0] = -c.u * ux - c.w * uz - cpth * px + ud;
+    k[1] = -c.u * wx_ - c.w * wz_ - cpth * pz + a.g_over_tb * c.t + wd_;
+    k[2] = -c.u * tx - c.w * tz + td;
+    k[3] = -c.u * px - c.w * (a.dpibar + pz) - a.rd_cv * (a.pibar[i] + c.p) * (ux + wz_) + ph;
+    if (fl & 1) k[1] = 0;   // w = 0 held on bottom/top walls
+    if (fl & 2) k[0] = 0;   // u = 0 held on left/right walls
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+        if (f % G != g) continue;   // lanes split the four fields' epilogues
+        const T kf = k[f];
+        const int64_t e = i * 4 + f;
+        if (a.stage < 0) {
+            a.dUdt[e] = kf;
+        } else {
+            const T un = a.Un[e];
+            if (a.stage == 0) {
+                a.K[e] = a.b_stage * kf;
+                a.Uout[e] = un + a.a_next * kf;
+            } else if (a.stage < 3) {
+                a.K[e] += a.b_stage * kf;
+                a.Uout[e] = un + a.a_next * kf;
+            } else {
+                a.Uout[e] = un + (a.K[e] + a.b_stage * kf);
+            }
+        }
+    }
+}
 
 // One RK4 stage (or the bare right-hand side when stage < 0) for G lanes per
 // node.  Each lane reads its operands as 16-byte vectors (V slots each) and
@@ -90,7 +122,7 @@ constexpr int kPrefetchVec = 3;   // operand vectors per lane held in registers 
 // table (neighbour = node + offset); the lanes of a warp whose nodes share a
 // class read the same table entries, which stay in L1.
 template <class T, int G, bool DIFF, int PF, bool LAT>
-__global__ void __launch_bounds__(256, (sizeof(T) == 4 && PF == 0) ? 4 : 1) ns_stage_kernel(NSArgs<T> a) {
+__global__ void __launch_bounds__(256, PF > 0 ? 1 : 4) ns_stage_kernel(NSArgs<T> a) {
     using VT = Vec<T>;
     using W = typename VT::W;
     using I = typename VT::I;
@@ -184,35 +216,72 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && PF == 0) ? 4 : 1) ns_s
     }
     if (!live) return;
     const Rec<T> c = DIFF ? fi : load_rec(U, i);
-    const unsigned char fl = a.flags[i];
-    const T cpth = a.cp * (a.theta_bar + c.t);
-    T k[4];
-    k[0] = -c.u * ux - c.w * uz - cpth * px + ud;
-    k[1] = -c.u * wx_ - c.w * wz_ - cpth * pz + a.g_over_tb * c.t + wd_;
-    k[2] = -c.u * tx - c.w * tz + td;
-    k[3] = -c.u * px - c.w * (a.dpibar + pz) - a.rd_cv * (a.pibar[i] + c.p) * (ux + wz_) + ph;
-    if (fl & 1) k[1] = 0;   // w = 0 held on bottom/top walls
-    if (fl & 2) k[0] = 0;   // u = 0 held on left/right walls
-#pragma unroll
-    for (int f = 0; f < 4; ++f) {
-        if (f % G != g) continue;   // lanes split the four fields' epilogues
-        const T kf = k[f];
-        const int64_t e = i * 4 + f;
-        if (a.stage < 0) {
-            a.dUdt[e] = kf;
-        } else {
-            const T un = a.Un[e];
-            if (a.stage == 0) {
-                a.K[e] = a.b_stage * kf;
-                a.Uout[e] = un + a.a_next * kf;
-            } else if (a.stage < 3) {
-                a.K[e] += a.b_stage * kf;
-                a.Uout[e] = un + a.a_next * kf;
-            } else {
-                a.Uout[e] = un + (a.K[e] + a.b_stage * kf);
-            }
-        }
+    finish_node<T, G>(a, i, g, c, ux, uz, ud, wx_, wz_, wd_, tx, tz, td, px, pz, ph);
+}
+
+// The FP64 stage (or bare right-hand side): the sums in fixed point
+// (fixdot.cuh), everything else in FP64.  On 308,097 scattered nodes with
+// n = 56 a launch took 365 us as 12 x 56 FP64 FMAs per node (0.95 of the FP64
+// pipe) and takes 173 us.  What bounds it now: the gathers through the L1 tags
+// (without the first pass 152 us, without the products 163 us, without the
+// operand stream 157 us) and, under them, 99 us of operand traffic at the copy
+// rate.  Seven blocks of 128 threads per SM (72 registers): six take 181 us,
+// eight, with spills, 181 us; one thread per node for all four fields (126
+// registers, 16 warps per SM) 225 us.
+template <int G, bool LAT>
+__global__ void __launch_bounds__(kFixThreads, 7) ns_stage_fixed_kernel(NSArgs<double> a) {
+    __shared__ FixRing ring;
+    const int64_t pair = (blockIdx.x * (int64_t)kFixThreads + threadIdx.x) >> 1;
+    const int h = threadIdx.x & 1, g = (int)(pair % G);
+    int64_t i = pair / G;
+    bool live;
+    if (a.nlist) {
+        live = i < a.n_list;
+        i = __ldg(a.nlist + (live ? i : a.n_list - 1));
+    } else {
+        live = i < a.n_prog;
+        if (!live) i = a.n_prog - 1;   // keep the lanes of the warp in the shuffles
     }
+    if (!__any_sync(0xffffffffu, live)) return;
+    FixStream s;
+    s.SLQ = a.SLQ;
+    s.step = a.n_prog * G;   // in vectors
+    s.ops = s.step * a.SLQ;
+    s.w = reinterpret_cast<const int4 *>(a.wx) + i * G + g;
+    s.idx = reinterpret_cast<const int2 *>(a.pidx) + i * G + g;
+    s.shift = 0;
+    short4 ew;
+    const int cl = LAT ? __ldg(a.lcls + i) : -1;
+    if (LAT && cl >= 0) {
+        s.step = G;
+        s.ops = (int64_t)a.n_cls * a.SLQ * G;
+        s.w = reinterpret_cast<const int4 *>(a.lw) + (int64_t)cl * a.SLQ * G + g;
+        s.idx = reinterpret_cast<const int2 *>(a.loff) + (int64_t)cl * a.SLQ * G + g;
+        s.shift = (int)i;
+        ew = __ldg(a.lexp + cl);
+    } else {
+        ew = __ldg(a.wexp + i);
+    }
+    FixFetch<LAT> fetch;
+    fetch.start(s, &ring[0][0][0], kFixThreads / 2);
+    fetch.copy(0);
+    fetch.copy(1);
+    grid_dep_wait();     // the stage input (and its ghosts) come from earlier kernels
+    grid_dep_launch();
+    FixHalf f;
+    fix_sums<G, LAT>(a.Uin, s, ring, fetch, f);
+    const HalfSums sums = fix_finish<G>(f, ew, h);
+    const Rec<double> c = load_rec(a.Uin, i);
+    const double2 k = fix_tendency(sums, {a.cp, a.g_over_tb, a.theta_bar, a.dpibar, a.rd_cv}, h,
+                                   make_double4(c.u, c.w, c.t, c.p), a.pibar[i], a.flags[i]);
+    if (!live || g != 0) return;
+    const int64_t e = 2 * i + h;   // the half record of both fields
+    if (a.stage < 0) {
+        reinterpret_cast<double2 *>(a.dUdt)[e] = k;
+        return;
+    }
+    fix_rk4_update(a.stage, a.a_next, a.b_stage, k, reinterpret_cast<const double2 *>(a.Un) + e,
+                   reinterpret_cast<double2 *>(a.K) + e, reinterpret_cast<double2 *>(a.Uout) + e);
 }
 
 // Velocity u(x, t) = sum_k c_k(t) (U_k, V_k)(x) with c_k(t) = fa_k + fb_k
@@ -322,6 +391,52 @@ __global__ void pack_kernel(const double *__restrict__ w64, const int32_t *__res
     }
 }
 
+// FP64 operators in fixed point (fixdot.cuh): one warp per node packs its rows
+// as pack_kernel does, with (Wh, Wl) pairs in place of the values, and writes
+// the rows' exponents.
+__global__ void __launch_bounds__(256) pack_fixed_kernel(const double *__restrict__ w64, const int32_t *__restrict__ idx,
+                                                         int64_t n_prog, int n, int nops, int first, int n_slots,
+                                                         int SLQ, int G, const double *__restrict__ comb,
+                                                         int2 *__restrict__ pw, int32_t *__restrict__ pidx,
+                                                         short4 *__restrict__ wexp) {
+    const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (i >= n_prog) return;
+    constexpr int V = 2;
+    const int per = SLQ * G * V;
+    const int64_t total = (int64_t)per * n_prog;
+    short ex[4];
+    for (int p = 0; p < 4; ++p) {
+        auto weight = [&](int slot) {
+            double val = 0.0;
+            for (int o = 0; o < nops; ++o) {
+                const double c = comb[p * nops + o];
+                if (c != 0.0) val += c * w64[((int64_t)o * n_prog + i) * n + slot + first];
+            }
+            return val;
+        };
+        double top = 0.0, sum = 0.0;
+        for (int t = lane; t < n_slots; t += 32) {
+            const double v = fabs(weight(t));
+            top = fmax(top, v);
+            sum += v;
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            top = fmax(top, __shfl_xor_sync(0xffffffffu, top, o));
+            sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        }
+        const int e = fix_exponent(top, sum);
+        ex[p] = (short)e;
+        for (int t = lane; t < per; t += 32) {
+            const int v = t % V, gq = t / V, g = gq % G, q = gq / G;
+            const int64_t dst = (((int64_t)q * n_prog + i) * G + g) * V + v;
+            pw[p * total + dst] = t < n_slots ? fix_weight(weight(t), e) : make_int2(0, 0);
+            if (p == 0) pidx[dst] = t < n_slots ? idx[i * n + t + first] : (int32_t)i;
+        }
+    }
+    if (lane == 0) wexp[i] = make_short4(ex[0], ex[1], ex[2], ex[3]);
+}
+
 // Advection: packed block k < NP = flux-form weights of velocity part k,
 // -(Dx_ij U_k(x_j) + Dy_ij V_k(x_j)); block NP = (-1)^(k+1) gamma Delta^k
 // weights; columns folded onto the source node of reflected nodes
@@ -380,9 +495,26 @@ __global__ void minmax_kernel(const T *U, int64_t n_prog, int F, double *out, in
     }
 }
 
+template <int G>
+void launch_ns_fixed(const NSArgs<double> &a, cudaStream_t s, bool pdl, int prio) {
+    const dim3 grid(div_up((a.nlist ? a.n_list : a.n_prog) * G * 2, kFixThreads)), blk(kFixThreads);   // two threads per lane
+    if (a.lcls) launch_kernel_prio(ns_stage_fixed_kernel<G, true>, grid, blk, s, pdl, prio, a);
+    else launch_kernel_prio(ns_stage_fixed_kernel<G, false>, grid, blk, s, pdl, prio, a);
+}
+
+void launch_ns(const NSArgs<double> &a, int G, int, cudaStream_t s, bool pdl, int prio = 0) {
+    switch (G) {
+        case 1: launch_ns_fixed<1>(a, s, pdl, prio); break;
+        case 2: launch_ns_fixed<2>(a, s, pdl, prio); break;
+        case 4: launch_ns_fixed<4>(a, s, pdl, prio); break;
+        case 8: launch_ns_fixed<8>(a, s, pdl, prio); break;
+        default: RBF_FAIL(RBF_E_ARG, "threads per node %d not in {1,2,4,8}", G);
+    }
+}
+
 template <class T, int G, int PF>
 void launch_ns_g(const NSArgs<T> &a, cudaStream_t s, bool pdl, int prio) {
-    constexpr bool kDiff = sizeof(T) == 4;   // FP32: difference form; FP64: plain sums
+    constexpr bool kDiff = true;   // difference form
     const dim3 grid(div_up((a.nlist ? a.n_list : a.n_prog) * G, 256)), blk(256);
     if (a.lcls) {
         if (PF == 0) launch_kernel_prio(ns_stage_kernel<T, G, kDiff, 0, true>, grid, blk, s, pdl, prio, a);
@@ -392,19 +524,18 @@ void launch_ns_g(const NSArgs<T> &a, cudaStream_t s, bool pdl, int prio) {
     }
 }
 
-template <class T>
-void launch_ns(const NSArgs<T> &a, int G, int pf, cudaStream_t s, bool pdl, int prio = 0) {
+void launch_ns(const NSArgs<float> &a, int G, int pf, cudaStream_t s, bool pdl, int prio = 0) {
     if (pf > 0 && a.SLQ > kPrefetchVec)
         RBF_FAIL(RBF_E_ARG, "prefetch variant needs <= %d operand vectors per lane", kPrefetchVec);
     switch (G * 2 + (pf > 0)) {
-        case 2: launch_ns_g<T, 1, 0>(a, s, pdl, prio); break;
-        case 3: launch_ns_g<T, 1, kPrefetchVec>(a, s, pdl, prio); break;
-        case 4: launch_ns_g<T, 2, 0>(a, s, pdl, prio); break;
-        case 5: launch_ns_g<T, 2, kPrefetchVec>(a, s, pdl, prio); break;
-        case 8: launch_ns_g<T, 4, 0>(a, s, pdl, prio); break;
-        case 9: launch_ns_g<T, 4, kPrefetchVec>(a, s, pdl, prio); break;
-        case 16: launch_ns_g<T, 8, 0>(a, s, pdl, prio); break;
-        case 17: launch_ns_g<T, 8, kPrefetchVec>(a, s, pdl, prio); break;
+        case 2: launch_ns_g<float, 1, 0>(a, s, pdl, prio); break;
+        case 3: launch_ns_g<float, 1, kPrefetchVec>(a, s, pdl, prio); break;
+        case 4: launch_ns_g<float, 2, 0>(a, s, pdl, prio); break;
+        case 5: launch_ns_g<float, 2, kPrefetchVec>(a, s, pdl, prio); break;
+        case 8: launch_ns_g<float, 4, 0>(a, s, pdl, prio); break;
+        case 9: launch_ns_g<float, 4, kPrefetchVec>(a, s, pdl, prio); break;
+        case 16: launch_ns_g<float, 8, 0>(a, s, pdl, prio); break;
+        case 17: launch_ns_g<float, 8, kPrefetchVec>(a, s, pdl, prio); break;
         default: RBF_FAIL(RBF_E_ARG, "threads per node %d not in {1,2,4,8}", G);
     }
 }
@@ -437,9 +568,11 @@ NSArgs<T> ns_args(Problem &pb) {
     a.wz = pw + total;
     a.wd = pw + 2 * total;
     a.wh = pw + 3 * total;
+    a.wexp = pb.wexp.p;
     a.pibar = (const T *)pb.pibar.p;
     a.flags = pb.flags.p;
     if (pb.lat.enabled) {
+        a.lexp = pb.lat.lexp.p;
         a.lcls = pb.lat.cls.p;
         a.loff = pb.lat.loff.p;
         a.lw = (const T *)pb.lat.lw.p;
@@ -514,20 +647,20 @@ void rk4_ns(Problem &pb, double dt, T *U, cudaStream_t s, bool rec, int step, bo
             ar.nlist = pb.rlist.p;
             ar.n_list = pb.n_prog - pb.n_wall;
             if (st > 0) RBF_CUDA(cudaStreamWaitEvent(pb.side, pb.ev_w[(st - 1) & 1], 0));
-            launch_ns<T>(ar, pb.G, pb.pf, pb.side, pb.pdl);
+            launch_ns(ar, pb.G, pb.pf, pb.side, pb.pdl);
             RBF_CUDA(cudaEventRecord(pb.ev_r[st & 1], pb.side));
             enqueue_ghost_fill(pb, in[st], s, pb.prio_hi);   // ahead of the other launch's blocks
             if (st > 0 || !first) RBF_CUDA(cudaStreamWaitEvent(s, pb.ev_r[(st + 3) & 1], 0));
             NSArgs<T> aw = a;   // the wall set, ahead of the other launch
             aw.nlist = pb.wlist.p;
             aw.n_list = pb.n_wall;
-            launch_ns<T>(aw, pb.G, pb.pf, s, pb.pdl, pb.prio_hi);
+            launch_ns(aw, pb.G, pb.pf, s, pb.pdl, pb.prio_hi);
             RBF_CUDA(cudaEventRecord(pb.ev_w[st & 1], s));
             continue;
         }
         enqueue_ghost_fill(pb, in[st], s);
         if (rec) RBF_CUDA(cudaEventRecordWithFlags(pb.rhs_ev[(step * 4 + st) * 2], s, cudaEventRecordExternal));
-        launch_ns<T>(a, pb.G, pb.pf, s, pb.pdl && !rec);
+        launch_ns(a, pb.G, pb.pf, s, pb.pdl && !rec);
         if (rec) RBF_CUDA(cudaEventRecordWithFlags(pb.rhs_ev[(step * 4 + st) * 2 + 1], s, cudaEventRecordExternal));
     }
     if (split && last) RBF_CUDA(cudaStreamWaitEvent(s, pb.ev_r[1], 0));
@@ -605,11 +738,12 @@ void pack_operators(Problem &pb) {
     DevBuf<double> dcomb(comb.size());
     RBF_CUDA(cudaMemcpyAsync(dcomb.p, comb.data(), dcomb.bytes(), cudaMemcpyHostToDevice, pb.st));
     pb.pw.alloc((size_t)pb.n_packed * total * pb.tsize());
-    if (pb.precision == 64)
-        pack_kernel<double><<<div_up(total, 256), 256, 0, pb.st>>>(pb.w64.p, pb.idx.p, pb.n_prog, pb.n, nops, pb.diff,
-                                                                   pb.n_slots, pb.SLQ, pb.G, pb.V, pb.n_packed,
-                                                                   dcomb.p, (double *)pb.pw.p, pb.pidx.p);
-    else
+    if (pb.precision == 64) {
+        pb.wexp.alloc(pb.n_prog);
+        pack_fixed_kernel<<<div_up(pb.n_prog, 8), 256, 0, pb.st>>>(pb.w64.p, pb.idx.p, pb.n_prog, pb.n, nops, pb.diff,
+                                                                   pb.n_slots, pb.SLQ, pb.G, dcomb.p, (int2 *)pb.pw.p,
+                                                                   pb.pidx.p, pb.wexp.p);
+    } else
         pack_kernel<float><<<div_up(total, 256), 256, 0, pb.st>>>(pb.w64.p, pb.idx.p, pb.n_prog, pb.n, nops, pb.diff,
                                                                   pb.n_slots, pb.SLQ, pb.G, pb.V, pb.n_packed,
                                                                   dcomb.p, (float *)pb.pw.p, pb.pidx.p);
@@ -638,13 +772,13 @@ void enqueue_rhs(Problem &pb, double t, void *U, void *dUdt, cudaStream_t s) {
             a.Uin = (const double *)U;
             a.dUdt = (double *)dUdt;
             a.stage = -1;
-            launch_ns<double>(a, pb.G, pb.pf, s, false);
+            launch_ns(a, pb.G, pb.pf, s, false);
         } else {
             NSArgs<float> a = ns_args<float>(pb);
             a.Uin = (const float *)U;
             a.dUdt = (float *)dUdt;
             a.stage = -1;
-            launch_ns<float>(a, pb.G, pb.pf, s, false);
+            launch_ns(a, pb.G, pb.pf, s, false);
         }
     } else {
         if (pb.precision == 64) {
@@ -687,7 +821,7 @@ void autotune_threads_per_node(Problem &pb) {
         pb.G = G;
         pack_operators(pb);
         for (int pf : {0, kPrefetchVec}) {
-            if (pf > 0 && (pb.kind != kNS || pb.SLQ > kPrefetchVec || pb.lat.enabled)) continue;
+            if (pf > 0 && (pb.kind != kNS || pb.precision == 64 || pb.SLQ > kPrefetchVec || pb.lat.enabled)) continue;
             pb.pf = pf;
             float ms = 1e30f;
             for (int rep = 0; rep < 3; ++rep) {

@@ -44,6 +44,7 @@
 #include <cstring>
 #include <vector>
 
+#include "fixdot.cuh"
 #include "problem.cuh"
 #include "records.cuh"
 
@@ -64,9 +65,8 @@ struct PV<float> {
 template <>
 struct PV<double> {
     static constexpr int V = 2;
-    using W = double2;
+    using W = int4;   // two fixed-point weights (fixdot.cuh)
     using L = ushort2;
-    __device__ static double at(const double2 &v, int k) { return k == 0 ? v.x : v.y; }
     __device__ static int at(const ushort2 &v, int k) { return k == 0 ? v.x : v.y; }
 };
 
@@ -97,6 +97,7 @@ __device__ __forceinline__ Rec<double> sh_rec(const double *S, int j) {
     const double2 b = reinterpret_cast<const double2 *>(S)[2 * j + 1];
     return {a.x, a.y, b.x, b.y};
 }
+__device__ __forceinline__ int4 sh_half(const double *S, int h) { return reinterpret_cast<const int4 *>(S)[h]; }
 __device__ __forceinline__ void sh_store(float *S, int j, const Rec<float> &r) {
     reinterpret_cast<float4 *>(S)[j] = make_float4(r.u, r.w, r.t, r.p);
 }
@@ -234,7 +235,8 @@ __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~size_t(
 template <class T>
 struct PArgs {
     T *U, *S0, *S1;                 // node-major records [n_all][4]
-    const T *pw;                    // [4][SLQ][lanes][G][V], lanes = grid * chunk
+    const T *pw;                    // [4][SLQ][lanes][G][V], lanes = grid * chunk (FP64: fixed-point pairs)
+    const short4 *wexp;             // FP64: row exponents of each node
     const uint16_t *lidx;           // [SLQ][lanes][G][V]
     const int32_t *hlist;
     const CtaInfo *cta;
@@ -243,6 +245,7 @@ struct PArgs {
     const unsigned char *flags;
     int64_t lanes, total;           // total = SLQ * lanes * G * V
     int SLQ, chunk, npad;
+    unsigned ring_off;              // FP64: byte offset of the operands' ring (0: streamed without)
     T cp_tb2, gconst;
     T cp, g_over_tb, theta_bar, dpibar, rd_cv;
     T an0, an1, an2, bs0, bs1, bs2, bs3;
@@ -466,7 +469,9 @@ __global__ void __launch_bounds__(MAXT, 1) rk4_persistent(const __grid_constant_
     using W = typename P::W;
     using L = typename P::L;
     constexpr int V = P::V;
-    constexpr bool DIFF = sizeof(T) == 4;   // FP32: difference form (self slot dropped)
+    constexpr bool FIX = sizeof(T) == 8;   // FP64: fixed-point sums on the integer units (fixdot.cuh)
+    constexpr int H = FIX ? 2 : 1;         // threads per lane
+    constexpr int NF = FIX ? 2 : 4;        // fields a thread steps
     extern __shared__ __align__(16) unsigned char smem_raw[];
 
     const CtaInfo ci = a.cta[blockIdx.x];
@@ -543,7 +548,9 @@ __global__ void __launch_bounds__(MAXT, 1) rk4_persistent(const __grid_constant_
     }
     const float *sD = reinterpret_cast<const float *>(mreg + ML.d);   // corrections of the own nodes
 
-    const int li = threadIdx.x / G, g = threadIdx.x % G;
+    // FP64: two threads per lane, h = 0 for the fields u, w and 1 for theta', pi'
+    const int lane = threadIdx.x / H, h = threadIdx.x % H;
+    const int li = lane / G, g = lane % G;
     const bool live = li < ci.n_own;
     const int self = live ? li : 0;            // idle lanes mirror the first node
     const int64_t i = __ldg(hl + self);
@@ -558,6 +565,15 @@ __global__ void __launch_bounds__(MAXT, 1) rk4_persistent(const __grid_constant_
     const W *wd = reinterpret_cast<const W *>(a.pw + 2 * a.total);
     const W *wh = reinterpret_cast<const W *>(a.pw + 3 * a.total);
     const L *lx = reinterpret_cast<const L *>(a.lidx);
+    // FP64: the operands' ring behind the CTA's other shared memory
+    int4 *const ring = reinterpret_cast<int4 *>(smem_raw + a.ring_off);
+    FixFetch<false> fetch;
+    const FixStream fs = {reinterpret_cast<const int4 *>(wx + off0), a.total / V, nullptr, stride, 0, a.SLQ};
+    if (FIX && a.ring_off) {
+        fetch.start(fs, ring, blockDim.x >> 1);
+        fetch.copy(0);
+        fetch.copy(1);
+    }
     constexpr int RR = R > 0 ? R : 1;
     L jr[RR];
     W rx[RR], rz[RR], rd[RR], rh[RR];
@@ -575,14 +591,21 @@ __global__ void __launch_bounds__(MAXT, 1) rk4_persistent(const __grid_constant_
         }
     }
     const T pib = __ldg(a.pibar + i);
+    short4 ew = make_short4(0, 0, 0, 0);
+    if (sizeof(T) == 8) ew = __ldg(a.wexp + i);
     const unsigned char fl = __ldg(a.flags + i);
-    T un[4], K[4] = {0, 0, 0, 0};
+    T un[NF], K[NF] = {};
     {
         const Rec<T> r0 = ld_rec_cg(a.U, i);
-        un[0] = r0.u; un[1] = r0.w; un[2] = r0.t; un[3] = r0.p;
+        if constexpr (FIX) {
+            un[0] = h ? r0.t : r0.u;
+            un[1] = h ? r0.p : r0.w;
+        } else {
+            un[0] = r0.u; un[1] = r0.w; un[2] = r0.t; un[3] = r0.p;
+        }
     }
     unsigned target = a.base, target2 = a.base2;
-    T o4[4] = {0, 0, 0, 0};   // the node's latest stage output
+    T o4[NF] = {};   // the node's latest stage output (its fields of this thread)
     const int32_t *ogp = reinterpret_cast<const int32_t *>(blob + ci.o_ogp);
     const int32_t *brow = reinterpret_cast<const int32_t *>(blob + ci.o_brow);
 
@@ -596,7 +619,10 @@ __global__ void __launch_bounds__(MAXT, 1) rk4_persistent(const __grid_constant_
             // group: the residuals and the ghost solve start once they have
             // landed, while the rest of the list is still in flight.
             const bool first = step == 0 && st == 0;
-            if (!first && live && g == 0) sh_store(halo, li, Rec<T>{o4[0], o4[1], o4[2], o4[3]});
+            if (!first && live && g == 0) {
+                if constexpr (FIX) reinterpret_cast<double2 *>(halo)[2 * li + h] = make_double2(o4[0], o4[1]);
+                else sh_store(halo, li, Rec<T>{o4[0], o4[1], o4[2], o4[3]});
+            }
             if (first) {
                 cp_async_wait();   // the constant block and the records issued at entry
             } else {
@@ -720,59 +746,111 @@ __global__ void __launch_bounds__(MAXT, 1) rk4_persistent(const __grid_constant_
                 if (st == 0) mlp_phase(a, halo, hl, ML, mreg, ci.n_own, NB);
             }
             // ---- stencil sums, tendencies, RK4 update ----------------------------
-            Rec<T> fi = {0, 0, 0, 0};
-            if (DIFF) fi = sh_rec(halo, self);
-            T ux = 0, uz = 0, ud = 0, wx_ = 0, wz_ = 0, wd_ = 0, tx = 0, tz = 0, td = 0, px = 0, pz = 0, ph = 0;
-            auto vec = [&](const L &jv, const W &cx, const W &cz, const W &cd, const W &ch) {
-#pragma unroll
-                for (int v = 0; v < V; ++v) {
-                    Rec<T> r = sh_rec(halo, P::at(jv, v));
-                    if (DIFF) { r.u -= fi.u; r.w -= fi.w; r.t -= fi.t; r.p -= fi.p; }
-                    const T x = P::at(cx, v), z = P::at(cz, v), d = P::at(cd, v), hh = P::at(ch, v);
-                    ux += x * r.u; uz += z * r.u; ud += d * r.u;
-                    wx_ += x * r.w; wz_ += z * r.w; wd_ += d * r.w;
-                    tx += x * r.t; tz += z * r.t; td += d * r.t;
-                    px += x * r.p; pz += z * r.p; ph += hh * r.p;
+            T k[NF];
+            const Rec<T> fi = sh_rec(halo, self);
+            if constexpr (FIX) {
+                FixLargest top;
+#pragma unroll 4
+                for (int q = 0; q < a.SLQ; ++q) {
+                    const L j = __ldg(lx + off0 + q * stride);
+                    top.take(sh_half(halo, 2 * j.x + h));
+                    top.take(sh_half(halo, 2 * j.y + h));
                 }
-            };
-            if (R > 0) {
-#pragma unroll
-                for (int q = 0; q < RR; ++q)
-                    if (q < a.SLQ) vec(jr[q], rx[q], rz[q], rd[q], rh[q]);
-            } else {
+                top.over_lanes<G>();
+                FixHalf f;
+                f.a.start(top.a);
+                f.b.start(top.b);
                 int64_t off = off0;
-#pragma unroll 2
-                for (int q = 0; q < a.SLQ; ++q, off += stride)
-                    vec(__ldg(lx + off), __ldg(wx + off), __ldg(wz + off), __ldg(wd + off), __ldg(wh + off));
-            }
+                if (a.ring_off) {
+                    // operands two steps ahead through the pair's ring slots (fixdot.cuh)
+                    const int4 *v = ring + (threadIdx.x >> 1);
+                    const int np = blockDim.x >> 1;
+                    L j = __ldg(lx + off);
+#pragma unroll 1
+                    for (int q0 = 0; q0 < a.SLQ; q0 += kFixRing) {
 #pragma unroll
-            for (int o = G / 2; o > 0; o >>= 1) {
-                ux += __shfl_xor_sync(0xffffffffu, ux, o, G);
-                uz += __shfl_xor_sync(0xffffffffu, uz, o, G);
-                ud += __shfl_xor_sync(0xffffffffu, ud, o, G);
-                wx_ += __shfl_xor_sync(0xffffffffu, wx_, o, G);
-                wz_ += __shfl_xor_sync(0xffffffffu, wz_, o, G);
-                wd_ += __shfl_xor_sync(0xffffffffu, wd_, o, G);
-                tx += __shfl_xor_sync(0xffffffffu, tx, o, G);
-                tz += __shfl_xor_sync(0xffffffffu, tz, o, G);
-                td += __shfl_xor_sync(0xffffffffu, td, o, G);
-                px += __shfl_xor_sync(0xffffffffu, px, o, G);
-                pz += __shfl_xor_sync(0xffffffffu, pz, o, G);
-                ph += __shfl_xor_sync(0xffffffffu, ph, o, G);
+                        for (int u = 0; u < kFixRing; ++u) {
+                            if (q0 + u >= a.SLQ) break;
+                            const int4 r0 = sh_half(halo, 2 * j.x + h), r1 = sh_half(halo, 2 * j.y + h);
+                            off += stride;
+                            if (q0 + u + 1 < a.SLQ) j = __ldg(lx + off);
+                            fetch.copy((u + 2) % kFixRing);
+                            asm volatile("cp.async.wait_group 2;" ::: "memory");
+                            __syncwarp();   // the other thread's vectors of this step
+                            const int4 *w = v + 4 * u * np;
+                            f.slots(r0, r1, w[0], w[np], w[2 * np], w[(2 + h) * np]);
+                        }
+                    }
+                    __syncwarp();   // every slot has been read
+                    fetch.start(fs, ring, np);
+                    fetch.copy(0);   // the next stage's first steps
+                    fetch.copy(1);
+                } else {
+                    const W *we = h ? wh : wd;
+#pragma unroll 2
+                    for (int q = 0; q < a.SLQ; ++q, off += stride) {
+                        const L j = __ldg(lx + off);
+                        f.slots(sh_half(halo, 2 * j.x + h), sh_half(halo, 2 * j.y + h), __ldg(wx + off),
+                                __ldg(wz + off), __ldg(wd + off), __ldg(we + off));
+                    }
+                }
+                const HalfSums sums = fix_finish<G>(f, ew, h);
+                const double2 kk = fix_tendency(sums, {a.cp, a.g_over_tb, a.theta_bar, a.dpibar, a.rd_cv}, h,
+                                                make_double4(fi.u, fi.w, fi.t, fi.p), pib, fl);
+                k[0] = kk.x;
+                k[1] = kk.y;
+            } else {
+                // FP32: difference form (self slot dropped)
+                T ux = 0, uz = 0, ud = 0, wx_ = 0, wz_ = 0, wd_ = 0, tx = 0, tz = 0, td = 0, px = 0, pz = 0, ph = 0;
+                auto vec = [&](const L &jv, const W &cx, const W &cz, const W &cd, const W &ch) {
+#pragma unroll
+                    for (int v = 0; v < V; ++v) {
+                        Rec<T> r = sh_rec(halo, P::at(jv, v));
+                        r.u -= fi.u; r.w -= fi.w; r.t -= fi.t; r.p -= fi.p;
+                        const T x = P::at(cx, v), z = P::at(cz, v), d = P::at(cd, v), hh = P::at(ch, v);
+                        ux += x * r.u; uz += z * r.u; ud += d * r.u;
+                        wx_ += x * r.w; wz_ += z * r.w; wd_ += d * r.w;
+                        tx += x * r.t; tz += z * r.t; td += d * r.t;
+                        px += x * r.p; pz += z * r.p; ph += hh * r.p;
+                    }
+                };
+                if (R > 0) {
+#pragma unroll
+                    for (int q = 0; q < RR; ++q)
+                        if (q < a.SLQ) vec(jr[q], rx[q], rz[q], rd[q], rh[q]);
+                } else {
+                    int64_t off = off0;
+#pragma unroll 2
+                    for (int q = 0; q < a.SLQ; ++q, off += stride)
+                        vec(__ldg(lx + off), __ldg(wx + off), __ldg(wz + off), __ldg(wd + off), __ldg(wh + off));
+                }
+#pragma unroll
+                for (int o = G / 2; o > 0; o >>= 1) {
+                    ux += __shfl_xor_sync(0xffffffffu, ux, o, G);
+                    uz += __shfl_xor_sync(0xffffffffu, uz, o, G);
+                    ud += __shfl_xor_sync(0xffffffffu, ud, o, G);
+                    wx_ += __shfl_xor_sync(0xffffffffu, wx_, o, G);
+                    wz_ += __shfl_xor_sync(0xffffffffu, wz_, o, G);
+                    wd_ += __shfl_xor_sync(0xffffffffu, wd_, o, G);
+                    tx += __shfl_xor_sync(0xffffffffu, tx, o, G);
+                    tz += __shfl_xor_sync(0xffffffffu, tz, o, G);
+                    td += __shfl_xor_sync(0xffffffffu, td, o, G);
+                    px += __shfl_xor_sync(0xffffffffu, px, o, G);
+                    pz += __shfl_xor_sync(0xffffffffu, pz, o, G);
+                    ph += __shfl_xor_sync(0xffffffffu, ph, o, G);
+                }
+                const T cpth = a.cp * (a.theta_bar + fi.t);
+                k[0] = -fi.u * ux - fi.w * uz - cpth * px + ud;
+                k[1] = -fi.u * wx_ - fi.w * wz_ - cpth * pz + a.g_over_tb * fi.t + wd_;
+                k[2] = -fi.u * tx - fi.w * tz + td;
+                k[3] = -fi.u * px - fi.w * (a.dpibar + pz) - a.rd_cv * (pib + fi.p) * (ux + wz_) + ph;
+                if (fl & 1) k[1] = 0;   // w = 0 held on bottom/top walls
+                if (fl & 2) k[0] = 0;   // u = 0 held on left/right walls
             }
-            const Rec<T> cr = DIFF ? fi : sh_rec(halo, self);
-            const T cpth = a.cp * (a.theta_bar + cr.t);
-            T k[4];
-            k[0] = -cr.u * ux - cr.w * uz - cpth * px + ud;
-            k[1] = -cr.u * wx_ - cr.w * wz_ - cpth * pz + a.g_over_tb * cr.t + wd_;
-            k[2] = -cr.u * tx - cr.w * tz + td;
-            k[3] = -cr.u * px - cr.w * (a.dpibar + pz) - a.rd_cv * (pib + cr.p) * (ux + wz_) + ph;
-            if (fl & 1) k[1] = 0;   // w = 0 held on bottom/top walls
-            if (fl & 2) k[0] = 0;   // u = 0 held on left/right walls
             const T an = st == 0 ? a.an0 : st == 1 ? a.an1 : a.an2;
             const T bs = st == 0 ? a.bs0 : st == 1 ? a.bs1 : st == 2 ? a.bs2 : a.bs3;
 #pragma unroll
-            for (int f = 0; f < 4; ++f) {
+            for (int f = 0; f < NF; ++f) {
                 const T kf = k[f];
                 if (st == 0) {
                     K[f] = bs * kf;
@@ -798,9 +876,12 @@ __global__ void __launch_bounds__(MAXT, 1) rk4_persistent(const __grid_constant_
             }
             if (st == 3) {
 #pragma unroll
-                for (int f = 0; f < 4; ++f) un[f] = o4[f];
+                for (int f = 0; f < NF; ++f) un[f] = o4[f];
             }
-            if (live && g == 0) st_rec(Uout, i, Rec<T>{o4[0], o4[1], o4[2], o4[3]});
+            if (live && g == 0) {
+                if constexpr (FIX) reinterpret_cast<double2 *>(Uout)[2 * i + h] = make_double2(o4[0], o4[1]);
+                else st_rec(Uout, i, Rec<T>{o4[0], o4[1], o4[2], o4[3]});
+            }
             const bool last = step + 1 == a.n_steps && st == 3;
             if (!last && !grid_barrier(a.arrive, a.abort, target, a.spin_limit)) return;
         }
@@ -929,7 +1010,10 @@ std::vector<Variant> variants() {
                 {4, 0, 512, true, (void *)rk4_persistent<float, 4, 0, 512, true>}};
     } else {
         return {{1, 0, 512, false, (void *)rk4_persistent<double, 1, 0, 512, false>},
+                {1, 0, 1024, false, (void *)rk4_persistent<double, 1, 0, 1024, false>},
                 {2, 0, 512, false, (void *)rk4_persistent<double, 2, 0, 512, false>},
+                {2, 0, 1024, false, (void *)rk4_persistent<double, 2, 0, 1024, false>},
+                {4, 0, 512, false, (void *)rk4_persistent<double, 4, 0, 512, false>},
                 {4, 0, 1024, false, (void *)rk4_persistent<double, 4, 0, 1024, false>}};
     }
 }
@@ -942,6 +1026,7 @@ PArgs<T> pargs(Problem &pb, T *U, double dt, int64_t n_steps) {
     a.S0 = (T *)pb.S0.p;
     a.S1 = (T *)pb.S1.p;
     a.pw = (const T *)ps.pw.p;
+    a.wexp = pb.wexp.p;
     a.lidx = ps.lidx.p;
     a.hlist = ps.hlist.p;
     a.cta = (const CtaInfo *)ps.cta.p;
@@ -949,10 +1034,11 @@ PArgs<T> pargs(Problem &pb, T *U, double dt, int64_t n_steps) {
     a.pibar = (const T *)pb.pibar.p;
     a.flags = pb.flags.p;
     a.lanes = (int64_t)ps.grid * ps.chunk;
-    a.total = (int64_t)ps.SLQ * a.lanes * ps.G * ps.V;
+    a.total = (int64_t)ps.SLQ * a.lanes * ps.S * ps.V;
     a.SLQ = ps.SLQ;
     a.chunk = ps.chunk;
     a.npad = pb.gh.npad;
+    a.ring_off = ps.ring_off;
     a.cp_tb2 = (T)(pb.cp * pb.theta_bar * pb.theta_bar);
     a.gconst = (T)pb.g;
     a.cp = (T)pb.cp;
@@ -985,7 +1071,7 @@ PArgs<T> pargs(Problem &pb, T *U, double dt, int64_t n_steps) {
 void *variant_fn(const PersistPlan &ps, int precision) {
     const std::vector<Variant> v = precision == 64 ? variants<double>() : variants<float>();
     for (const Variant &x : v)
-        if (!x.mlp && x.G == ps.G && x.R == ps.R && x.maxt == ps.maxt) return x.fn;
+        if (!x.mlp && x.G == ps.S && x.R == ps.R && x.maxt == ps.maxt) return x.fn;
     return nullptr;
 }
 
@@ -993,7 +1079,7 @@ void *variant_fn(const PersistPlan &ps, int precision) {
 void *mlp_variant_fn(const PersistPlan &ps, int precision) {
     if (precision != 32) return nullptr;
     for (const Variant &x : variants<float>())
-        if (x.mlp && x.G == ps.G && x.R == ps.R && ps.threads <= x.maxt) return x.fn;
+        if (x.mlp && x.G == ps.S && x.R == ps.R && ps.threads <= x.maxt) return x.fn;
     return nullptr;
 }
 
@@ -1047,7 +1133,12 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
     const int64_t P = pb.n_prog;
     const int grid = (int)std::min<int64_t>(ctas > 0 ? ctas : nsm, P);
     const int chunk = div_up(P, grid) + 1;   // bisection blocks differ by at most one node
-    const int threads = div_up((int64_t)chunk * G, 32) * 32;
+    // Slot lanes per node.  FP64 uses two threads per lane; its sums do not
+    // depend on the number of lanes, so 4 lanes become 2 where 8 threads per
+    // node would not fit a CTA.
+    const bool fp64 = pb.precision == 64;
+    const int S = fp64 && G == 4 && chunk * 8 > 1024 ? 2 : G;
+    const int threads = div_up((int64_t)chunk * S * (fp64 ? 2 : 1), 32) * 32;
     if (threads > 1024) return false;
     RBF_CUDA(cudaStreamSynchronize(pb.st));
 
@@ -1069,7 +1160,7 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
     std::vector<unsigned char> hw;
     int SLQ = 0, V = 0;
     try {
-        pb.G = G;
+        pb.G = S;
         pack_operators(pb);
         hp = to_host(pb.pidx);
         hw = to_host(pb.pw);
@@ -1081,7 +1172,7 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
     }
     restore();
     const size_t ts = pb.tsize();
-    const int GV = G * V;                       // slots of one node per operand vector
+    const int GV = S * V;                       // slots of one node per operand vector
 
     // ---- blocks -----------------------------------------------------------------
     std::vector<double> x(P), z(P);
@@ -1373,13 +1464,22 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
         smem_max = std::max(smem_max, sm);
     }
     if (smem_max > (size_t)smem_optin) return false;
+    // FP64: room for the operands' ring, where shared memory has it
+    unsigned ring_off = 0;
+    if (fp64) {
+        const size_t ring = (size_t)kFixRing * 4 * sizeof(int4) * (threads / 2);
+        if (align16(smem_max) + ring + 1024 <= (size_t)smem_optin) {   // beside the kernel's static words
+            ring_off = (unsigned)align16(smem_max);
+            smem_max = ring_off + ring;
+        }
+    }
 
     // ---- kernel variant: operators in registers when they fit ----------------------
     const std::vector<Variant> vs = pb.precision == 64 ? variants<double>() : variants<float>();
     int pick = -1;
     for (int k = 0; k < (int)vs.size(); ++k) {
         const Variant &v = vs[k];
-        if (v.mlp || v.G != G || threads > v.maxt) continue;
+        if (v.mlp || v.G != S || threads > v.maxt) continue;
         if (v.R > 0 && SLQ > v.R) continue;
         if (pick < 0 || (v.R > 0 && vs[pick].R == 0)) pick = k;
     }
@@ -1390,6 +1490,7 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
     if ((int64_t)per_sm * nsm < grid) return false;
 
     ps.G = G;
+    ps.S = S;
     ps.SLQ = SLQ;
     ps.V = V;
     ps.R = vs[pick].R;
@@ -1400,6 +1501,7 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
     ps.halo_max = halo_max;
     ps.rows_max = rows_max;
     ps.smem = smem_max;
+    ps.ring_off = ring_off;
     ps.pw.alloc(pwp.size());
     ps.lidx.alloc(lidx.size());
     ps.hlist.alloc(hlist.size());

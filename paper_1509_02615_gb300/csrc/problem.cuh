@@ -79,6 +79,7 @@ void build_ghost_bands(GhostPlan &gh, int precision, cudaStream_t st);
 struct PersistPlan {
     bool ready = false;
     int G = 0;                   // lanes per node
+    int S = 0;                   // slot lanes per node of the kernel (FP64: two threads each)
     int R = 0;                   // operand vectors held in registers (0: read each stage)
     int maxt = 0;                // thread limit of the kernel variant
     int SLQ = 0, V = 0;          // packing of pw / lidx (as Problem::SLQ, V)
@@ -87,8 +88,9 @@ struct PersistPlan {
     int halo_max = 0;            // largest record list
     int rows_max = 0;            // most ghost rows one CTA solves
     size_t smem = 0;
-    DevBuf<unsigned char> pw;    // T [4][SLQ][grid * chunk][G][V]
-    DevBuf<uint16_t> lidx;       // [SLQ][grid * chunk][G][V] list position of each slot
+    unsigned ring_off = 0;       // FP64: where the operands' ring starts in it (0: none)
+    DevBuf<unsigned char> pw;    // T [4][SLQ][grid * chunk][S][V], as Problem::pw
+    DevBuf<uint16_t> lidx;       // [SLQ][grid * chunk][S][V] list position of each slot
     DevBuf<int32_t> hlist;       // record lists of all CTAs
     DevBuf<unsigned char> cta;   // per-CTA layout records
     DevBuf<unsigned char> blob;  // per-CTA ghost-row and ghost-value data
@@ -142,7 +144,9 @@ struct Problem {
     // packed operators, precision T
     int n_packed = 4;
     DevBuf<int32_t> pidx;         // [SLQ][n_prog][G][V]
-    DevBuf<unsigned char> pw;     // T [n_packed][SLQ][n_prog][G][V]
+    DevBuf<unsigned char> pw;     // T [n_packed][SLQ][n_prog][G][V]; NS in FP64: fixed-point
+                                  // pairs int2 (fixdot.cuh) in place of the doubles
+    DevBuf<short4> wexp;          // [n_prog] NS in FP64: exponents of the packed rows
     DevBuf<unsigned char> pibar;  // T [n_prog]
     DevBuf<unsigned char> flags;  // [n_prog]: bit0 w Dirichlet, bit1 u Dirichlet, bit2 wall set
 
@@ -189,7 +193,8 @@ struct Problem {
         std::vector<double> rep_w;    // [nops][n_cls][n] its FP64 weights
         DevBuf<int32_t> cls;          // [n_prog] class of each node, -1: per-node operators
         DevBuf<int32_t> loff;         // [n_cls][SLQ][G][V] relative index of each slot
-        DevBuf<unsigned char> lw;     // T [4][n_cls][SLQ][G][V] packed operators
+        DevBuf<unsigned char> lw;     // T [4][n_cls][SLQ][G][V] packed operators (FP64: as pw)
+        DevBuf<short4> lexp;          // [n_cls] FP64: exponents of the packed rows
     } lat;
 
     float weight_build_ms = 0.f, ghost_setup_ms = 0.f;
