@@ -732,8 +732,9 @@ void mlp_init(Mlp &m, Problem &pb, void *stream) {
     RBF_CUDA(cudaMemsetAsync(m.V.p, 0, m.V.bytes(), m.st));
     const float ones[12] = {1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1};
     RBF_CUDA(cudaMemcpyAsync(m.scales.p, ones, sizeof(ones), cudaMemcpyHostToDevice, m.st));
+    // the widest network's need: a later, narrower one must not lower the limit
     RBF_CUDA(cudaFuncSetAttribute(mlp_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)train_smem(m.n_in)));
+                                  (int)train_smem(kMaxInputs)));
     RBF_CUDA(cudaStreamSynchronize(m.st));
 }
 

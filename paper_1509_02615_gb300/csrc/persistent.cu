@@ -16,10 +16,10 @@
 // exponentially along the wall (the wall rows couple only nearby ghosts), so
 // each row is kept where its entries exceed 2^-8 eps of the row's largest:
 // the dropped part is below the rounding of the kept sum.  A CTA whose
-// stencils read ghosts forms, from its shared-memory records, the residuals
-// of every wall row in those ghosts' bands, then the ghost values it needs
-// (every field of an operator class at once; the lanes per row and per
-// ghost are chosen so that one pass of the CTA's threads covers them).
+// stencils read ghosts solves for them itself from its shared-memory records:
+// in FP32 straight (ghosts_from_records), in FP64 by the residuals of the wall
+// rows, each formed by the CTA that owns its wall node and passed through
+// global memory, then the banded rows.
 //
 // Learned correction (a9, MLP variants): at stage 0 of every step the CTA's
 // shared memory holds the step-start records of its stencils, ghosts
@@ -36,7 +36,7 @@
 // evaluate Eqs. (uEq)-(piEq) and the RK4 update for its nodes, write them,
 // and meet every other CTA at a grid barrier.  Every barrier wait is
 // bounded: after spin_limit polls a CTA raises the abort flag, every CTA
-// leaves at its next barrier, and the host reports RBF_E_TIMEOUT.
+// leaves at a later barrier, and the host reports RBF_E_TIMEOUT.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -147,45 +147,28 @@ __device__ __forceinline__ void st_relaxed(int *p, int v) {
     asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// Grid barrier with a bounded wait.  `target` counts the arrivals expected
-// so far (gridDim.x per barrier on top of the counter's value at launch; the
-// comparison tolerates wrap-around, so the counter is never reset between
-// launches).  Returns false if this or another CTA gave up; the caller then
-// returns.
+// Barrier among `members` CTAs (the whole grid, or the CTAs that solve ghosts;
+// the others never call it) with a bounded wait.  `target` counts the arrivals
+// expected so far (`members` per barrier on top of the counter's value at
+// launch; the comparison tolerates wrap-around, so the counter is never reset
+// between launches).  Returns false if this or another CTA gave up; the caller
+// then returns.
 //
 // Ordering: the CTA barrier orders every thread's stage outputs before
 // thread 0's arrival, a release add at gpu scope; the poll that sees the last
 // arrival is an acquire at gpu scope, and the closing CTA barrier orders it
 // before every thread's next reads.  Release and acquire are cumulative
 // through the CTA barriers, so no separate fences are needed.
-__device__ bool grid_barrier(unsigned *arrive, int *abort, unsigned &target, long long limit) {
+//
+// What bounds it: round trips to L2 (about 700 clocks each).  A poll is one;
+// the abort flag is read every 16th poll only, not beside each poll and once
+// more after the last, so that a CTA that sees every arrival goes on even if
+// another one gave up: it leaves at a later barrier, where that one is missing.
+// On 38 balanced CTAs a barrier takes 2,550 clocks (940 until the stores before
+// the release are acknowledged, then polls); with the flag read beside each poll
+// and 32 ns of sleep between polls it took 3,200.
+__device__ bool cta_barrier(unsigned *arrive, int *abort, unsigned &target, unsigned members, long long limit) {
     __shared__ int s_ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        target += gridDim.x;
-        red_release_add(arrive, 1u);
-        int ok = 1;
-        long long polls = 0;
-        while ((int)(ld_acquire(arrive) - target) < 0) {
-            if (ld_relaxed(abort)) { ok = 0; break; }
-            if (++polls > limit) {
-                st_relaxed(abort, 1);
-                ok = 0;
-                break;
-            }
-            __nanosleep(32);
-        }
-        if (ok && ld_relaxed(abort)) ok = 0;
-        s_ok = ok;
-    }
-    __syncthreads();
-    return s_ok != 0;
-}
-
-// Barrier among `members` CTAs only (the others never call it), with the same
-// bounded wait and abort protocol as grid_barrier.
-__device__ bool group_barrier(unsigned *arrive, int *abort, unsigned &target, unsigned members, long long limit) {
-    __shared__ int s_ok2;
     __syncthreads();
     if (threadIdx.x == 0) {
         target += members;
@@ -193,19 +176,20 @@ __device__ bool group_barrier(unsigned *arrive, int *abort, unsigned &target, un
         int ok = 1;
         long long polls = 0;
         while ((int)(ld_acquire(arrive) - target) < 0) {
-            if (ld_relaxed(abort)) { ok = 0; break; }
             if (++polls > limit) {
                 st_relaxed(abort, 1);
                 ok = 0;
                 break;
             }
-            __nanosleep(32);
+            if ((polls & 15) == 0 && ld_relaxed(abort)) {
+                ok = 0;
+                break;
+            }
         }
-        if (ok && ld_relaxed(abort)) ok = 0;
-        s_ok2 = ok;
+        s_ok = ok;
     }
     __syncthreads();
-    return s_ok2 != 0;
+    return s_ok != 0;
 }
 
 // Layout of one CTA's block (host-built, identical on both sides).
@@ -220,7 +204,7 @@ struct CtaInfo {
     int32_t n_crows;    // wall rows whose residuals it forms: the band rows, or in
                         // owned-rows mode the rows of its own wall nodes
     int32_t o_ogp, o_brow;   // owned-rows mode: global row of each formed row, of each band row
-    int32_t n_gc;       // (ghost, operator class) pairs it solves
+    int32_t n_gc;       // (ghost, field) items it solves
     int32_t n_set;      // weight sets per wall row
     int32_t n_coef;     // band coefficients of all its pairs
     int32_t row_pad;    // row stride of the slot-major row arrays (bank-conflict free)
@@ -228,6 +212,21 @@ struct CtaInfo {
     int64_t blob_off;   // byte offset of its constant block
     int32_t blob_bytes;
     int32_t o_rw, o_rinfo, o_gc, o_cidx, o_cval;   // sections of the block (row slots at 0)
+    // FP32: ghost values straight from the records (n_gh > 0; the row sections
+    // above are then empty): pairs of ghosts at 0, list positions, coefficients
+    int32_t n_gh, o_pos, o_comp;
+    int32_t n_hy, o_hy, o_b;   // hydrostatic wall nodes of all pairs (records), their b of the stage
+};
+
+constexpr int kGhostPad = 96;   // three records for each lane of a warp
+
+// Two ghosts of a CTA (FP32): the records they read and their coefficients.
+struct GhostPair {
+    int32_t pos, n_j;      // first list position, number of records (a multiple of kGhostPad)
+    int32_t comp;          // coefficients [class][2][n_j]
+    int32_t tb, n_tb;      // hydrostatic wall nodes in their bands (index among the CTA's) and
+    int32_t binv;          // the inverse rows' entries there [2][n_tb]
+    int32_t unused[2];
 };
 
 __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~size_t(15); }
@@ -246,7 +245,8 @@ struct PArgs {
     int64_t lanes, total;           // total = SLQ * lanes * G * V
     int SLQ, chunk, npad;
     unsigned ring_off;              // FP64: byte offset of the operands' ring (0: streamed without)
-    T cp_tb2, gconst;
+    T cp_tb2, cp_tb, gconst;        // c_p theta_bar^2, c_p theta_bar, g
+    int4 field_class;               // boundary-operator class of each field
     T cp, g_over_tb, theta_bar, dpibar, rd_cv;
     T an0, an1, an2, bs0, bs1, bs2, bs3;
     int64_t n_steps;
@@ -365,8 +365,10 @@ __device__ __forceinline__ void mma_layer(const __nv_bfloat16 *xh, const __nv_bf
     }
 }
 
-constexpr int kRowLanes = 8;    // most lanes per wall row in the residuals
-constexpr int kPairLanes = 8;   // most lanes per (ghost, class) pair in the ghost values
+// most lanes per wall row in the residuals: an FP64 instruction of a warp takes
+// 16 clocks of the SM's FP64 pipe, so its lane reductions are kept short
+__host__ __device__ constexpr int row_lanes(bool fp64) { return fp64 ? 4 : 8; }
+constexpr int kPairLanes = 8;   // most lanes per (ghost, field) item in the ghost values
 
 // Lanes per item: the largest power of two up to `most` with items * lanes
 // within one pass of the CTA's threads (at least one lane).
@@ -374,6 +376,106 @@ __host__ __device__ __forceinline__ int lanes_for(int items, int threads, int mo
     int l = most;
     while (l > 1 && items * l > threads) l >>= 1;
     return l;
+}
+
+// FP32: the CTA's ghost values from its records in one step.  The solve
+// u_G = W_G^{-1} (b - W_I u_I - W_B u_B) is linear in the records apart from b,
+// so the plan holds per ghost and operator class the products of its banded
+// inverse row with the wall rows' weights (in FP64, rounded once), one
+// coefficient per record that any of its rows reads; the pi' rows'
+// hydrostatic b enters with the inverse row itself.  A warp takes two ghosts,
+// its lanes the records.  The two-step form (residuals of every wall row in
+// the bands, a CTA barrier, the banded rows) took 3,680 of a stage's 11,700
+// clocks in the 400 m density current (38 CTAs); this one takes 1,750 of 8,700.
+// It stays for FP64, whose coefficients would not fit shared memory.
+//
+// What bounds it: chains of dependent shared-memory reads in few warps.  L lanes
+// take a pair, three records each per pass, so that three chains overlap.
+template <int L>
+__device__ __forceinline__ void ghosts_from_records(const PArgs<float> &a, const CtaInfo &ci, float *halo,
+                                                    const unsigned char *blob) {
+    const GhostPair *pairs = reinterpret_cast<const GhostPair *>(blob);
+    const uint16_t *pos = reinterpret_cast<const uint16_t *>(blob + ci.o_pos);
+    const float *coef = reinterpret_cast<const float *>(blob + ci.o_comp);
+    const float *hydro = reinterpret_cast<const float *>(blob + ci.o_b);
+    const int np = (ci.n_gh + 1) / 2, lane = threadIdx.x & (L - 1), step = blockDim.x / L;
+    const int4 fc = a.field_class;
+    const bool c2 = fc.z != fc.x, c3 = fc.w != fc.z;   // classes of theta', pi' of their own
+    for (int q0 = threadIdx.x / L; (q0 & ~(32 / L - 1)) < np; q0 += step) {   // uniform per warp: it holds 32 / L pairs
+        const int q = min(q0, np - 1);
+        const GhostPair g = pairs[q];
+        const int n_j = g.n_j;
+        const uint16_t *J = pos + g.pos, *tb = pos + g.tb;
+        const float *p0 = coef + g.comp + fc.x * 2 * n_j, *p1 = coef + g.comp + fc.y * 2 * n_j;
+        const float *p2 = coef + g.comp + fc.z * 2 * n_j, *p3 = coef + g.comp + fc.w * 2 * n_j;
+        const float *binv = coef + g.binv;
+        float s[8] = {};   // [ghost][field]
+#pragma unroll 1
+        for (int j0 = lane; j0 < n_j; j0 += 3 * L) {
+#pragma unroll
+            for (int u = 0; u < 3; ++u) {
+                const int j = j0 + u * L;
+                const Rec<float> r = sh_rec(halo, J[j]);
+                float v0 = p0[j], v1 = p0[j + n_j];
+                s[0] += v0 * r.u;
+                s[4] += v1 * r.u;
+                s[1] += p1[j] * r.w;
+                s[5] += p1[j + n_j] * r.w;
+                if (c2) {
+                    v0 = p2[j];
+                    v1 = p2[j + n_j];
+                }
+                s[2] += v0 * r.t;
+                s[6] += v1 * r.t;
+                if (c3) {
+                    v0 = p3[j];
+                    v1 = p3[j + n_j];
+                }
+                s[3] += v0 * r.p;
+                s[7] += v1 * r.p;
+            }
+        }
+#pragma unroll 2
+        for (int r = lane; r < g.n_tb; r += L) {
+            const float b = hydro[tb[r]];
+            s[3] += binv[r] * b;
+            s[7] += binv[g.n_tb + r] * b;
+        }
+        // the eight sums over the lanes: each exchange halves the values a lane holds
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const int o = L >> (k + 1), n = 4 >> k;
+            const bool up = lane & o;
+#pragma unroll
+            for (int v = 0; v < n; ++v) {
+                const float send = up ? s[v] : s[v + n], keep = up ? s[v + n] : s[v];
+                s[v] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+        }
+#pragma unroll
+        for (int k = L / 16; k > 0; k >>= 1) s[0] += __shfl_xor_sync(0xffffffffu, s[0], k);
+        const int v = lane / (L / 8);   // the sum this lane holds: ghost * 4 + field
+        if (q0 < np && lane % (L / 8) == 0 && (v < 4 || 2 * q + 1 < ci.n_gh))
+            halo[(size_t)(ci.n_load + 2 * q + (v >> 2)) * 4 + (v & 3)] = s[0];
+    }
+}
+
+// pi'_z = g theta' / (c_p theta_bar (theta_bar + theta')) at the CTA's
+// hydrostatic wall nodes, from the stage input itself: the first read goes out
+// ahead of the record copies (th0), the division runs while they are in flight
+// (formed per pair of ghosts, the divisions took 650 clocks).
+__device__ __forceinline__ float hydrostatic_read(const CtaInfo &ci, const float *Uin, const unsigned char *blob, int r) {
+    const int32_t *rec = reinterpret_cast<const int32_t *>(blob + ci.o_hy);
+    return r < ci.n_hy ? __ldcg(Uin + (int64_t)rec[r] * 4 + 2) : 0.f;
+}
+__device__ __forceinline__ void hydrostatic(const PArgs<float> &a, const CtaInfo &ci, const float *Uin,
+                                            unsigned char *blob, float th0) {
+    float *b = reinterpret_cast<float *>(blob + ci.o_b);
+    for (int r = threadIdx.x; r < ci.n_hy; r += blockDim.x) {
+        const float th = r < (int)blockDim.x ? th0 : hydrostatic_read(ci, Uin, blob, r);
+        b[r] = a.gconst * th / (a.cp_tb2 + a.cp_tb * th);
+    }
 }
 
 // a9 at stage 0: delta of the CTA's own nodes from the records in shared
@@ -552,6 +654,7 @@ __global__ void __launch_bounds__(MAXT, 1) rk4_persistent(const __grid_constant_
     const int lane = threadIdx.x / H, h = threadIdx.x % H;
     const int li = lane / G, g = lane % G;
     const bool live = li < ci.n_own;
+    const bool busy = __any_sync(0xffffffffu, live);   // the warp has nodes to step
     const int self = live ? li : 0;            // idle lanes mirror the first node
     const int64_t i = __ldg(hl + self);
 
@@ -626,119 +729,126 @@ __global__ void __launch_bounds__(MAXT, 1) rk4_persistent(const __grid_constant_
             if (first) {
                 cp_async_wait();   // the constant block and the records issued at entry
             } else {
+                T th0 = 0;
+                if constexpr (!FIX) {
+                    if (ci.n_gh > 0) th0 = hydrostatic_read(ci, Uin, blob, threadIdx.x);
+                }
                 const int wend = ci.n_own + ci.n_wload;
                 for (int k = ci.n_own + threadIdx.x; k < wend; k += blockDim.x) cp_rec(halo, k, Uin, __ldg(hl + k));
                 cp_async_commit();
                 for (int k = wend + threadIdx.x; k < ci.n_load; k += blockDim.x) cp_rec(halo, k, Uin, __ldg(hl + k));
                 cp_async_commit();
-                if (ci.n_rows > 0 || ci.n_crows > 0) cp_async_wait_pending<1>();
+                if constexpr (!FIX) {
+                    if (ci.n_gh > 0) hydrostatic(a, ci, Uin, blob, th0);
+                }
+                if (ci.n_gh > 0 || ci.n_crows > 0) cp_async_wait_pending<1>();
                 else cp_async_wait_pending<0>();
             }
             __syncthreads();
-            if (ci.n_crows > 0) {
-                // ---- residuals b - W_I u_I - W_B u_B of its wall rows -----------
-                // L lanes per row, L the largest of 8, 4, 2, 1 that lets one pass
-                // of the CTA's threads cover every row
-                const int L = lanes_for(ci.n_crows, blockDim.x, kRowLanes);
-                const int per = a.npad / L;
-                const int nlr = (ci.n_crows * L + 31) & ~31;
-                for (int e = threadIdx.x; e < nlr; e += blockDim.x) {
-                    int r = e / L;
-                    const int ln = e % L;
-                    const bool rl = r < ci.n_crows;
-                    if (!rl) r = ci.n_crows - 1;
-                    const int inf = rinfo[r];
-                    // slot-major [set][slot][row_pad]: the lanes of a warp read
-                    // consecutive rows of one slot
-                    const size_t RP = ci.row_pad, step = (size_t)L * RP;
-                    const T *w0 = rw + ((size_t)((inf >> 17) & 3) * a.npad + ln) * RP + r;
-                    const T *w1 = rw + ((size_t)((inf >> 19) & 3) * a.npad + ln) * RP + r;
-                    const T *w2 = rw + ((size_t)((inf >> 21) & 3) * a.npad + ln) * RP + r;
-                    const T *w3 = rw + ((size_t)((inf >> 23) & 3) * a.npad + ln) * RP + r;
-                    const uint16_t *rj = ridx + (size_t)ln * RP + r;
-                    T a0 = 0, a1 = 0, a2 = 0, a3 = 0;
+            bool solved = false;
+            if constexpr (!FIX) {
+                if (ci.n_gh > 0) {
+                    if (first) {   // the block has only just arrived
+                        hydrostatic(a, ci, Uin, blob, hydrostatic_read(ci, Uin, blob, threadIdx.x));
+                        __syncthreads();
+                    }
+                    // lanes per pair: a warp's, or half or a quarter where one pass
+                    // of the CTA's warps then covers every pair
+                    const int np = (ci.n_gh + 1) / 2;
+                    if (np * 32 <= (int)blockDim.x) ghosts_from_records<32>(a, ci, halo, blob);
+                    else if (np * 16 <= (int)blockDim.x) ghosts_from_records<16>(a, ci, halo, blob);
+                    else ghosts_from_records<8>(a, ci, halo, blob);
+                    __syncthreads();
+                    solved = true;
+                }
+            }
+            if (!solved) {   // FP64, and FP32 CTAs whose coefficients do not fit
+                if (ci.n_crows > 0) {
+                    // ---- residuals b - W_I u_I - W_B u_B of its wall rows -----------
+                    // L lanes per row, L the largest of 8, 4, 2, 1 that lets one pass
+                    // of the CTA's threads cover every row
+                    const int L = lanes_for(ci.n_crows, blockDim.x, row_lanes(FIX));
+                    const int per = a.npad / L;
+                    const int nlr = (ci.n_crows * L + 31) & ~31;
+                    for (int e = threadIdx.x; e < nlr; e += blockDim.x) {
+                        int r = e / L;
+                        const int ln = e % L;
+                        const bool rl = r < ci.n_crows;
+                        if (!rl) r = ci.n_crows - 1;
+                        const int inf = rinfo[r];
+                        // slot-major [set][slot][row_pad]: the lanes of a warp read
+                        // consecutive rows of one slot
+                        const size_t RP = ci.row_pad, step = (size_t)L * RP;
+                        const T *w0 = rw + ((size_t)((inf >> 17) & 3) * a.npad + ln) * RP + r;
+                        const T *w1 = rw + ((size_t)((inf >> 19) & 3) * a.npad + ln) * RP + r;
+                        const T *w2 = rw + ((size_t)((inf >> 21) & 3) * a.npad + ln) * RP + r;
+                        const T *w3 = rw + ((size_t)((inf >> 23) & 3) * a.npad + ln) * RP + r;
+                        const uint16_t *rj = ridx + (size_t)ln * RP + r;
+                        T a0 = 0, a1 = 0, a2 = 0, a3 = 0;
 #pragma unroll 4
-                    for (int t = 0; t < per; ++t) {
-                        const Rec<T> v = sh_rec(halo, rj[t * step]);
-                        a0 += w0[t * step] * v.u;
-                        a1 += w1[t * step] * v.w;
-                        a2 += w2[t * step] * v.t;
-                        a3 += w3[t * step] * v.p;
-                    }
-                    for (int o = L / 2; o > 0; o >>= 1) {
-                        a0 += __shfl_xor_sync(0xffffffffu, a0, o, L);
-                        a1 += __shfl_xor_sync(0xffffffffu, a1, o, L);
-                        a2 += __shfl_xor_sync(0xffffffffu, a2, o, L);
-                        a3 += __shfl_xor_sync(0xffffffffu, a3, o, L);
-                    }
-                    if (rl) {
+                        for (int t = 0; t < per; ++t) {
+                            const Rec<T> v = sh_rec(halo, rj[t * step]);
+                            a0 += w0[t * step] * v.u;
+                            a1 += w1[t * step] * v.w;
+                            a2 += w2[t * step] * v.t;
+                            a3 += w3[t * step] * v.p;
+                        }
+                        for (int o = L / 2; o > 0; o >>= 1) {
+                            a0 += __shfl_xor_sync(0xffffffffu, a0, o, L);
+                            a1 += __shfl_xor_sync(0xffffffffu, a1, o, L);
+                            a2 += __shfl_xor_sync(0xffffffffu, a2, o, L);
+                            a3 += __shfl_xor_sync(0xffffffffu, a3, o, L);
+                        }
+                        if (rl) {
 #pragma unroll
-                        for (int f = 0; f < 4; ++f) {
-                            if (f % L != ln) continue;
-                            const T acc = f == 0 ? a0 : f == 1 ? a1 : f == 2 ? a2 : a3;
-                            T b = 0;
-                            if (f == 3 && (inf & (1 << 16))) {
-                                // pi'_z = g theta' / (c_p theta_bar (theta_bar + theta')) at the wall node
-                                const T th = halo[(size_t)(inf & 0xffff) * 4 + 2];
-                                b = a.gconst * th / (a.cp_tb2 + a.cp_tb2 / a.theta_bar * th);
+                            for (int f = 0; f < 4; ++f) {
+                                if (f % L != ln) continue;
+                                const T acc = f == 0 ? a0 : f == 1 ? a1 : f == 2 ? a2 : a3;
+                                T b = 0;
+                                if (f == 3 && (inf & (1 << 16))) {
+                                    // pi'_z = g theta' / (c_p theta_bar (theta_bar + theta')) at the wall node
+                                    const T th = halo[(size_t)(inf & 0xffff) * 4 + 2];
+                                    b = a.gconst * th / (a.cp_tb2 + a.cp_tb * th);
+                                }
+                                if (a.own_rows) a.resg[f * a.ng + ogp[r]] = b - acc;
+                                else res[f * ci.n_rows + r] = b - acc;
                             }
-                            if (a.own_rows) a.resg[f * a.ng + ogp[r]] = b - acc;
-                            else res[f * ci.n_rows + r] = b - acc;
                         }
                     }
+                    __syncthreads();
                 }
-                __syncthreads();
-            }
-            if (a.own_rows && (ci.n_rows > 0 || ci.n_crows > 0)) {
-                // ---- the band rows' residuals, formed by the CTAs owning their
-                // wall nodes, once every CTA that forms or reads them is here
-                if (!group_barrier(a.arrive2, a.abort, target2, (unsigned)a.wall_ctas, a.spin_limit)) return;
-                for (int e = threadIdx.x; e < 4 * ci.n_rows; e += blockDim.x) {
-                    const int f = e / ci.n_rows, k = e % ci.n_rows;
-                    res[e] = __ldcg(a.resg + f * a.ng + brow[k]);
+                if (a.own_rows && (ci.n_rows > 0 || ci.n_crows > 0)) {
+                    // ---- the band rows' residuals, formed by the CTAs owning their
+                    // wall nodes, once every CTA that forms or reads them is here
+                    if (!cta_barrier(a.arrive2, a.abort, target2, (unsigned)a.wall_ctas, a.spin_limit)) return;
+                    for (int e = threadIdx.x; e < 4 * ci.n_rows; e += blockDim.x) {
+                        const int f = e / ci.n_rows, k = e % ci.n_rows;
+                        res[e] = __ldcg(a.resg + f * a.ng + brow[k]);
+                    }
+                    __syncthreads();
                 }
-                __syncthreads();
-            }
-            if (ci.n_rows > 0) {
-                // ---- ghost values from the banded inverse rows -------------------
-                // M lanes per (ghost, class) pair, every field of the class at once
-                const int M = lanes_for(ci.n_gc, blockDim.x, kPairLanes);
-                const int npl = (ci.n_gc * M + 31) & ~31;
-                for (int e = threadIdx.x; e < npl; e += blockDim.x) {
-                    const int k0 = e / M, ln = e % M;
-                    const int k = k0 < ci.n_gc ? k0 : ci.n_gc - 1;
-                    const int4 gc = gcs[k];   // list position, field mask, -, count
-                    T s0 = 0, s1 = 0, s2 = 0, s3 = 0;
-                    // pair-interleaved [coefficient][pair_pad]: the lanes of a warp
-                    // read consecutive pairs
-                    const size_t PP = ci.pair_pad;
-                    const uint16_t *cj = cidx + k;
-                    const T *cv = cval + k;
+                if (ci.n_rows > 0) {
+                    // ---- ghost values from the banded inverse rows -------------------
+                    // M lanes per (ghost, field): every lane of a warp has the same
+                    // work, so no FP64 instruction runs for idle lanes
+                    const int M = lanes_for(ci.n_gc, blockDim.x, kPairLanes);
+                    const int npl = (ci.n_gc * M + 31) & ~31;
+                    for (int e = threadIdx.x; e < npl; e += blockDim.x) {
+                        const int k0 = e / M, ln = e % M;
+                        const int4 gc = gcs[k0 < ci.n_gc ? k0 : ci.n_gc - 1];   // list position, field, coefficients, count
+                        const size_t PP = ci.pair_pad;   // coefficients [entry][pair_pad]
+                        const uint16_t *cj = cidx + gc.z;
+                        const T *cv = cval + gc.z, *rf = res + gc.y * ci.n_rows;
+                        T sum = 0;
 #pragma unroll 4
-                    for (int j = ln; j < gc.w; j += M) {
-                        const T c = cv[j * PP];
-                        const int rr = cj[j * PP];
-                        if (gc.y & 1) s0 += c * res[rr];
-                        if (gc.y & 2) s1 += c * res[ci.n_rows + rr];
-                        if (gc.y & 4) s2 += c * res[2 * ci.n_rows + rr];
-                        if (gc.y & 8) s3 += c * res[3 * ci.n_rows + rr];
+                        for (int j = ln; j < gc.w; j += M) sum += cv[j * PP] * rf[cj[j * PP]];
+                        for (int o = M / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o, M);
+                        if (k0 < ci.n_gc && ln == 0) halo[(size_t)gc.x * 4 + gc.y] = sum;
                     }
-                    for (int o = M / 2; o > 0; o >>= 1) {
-                        s0 += __shfl_xor_sync(0xffffffffu, s0, o, M);
-                        s1 += __shfl_xor_sync(0xffffffffu, s1, o, M);
-                        s2 += __shfl_xor_sync(0xffffffffu, s2, o, M);
-                        s3 += __shfl_xor_sync(0xffffffffu, s3, o, M);
-                    }
-                    if (k0 < ci.n_gc) {
-#pragma unroll
-                        for (int f = 0; f < 4; ++f)
-                            if (f % M == ln && (gc.y & (1 << f)))
-                                halo[(size_t)gc.x * 4 + f] = f == 0 ? s0 : f == 1 ? s1 : f == 2 ? s2 : s3;
-                    }
+                    __syncthreads();
                 }
-                __syncthreads();
             }
-            if (ci.n_rows > 0 || ci.n_crows > 0) {
+            if (ci.n_gh > 0 || ci.n_crows > 0) {
                 cp_async_wait_pending<0>();   // the rest of the list (no-op at the first stage)
                 __syncthreads();
             }
@@ -746,144 +856,146 @@ __global__ void __launch_bounds__(MAXT, 1) rk4_persistent(const __grid_constant_
                 if (st == 0) mlp_phase(a, halo, hl, ML, mreg, ci.n_own, NB);
             }
             // ---- stencil sums, tendencies, RK4 update ----------------------------
-            T k[NF];
-            const Rec<T> fi = sh_rec(halo, self);
-            if constexpr (FIX) {
-                FixLargest top;
+            if (busy) {   // a warp of helper threads has no nodes
+                T k[NF];
+                const Rec<T> fi = sh_rec(halo, self);
+                if constexpr (FIX) {
+                    FixLargest top;
 #pragma unroll 4
-                for (int q = 0; q < a.SLQ; ++q) {
-                    const L j = __ldg(lx + off0 + q * stride);
-                    top.take(sh_half(halo, 2 * j.x + h));
-                    top.take(sh_half(halo, 2 * j.y + h));
-                }
-                top.over_lanes<G>();
-                FixHalf f;
-                f.a.start(top.a);
-                f.b.start(top.b);
-                int64_t off = off0;
-                if (a.ring_off) {
-                    // operands two steps ahead through the pair's ring slots (fixdot.cuh)
-                    const int4 *v = ring + (threadIdx.x >> 1);
-                    const int np = blockDim.x >> 1;
-                    L j = __ldg(lx + off);
+                    for (int q = 0; q < a.SLQ; ++q) {
+                        const L j = __ldg(lx + off0 + q * stride);
+                        top.take(sh_half(halo, 2 * j.x + h));
+                        top.take(sh_half(halo, 2 * j.y + h));
+                    }
+                    top.over_lanes<G>();
+                    FixHalf f;
+                    f.a.start(top.a);
+                    f.b.start(top.b);
+                    int64_t off = off0;
+                    if (a.ring_off) {
+                        // operands two steps ahead through the pair's ring slots (fixdot.cuh)
+                        const int4 *v = ring + (threadIdx.x >> 1);
+                        const int np = blockDim.x >> 1;
+                        L j = __ldg(lx + off);
 #pragma unroll 1
-                    for (int q0 = 0; q0 < a.SLQ; q0 += kFixRing) {
+                        for (int q0 = 0; q0 < a.SLQ; q0 += kFixRing) {
 #pragma unroll
-                        for (int u = 0; u < kFixRing; ++u) {
-                            if (q0 + u >= a.SLQ) break;
-                            const int4 r0 = sh_half(halo, 2 * j.x + h), r1 = sh_half(halo, 2 * j.y + h);
-                            off += stride;
-                            if (q0 + u + 1 < a.SLQ) j = __ldg(lx + off);
-                            fetch.copy((u + 2) % kFixRing);
-                            asm volatile("cp.async.wait_group 2;" ::: "memory");
-                            __syncwarp();   // the other thread's vectors of this step
-                            const int4 *w = v + 4 * u * np;
-                            f.slots(r0, r1, w[0], w[np], w[2 * np], w[(2 + h) * np]);
+                            for (int u = 0; u < kFixRing; ++u) {
+                                if (q0 + u >= a.SLQ) break;
+                                const int4 r0 = sh_half(halo, 2 * j.x + h), r1 = sh_half(halo, 2 * j.y + h);
+                                off += stride;
+                                if (q0 + u + 1 < a.SLQ) j = __ldg(lx + off);
+                                fetch.copy((u + 2) % kFixRing);
+                                asm volatile("cp.async.wait_group 2;" ::: "memory");
+                                __syncwarp();   // the other thread's vectors of this step
+                                const int4 *w = v + 4 * u * np;
+                                f.slots(r0, r1, w[0], w[np], w[2 * np], w[(2 + h) * np]);
+                            }
+                        }
+                        __syncwarp();   // every slot has been read
+                        fetch.start(fs, ring, np);
+                        fetch.copy(0);   // the next stage's first steps
+                        fetch.copy(1);
+                    } else {
+                        const W *we = h ? wh : wd;
+#pragma unroll 2
+                        for (int q = 0; q < a.SLQ; ++q, off += stride) {
+                            const L j = __ldg(lx + off);
+                            f.slots(sh_half(halo, 2 * j.x + h), sh_half(halo, 2 * j.y + h), __ldg(wx + off),
+                                    __ldg(wz + off), __ldg(wd + off), __ldg(we + off));
                         }
                     }
-                    __syncwarp();   // every slot has been read
-                    fetch.start(fs, ring, np);
-                    fetch.copy(0);   // the next stage's first steps
-                    fetch.copy(1);
+                    const HalfSums sums = fix_finish<G>(f, ew, h);
+                    const double2 kk = fix_tendency(sums, {a.cp, a.g_over_tb, a.theta_bar, a.dpibar, a.rd_cv}, h,
+                                                    make_double4(fi.u, fi.w, fi.t, fi.p), pib, fl);
+                    k[0] = kk.x;
+                    k[1] = kk.y;
                 } else {
-                    const W *we = h ? wh : wd;
+                    // FP32: difference form (self slot dropped)
+                    T ux = 0, uz = 0, ud = 0, wx_ = 0, wz_ = 0, wd_ = 0, tx = 0, tz = 0, td = 0, px = 0, pz = 0, ph = 0;
+                    auto vec = [&](const L &jv, const W &cx, const W &cz, const W &cd, const W &ch) {
+#pragma unroll
+                        for (int v = 0; v < V; ++v) {
+                            Rec<T> r = sh_rec(halo, P::at(jv, v));
+                            r.u -= fi.u; r.w -= fi.w; r.t -= fi.t; r.p -= fi.p;
+                            const T x = P::at(cx, v), z = P::at(cz, v), d = P::at(cd, v), hh = P::at(ch, v);
+                            ux += x * r.u; uz += z * r.u; ud += d * r.u;
+                            wx_ += x * r.w; wz_ += z * r.w; wd_ += d * r.w;
+                            tx += x * r.t; tz += z * r.t; td += d * r.t;
+                            px += x * r.p; pz += z * r.p; ph += hh * r.p;
+                        }
+                    };
+                    if (R > 0) {
+#pragma unroll
+                        for (int q = 0; q < RR; ++q)
+                            if (q < a.SLQ) vec(jr[q], rx[q], rz[q], rd[q], rh[q]);
+                    } else {
+                        int64_t off = off0;
 #pragma unroll 2
-                    for (int q = 0; q < a.SLQ; ++q, off += stride) {
-                        const L j = __ldg(lx + off);
-                        f.slots(sh_half(halo, 2 * j.x + h), sh_half(halo, 2 * j.y + h), __ldg(wx + off),
-                                __ldg(wz + off), __ldg(wd + off), __ldg(we + off));
+                        for (int q = 0; q < a.SLQ; ++q, off += stride)
+                            vec(__ldg(lx + off), __ldg(wx + off), __ldg(wz + off), __ldg(wd + off), __ldg(wh + off));
+                    }
+#pragma unroll
+                    for (int o = G / 2; o > 0; o >>= 1) {
+                        ux += __shfl_xor_sync(0xffffffffu, ux, o, G);
+                        uz += __shfl_xor_sync(0xffffffffu, uz, o, G);
+                        ud += __shfl_xor_sync(0xffffffffu, ud, o, G);
+                        wx_ += __shfl_xor_sync(0xffffffffu, wx_, o, G);
+                        wz_ += __shfl_xor_sync(0xffffffffu, wz_, o, G);
+                        wd_ += __shfl_xor_sync(0xffffffffu, wd_, o, G);
+                        tx += __shfl_xor_sync(0xffffffffu, tx, o, G);
+                        tz += __shfl_xor_sync(0xffffffffu, tz, o, G);
+                        td += __shfl_xor_sync(0xffffffffu, td, o, G);
+                        px += __shfl_xor_sync(0xffffffffu, px, o, G);
+                        pz += __shfl_xor_sync(0xffffffffu, pz, o, G);
+                        ph += __shfl_xor_sync(0xffffffffu, ph, o, G);
+                    }
+                    const T cpth = a.cp * (a.theta_bar + fi.t);
+                    k[0] = -fi.u * ux - fi.w * uz - cpth * px + ud;
+                    k[1] = -fi.u * wx_ - fi.w * wz_ - cpth * pz + a.g_over_tb * fi.t + wd_;
+                    k[2] = -fi.u * tx - fi.w * tz + td;
+                    k[3] = -fi.u * px - fi.w * (a.dpibar + pz) - a.rd_cv * (pib + fi.p) * (ux + wz_) + ph;
+                    if (fl & 1) k[1] = 0;   // w = 0 held on bottom/top walls
+                    if (fl & 2) k[0] = 0;   // u = 0 held on left/right walls
+                }
+                const T an = st == 0 ? a.an0 : st == 1 ? a.an1 : a.an2;
+                const T bs = st == 0 ? a.bs0 : st == 1 ? a.bs1 : st == 2 ? a.bs2 : a.bs3;
+#pragma unroll
+                for (int f = 0; f < NF; ++f) {
+                    const T kf = k[f];
+                    if (st == 0) {
+                        K[f] = bs * kf;
+                        o4[f] = un[f] + an * kf;
+                    } else if (st < 3) {
+                        K[f] += bs * kf;
+                        o4[f] = un[f] + an * kf;
+                    } else {
+                        o4[f] = un[f] + (K[f] + bs * kf);
                     }
                 }
-                const HalfSums sums = fix_finish<G>(f, ew, h);
-                const double2 kk = fix_tendency(sums, {a.cp, a.g_over_tb, a.theta_bar, a.dpibar, a.rd_cv}, h,
-                                                make_double4(fi.u, fi.w, fi.t, fi.p), pib, fl);
-                k[0] = kk.x;
-                k[1] = kk.y;
-            } else {
-                // FP32: difference form (self slot dropped)
-                T ux = 0, uz = 0, ud = 0, wx_ = 0, wz_ = 0, wd_ = 0, tx = 0, tz = 0, td = 0, px = 0, pz = 0, ph = 0;
-                auto vec = [&](const L &jv, const W &cx, const W &cz, const W &cd, const W &ch) {
+                if constexpr (MLP) {
+                    if (st == 3 && live) {
+                        // U += alpha dt delta; a non-finite correction is skipped and counted
+                        const float al[4] = {a.malpha.x, a.malpha.y, a.malpha.z, a.malpha.w};
 #pragma unroll
-                    for (int v = 0; v < V; ++v) {
-                        Rec<T> r = sh_rec(halo, P::at(jv, v));
-                        r.u -= fi.u; r.w -= fi.w; r.t -= fi.t; r.p -= fi.p;
-                        const T x = P::at(cx, v), z = P::at(cz, v), d = P::at(cd, v), hh = P::at(ch, v);
-                        ux += x * r.u; uz += z * r.u; ud += d * r.u;
-                        wx_ += x * r.w; wz_ += z * r.w; wd_ += d * r.w;
-                        tx += x * r.t; tz += z * r.t; td += d * r.t;
-                        px += x * r.p; pz += z * r.p; ph += hh * r.p;
-                    }
-                };
-                if (R > 0) {
-#pragma unroll
-                    for (int q = 0; q < RR; ++q)
-                        if (q < a.SLQ) vec(jr[q], rx[q], rz[q], rd[q], rh[q]);
-                } else {
-                    int64_t off = off0;
-#pragma unroll 2
-                    for (int q = 0; q < a.SLQ; ++q, off += stride)
-                        vec(__ldg(lx + off), __ldg(wx + off), __ldg(wz + off), __ldg(wd + off), __ldg(wh + off));
-                }
-#pragma unroll
-                for (int o = G / 2; o > 0; o >>= 1) {
-                    ux += __shfl_xor_sync(0xffffffffu, ux, o, G);
-                    uz += __shfl_xor_sync(0xffffffffu, uz, o, G);
-                    ud += __shfl_xor_sync(0xffffffffu, ud, o, G);
-                    wx_ += __shfl_xor_sync(0xffffffffu, wx_, o, G);
-                    wz_ += __shfl_xor_sync(0xffffffffu, wz_, o, G);
-                    wd_ += __shfl_xor_sync(0xffffffffu, wd_, o, G);
-                    tx += __shfl_xor_sync(0xffffffffu, tx, o, G);
-                    tz += __shfl_xor_sync(0xffffffffu, tz, o, G);
-                    td += __shfl_xor_sync(0xffffffffu, td, o, G);
-                    px += __shfl_xor_sync(0xffffffffu, px, o, G);
-                    pz += __shfl_xor_sync(0xffffffffu, pz, o, G);
-                    ph += __shfl_xor_sync(0xffffffffu, ph, o, G);
-                }
-                const T cpth = a.cp * (a.theta_bar + fi.t);
-                k[0] = -fi.u * ux - fi.w * uz - cpth * px + ud;
-                k[1] = -fi.u * wx_ - fi.w * wz_ - cpth * pz + a.g_over_tb * fi.t + wd_;
-                k[2] = -fi.u * tx - fi.w * tz + td;
-                k[3] = -fi.u * px - fi.w * (a.dpibar + pz) - a.rd_cv * (pib + fi.p) * (ux + wz_) + ph;
-                if (fl & 1) k[1] = 0;   // w = 0 held on bottom/top walls
-                if (fl & 2) k[0] = 0;   // u = 0 held on left/right walls
-            }
-            const T an = st == 0 ? a.an0 : st == 1 ? a.an1 : a.an2;
-            const T bs = st == 0 ? a.bs0 : st == 1 ? a.bs1 : st == 2 ? a.bs2 : a.bs3;
-#pragma unroll
-            for (int f = 0; f < NF; ++f) {
-                const T kf = k[f];
-                if (st == 0) {
-                    K[f] = bs * kf;
-                    o4[f] = un[f] + an * kf;
-                } else if (st < 3) {
-                    K[f] += bs * kf;
-                    o4[f] = un[f] + an * kf;
-                } else {
-                    o4[f] = un[f] + (K[f] + bs * kf);
-                }
-            }
-            if constexpr (MLP) {
-                if (st == 3 && live) {
-                    // U += alpha dt delta; a non-finite correction is skipped and counted
-                    const float al[4] = {a.malpha.x, a.malpha.y, a.malpha.z, a.malpha.w};
-#pragma unroll
-                    for (int f = 0; f < 4; ++f) {
-                        const T d = (T)sD[li * 4 + f];
-                        if (isfinite((double)d)) o4[f] += (T)al[f] * (T)a.mdt * d;
-                        else if (g == 0) atomicAdd(a.mbad, 1ull);
+                        for (int f = 0; f < 4; ++f) {
+                            const T d = (T)sD[li * 4 + f];
+                            if (isfinite((double)d)) o4[f] += (T)al[f] * (T)a.mdt * d;
+                            else if (g == 0) atomicAdd(a.mbad, 1ull);
+                        }
                     }
                 }
-            }
-            if (st == 3) {
+                if (st == 3) {
 #pragma unroll
-                for (int f = 0; f < NF; ++f) un[f] = o4[f];
-            }
-            if (live && g == 0) {
-                if constexpr (FIX) reinterpret_cast<double2 *>(Uout)[2 * i + h] = make_double2(o4[0], o4[1]);
-                else st_rec(Uout, i, Rec<T>{o4[0], o4[1], o4[2], o4[3]});
+                    for (int f = 0; f < NF; ++f) un[f] = o4[f];
+                }
+                if (live && g == 0) {
+                    if constexpr (FIX) reinterpret_cast<double2 *>(Uout)[2 * i + h] = make_double2(o4[0], o4[1]);
+                    else st_rec(Uout, i, Rec<T>{o4[0], o4[1], o4[2], o4[3]});
+                }
             }
             const bool last = step + 1 == a.n_steps && st == 3;
-            if (!last && !grid_barrier(a.arrive, a.abort, target, a.spin_limit)) return;
+            if (!last && !cta_barrier(a.arrive, a.abort, target, gridDim.x, a.spin_limit)) return;
         }
     }
 }
@@ -981,7 +1093,7 @@ __global__ void __launch_bounds__(256, 1) adv_persistent(const __grid_constant__
             }
             if (live && g == 0) Uout[i] = o;
             const bool last = step + 1 == a.n_steps && st == 3;
-            if (!last && !grid_barrier(a.arrive, a.abort, target, a.spin_limit)) return;
+            if (!last && !cta_barrier(a.arrive, a.abort, target, gridDim.x, a.spin_limit)) return;
         }
         tcur += a.dt;
     }
@@ -1040,6 +1152,8 @@ PArgs<T> pargs(Problem &pb, T *U, double dt, int64_t n_steps) {
     a.npad = pb.gh.npad;
     a.ring_off = ps.ring_off;
     a.cp_tb2 = (T)(pb.cp * pb.theta_bar * pb.theta_bar);
+    a.cp_tb = a.cp_tb2 / (T)pb.theta_bar;
+    a.field_class = make_int4(pb.gh.field_class[0], pb.gh.field_class[1], pb.gh.field_class[2], pb.gh.field_class[3]);
     a.gconst = (T)pb.g;
     a.cp = (T)pb.cp;
     a.g_over_tb = (T)(pb.g / pb.theta_bar);
@@ -1118,6 +1232,145 @@ void put(std::vector<unsigned char> &b, size_t at, const void *src, size_t bytes
     if (bytes) memcpy(b.data() + at, src, bytes);
 }
 
+// Lets a kernel use all the dynamic shared memory a block may have (`optin`
+// with its static part) and returns that size.  Plans of several problems share
+// a kernel, so the limit is not each plan's own need: a later, smaller plan
+// would make the earlier one's launches fail.
+int allow_dynamic_smem(void *fn, int optin) {
+    cudaFuncAttributes fa{};
+    RBF_CUDA(cudaFuncGetAttributes(&fa, fn));
+    const int most = optin - (int)fa.sharedSizeBytes;
+    RBF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    return most;
+}
+
+// Rows of the ghost values as functions of the records, [class * ng + position]:
+// (record, coefficient) with the coefficients -sum over the banded inverse row's
+// wall rows of its entry times the wall row's weight, formed in FP64.
+std::vector<std::vector<std::pair<int32_t, double>>> ghost_rows(
+    const GhostPlan &gh, int64_t ng, int npad, int64_t n_all,
+    const std::vector<std::vector<std::pair<int32_t, double>>> &band, const std::vector<int32_t> &at,
+    const std::vector<int32_t> &gidx, const std::vector<unsigned char> &gw) {
+    const float *w = reinterpret_cast<const float *>(gw.data());   // [4][ng][npad]
+    std::vector<std::vector<std::pair<int32_t, double>>> out((size_t)gh.n_class * ng);
+    std::vector<double> sum(n_all, 0.0);
+    std::vector<char> seen(n_all, 0);
+    std::vector<int32_t> used;
+    for (int f = 3; f >= 0; --f) {   // one field per class: its fields share their weights
+        const int cl = gh.field_class[f];
+        if (!out[(size_t)cl * ng].empty()) continue;
+        for (int64_t q = 0; q < ng; ++q) {
+            used.clear();
+            for (const auto &e : band[(size_t)cl * ng + q]) {
+                const int32_t r = at[e.first];
+                for (int t = 0; t < npad; ++t) {
+                    const double v = w[((size_t)f * ng + r) * npad + t];
+                    if (v == 0.0) continue;
+                    const int32_t j = gidx[(size_t)r * npad + t];
+                    if (!seen[j]) {
+                        seen[j] = 1;
+                        used.push_back(j);
+                    }
+                    sum[j] -= e.second * v;
+                }
+            }
+            auto &row = out[(size_t)cl * ng + q];
+            row.reserve(used.size());
+            for (int32_t j : used) {
+                row.emplace_back(j, sum[j]);
+                sum[j] = 0.0;
+                seen[j] = 0;
+            }
+        }
+    }
+    return out;
+}
+
+// The ghost block of an FP32 CTA (ghosts_from_records): per pair of its ghosts
+// the records they read, the coefficients (rounded once) and the pi' rows'
+// entries at the hydrostatic wall nodes.  Fills ci's section offsets.
+std::vector<unsigned char> ghost_pairs(const std::vector<int32_t> &ghosts, const GhostPlan &gh, int64_t ng, int64_t P,
+                                       const std::vector<std::vector<std::pair<int32_t, double>>> &band,
+                                       const std::vector<std::vector<std::pair<int32_t, double>>> &rows,
+                                       const std::vector<int32_t> &posv, const std::vector<int32_t> &at,
+                                       const std::vector<int32_t> &owner, const std::vector<unsigned char> &tbv,
+                                       const std::vector<int32_t> &loc, CtaInfo &ci) {
+    std::vector<int32_t> hydro;            // records of the CTA's hydrostatic wall nodes
+    std::vector<int32_t> index(ng, -1);    // their index by wall row
+    std::vector<GhostPair> pairs;
+    std::vector<uint16_t> pos;
+    std::vector<float> coef;
+    std::vector<int32_t> used, hyd;        // list positions and hydrostatic nodes of the pair
+    std::vector<char> seen(ci.n_list, 0);
+    // [class * 2 + ghost][list position], [ghost][hydrostatic node]
+    std::vector<std::vector<double>> c((size_t)gh.n_class * 2, std::vector<double>(ci.n_list, 0.0)), hb(2);
+    for (size_t k = 0; k < ghosts.size(); k += 2) {
+        used.clear();
+        hyd.clear();
+        for (int s = 0; s < 2 && k + s < ghosts.size(); ++s) {
+            const int64_t q = posv[ghosts[k + s] - P];
+            for (int cl = 0; cl < gh.n_class; ++cl)
+                for (const auto &e : rows[(size_t)cl * ng + q]) {
+                    const int32_t l = loc[e.first];
+                    seen[l] = 1;
+                    c[(size_t)cl * 2 + s][l] = e.second;
+                }
+            for (const auto &e : band[(size_t)gh.field_class[3] * ng + q]) {
+                const int32_t r = at[e.first];
+                if (!tbv[r]) continue;
+                if (index[r] < 0) {
+                    index[r] = (int32_t)hydro.size();
+                    hydro.push_back(owner[r]);
+                    hb[0].push_back(0.0);
+                    hb[1].push_back(0.0);
+                }
+                if (hb[0][index[r]] == 0.0 && hb[1][index[r]] == 0.0) hyd.push_back(index[r]);
+                hb[s][index[r]] = e.second;   // kept entries are not zero
+            }
+        }
+        for (int32_t l = 0; l < ci.n_list; ++l)
+            if (seen[l]) used.push_back(l);
+        const size_t real = used.size();
+        while (used.size() % kGhostPad) used.push_back(used[0]);   // padded with a record it reads anyway, coefficient 0
+        GhostPair g{};
+        g.pos = (int32_t)pos.size();
+        g.n_j = (int32_t)used.size();
+        for (int32_t l : used) pos.push_back((uint16_t)l);
+        g.comp = (int32_t)coef.size();
+        coef.resize(coef.size() + c.size() * used.size(), 0.f);
+        for (size_t r = 0; r < c.size(); ++r) {
+            float *to = coef.data() + g.comp + r * used.size();
+            for (size_t j = 0; j < real; ++j) {
+                to[j] = (float)c[r][used[j]];
+                c[r][used[j]] = 0.0;
+            }
+        }
+        for (int32_t l : used) seen[l] = 0;
+        g.tb = (int32_t)pos.size();
+        g.n_tb = (int32_t)hyd.size();
+        g.binv = (int32_t)coef.size();
+        for (int32_t h : hyd) pos.push_back((uint16_t)h);
+        for (auto &row : hb)
+            for (int32_t h : hyd) {
+                coef.push_back((float)row[h]);
+                row[h] = 0.0;
+            }
+        pairs.push_back(g);
+    }
+    std::vector<unsigned char> b;
+    put(b, 0, pairs.data(), pairs.size() * sizeof(GhostPair));
+    ci.o_pos = (int32_t)align16(b.size());
+    put(b, ci.o_pos, pos.data(), pos.size() * 2);
+    ci.o_comp = (int32_t)align16(b.size());
+    put(b, ci.o_comp, coef.data(), coef.size() * 4);
+    ci.n_hy = (int32_t)hydro.size();
+    ci.o_hy = (int32_t)align16(b.size());
+    put(b, ci.o_hy, hydro.data(), hydro.size() * 4);
+    ci.o_b = (int32_t)align16(b.size());
+    b.resize(align16((size_t)ci.o_b + hydro.size() * 4), 0);
+    return b;
+}
+
 }  // namespace
 
 bool persistent_plan(Problem &pb, int G, int ctas) {
@@ -1138,7 +1391,7 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
     // node would not fit a CTA.
     const bool fp64 = pb.precision == 64;
     const int S = fp64 && G == 4 && chunk * 8 > 1024 ? 2 : G;
-    const int threads = div_up((int64_t)chunk * S * (fp64 ? 2 : 1), 32) * 32;
+    int threads = div_up((int64_t)chunk * S * (fp64 ? 2 : 1), 32) * 32;
     if (threads > 1024) return false;
     RBF_CUDA(cudaStreamSynchronize(pb.st));
 
@@ -1173,6 +1426,22 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
     restore();
     const size_t ts = pb.tsize();
     const int GV = S * V;                       // slots of one node per operand vector
+
+    // ---- kernel variant: operators in registers when they fit.  Threads beyond the
+    // nodes' own help with the record copies and the ghost solve, whose chains of
+    // shared-memory reads need warps to overlap (400 m, one lane per node, 76 CTAs:
+    // 29.1 us per step with the nodes' two warps alone, 17.0 with eight).
+    const std::vector<Variant> vs = pb.precision == 64 ? variants<double>() : variants<float>();
+    int pick = -1;
+    for (int k = 0; k < (int)vs.size(); ++k) {
+        const Variant &v = vs[k];
+        if (v.mlp || v.G != S || threads > v.maxt) continue;
+        if (v.R > 0 && SLQ > v.R) continue;
+        if (pick < 0 || (v.R > 0 && vs[pick].R == 0)) pick = k;
+    }
+    if (pick < 0) return false;
+    threads = std::max(threads, std::min(vs[pick].maxt, 512));
+    smem_optin = allow_dynamic_smem(vs[pick].fn, smem_optin);
 
     // ---- blocks -----------------------------------------------------------------
     std::vector<double> x(P), z(P);
@@ -1336,16 +1605,31 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
         for (int li = 0; li < chunk; ++li) {
             const int64_t i = ids[b0 + (li < n_own ? li : 0)];
             const int64_t p = (int64_t)c * chunk + li;
-            for (int q = 0; q < SLQ; ++q)
-                for (int s = 0; s < GV; ++s) {
-                    const int64_t eo = ((int64_t)q * P + i) * GV + s, en = ((int64_t)q * lanes + p) * GV + s;
-                    lidx[en] = (uint16_t)loc[hp[eo]];
-                    for (int f = 0; f < 4; ++f)
-                        memcpy(pwp.data() + ((size_t)f * tot_new + en) * ts,
-                               hw.data() + ((size_t)f * tot_old + eo) * ts, ts);
-                }
+            for (int q = 0; q < SLQ; ++q) {
+                // a node's slots of one step are contiguous in both packings
+                const int64_t eo = ((int64_t)q * P + i) * GV, en = ((int64_t)q * lanes + p) * GV;
+                for (int s = 0; s < GV; ++s) lidx[en + s] = (uint16_t)loc[hp[eo + s]];
+                for (int f = 0; f < 4; ++f)
+                    memcpy(pwp.data() + ((size_t)f * tot_new + en) * ts, hw.data() + ((size_t)f * tot_old + eo) * ts,
+                           (size_t)GV * ts);
+            }
         }
 
+        // FP32: ghost values straight from the records, where the coefficients fit
+        const size_t list_bytes = align16((size_t)n_list * 4 * ts);
+        if (!own && !ghosts.empty()) {
+            if (ps.ghost_rows.empty()) ps.ghost_rows = ghost_rows(gh, ng, npad, pb.n_all, band, at, gidx, gwv);
+            const std::vector<unsigned char> b =
+                ghost_pairs(ghosts, gh, ng, P, band, ps.ghost_rows, posv, at, owner, tbv, loc, ci);
+            if (list_bytes + b.size() <= (size_t)smem_optin) {
+                ci.n_gh = (int32_t)ghosts.size();
+                ci.blob_off = (int64_t)blob.size();
+                ci.blob_bytes = (int32_t)b.size();
+                blob.insert(blob.end(), b.begin(), b.end());
+                smem_max = std::max(smem_max, list_bytes + b.size());
+                continue;
+            }
+        }
         // ghost block: row slots, weight sets, row info, pairs, band coefficients
         const int n_rows = (int)rows.size(), n_crows = (int)crows.size();
         ci.n_rows = n_rows;
@@ -1379,7 +1663,7 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
             ci.n_set = n_set;
             // row stride: the L lane groups of a warp (32 / L consecutive rows
             // each) start 32 / L banks apart
-            const int L = lanes_for(std::max(n_crows, 1), threads, kRowLanes);
+            const int L = lanes_for(std::max(n_crows, 1), threads, row_lanes(fp64));
             int RP = std::max(n_crows, 1);
             while (RP % 32 != (32 / L) % 32) ++RP;
             ci.row_pad = RP;
@@ -1421,22 +1705,26 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
                     maxlen = std::max(maxlen, len);
                     ncoef += len;
                 }
-            const int n_gc = (int)pairs.size();
+            const int n_pair = (int)pairs.size();
+            const int n_gc = 4 * (int)ghosts.size();   // (ghost, field) items: every field has one class
             const int Mp = lanes_for(n_gc, threads, kPairLanes);
-            int PPd = std::max(n_gc, 1);
+            int PPd = std::max(n_pair, 1);
             while (PPd % 32 != (32 / Mp) % 32) ++PPd;
             ci.pair_pad = PPd;
             std::vector<int32_t> gcv;
             std::vector<uint16_t> cix(maxlen * PPd, 0);
             std::vector<unsigned char> cvl(maxlen * PPd * ts, 0);
-            for (int k = 0; k < n_gc; ++k) {
+            for (int k = 0; k < n_pair; ++k) {
                 const int32_t gr = pairs[k].first;
                 const int cl = pairs[k].second;
                 const auto &bd = band[(size_t)cl * ng + posv[gr - P]];
-                gcv.push_back(loc[gr]);
-                gcv.push_back(cls_fields[cl]);
-                gcv.push_back(0);
-                gcv.push_back((int32_t)bd.size());
+                for (int f = 0; f < 4; ++f) {
+                    if (!(cls_fields[cl] & (1 << f))) continue;
+                    gcv.push_back(loc[gr]);
+                    gcv.push_back(f);
+                    gcv.push_back(k);
+                    gcv.push_back((int32_t)bd.size());
+                }
                 for (size_t j = 0; j < bd.size(); ++j) {
                     cix[j * PPd + k] = (uint16_t)rloc[bd[j].first];
                     if (pb.precision == 64) {
@@ -1460,7 +1748,7 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
             ci.blob_bytes = (int32_t)b.size();
             blob.insert(blob.end(), b.begin(), b.end());
         }
-        const size_t sm = align16((size_t)n_list * 4 * ts) + align16((size_t)n_rows * 4 * ts) + ci.blob_bytes;
+        const size_t sm = list_bytes + align16((size_t)n_rows * 4 * ts) + ci.blob_bytes;
         smem_max = std::max(smem_max, sm);
     }
     if (smem_max > (size_t)smem_optin) return false;
@@ -1468,23 +1756,12 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
     unsigned ring_off = 0;
     if (fp64) {
         const size_t ring = (size_t)kFixRing * 4 * sizeof(int4) * (threads / 2);
-        if (align16(smem_max) + ring + 1024 <= (size_t)smem_optin) {   // beside the kernel's static words
+        if (align16(smem_max) + ring <= (size_t)smem_optin) {
             ring_off = (unsigned)align16(smem_max);
             smem_max = ring_off + ring;
         }
     }
 
-    // ---- kernel variant: operators in registers when they fit ----------------------
-    const std::vector<Variant> vs = pb.precision == 64 ? variants<double>() : variants<float>();
-    int pick = -1;
-    for (int k = 0; k < (int)vs.size(); ++k) {
-        const Variant &v = vs[k];
-        if (v.mlp || v.G != S || threads > v.maxt) continue;
-        if (v.R > 0 && SLQ > v.R) continue;
-        if (pick < 0 || (v.R > 0 && vs[pick].R == 0)) pick = k;
-    }
-    if (pick < 0) return false;
-    RBF_CUDA(cudaFuncSetAttribute(vs[pick].fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
     int per_sm = 0;
     RBF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, vs[pick].fn, threads, smem_max));
     if ((int64_t)per_sm * nsm < grid) return false;
@@ -1678,8 +1955,8 @@ void persistent_run_mlp(Problem &pb, double dt, int64_t n_steps, void *U, cudaSt
     RBF_CUDA(cudaGetDevice(&dev));
     RBF_CUDA(cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     const size_t smem = ps.smem + mlp_layout(mv.n_in, ps.chunk, pb.n_slots).end;
+    smem_optin = allow_dynamic_smem(fn, smem_optin);
     RBF_REQUIRE(smem <= (size_t)smem_optin, "network does not fit shared memory beside the record lists");
-    RBF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     PArgs<float> a = pargs<float>(pb, (float *)U, dt, n_steps);
     a.mW = reinterpret_cast<const __nv_bfloat16 *>(mv.Pb);
     a.mP = mv.P;
