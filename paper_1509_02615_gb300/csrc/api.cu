@@ -47,8 +47,6 @@ __global__ void pibar_kernel(const double *z, int64_t n_prog, double g, double c
     if (i < n_prog) out[i] = (T)(1.0 - g * z[i] / (cp * theta_bar));   // Sec. 6.3 background Exner
 }
 
-__global__ void set_time(double *t, double v) { *t = v; }
-
 void common_setup(Problem &pb, const double *x, const double *z, int64_t n_prog, int64_t n_all, void *stream) {
     RBF_REQUIRE(n_prog >= 1 && n_all >= n_prog, "need 1 <= n_prog <= n_all (got %lld, %lld)", (long long)n_prog,
                 (long long)n_all);
@@ -67,7 +65,7 @@ void common_setup(Problem &pb, const double *x, const double *z, int64_t n_prog,
     pb.z.alloc(n_all);
     RBF_CUDA(cudaMemcpyAsync(pb.x.p, x, n_all * 8, cudaMemcpyHostToDevice, pb.st));
     RBF_CUDA(cudaMemcpyAsync(pb.z.p, z, n_all * 8, cudaMemcpyHostToDevice, pb.st));
-    pb.tdev.alloc(1);
+    pb.tdev.alloc(16);
 }
 
 }  // namespace
@@ -176,8 +174,7 @@ void run(Problem &pb, double t0, double dt, int64_t n_steps, void *U) {
     // order the private stream after the caller's stream
     RBF_CUDA(cudaEventRecord(ev, pb.st));
     RBF_CUDA(cudaStreamWaitEvent(pb.cap, ev, 0));
-    set_time<<<1, 1, 0, pb.cap>>>(pb.tdev.p, t0);
-    RBF_CHECK_LAUNCH();
+    enqueue_set_time(pb, t0, dt, pb.cap);
     int64_t done = 0;
     while (done + chunk <= n_steps) {
         RBF_CUDA(cudaGraphLaunch(pb.graph, pb.cap));
@@ -219,8 +216,8 @@ float time_run(Problem &pb, void *U, int steps) {
 }
 
 // Run-mode autotuner of an advection problem: graph replay (with the lanes
-// per node it was packed for) against the persistent kernel for 2, 4 and 8
-// lanes per node (operators repacked for each) and CTAs of 64, 128 and 256
+// per node it was packed for) against the persistent kernel for 1 (FP32), 2, 4
+// and 8 lanes per node (operators repacked for each) and CTAs of 64, 128 and 256
 // threads, on a zero state; keeps the fastest.  lanes > 0 restricts the
 // persistent candidates to that lane count.
 void choose_run_mode_adv(Problem &pb, int mode, int lanes, int ctas) {
@@ -248,8 +245,8 @@ void choose_run_mode_adv(Problem &pb, int mode, int lanes, int ctas) {
         best = time_run(pb, U.p, steps);
         invalidate_graph(pb);
     }
-    for (int G : {2, 4, 8}) {
-        if (lanes && G != lanes) continue;
+    for (int G : {1, 2, 4, 8}) {
+        if (lanes ? G != lanes : G == 1 && pb.precision == 64) continue;
         pb.G = G;
         pack_operators(pb);
         for (int threads : {64, 128, 256}) {

@@ -287,7 +287,8 @@ __global__ void __launch_bounds__(kFixThreads, 7) ns_stage_fixed_kernel(NSArgs<d
 // Velocity u(x, t) = sum_k c_k(t) (U_k, V_k)(x) with c_k(t) = fa_k + fb_k
 // cos(fm_k pi t / T): one separable part for the deformational flow, two for
 // the vortex flow of Sec. 6.1.  Packed block k holds part k's flux-form
-// weights; the hyperviscosity block follows the parts.
+// weights; the hyperviscosity block follows the parts.  Operand vectors hold
+// two slots ([SLQ][n_prog][G][2]).
 template <class T>
 struct AdvArgs {
     const T *Uin, *Un;
@@ -295,37 +296,95 @@ struct AdvArgs {
     const int32_t *pidx;
     const T *wa, *wa2, *wh;
     int64_t n_prog;
-    int SL, stage;
+    int SLQ, stage;
     T a_next, b_stage;
-    const double *tdev;   // device time (graph replays) or nullptr
+    const double *ff;     // the stage's time factors (graph replays) or nullptr
     double t_host, t_frac_dt, period_T;
     double fa[2], fb[2], fm[2];
 };
 
-__device__ __forceinline__ double flow_factor(double a, double b, double m, double t, double T) {
-    return b == 0.0 ? a : a + b * cos(m * 3.141592653589793 * t / T);
+// Time factors of the four stages of the step at time *t (device), after
+// setting it to t0 or moving it on by dt: ff[stage][part].  One warp; an FP64
+// cosine costs a warp some 1,600 clocks of its SM's FP64 pipe, too much for
+// every block of every stage.
+struct AdvTimes {
+    double t0, dt, frac[4], period_T, fa[2], fb[2], fm[2];
+    int set, parts;
+};
+__global__ void adv_times_kernel(double *t, double *ff, AdvTimes a) {
+    grid_dep_wait();
+    const double now = a.set ? a.t0 : *t + a.dt;
+    __syncwarp();
+    if (threadIdx.x == 0) *t = now;
+    const int st = threadIdx.x >> 1, k = threadIdx.x & 1;
+    if (st < 4 && k < a.parts)
+        ff[threadIdx.x] = velocity_time_factor(a.fa[k], a.fb[k], a.fm[k], now + a.frac[st], a.period_T);
 }
 
+template <class T>
+struct Pair;
+template <>
+struct Pair<float> {
+    using W = float2;
+};
+template <>
+struct Pair<double> {
+    using W = double2;
+};
+
+constexpr int kAdvAhead = 5;   // operand vectors loaded before the wait for the preceding kernel
+
+// One stage of the advection problem.  Its operands (16 to 28 bytes per slot
+// and velocity part) stay in L2 between stages for the problems of Sec. 6.1,
+// so a launch is bound by L2 latency and by the gaps between launches: the
+// first operand vectors, constant data, load before the wait, two slots each.
 template <class T, int G, int NP>
 __global__ void __launch_bounds__(256) adv_stage_kernel(AdvArgs<T> a) {
+    using W = typename Pair<T>::W;
+    __shared__ double s_ff[2];
     const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int g = (int)(tid % G);
     int64_t i = tid / G;
     const bool live = i < a.n_prog;
     if (!live) i = a.n_prog - 1;
+    const int64_t stride = a.n_prog * G, off0 = i * G + g;   // in vectors
+    const int2 *pidx = reinterpret_cast<const int2 *>(a.pidx) + off0;
+    const W *wa = reinterpret_cast<const W *>(a.wa) + off0, *wh = reinterpret_cast<const W *>(a.wh) + off0;
+    const W *wb = NP == 2 ? reinterpret_cast<const W *>(a.wa2) + off0 : nullptr;
+    int2 j[kAdvAhead];
+    W ra[kAdvAhead], rb[kAdvAhead], rh[kAdvAhead];
+#pragma unroll
+    for (int q = 0; q < kAdvAhead; ++q) {
+        if (q < a.SLQ) {
+            j[q] = __ldg(pidx + q * stride);
+            ra[q] = __ldg(wa + q * stride);
+            if (NP == 2) rb[q] = __ldg(wb + q * stride);
+            rh[q] = __ldg(wh + q * stride);
+        }
+    }
+    if (!a.ff && threadIdx.x < NP)   // velocity time factors at this stage's time
+        s_ff[threadIdx.x] = velocity_time_factor(a.fa[threadIdx.x], a.fb[threadIdx.x], a.fm[threadIdx.x],
+                                                 a.t_host + a.t_frac_dt, a.period_T);
+    __syncthreads();
     grid_dep_wait();
     grid_dep_launch();
     T sa = 0, sb = 0, sh = 0;
-    const int64_t stride = a.n_prog * G;
-    int64_t off = i * G + g;
+    auto add = [&](const int2 &jv, const W &ca, const W &cb, const W &ch) {
+        const T v0 = a.Uin[jv.x], v1 = a.Uin[jv.y];
+        sa += ca.x * v0;
+        if (NP == 2) sb += cb.x * v0;
+        sh += ch.x * v0;
+        sa += ca.y * v1;
+        if (NP == 2) sb += cb.y * v1;
+        sh += ch.y * v1;
+    };
+#pragma unroll
+    for (int q = 0; q < kAdvAhead; ++q)
+        if (q < a.SLQ) add(j[q], ra[q], NP == 2 ? rb[q] : W{}, rh[q]);
 #pragma unroll 4
-    for (int s = 0; s < a.SL; ++s, off += stride) {
-        const int j = __ldg(a.pidx + off);
-        const T v = a.Uin[j];
-        sa += __ldg(a.wa + off) * v;
-        if (NP == 2) sb += __ldg(a.wa2 + off) * v;
-        sh += __ldg(a.wh + off) * v;
-    }
+    for (int q = kAdvAhead; q < a.SLQ; ++q)
+        add(__ldg(pidx + q * stride), __ldg(wa + q * stride), NP == 2 ? __ldg(wb + q * stride) : W{},
+            __ldg(wh + q * stride));
 #pragma unroll
     for (int o = G / 2; o > 0; o >>= 1) {
         sa += __shfl_xor_sync(0xffffffffu, sa, o, G);
@@ -333,10 +392,9 @@ __global__ void __launch_bounds__(256) adv_stage_kernel(AdvArgs<T> a) {
         sh += __shfl_xor_sync(0xffffffffu, sh, o, G);
     }
     if (!live || g != 0) return;
-    // velocity time factors at this stage's time
-    double t = (a.tdev ? *a.tdev : a.t_host) + a.t_frac_dt;
-    T kf = (T)flow_factor(a.fa[0], a.fb[0], a.fm[0], t, a.period_T) * sa + sh;
-    if (NP == 2) kf += (T)flow_factor(a.fa[1], a.fb[1], a.fm[1], t, a.period_T) * sb;
+    const double *ff = a.ff ? a.ff : s_ff;
+    T kf = (T)ff[0] * sa + sh;
+    if (NP == 2) kf += (T)ff[1] * sb;
     if (a.stage < 0) {
         a.dUdt[i] = kf;
     } else {
@@ -351,11 +409,6 @@ __global__ void __launch_bounds__(256) adv_stage_kernel(AdvArgs<T> a) {
             a.Uout[i] = un + (a.K[i] + a.b_stage * kf);
         }
     }
-}
-
-__global__ void advance_time(double *t, double dt) {
-    grid_dep_wait();
-    *t += dt;
 }
 
 // Packs FP64 weights [ops][n_prog][n] into [n_packed][SLQ][n_prog][G][V] of T
@@ -445,15 +498,18 @@ __global__ void __launch_bounds__(256) pack_fixed_kernel(const double *__restric
 template <class T>
 __global__ void pack_adv_kernel(const double *__restrict__ w64, const int32_t *__restrict__ idx, int64_t n_prog,
                                 int64_t n_all, int n, int has_hv, double hvc, const double *__restrict__ vel, int NP,
-                                const int32_t *__restrict__ src, int SL, int G, T *__restrict__ pw,
+                                const int32_t *__restrict__ src, int SLQ, int G, T *__restrict__ pw,
                                 int32_t *__restrict__ pidx) {
     int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    int64_t total = (int64_t)SL * G * n_prog;
+    constexpr int V = 2;
+    const int per = SLQ * G * V;
+    int64_t total = (int64_t)per * n_prog;
     if (t >= total) return;
-    int64_t i = t / ((int64_t)SL * G);
-    int slot = (int)(t - i * SL * G);
-    int s = slot / G, g = slot - s * G;
-    int64_t dst = ((int64_t)s * n_prog + i) * G + g;
+    int64_t i = t / per;
+    int slot = (int)(t - i * per);
+    int v = slot % V, gq = slot / V;
+    int g = gq % G, q = gq / G;
+    int64_t dst = (((int64_t)q * n_prog + i) * G + g) * V + v;
     if (slot < n) {
         int j = idx[i * n + slot];
         pidx[dst] = src[j];
@@ -599,7 +655,7 @@ AdvArgs<T> adv_args(Problem &pb) {
     a.wa2 = pb.n_vparts == 2 ? pw + total : nullptr;
     a.wh = pw + pb.n_vparts * total;
     a.n_prog = pb.n_prog;
-    a.SL = pb.SL;
+    a.SLQ = pb.SLQ;
     a.period_T = pb.period_T;
     for (int k = 0; k < 2; ++k) {
         a.fa[k] = pb.vpart[k][0];
@@ -666,6 +722,26 @@ void rk4_ns(Problem &pb, double dt, T *U, cudaStream_t s, bool rec, int step, bo
     if (split && last) RBF_CUDA(cudaStreamWaitEvent(s, pb.ev_r[1], 0));
 }
 
+// device time factors of the current step, [stage][part], behind the time
+double *adv_factors(Problem &pb) { return pb.tdev.p + 8; }
+
+void launch_adv_times(Problem &pb, bool set, double t0, double dt, cudaStream_t s, bool pdl) {
+    AdvTimes a{};
+    a.t0 = t0;
+    a.dt = dt;
+    const double frac[4] = {0.0, 0.5, 0.5, 1.0};
+    for (int k = 0; k < 4; ++k) a.frac[k] = frac[k] * dt;
+    a.period_T = pb.period_T;
+    a.parts = pb.n_vparts;
+    a.set = set;
+    for (int k = 0; k < 2; ++k) {
+        a.fa[k] = pb.vpart[k][0];
+        a.fb[k] = pb.vpart[k][1];
+        a.fm[k] = pb.vpart[k][2];
+    }
+    launch_kernel(adv_times_kernel, dim3(1), dim3(32), s, pdl, pb.tdev.p, adv_factors(pb), a);
+}
+
 template <class T>
 void rk4_adv(Problem &pb, double t, double dt, T *U, cudaStream_t s, bool use_tdev, bool rec, int step) {
     AdvArgs<T> a = adv_args<T>(pb);
@@ -675,7 +751,6 @@ void rk4_adv(Problem &pb, double t, double dt, T *U, cudaStream_t s, bool use_td
     const double frac[4] = {0.0, 0.5, 0.5, 1.0};
     a.Un = U;
     a.K = (T *)pb.K.p;
-    a.tdev = use_tdev ? pb.tdev.p : nullptr;
     a.t_host = t;
     for (int st = 0; st < 4; ++st) {
         a.Uin = in[st];
@@ -684,13 +759,12 @@ void rk4_adv(Problem &pb, double t, double dt, T *U, cudaStream_t s, bool use_td
         a.a_next = (T)(kA[st] * dt);
         a.b_stage = (T)(kB[st] * dt);
         a.t_frac_dt = frac[st] * dt;
+        a.ff = use_tdev ? adv_factors(pb) + 2 * st : nullptr;
         if (rec) RBF_CUDA(cudaEventRecordWithFlags(pb.rhs_ev[(step * 4 + st) * 2], s, cudaEventRecordExternal));
         launch_adv<T>(a, pb.G, s, pb.pdl && !rec);
         if (rec) RBF_CUDA(cudaEventRecordWithFlags(pb.rhs_ev[(step * 4 + st) * 2 + 1], s, cudaEventRecordExternal));
     }
-    if (use_tdev) {
-        launch_kernel(advance_time, dim3(1), dim3(1), s, pb.pdl && !rec, pb.tdev.p, dt);
-    }
+    if (use_tdev) launch_adv_times(pb, false, 0.0, dt, s, pb.pdl && !rec);
 }
 
 }  // namespace
@@ -698,8 +772,9 @@ void rk4_adv(Problem &pb, double t, double dt, T *U, cudaStream_t s, bool use_td
 void pack_operators(Problem &pb) {
     const int nops = (int)pb.ops.size();
     pb.n_slots = pb.diff ? pb.n - 1 : pb.n;
-    // NS: 16-byte operand vectors; advection: one slot per load
-    pb.V = pb.kind == kNS ? (int)(16 / pb.tsize()) : 1;
+    // NS: 16-byte operand vectors; advection: two slots per load (37 slots on 4
+    // lanes then pad to 40, as with one)
+    pb.V = pb.kind == kNS ? (int)(16 / pb.tsize()) : 2;
     pb.SLQ = div_up(pb.n_slots, pb.G * pb.V);
     pb.SL = pb.SLQ * pb.V;
     const int64_t total = (int64_t)pb.SL * pb.G * pb.n_prog;
@@ -711,11 +786,11 @@ void pack_operators(Problem &pb) {
         if (pb.precision == 64)
             pack_adv_kernel<double><<<div_up(total, 256), 256, 0, pb.st>>>(
                 pb.w64.p, pb.idx.p, pb.n_prog, pb.n_all, pb.n, has_hv, pb.hvc, pb.vel.p, pb.n_vparts, pb.src.p,
-                pb.SL, pb.G, (double *)pb.pw.p, pb.pidx.p);
+                pb.SLQ, pb.G, (double *)pb.pw.p, pb.pidx.p);
         else
             pack_adv_kernel<float><<<div_up(total, 256), 256, 0, pb.st>>>(
                 pb.w64.p, pb.idx.p, pb.n_prog, pb.n_all, pb.n, has_hv, pb.hvc, pb.vel.p, pb.n_vparts, pb.src.p,
-                pb.SL, pb.G, (float *)pb.pw.p, pb.pidx.p);
+                pb.SLQ, pb.G, (float *)pb.pw.p, pb.pidx.p);
         RBF_CHECK_LAUNCH();
         RBF_CUDA(cudaStreamSynchronize(pb.st));
         return;
@@ -750,6 +825,10 @@ void pack_operators(Problem &pb) {
     RBF_CHECK_LAUNCH();
     RBF_CUDA(cudaStreamSynchronize(pb.st));
     if (pb.lat.enabled) pack_lattice(pb, comb, nops);
+}
+
+void enqueue_set_time(Problem &pb, double t0, double dt, cudaStream_t s) {
+    if (pb.kind == kAdvection) launch_adv_times(pb, true, t0, dt, s, false);
 }
 
 void enqueue_rk4_step(Problem &pb, double t, double dt, void *U, cudaStream_t s, bool rec, int step, bool first,

@@ -130,6 +130,18 @@ __device__ __forceinline__ void cp_rec(double *S, int k, const double *U, int64_
     cp_async16(S + (size_t)k * 4 + 2, U + j * 4 + 2);
 }
 
+// ordinary (weak) load through L1 of data that other CTAs wrote before a
+// barrier: the barrier's acquire orders it after their stores
+__device__ __forceinline__ float ld_weak(const float *p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ double ld_weak(const double *p) {
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+    return v;
+}
 __device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
     unsigned v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -1014,7 +1026,7 @@ __global__ void __launch_bounds__(MAXT, 1) rk4_persistent(const __grid_constant_
 template <class T>
 struct AdvPArgs {
     T *U, *S0, *S1;                // [n_prog] scalar state and stage buffers
-    const int32_t *pidx;           // packed as for the stage kernel: [SL][n_prog][G]
+    const int32_t *pidx;           // packed as for the stage kernel: [SL / 2][n_prog][G][2]
     const T *wa, *wa2, *wh;
     int64_t n_prog;
     int SL;
@@ -1028,21 +1040,27 @@ struct AdvPArgs {
     long long spin_limit;
 };
 
-template <class T, int G, int R, int NP>
-__global__ void __launch_bounds__(256, 1) adv_persistent(const __grid_constant__ AdvPArgs<T> a) {
+//
+// P16: the two indices of a vector share a register (at most 65,536 nodes), for
+// the variants that fill the register file.
+template <class T, int G, int R, int NP, int MAXT, int MINB, bool P16>
+__global__ void __launch_bounds__(MAXT, MINB) adv_persistent(const __grid_constant__ AdvPArgs<T> a) {
     const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int g = (int)(tid % G);
     int64_t i = tid / G;
     const bool live = i < a.n_prog;
     if (!live) i = a.n_prog - 1;   // idle lanes mirror the last node and write nothing
-    const int64_t stride = a.n_prog * G;
-    int jr[R];
+    const int64_t stride = a.n_prog * G;   // in vectors of two slots
+    int jr[P16 ? 1 : R];
+    unsigned jp[P16 ? R / 2 : 1];
     T ra[R], rb[R], rh[R];
 #pragma unroll
     for (int s = 0; s < R; ++s) {
-        const int64_t off = i * G + g + s * stride;
+        const int64_t off = 2 * (i * G + g + (s / 2) * stride) + s % 2;
         const bool in = s < a.SL;
-        jr[s] = in ? __ldg(a.pidx + off) : 0;
+        const int j = in ? __ldg(a.pidx + off) : 0;
+        if (!P16) jr[s] = j;
+        else jp[s / 2] = s % 2 ? jp[s / 2] | (unsigned)j << 16 : (unsigned)j;
         ra[s] = in ? __ldg(a.wa + off) : T(0);
         rb[s] = (in && NP == 2) ? __ldg(a.wa2 + off) : T(0);
         rh[s] = in ? __ldg(a.wh + off) : T(0);
@@ -1066,7 +1084,8 @@ __global__ void __launch_bounds__(256, 1) adv_persistent(const __grid_constant__
 #pragma unroll
             for (int s = 0; s < R; ++s) {
                 if (s < a.SL) {
-                    const T v = __ldcg(Uin + jr[s]);   // written by other CTAs in this launch: through L2
+                    const unsigned j = P16 ? (s % 2 ? jp[s / 2] >> 16 : jp[s / 2] & 0xffffu) : (unsigned)jr[s];
+                    const T v = ld_weak(Uin + j);
                     sa += ra[s] * v;
                     if (NP == 2) sb += rb[s] * v;
                     sh += rh[s] * v;
@@ -1832,25 +1851,37 @@ void persistent_run(Problem &pb, double dt, int64_t n_steps, void *U, cudaStream
 // ---- advection (a6 + a7): plan, launch and choice of lanes and CTA size -------
 
 // Register-resident slots per lane of each lane count: a 37-node stencil
-// needs 19 (2 lanes), 10 (4 lanes) or 5 (8 lanes).
-constexpr int kAdvR2 = 19, kAdvR4 = 10, kAdvR8 = 5;
+// needs 38 (one lane), 20 (2 lanes), 10 (4 lanes) or 6 (8 lanes).  One lane
+// (FP32 only: 38 slots with three weights and 16-bit indices are 133 registers)
+// is bounded to three CTAs of 128 threads per SM (168 registers: a scheduler's
+// quarter of the file for three warps), two lanes to five, so that up to 384
+// (320) nodes per SM keep their operators in registers: the hexagonal vortex
+// nodes at h = 0.005 (46,516) take 14.2 us per step (graph replay 22.3; 44.3
+// with one slot per load and a cosine in every warp of every stage).
+constexpr int kAdvR1 = 38, kAdvR2 = 20, kAdvR4 = 10, kAdvR8 = 6;
 
 template <class T, int NP>
-void *adv_fn(int G) {
+void *adv_fn(int G, int threads, bool p16) {
+    if constexpr (sizeof(T) == 4) {
+        if (G == 1) return threads == 128 && p16 ? (void *)adv_persistent<T, 1, kAdvR1, NP, 128, 3, true> : nullptr;
+        if (G == 2 && threads == 128 && p16) return (void *)adv_persistent<T, 2, kAdvR2, NP, 128, 5, true>;
+    }
     switch (G) {
-        case 2: return (void *)adv_persistent<T, 2, kAdvR2, NP>;
-        case 4: return (void *)adv_persistent<T, 4, kAdvR4, NP>;
-        case 8: return (void *)adv_persistent<T, 8, kAdvR8, NP>;
+        case 2: return (void *)adv_persistent<T, 2, kAdvR2, NP, 256, 1, false>;
+        case 4: return (void *)adv_persistent<T, 4, kAdvR4, NP, 256, 1, false>;
+        case 8: return (void *)adv_persistent<T, 8, kAdvR8, NP, 256, 1, false>;
     }
     return nullptr;
 }
 
-void *adv_variant(const Problem &pb, int G) {
-    if (pb.precision == 64) return pb.n_vparts == 2 ? adv_fn<double, 2>(G) : adv_fn<double, 1>(G);
-    return pb.n_vparts == 2 ? adv_fn<float, 2>(G) : adv_fn<float, 1>(G);
+// the kernel for the problem with G lanes and CTAs of `threads` threads, if any
+void *adv_variant(const Problem &pb, int G, int threads) {
+    const bool p16 = pb.n_prog <= 65536;
+    if (pb.precision == 64) return pb.n_vparts == 2 ? adv_fn<double, 2>(G, threads, p16) : adv_fn<double, 1>(G, threads, p16);
+    return pb.n_vparts == 2 ? adv_fn<float, 2>(G, threads, p16) : adv_fn<float, 1>(G, threads, p16);
 }
 
-int adv_regs(int G) { return G == 2 ? kAdvR2 : G == 4 ? kAdvR4 : G == 8 ? kAdvR8 : 0; }
+int adv_regs(int G) { return G == 1 ? kAdvR1 : G == 2 ? kAdvR2 : G == 4 ? kAdvR4 : G == 8 ? kAdvR8 : 0; }
 
 // Plan for the problem's current packing (pb.G lanes per node) with CTAs of
 // `threads` threads; false if the slots of a lane exceed the variant's
@@ -1866,7 +1897,8 @@ bool adv_persistent_plan(Problem &pb, int threads) {
     RBF_CUDA(cudaGetDevice(&dev));
     RBF_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
     if (!coop) return false;
-    void *fn = adv_variant(pb, G);
+    void *fn = adv_variant(pb, G, threads);
+    if (!fn) return false;
     const int64_t grid = div_up(pb.n_prog * G, threads);
     int per_sm = 0;
     RBF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, 0));
@@ -1926,7 +1958,7 @@ void adv_launch(Problem &pb, double t0, double dt, int64_t n_steps, T *U, cudaSt
     a.base = ps.base;
     a.abort = ps.abort.p;
     a.spin_limit = ps.spin_limit;
-    void *fn = adv_variant(pb, ps.G);
+    void *fn = adv_variant(pb, ps.G, ps.threads);
     RBF_REQUIRE(fn != nullptr, "persistent advection variant missing");
     void *args[] = {&a};
     RBF_CUDA(cudaLaunchCooperativeKernel(fn, dim3(ps.grid), dim3(ps.threads), args, 0, s));

@@ -58,9 +58,8 @@ struct GhostPlan {
 };
 
 // Time factor c_k(t) = a + b cos(m pi t / T) of a separable velocity part
-// (advection, Sec. 6.1), as the persistent advection kernel evaluates it.  It
-// is the same expression as the stage kernel's flow_factor (csrc/ns.cu), so
-// the two run modes agree bit for bit (tests/test_gpu_adv_persistent.py).
+// (advection, Sec. 6.1), one expression for the launch-per-stage and the
+// persistent form, which agree bit for bit (tests/test_gpu_adv_persistent.py).
 __device__ __forceinline__ double velocity_time_factor(double a, double b, double m, double t, double T) {
     return b == 0.0 ? a : a + b * cos(m * 3.141592653589793 * t / T);
 }
@@ -169,7 +168,8 @@ struct Problem {
 
     // RK4 scratch, precision T, node-major records [rows][F]
     DevBuf<unsigned char> S0, S1, K;
-    DevBuf<double> tdev;          // device time for graph replays (advection)
+    DevBuf<double> tdev;          // advection: device time of graph replays, and at [8] the step's
+                                  // time factors [stage][part]
     DevBuf<unsigned char> host_state;  // device copy used by rbf_run_host
 
     // graph cache
@@ -213,6 +213,8 @@ struct Problem {
 // leaves it open (the sequence's last step must pass last = true).
 void enqueue_rk4_step(Problem &pb, double t, double dt, void *U, cudaStream_t s, bool record_events, int step_in_graph,
                       bool first = true, bool last = true);
+// Sets an advection problem's device time to t0 (graph replays with step dt).
+void enqueue_set_time(Problem &pb, double t0, double dt, cudaStream_t s);
 void enqueue_rhs(Problem &pb, double t, void *U, void *dUdt, cudaStream_t s);
 void autotune_threads_per_node(Problem &pb);
 void pack_operators(Problem &pb);
