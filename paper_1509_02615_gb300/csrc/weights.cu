@@ -89,10 +89,10 @@ __device__ double poly_rhs(int op, int k, int a, int b) {
 
 // Look-ahead step of weights_kernel, run by one warp: the pivot of column
 // col among logical rows col.. (permutation pc), the permutation with the
-// pivot row moved to col (pn; pn == pc allowed), the pivot, its failure flag
-// (by the step's parity) and the multipliers of the rows below it.
+// pivot row moved to col (pn; pn == pc allowed), the pivot's reciprocal, its
+// failure flag (by the step's parity) and the multipliers of the rows below it.
 __device__ __forceinline__ void pivot_step(double *A, int ld, int S, int col, const int *pc, int *pn, double *mvn,
-                                           double *diag, int *s_bad, int lane) {
+                                           double *rdiag, int *s_bad, int lane) {
     const long long kTiny = __double_as_longlong(1e-14);
     const long long kInf = 0x7ff0000000000000LL;
     long long best = -1;
@@ -113,14 +113,14 @@ __device__ __forceinline__ void pivot_step(double *A, int ld, int S, int col, co
     if (pn != pc)   // entries from col - 1 on: pn then holds every settled entry
         for (int i = col - 1 + lane; i < S; i += 32) pn[i] = pc[i];
     __syncwarp();
+    const double inv = bad ? 0.0 : 1.0 / piv;
     if (lane == 0) {
         pn[col] = rb;
         pn[bi] = rc;
-        diag[col] = piv;
+        rdiag[col] = inv;
         s_bad[col & 1] = bad;
     }
     __syncwarp();
-    const double inv = bad ? 0.0 : 1.0 / piv;
     for (int i = col + 1 + lane; i < S; i += 32) mvn[i] = A[pn[i] * ld + col] * inv;
 }
 
@@ -147,8 +147,8 @@ __global__ void __launch_bounds__(NT) weights_kernel(const double *__restrict__ 
     double *xi = A + S * ld;        // n shifted, scaled coordinates
     double *eta = xi + n;
     double *const mv0 = eta + n, *const mv1 = mv0 + S;   // multipliers, double-buffered by step
-    double *const diag = mv1 + S;                         // S pivots (the diagonal of U)
-    int *const pm0 = reinterpret_cast<int *>(diag + S), *const pm1 = pm0 + S;   // permutations, likewise
+    double *const rdiag = mv1 + S;                        // reciprocals of the S pivots (the diagonal of U)
+    int *const pm0 = reinterpret_cast<int *>(rdiag + S), *const pm1 = pm0 + S;   // permutations, likewise
 
     const int32_t *row = idx + c * n;
     const double xc = x[c], zc = z[c];
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(NT) weights_kernel(const double *__restrict__ 
     }
     __syncthreads();
 
-    if (warp == 0) pivot_step(A, ld, S, 0, pm0, pm0, mv0, diag, s_bad, lane);
+    if (warp == 0) pivot_step(A, ld, S, 0, pm0, pm0, mv0, rdiag, s_bad, lane);
     __syncthreads();
     int cur = 0;
     int failed = s_bad[0];
@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(NT) weights_kernel(const double *__restrict__ 
                     const double pk = prow[kk + 1];
                     for (int i = kk + 1 + lane; i < S; i += 32) A[pc[i] * ld + kk + 1] -= mc[i] * pk;
                     __syncwarp();
-                    pivot_step(A, ld, S, kk + 1, pc, cur ? pm0 : pm1, cur ? mv0 : mv1, diag, s_bad, lane);
+                    pivot_step(A, ld, S, kk + 1, pc, cur ? pm0 : pm1, cur ? mv0 : mv1, rdiag, s_bad, lane);
                 }
             } else {
                 // A[i][j] -= m_i p_j, logical rows i > kk, columns j >= kk+2,
@@ -277,8 +277,12 @@ __global__ void __launch_bounds__(NT) weights_kernel(const double *__restrict__ 
         return;
     }
     const int *P = cur ? pm1 : pm0;   // the last step's permutation: every entry settled
+    // (a division here would run for every row once more: an FP64 division is
+    // some nine instructions of 16 clocks each for the warp; with the pivots'
+    // reciprocals, formed for the multipliers anyway, 42.1 -> 40.5 ms for 77,235
+    // systems with S = 77)
     for (int i = S - 1; i >= 0; --i) {
-        if (tid < K) A[P[i] * ld + S + tid] /= diag[i];
+        if (tid < K) A[P[i] * ld + S + tid] *= rdiag[i];
         __syncthreads();
         const double *xr = A + P[i] * ld + S;
         for (int e = tid; e < i * K; e += NT) {
