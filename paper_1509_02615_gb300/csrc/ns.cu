@@ -846,18 +846,22 @@ void enqueue_rk4_step(Problem &pb, double t, double dt, void *U, cudaStream_t s,
 void enqueue_rhs(Problem &pb, double t, void *U, void *dUdt, cudaStream_t s) {
     if (pb.kind == kNS) {
         enqueue_ghost_fill(pb, U, s);
+        // after the ghost kernels the stage launches early, as in a run, and
+        // brings its first operands in while they finish: 26.6 -> 24.6 us per
+        // call in FP64 (the 10 km x 10 km box at 125 m)
+        const bool pdl = pb.pdl && pb.gh.n_ghost > 0;
         if (pb.precision == 64) {
             NSArgs<double> a = ns_args<double>(pb);
             a.Uin = (const double *)U;
             a.dUdt = (double *)dUdt;
             a.stage = -1;
-            launch_ns(a, pb.G, pb.pf, s, false);
+            launch_ns(a, pb.G, pb.pf, s, pdl);
         } else {
             NSArgs<float> a = ns_args<float>(pb);
             a.Uin = (const float *)U;
             a.dUdt = (float *)dUdt;
             a.stage = -1;
-            launch_ns(a, pb.G, pb.pf, s, false);
+            launch_ns(a, pb.G, pb.pf, s, pdl);
         }
     } else {
         if (pb.precision == 64) {
