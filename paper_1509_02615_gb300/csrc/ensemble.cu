@@ -17,6 +17,7 @@
 #include <numeric>
 
 #include "fixdot.cuh"
+#include "stream32.cuh"
 #include "problem.cuh"
 #include "records.cuh"
 
@@ -27,6 +28,7 @@ namespace {
 template <class T>
 struct BlockDesc {
     const int32_t *pidx;
+    const short4 *pnear;          // FP32: indices relative to the node (nodes without kFarFlag)
     const T *wx, *wz, *wd, *wh;   // FP64: fixed-point pairs (fixdot.cuh)
     const short4 *wexp, *lexp;    // FP64: row exponents of the member's nodes, of its classes
     const T *pibar;
@@ -100,7 +102,7 @@ __device__ __forceinline__ void finish_node(const BlockDesc<T> &d, const EnsArgs
 // stage kernel with streamed operands).  LAT: members with lattice storage
 // take a class node's operands from the member's class table.
 template <class T, int G, bool DIFF, bool LAT>
-__global__ void __launch_bounds__(256, 4) ens_stage_kernel(const BlockDesc<T> *__restrict__ descs, EnsArgs<T> a) {
+__global__ void __launch_bounds__(kThreads32, 1024 / kThreads32) ens_stage_kernel(const BlockDesc<T> *__restrict__ descs, EnsArgs<T> a) {
     using VT = VecE<T>;
     using W = typename VT::W;
     using I = typename VT::I;
@@ -115,6 +117,15 @@ __global__ void __launch_bounds__(256, 4) ens_stage_kernel(const BlockDesc<T> *_
     const I *pidx = reinterpret_cast<const I *>(d.pidx);
     const W *wx = reinterpret_cast<const W *>(d.wx), *wz = reinterpret_cast<const W *>(d.wz);
     const W *wd = reinterpret_cast<const W *>(d.wd), *wh = reinterpret_cast<const W *>(d.wh);
+    // neighbour indices: 16 bits relative to the node where that suffices
+    const bool near = !LAT && !(__ldg(d.flags + i) & kFarFlag);
+    auto nbr = [&](int q) {
+        const int64_t off = off0 + q * stride;
+        return near ? near_at(__ldg(d.pnear + off), (int)i) : __ldg(pidx + off);
+    };
+    __shared__ Stage32<!LAT> ring;
+    Stream32 st;
+    if constexpr (!LAT) st.start(d.wx, off0, stride * d.SLQ, stride, d.SLQ, ring.at);
     grid_dep_wait();
     grid_dep_launch();
     const T *U = a.Uin + d.rec0 * 4;   // member-local record indices from here on
@@ -134,7 +145,9 @@ __global__ void __launch_bounds__(256, 4) ens_stage_kernel(const BlockDesc<T> *_
         }
     };
     const int cl = (LAT && d.lcls) ? __ldg(d.lcls + i) : -1;
-    if (LAT && cl >= 0) {
+    if constexpr (!LAT) {
+        stream_steps(st, ring.at, d.SLQ, nbr, vec);
+    } else if (cl >= 0) {
         const I *lo = reinterpret_cast<const I *>(d.loff);
         const W *lw = reinterpret_cast<const W *>(d.lw);
         const int64_t ls = (int64_t)d.n_cls * d.SLQ * G;   // in vectors, between operators
@@ -222,7 +235,7 @@ const double kA[4] = {0.5, 0.5, 1.0, 0.0};
 const double kB[4] = {1.0 / 6.0, 1.0 / 3.0, 1.0 / 3.0, 1.0 / 6.0};
 
 // threads of a stage block
-int block_threads(const Problem &pb) { return pb.precision == 64 ? kFixThreads : 256; }
+int block_threads(const Problem &pb) { return pb.precision == 64 ? kFixThreads : kThreads32; }
 
 template <class T>
 void fill_descs(Problem &pb) {
@@ -237,6 +250,7 @@ void fill_descs(Problem &pb) {
         for (int64_t n0 = 0; n0 < m.n_prog; n0 += C) {
             BlockDesc<T> d{};
             d.pidx = m.pidx.p;
+            d.pnear = m.pnear.p;
             d.wx = pw;
             d.wz = pw + total;
             d.wd = pw + 2 * total;

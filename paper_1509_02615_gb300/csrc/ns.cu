@@ -24,6 +24,7 @@
 #include <cstring>
 
 #include "fixdot.cuh"
+#include "stream32.cuh"
 #include "problem.cuh"
 #include "records.cuh"
 
@@ -39,6 +40,7 @@ struct NSArgs {
     T *K;             // [n_prog][4] RK4 accumulator
     T *dUdt;          // [n_prog][4] tendency (stage < 0)
     const int32_t *pidx;
+    const short4 *pnear;          // FP32: indices relative to the node (nodes without kFarFlag)
     const T *wx, *wz, *wd, *wh;   // FP64: fixed-point pairs (fixdot.cuh), not doubles
     const short4 *wexp;           // FP64: row exponents of each node, or of each class
     const T *pibar;
@@ -113,16 +115,20 @@ __device__ __forceinline__ void finish_node(const NSArgs<T> &a, int64_t i, int g
     }
 }
 
-// One RK4 stage (or the bare right-hand side when stage < 0) for G lanes per
-// node.  Each lane reads its operands as 16-byte vectors (V slots each) and
-// gathers one node record per neighbour.  PF > 0: the lane's operand vectors
+// One FP32 RK4 stage (or the bare right-hand side when stage < 0) for G lanes
+// per node.  Each lane reads its operands as 16-byte vectors (four slots each)
+// and gathers one node record per neighbour.  PF > 0: the lane's operand vectors
 // (constant data) are loaded into registers before grid_dep_wait(), so they
-// stream in while the preceding ghost kernels finish; PF == 0 streams them.
-// LAT: a node of a lattice class takes its operand vectors from the class
-// table (neighbour = node + offset); the lanes of a warp whose nodes share a
-// class read the same table entries, which stay in L1.
+// stream in while the preceding ghost kernels finish; PF == 0 streams them
+// through a ring in shared memory, with 16-bit indices where they suffice
+// (stream32.cuh has the figures).  LAT: a node of a lattice class takes its
+// operand vectors from the class table (neighbour = node + offset); the lanes of
+// a warp whose nodes share a class read the same table entries, which stay in
+// L1, and the nodes outside all classes are few and load plainly.
+template <int PF, bool LAT>
+constexpr int kStageThreads = PF == 0 && !LAT ? kThreads32 : 256;
 template <class T, int G, bool DIFF, int PF, bool LAT>
-__global__ void __launch_bounds__(256, PF > 0 ? 1 : 4) ns_stage_kernel(NSArgs<T> a) {
+__global__ void __launch_bounds__(kStageThreads<PF, LAT>, PF > 0 ? 1 : 1024 / kStageThreads<PF, LAT>) ns_stage_kernel(NSArgs<T> a) {
     using VT = Vec<T>;
     using W = typename VT::W;
     using I = typename VT::I;
@@ -145,6 +151,16 @@ __global__ void __launch_bounds__(256, PF > 0 ? 1 : 4) ns_stage_kernel(NSArgs<T>
     const I *pidx = reinterpret_cast<const I *>(a.pidx);
     const W *wx = reinterpret_cast<const W *>(a.wx), *wz = reinterpret_cast<const W *>(a.wz);
     const W *wd = reinterpret_cast<const W *>(a.wd), *wh = reinterpret_cast<const W *>(a.wh);
+    constexpr bool RING = PF == 0 && !LAT;
+    // neighbour indices: 16 bits relative to the node where that suffices
+    const bool near = RING && !(__ldg(a.flags + i) & kFarFlag);
+    auto nbr = [&](int q) {
+        const int64_t off = off0 + q * stride;
+        return near ? near_at(__ldg(a.pnear + off), (int)i) : __ldg(pidx + off);
+    };
+    __shared__ Stage32<RING> ring;
+    Stream32 st;
+    if constexpr (RING) st.start(a.wx, off0, stride * a.SLQ, stride, a.SLQ, ring.at);
     constexpr int R = PF > 0 ? PF : 1;
     I jr[R];
     W rx[R], rz[R], rd[R], rh[R];
@@ -179,7 +195,9 @@ __global__ void __launch_bounds__(256, PF > 0 ? 1 : 4) ns_stage_kernel(NSArgs<T>
             px += x * r.p; pz += z * r.p; ph += h * r.p;
         }
     };
-    if (PF > 0) {
+    if constexpr (RING) {
+        stream_steps(st, ring.at, a.SLQ, nbr, vec);
+    } else if (PF > 0) {
 #pragma unroll
         for (int q = 0; q < R; ++q)
             if (q < a.SLQ) vec(jr[q], rx[q], rz[q], rd[q], rh[q]);
@@ -490,6 +508,27 @@ __global__ void __launch_bounds__(256) pack_fixed_kernel(const double *__restric
     if (lane == 0) wexp[i] = make_short4(ex[0], ex[1], ex[2], ex[3]);
 }
 
+// Neighbour indices relative to the node in 16 bits, in the layout of pidx
+// (four slots each), and kFarFlag for the nodes one of whose neighbours is too
+// far (ghosts, which follow all prognostic nodes, and the seams of the node
+// order), or for all of them without `out`; counts them.  One thread per node.
+__global__ void near_indices(const int32_t *__restrict__ pidx, int64_t n_prog, int SLQ, int G, short4 *__restrict__ out,
+                             unsigned char *__restrict__ flags, unsigned long long *n_far) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= n_prog) return;
+    bool far = out == nullptr;
+    for (int q = 0; q < SLQ; ++q)
+        for (int g = 0; g < G; ++g) {
+            const int64_t at = ((int64_t)q * n_prog + i) * G + g;
+            const int4 j = reinterpret_cast<const int4 *>(pidx)[at];
+            const int64_t d[4] = {j.x - i, j.y - i, j.z - i, j.w - i};
+            for (int v = 0; v < 4; ++v) far = far || d[v] < -32768 || d[v] > 32767;
+            if (out) out[at] = make_short4((short)d[0], (short)d[1], (short)d[2], (short)d[3]);
+        }
+    flags[i] = (unsigned char)((flags[i] & ~kFarFlag) | (far ? kFarFlag : 0));
+    if (far) atomicAdd(n_far, 1ull);
+}
+
 // Advection: packed block k < NP = flux-form weights of velocity part k,
 // -(Dx_ij U_k(x_j) + Dy_ij V_k(x_j)); block NP = (-1)^(k+1) gamma Delta^k
 // weights; columns folded onto the source node of reflected nodes
@@ -571,7 +610,8 @@ void launch_ns(const NSArgs<double> &a, int G, int, cudaStream_t s, bool pdl, in
 template <class T, int G, int PF>
 void launch_ns_g(const NSArgs<T> &a, cudaStream_t s, bool pdl, int prio) {
     constexpr bool kDiff = true;   // difference form
-    const dim3 grid(div_up((a.nlist ? a.n_list : a.n_prog) * G, 256)), blk(256);
+    const int threads = a.lcls ? kStageThreads<0, true> : kStageThreads<PF, false>;
+    const dim3 grid(div_up((a.nlist ? a.n_list : a.n_prog) * G, threads)), blk(threads);
     if (a.lcls) {
         if (PF == 0) launch_kernel_prio(ns_stage_kernel<T, G, kDiff, 0, true>, grid, blk, s, pdl, prio, a);
         else RBF_FAIL(RBF_E_ARG, "the lattice storage has no prefetch variant");
@@ -620,6 +660,7 @@ NSArgs<T> ns_args(Problem &pb) {
     const int64_t total = (int64_t)pb.SLQ * pb.V * pb.G * pb.n_prog;
     const T *pw = (const T *)pb.pw.p;
     a.pidx = pb.pidx.p;
+    a.pnear = pb.pnear.p;
     a.wx = pw;
     a.wz = pw + total;
     a.wd = pw + 2 * total;
@@ -769,7 +810,7 @@ void rk4_adv(Problem &pb, double t, double dt, T *U, cudaStream_t s, bool use_td
 
 }  // namespace
 
-void pack_operators(Problem &pb) {
+void pack_operators(Problem &pb, bool near) {
     const int nops = (int)pb.ops.size();
     pb.n_slots = pb.diff ? pb.n - 1 : pb.n;
     // NS: 16-byte operand vectors; advection: two slots per load (37 slots on 4
@@ -823,6 +864,23 @@ void pack_operators(Problem &pb) {
                                                                   pb.n_slots, pb.SLQ, pb.G, pb.V, pb.n_packed,
                                                                   dcomb.p, (float *)pb.pw.p, pb.pidx.p);
     RBF_CHECK_LAUNCH();
+    if (near && pb.precision == 32) {
+        // a tenth more operand storage, where it leaves room for the states;
+        // without it every node is marked far
+        size_t free_b = 0, total_b = 0;
+        RBF_CUDA(cudaMemGetInfo(&free_b, &total_b));
+        pb.pnear.release();
+        if (!pb.lat.enabled && free_b >= 8 * (size_t)total) pb.pnear.alloc((size_t)total / 4);
+        unsigned long long far = 0;
+        DevBuf<unsigned long long> dfar(1);
+        RBF_CUDA(cudaMemsetAsync(dfar.p, 0, sizeof(far), pb.st));
+        near_indices<<<div_up(pb.n_prog, 256), 256, 0, pb.st>>>(pb.pidx.p, pb.n_prog, pb.SLQ, pb.G, pb.pnear.p,
+                                                                pb.flags.p, dfar.p);
+        RBF_CHECK_LAUNCH();
+        RBF_CUDA(cudaMemcpyAsync(&far, dfar.p, sizeof(far), cudaMemcpyDeviceToHost, pb.st));
+        RBF_CUDA(cudaStreamSynchronize(pb.st));
+        pb.n_far = (int64_t)far;
+    }
     RBF_CUDA(cudaStreamSynchronize(pb.st));
     if (pb.lat.enabled) pack_lattice(pb, comb, nops);
 }

@@ -1433,7 +1433,7 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
     int SLQ = 0, V = 0;
     try {
         pb.G = S;
-        pack_operators(pb);
+        pack_operators(pb, false);
         hp = to_host(pb.pidx);
         hw = to_host(pb.pw);
         SLQ = pb.SLQ;

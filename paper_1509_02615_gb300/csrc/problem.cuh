@@ -64,8 +64,10 @@ __device__ __forceinline__ double velocity_time_factor(double a, double b, doubl
     return b == 0.0 ? a : a + b * cos(m * 3.141592653589793 * t / T);
 }
 
-// flags bit of the wall set (split stage launches)
-constexpr unsigned char kWallSetFlag = 4;
+// flags bits: the wall set (split stage launches); a neighbour's index is more
+// than 16 bits away from the node's
+constexpr unsigned char kWallSetFlag = 4, kFarFlag = 8;
+__device__ __forceinline__ int4 near_at(short4 d, int i) { return make_int4(i + d.x, i + d.y, i + d.z, i + d.w); }
 
 // Builds gh.brow / bcol / bval from the dense inverse blocks.
 void build_ghost_bands(GhostPlan &gh, int precision, cudaStream_t st);
@@ -146,6 +148,9 @@ struct Problem {
     // packed operators, precision T
     int n_packed = 4;
     DevBuf<int32_t> pidx;         // [SLQ][n_prog][G][V]
+    DevBuf<short4> pnear;         // NS in FP32: pidx relative to the node, in 16 bits, for the
+                                  // nodes without kFarFlag
+    int64_t n_far = 0;            // nodes with it
     DevBuf<unsigned char> pw;     // T [n_packed][SLQ][n_prog][G][V]; NS in FP64: fixed-point
                                   // pairs int2 (fixdot.cuh) in place of the doubles
     DevBuf<short4> wexp;          // [n_prog] NS in FP64: exponents of the packed rows
@@ -217,7 +222,7 @@ void enqueue_rk4_step(Problem &pb, double t, double dt, void *U, cudaStream_t s,
 void enqueue_set_time(Problem &pb, double t0, double dt, cudaStream_t s);
 void enqueue_rhs(Problem &pb, double t, void *U, void *dUdt, cudaStream_t s);
 void autotune_threads_per_node(Problem &pb);
-void pack_operators(Problem &pb);
+void pack_operators(Problem &pb, bool near = true);   // near: with pnear (the stage kernels)
 void pack_lattice(Problem &pb, const std::vector<double> &comb, int nops);
 double ns_rhs_bytes(const Problem &pb);
 // gamma of Sec. 5.3 from a problem's gamma or (gamma_c, spacing) (api.cu)
