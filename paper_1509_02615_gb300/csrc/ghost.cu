@@ -126,10 +126,16 @@ __global__ void to_t(const double *src, T *dst, int64_t n) {
 
 constexpr int kRowLanes = 8;    // lanes per wall row in the residual kernel
 constexpr int kRowPf = 16;      // slots per lane held in registers
+constexpr int kRowBatch = 4;    // record gathers in flight together
 
 // r[f][pos(r)] = b_f(r) - sum over the row's non-ghost stencil nodes, all four
 // fields at once from one record gather per slot; 8 lanes per row share the
 // stencil slots (layout [row][slot]).  U holds node-major records [n_all][4].
+// The two ghost kernels are chains of memory latencies between the stages, not
+// work, so every constant (the wall rows' owners and positions too) loads before
+// the wait and the gathers go out in batches.  That and the same in
+// ghost_apply_band: 82.7 -> 80.5 us per FP32 stage on 608,256 nodes (4,096 wall
+// rows), 21.7 -> 19.8 us per FP64 right-hand side of a 125 m box.
 template <class T>
 __global__ void __launch_bounds__(256) ghost_residual(const T *__restrict__ U, int64_t ng, int64_t rows, int npad,
                                                       const int32_t *__restrict__ gidx, const T *__restrict__ gw,
@@ -157,17 +163,28 @@ __global__ void __launch_bounds__(256) ghost_residual(const T *__restrict__ U, i
             w3[t] = __ldg(gw + 3 * ng * npad + o);
         }
     }
+    const bool wall = ln == 3 && __ldg(tb + r);   // the row of pi' on a bottom or top wall
+    const int64_t own = wall ? __ldg(owner + r) : 0;
+    const int at = ln < 4 ? __ldg(pos + r) : 0;
     grid_dep_wait();
     grid_dep_launch();
+    const T th = wall ? U[own * 4 + 2] : (T)0;
     T a0 = 0, a1 = 0, a2 = 0, a3 = 0;
 #pragma unroll
-    for (int t = 0; t < kRowPf; ++t) {
-        if (t < per) {
-            const Rec<T> v = load_rec(U, jj[t]);
-            a0 += w0[t] * v.u;
-            a1 += w1[t] * v.w;
-            a2 += w2[t] * v.t;
-            a3 += w3[t] * v.p;
+    for (int t0 = 0; t0 < kRowPf; t0 += kRowBatch) {
+        if (t0 >= per) break;
+        Rec<T> v[kRowBatch];
+#pragma unroll
+        for (int t = 0; t < kRowBatch; ++t)
+            v[t] = t0 + t < per ? load_rec(U, jj[t0 + t]) : Rec<T>{0, 0, 0, 0};
+#pragma unroll
+        for (int t = 0; t < kRowBatch; ++t) {
+            if (t0 + t < per) {
+                a0 += w0[t0 + t] * v[t].u;
+                a1 += w1[t0 + t] * v[t].w;
+                a2 += w2[t0 + t] * v[t].t;
+                a3 += w3[t0 + t] * v[t].p;
+            }
         }
     }
 #pragma unroll
@@ -180,12 +197,8 @@ __global__ void __launch_bounds__(256) ghost_residual(const T *__restrict__ U, i
     if (!live || ln >= 4) return;
     T acc = ln == 0 ? a0 : ln == 1 ? a1 : ln == 2 ? a2 : a3;
     T b = 0;
-    if (ln == 3 && tb[r]) {
-        // pi'_z = g theta' / (c_p theta_bar (theta_bar + theta')) at the wall node
-        T th = U[(int64_t)owner[r] * 4 + 2];
-        b = gconst * th / (cp_tb2 + cp_tb * th);
-    }
-    res[ln * ng + pos[r]] = b - acc;
+    if (wall) b = gconst * th / (cp_tb2 + cp_tb * th);   // pi'_z = g theta' / (c_p theta_bar (theta_bar + theta'))
+    res[ln * ng + at] = b - acc;
 }
 
 // u_G = W_G^{-1} r within each component, one warp per (class, position)
@@ -195,7 +208,10 @@ __global__ void __launch_bounds__(256) ghost_residual(const T *__restrict__ U, i
 // kBandPf * 32 entries of a row are loaded before the wait.  Lanes past the
 // row's end skip the product instead of multiplying a zero by some other
 // component's residual: a non-finite residual (a member that has blown up
-// in a batched ensemble) then stays within its own component.
+// in a batched ensemble) then stays within its own component.  An FP64 addition
+// takes a warp 16 clocks of its SM's pipe: with four butterflies and products
+// for all four fields the 4,800 warps of the 25 m bubble took 9 us, 8 of them
+// on the step's critical path.
 constexpr int kBandPf = 4;
 
 template <class T>
@@ -222,21 +238,41 @@ __global__ void __launch_bounds__(256) ghost_apply_band(T *__restrict__ U, int64
         col[t] = in ? __ldg(bcol + e) : -1;
     }
     const int fm = cls == 0 ? cls_fields.x : cls == 1 ? cls_fields.y : cls == 2 ? cls_fields.z : cls_fields.w;
+    const int64_t rec = __ldg(grec + q);
     grid_dep_wait();
     grid_dep_launch();
     if (!live) return;
+    // the residuals of all fields of the class together: one L2 round trip
+    T v[4][kBandPf], s[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int f = 0; f < 4; ++f)
+#pragma unroll
+        for (int t = 0; t < kBandPf; ++t) v[f][t] = (fm >> f & 1) && col[t] >= 0 ? res[f * ng + col[t]] : (T)0;
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
-        if (!(fm & (1 << f))) continue;
-        const T *rr = res + f * ng;
-        T s = 0;
+        if (!(fm >> f & 1)) continue;   // the same for the whole warp: no FP64 work for other classes' fields
 #pragma unroll
         for (int t = 0; t < kBandPf; ++t)
-            if (col[t] >= 0) s += a[t] * rr[col[t]];
-        for (int64_t e = b0 + lane + 32 * kBandPf; e < b1; e += 32) s += __ldg(bval + e) * rr[__ldg(bcol + e)];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) U[grec[q] * 4 + f] = s;
+            if (b0 + 32 * t < b1 && col[t] >= 0) s[f] += a[t] * v[f][t];
     }
+    for (int64_t e = b0 + lane + 32 * kBandPf; e < b1; e += 32) {
+        const T av = __ldg(bval + e);
+        const int c = __ldg(bcol + e);
+#pragma unroll
+        for (int f = 0; f < 4; ++f)
+            if (fm >> f & 1) s[f] += av * res[f * ng + c];
+    }
+    // four sums over the warp in six additions: a lane keeps two fields after the
+    // first exchange and one after the second (the same tree of additions per
+    // field as four separate butterflies)
+    const bool h4 = lane & 16, h3 = lane & 8;
+    const T x0 = (h4 ? s[2] : s[0]) + __shfl_xor_sync(0xffffffffu, h4 ? s[0] : s[2], 16);
+    const T x1 = (h4 ? s[3] : s[1]) + __shfl_xor_sync(0xffffffffu, h4 ? s[1] : s[3], 16);
+    T y = (h3 ? x1 : x0) + __shfl_xor_sync(0xffffffffu, h3 ? x0 : x1, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
+    const int f = lane >> 3;   // 2 h4 + h3
+    if ((lane & 7) == 0 && (fm >> f & 1)) U[rec * 4 + f] = y;
 }
 
 struct UnionFind {
