@@ -13,8 +13,9 @@ Metric: node-RHS evaluations per second (4 per node per RK4 step).  The
 headline's working set (operators, records, RK4 buffers: ~0.7 GB in FP64) is
 several times larger than L2, so steps are timed back to back without an L2
 flush, each with CUDA events on the problem's stream.  The dominant kernel is
-the FP64 stage kernel, bound by the FP64 pipe: its roofline is in TFLOP/s
-against a DGEMM measured in the same run.
+the FP64 stage kernel, whose stencil sums run in fixed point on the integer
+units: its roofline is its operand traffic against HBM, with its FP64-equivalent
+rate and a DGEMM measured in the same run beside it.
 
 Beside the headline, in the same JSON line:
   bubble_fp32      the same workload with FP64-built weights stored in FP32
@@ -156,7 +157,7 @@ def kernel_source_hash(key=""):
     h = hashlib.sha256()
     unit = ("persistent.cu" if key.startswith("persistent") else
             "ensemble.cu" if key.startswith("ens_stage") else "ns.cu")
-    for fn in (unit, "records.cuh", "common.cuh"):
+    for fn in (unit, "records.cuh", "common.cuh", "fixdot.cuh", "stream32.cuh"):
         with open(os.path.join(ROOT, "paper_1509_02615_gb300", "csrc", fn), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
@@ -298,17 +299,18 @@ def headline_case(torch, args, wl, world, local, p64):
     else:
         avg_ms = float(np.mean(stage_ms)) / 4.0
         flops = info["rhs_flops_per_node"] * nodes.n_prog
-        kernel, share = "ns_stage_kernel<double>", float(np.sum(stage_ms) / np.sum(step_ms))
+        kernel, share = "ns_stage_fixed_kernel", float(np.sum(stage_ms) / np.sum(step_ms))
     ach = flops / (avg_ms / 1e3) / 1e12
     key = f"ns_stage_fp64_bubble{int(nodes.h)}"
-    roof = {"bound": "alu", "achieved": ach, "peak": p64, "unit": "TFLOP/s", "frac": ach / p64,
+    bpl = info["rhs_bytes_per_node"] * nodes.n_prog * (4 if persistent else 1)
+    hbm, pk = bpl / (avg_ms / 1e3) / 1e9, peaks()[0]
+    roof = {"bound": "hbm", "achieved": hbm, "peak": pk["hbm_gbs"], "unit": "GB/s", "frac": hbm / pk["hbm_gbs"],
             "traffic": None if persistent else profiled_traffic(key, threads_per_node=info["threads_per_node"]),
-            "kernel": kernel, "algorithmic_flops_per_launch": flops,
-            "algorithmic_bytes_per_launch": info["rhs_bytes_per_node"] * nodes.n_prog * (4 if persistent else 1),
+            "kernel": kernel, "algorithmic_flops_per_launch": flops, "algorithmic_bytes_per_launch": bpl,
             "avg_launch_ms": avg_ms, "kernel_share_of_step": share,
-            "peak_source": "FP64 DGEMM (cuBLAS via torch.matmul, 4096^3) measured in this run; GB300 nominal FP64 "
-                           "1.25 TFLOP/s", "frac_of_nominal": ach / 1.25,
-            "hbm_GBps": info["rhs_bytes_per_node"] * nodes.n_prog * (4 if persistent else 1) / (avg_ms / 1e3) / 1e9}
+            "fp64_equivalent_tflops": ach, "fp64_dgemm_tflops": p64,
+            "note": "the stencil sums are exact products of 28-bit integers on the integer units, no FP64 FMAs; the "
+                    "DGEMM (cuBLAS via torch.matmul, 4096^3, this run) is the rate they would be bound by"}
     # end to end through the C ABI: pinned host state -> device, one RK4 step, device -> host
     Uh = rbffd.state_tensor(wl.U0, 64, device="cpu").pin_memory()
     n_e2e = max(5, args.steps // 4)
@@ -444,7 +446,8 @@ def density_current_case(torch, args, pk, pk_kind, p64, flush):
                    "run_mode": "persistent" if i64["run_mode"] == 2 else "graph",
                    "roofline": {"bound": "alu", "achieved": flops / (avg64 / 1e3) / 1e12, "peak": p64,
                                 "unit": "TFLOP/s", "frac": flops / (avg64 / 1e3) / 1e12 / p64,
-                                "peak_source": "measured FP64 DGEMM in this run", "avg_launch_ms": avg64}}
+                                "peak_source": "measured FP64 DGEMM in this run (the stencil sums run on the integer "
+                                               "units, so this may exceed 1)", "avg_launch_ms": avg64}}
     if not args.no_final_error:
         n_end = int(round(900.0 / dt))
         A64 = rbffd.state_tensor(U0, 64)

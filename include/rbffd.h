@@ -142,10 +142,12 @@ typedef struct rbf_ns_params {
     int32_t poly_l;     /* polynomial degree l (4)                            */
     int32_t hv_k;       /* hyperviscosity Laplacian power k (3); 0 = none     */
     int32_t hv_p;       /* PHS exponent of the Delta^k weights (>= 2k+1)      */
-    int32_t precision;  /* 64: FP64 storage and arithmetic; 32: FP64-built
+    int32_t precision;  /* 64: FP64 storage and arithmetic, the stencil sums
+                           in 55-bit fixed point per stencil (closer to the
+                           exact sums than sums in FP64); 32: FP64-built
                            weights stored in FP32, FP32 RHS and RK4           */
-    int32_t threads_per_node; /* 0 = autotuned (lanes per node and register
-                                 prefetch); else 1, 2, 4 or 8 lanes        */
+    int32_t threads_per_node; /* 0 = autotuned (lanes per node and, in FP32,
+                                 register prefetch); else 1, 2, 4 or 8 lanes */
     int32_t storage;    /* RBF_STORE_PER_NODE (0, Sec. 3's rows) or
                            RBF_STORE_LATTICE (1, one row per class of
                            translated stencils; see rbf_set_operator_storage);
@@ -408,7 +410,7 @@ int rbf_run(rbf_problem *pb, double t0, double dt, int64_t n_steps, void *U);
  *                       always for advection problems).
  * lanes: lanes per node of the persistent kernel (Navier-Stokes 1, 2 or 4;
  *        advection 2, 4 or 8, which also become the lanes of the graph
- *        mode; 0 = fastest).
+ *        mode; 0 = fastest, for FP32 advection also one lane).
  * ctas:  CTAs of the persistent kernel (0: fastest of 1, 1/2, 1/4, 1/8 per
  *        SM; with lanes > 0 and RBF_RUN_PERSISTENT, one per SM untimed).
  *        Advection problems take 0: their CTA count follows from the lanes

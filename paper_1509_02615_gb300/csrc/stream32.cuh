@@ -4,7 +4,7 @@
 // the stream from memory runs on while the thread waits for its gathers.
 //
 // The stage is bound by HBM: on 608,256 nodes with n = 37 it moves 437 MB in
-// 74 us (0.85 of the copy rate).  With 32-bit indices and plain loads, two steps
+// 74 us (0.87 of the copy rate).  With 32-bit indices and plain loads, two steps
 // unrolled, a stage of a run (with its ghost kernels) took 84.9 us there, 28.1
 // us on 152,576 nodes, whose operands stay in L2, and the 12-member ensemble
 // 2.92 ms; with 16-bit indices 84.3 us, 25.7 us and 2.69 ms; with the ring as
