@@ -295,6 +295,7 @@ void choose_run_mode(Problem &pb, int mode, int lanes, int ctas) {
         pb.run_mode = RBF_RUN_GRAPH;
         return;
     }
+    invalidate_graph(pb);   // the plans below pack operands of their own
     const int nsm = sm_count();
     std::vector<std::pair<int, int>> cands;
     for (int G : {1, 2, 4}) {

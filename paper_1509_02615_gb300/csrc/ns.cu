@@ -855,7 +855,9 @@ void pack_operators(Problem &pb, bool near) {
     RBF_CUDA(cudaMemcpyAsync(dcomb.p, comb.data(), dcomb.bytes(), cudaMemcpyHostToDevice, pb.st));
     pb.pw.alloc((size_t)pb.n_packed * total * pb.tsize());
     if (pb.precision == 64) {
-        pb.wexp.alloc(pb.n_prog);
+        // the exponents do not depend on the lanes: one buffer for good, which captured
+        // graphs keep reading when a persistent plan packs its own operands
+        if (pb.wexp.n != (size_t)pb.n_prog) pb.wexp.alloc(pb.n_prog);
         pack_fixed_kernel<<<div_up(pb.n_prog, 8), 256, 0, pb.st>>>(pb.w64.p, pb.idx.p, pb.n_prog, pb.n, nops, pb.diff,
                                                                    pb.n_slots, pb.SLQ, pb.G, dcomb.p, (int2 *)pb.pw.p,
                                                                    pb.pidx.p, pb.wexp.p);
