@@ -17,9 +17,13 @@
 // each row is kept where its entries exceed 2^-8 eps of the row's largest:
 // the dropped part is below the rounding of the kept sum.  A CTA whose
 // stencils read ghosts solves for them itself from its shared-memory records:
-// in FP32 straight (ghosts_from_records), in FP64 by the residuals of the wall
-// rows, each formed by the CTA that owns its wall node and passed through
-// global memory, then the banded rows.
+// the residuals of the wall rows in the bands (in FP64 each formed by the CTA
+// that owns its wall node and passed through global memory), then the banded
+// rows.  The two steps stay apart: coefficients of the ghosts on the records
+// (products of the two, formed in FP64 and rounded once) took 770 in place of
+// 950 us for 50 steps at 400 m in FP32, but their sums do not keep the
+// residuals small, and runs in walled boxes were 1.3 to 1.7 times further from
+// FP64 (tests/test_gpu_persistent_accuracy.py).
 //
 // Learned correction (a9, MLP variants): at stage 0 of every step the CTA's
 // shared memory holds the step-start records of its stencils, ghosts
@@ -224,21 +228,6 @@ struct CtaInfo {
     int64_t blob_off;   // byte offset of its constant block
     int32_t blob_bytes;
     int32_t o_rw, o_rinfo, o_gc, o_cidx, o_cval;   // sections of the block (row slots at 0)
-    // FP32: ghost values straight from the records (n_gh > 0; the row sections
-    // above are then empty): pairs of ghosts at 0, list positions, coefficients
-    int32_t n_gh, o_pos, o_comp;
-    int32_t n_hy, o_hy, o_b;   // hydrostatic wall nodes of all pairs (records), their b of the stage
-};
-
-constexpr int kGhostPad = 96;   // three records for each lane of a warp
-
-// Two ghosts of a CTA (FP32): the records they read and their coefficients.
-struct GhostPair {
-    int32_t pos, n_j;      // first list position, number of records (a multiple of kGhostPad)
-    int32_t comp;          // coefficients [class][2][n_j]
-    int32_t tb, n_tb;      // hydrostatic wall nodes in their bands (index among the CTA's) and
-    int32_t binv;          // the inverse rows' entries there [2][n_tb]
-    int32_t unused[2];
 };
 
 __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~size_t(15); }
@@ -258,7 +247,6 @@ struct PArgs {
     int SLQ, chunk, npad;
     unsigned ring_off;              // FP64: byte offset of the operands' ring (0: streamed without)
     T cp_tb2, cp_tb, gconst;        // c_p theta_bar^2, c_p theta_bar, g
-    int4 field_class;               // boundary-operator class of each field
     T cp, g_over_tb, theta_bar, dpibar, rd_cv;
     T an0, an1, an2, bs0, bs1, bs2, bs3;
     int64_t n_steps;
@@ -388,106 +376,6 @@ __host__ __device__ __forceinline__ int lanes_for(int items, int threads, int mo
     int l = most;
     while (l > 1 && items * l > threads) l >>= 1;
     return l;
-}
-
-// FP32: the CTA's ghost values from its records in one step.  The solve
-// u_G = W_G^{-1} (b - W_I u_I - W_B u_B) is linear in the records apart from b,
-// so the plan holds per ghost and operator class the products of its banded
-// inverse row with the wall rows' weights (in FP64, rounded once), one
-// coefficient per record that any of its rows reads; the pi' rows'
-// hydrostatic b enters with the inverse row itself.  A warp takes two ghosts,
-// its lanes the records.  The two-step form (residuals of every wall row in
-// the bands, a CTA barrier, the banded rows) took 3,680 of a stage's 11,700
-// clocks in the 400 m density current (38 CTAs); this one takes 1,750 of 8,700.
-// It stays for FP64, whose coefficients would not fit shared memory.
-//
-// What bounds it: chains of dependent shared-memory reads in few warps.  L lanes
-// take a pair, three records each per pass, so that three chains overlap.
-template <int L>
-__device__ __forceinline__ void ghosts_from_records(const PArgs<float> &a, const CtaInfo &ci, float *halo,
-                                                    const unsigned char *blob) {
-    const GhostPair *pairs = reinterpret_cast<const GhostPair *>(blob);
-    const uint16_t *pos = reinterpret_cast<const uint16_t *>(blob + ci.o_pos);
-    const float *coef = reinterpret_cast<const float *>(blob + ci.o_comp);
-    const float *hydro = reinterpret_cast<const float *>(blob + ci.o_b);
-    const int np = (ci.n_gh + 1) / 2, lane = threadIdx.x & (L - 1), step = blockDim.x / L;
-    const int4 fc = a.field_class;
-    const bool c2 = fc.z != fc.x, c3 = fc.w != fc.z;   // classes of theta', pi' of their own
-    for (int q0 = threadIdx.x / L; (q0 & ~(32 / L - 1)) < np; q0 += step) {   // uniform per warp: it holds 32 / L pairs
-        const int q = min(q0, np - 1);
-        const GhostPair g = pairs[q];
-        const int n_j = g.n_j;
-        const uint16_t *J = pos + g.pos, *tb = pos + g.tb;
-        const float *p0 = coef + g.comp + fc.x * 2 * n_j, *p1 = coef + g.comp + fc.y * 2 * n_j;
-        const float *p2 = coef + g.comp + fc.z * 2 * n_j, *p3 = coef + g.comp + fc.w * 2 * n_j;
-        const float *binv = coef + g.binv;
-        float s[8] = {};   // [ghost][field]
-#pragma unroll 1
-        for (int j0 = lane; j0 < n_j; j0 += 3 * L) {
-#pragma unroll
-            for (int u = 0; u < 3; ++u) {
-                const int j = j0 + u * L;
-                const Rec<float> r = sh_rec(halo, J[j]);
-                float v0 = p0[j], v1 = p0[j + n_j];
-                s[0] += v0 * r.u;
-                s[4] += v1 * r.u;
-                s[1] += p1[j] * r.w;
-                s[5] += p1[j + n_j] * r.w;
-                if (c2) {
-                    v0 = p2[j];
-                    v1 = p2[j + n_j];
-                }
-                s[2] += v0 * r.t;
-                s[6] += v1 * r.t;
-                if (c3) {
-                    v0 = p3[j];
-                    v1 = p3[j + n_j];
-                }
-                s[3] += v0 * r.p;
-                s[7] += v1 * r.p;
-            }
-        }
-#pragma unroll 2
-        for (int r = lane; r < g.n_tb; r += L) {
-            const float b = hydro[tb[r]];
-            s[3] += binv[r] * b;
-            s[7] += binv[g.n_tb + r] * b;
-        }
-        // the eight sums over the lanes: each exchange halves the values a lane holds
-        __syncwarp();
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const int o = L >> (k + 1), n = 4 >> k;
-            const bool up = lane & o;
-#pragma unroll
-            for (int v = 0; v < n; ++v) {
-                const float send = up ? s[v] : s[v + n], keep = up ? s[v + n] : s[v];
-                s[v] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-            }
-        }
-#pragma unroll
-        for (int k = L / 16; k > 0; k >>= 1) s[0] += __shfl_xor_sync(0xffffffffu, s[0], k);
-        const int v = lane / (L / 8);   // the sum this lane holds: ghost * 4 + field
-        if (q0 < np && lane % (L / 8) == 0 && (v < 4 || 2 * q + 1 < ci.n_gh))
-            halo[(size_t)(ci.n_load + 2 * q + (v >> 2)) * 4 + (v & 3)] = s[0];
-    }
-}
-
-// pi'_z = g theta' / (c_p theta_bar (theta_bar + theta')) at the CTA's
-// hydrostatic wall nodes, from the stage input itself: the first read goes out
-// ahead of the record copies (th0), the division runs while they are in flight
-// (formed per pair of ghosts, the divisions took 650 clocks).
-__device__ __forceinline__ float hydrostatic_read(const CtaInfo &ci, const float *Uin, const unsigned char *blob, int r) {
-    const int32_t *rec = reinterpret_cast<const int32_t *>(blob + ci.o_hy);
-    return r < ci.n_hy ? __ldcg(Uin + (int64_t)rec[r] * 4 + 2) : 0.f;
-}
-__device__ __forceinline__ void hydrostatic(const PArgs<float> &a, const CtaInfo &ci, const float *Uin,
-                                            unsigned char *blob, float th0) {
-    float *b = reinterpret_cast<float *>(blob + ci.o_b);
-    for (int r = threadIdx.x; r < ci.n_hy; r += blockDim.x) {
-        const float th = r < (int)blockDim.x ? th0 : hydrostatic_read(ci, Uin, blob, r);
-        b[r] = a.gconst * th / (a.cp_tb2 + a.cp_tb * th);
-    }
 }
 
 // a9 at stage 0: delta of the CTA's own nodes from the records in shared
@@ -741,126 +629,100 @@ __global__ void __launch_bounds__(MAXT, 1) rk4_persistent(const __grid_constant_
             if (first) {
                 cp_async_wait();   // the constant block and the records issued at entry
             } else {
-                T th0 = 0;
-                if constexpr (!FIX) {
-                    if (ci.n_gh > 0) th0 = hydrostatic_read(ci, Uin, blob, threadIdx.x);
-                }
                 const int wend = ci.n_own + ci.n_wload;
                 for (int k = ci.n_own + threadIdx.x; k < wend; k += blockDim.x) cp_rec(halo, k, Uin, __ldg(hl + k));
                 cp_async_commit();
                 for (int k = wend + threadIdx.x; k < ci.n_load; k += blockDim.x) cp_rec(halo, k, Uin, __ldg(hl + k));
                 cp_async_commit();
-                if constexpr (!FIX) {
-                    if (ci.n_gh > 0) hydrostatic(a, ci, Uin, blob, th0);
-                }
-                if (ci.n_gh > 0 || ci.n_crows > 0) cp_async_wait_pending<1>();
+                if (ci.n_crows > 0) cp_async_wait_pending<1>();
                 else cp_async_wait_pending<0>();
             }
             __syncthreads();
-            bool solved = false;
-            if constexpr (!FIX) {
-                if (ci.n_gh > 0) {
-                    if (first) {   // the block has only just arrived
-                        hydrostatic(a, ci, Uin, blob, hydrostatic_read(ci, Uin, blob, threadIdx.x));
-                        __syncthreads();
-                    }
-                    // lanes per pair: a warp's, or half or a quarter where one pass
-                    // of the CTA's warps then covers every pair
-                    const int np = (ci.n_gh + 1) / 2;
-                    if (np * 32 <= (int)blockDim.x) ghosts_from_records<32>(a, ci, halo, blob);
-                    else if (np * 16 <= (int)blockDim.x) ghosts_from_records<16>(a, ci, halo, blob);
-                    else ghosts_from_records<8>(a, ci, halo, blob);
-                    __syncthreads();
-                    solved = true;
-                }
-            }
-            if (!solved) {   // FP64, and FP32 CTAs whose coefficients do not fit
-                if (ci.n_crows > 0) {
-                    // ---- residuals b - W_I u_I - W_B u_B of its wall rows -----------
-                    // L lanes per row, L the largest of 8, 4, 2, 1 that lets one pass
-                    // of the CTA's threads cover every row
-                    const int L = lanes_for(ci.n_crows, blockDim.x, row_lanes(FIX));
-                    const int per = a.npad / L;
-                    const int nlr = (ci.n_crows * L + 31) & ~31;
-                    for (int e = threadIdx.x; e < nlr; e += blockDim.x) {
-                        int r = e / L;
-                        const int ln = e % L;
-                        const bool rl = r < ci.n_crows;
-                        if (!rl) r = ci.n_crows - 1;
-                        const int inf = rinfo[r];
-                        // slot-major [set][slot][row_pad]: the lanes of a warp read
-                        // consecutive rows of one slot
-                        const size_t RP = ci.row_pad, step = (size_t)L * RP;
-                        const T *w0 = rw + ((size_t)((inf >> 17) & 3) * a.npad + ln) * RP + r;
-                        const T *w1 = rw + ((size_t)((inf >> 19) & 3) * a.npad + ln) * RP + r;
-                        const T *w2 = rw + ((size_t)((inf >> 21) & 3) * a.npad + ln) * RP + r;
-                        const T *w3 = rw + ((size_t)((inf >> 23) & 3) * a.npad + ln) * RP + r;
-                        const uint16_t *rj = ridx + (size_t)ln * RP + r;
-                        T a0 = 0, a1 = 0, a2 = 0, a3 = 0;
+            if (ci.n_crows > 0) {
+                // ---- residuals b - W_I u_I - W_B u_B of its wall rows -----------
+                // L lanes per row, L the largest of 8, 4, 2, 1 that lets one pass
+                // of the CTA's threads cover every row
+                const int L = lanes_for(ci.n_crows, blockDim.x, row_lanes(FIX));
+                const int per = a.npad / L;
+                const int nlr = (ci.n_crows * L + 31) & ~31;
+                for (int e = threadIdx.x; e < nlr; e += blockDim.x) {
+                    int r = e / L;
+                    const int ln = e % L;
+                    const bool rl = r < ci.n_crows;
+                    if (!rl) r = ci.n_crows - 1;
+                    const int inf = rinfo[r];
+                    // slot-major [set][slot][row_pad]: the lanes of a warp read
+                    // consecutive rows of one slot
+                    const size_t RP = ci.row_pad, step = (size_t)L * RP;
+                    const T *w0 = rw + ((size_t)((inf >> 17) & 3) * a.npad + ln) * RP + r;
+                    const T *w1 = rw + ((size_t)((inf >> 19) & 3) * a.npad + ln) * RP + r;
+                    const T *w2 = rw + ((size_t)((inf >> 21) & 3) * a.npad + ln) * RP + r;
+                    const T *w3 = rw + ((size_t)((inf >> 23) & 3) * a.npad + ln) * RP + r;
+                    const uint16_t *rj = ridx + (size_t)ln * RP + r;
+                    T a0 = 0, a1 = 0, a2 = 0, a3 = 0;
 #pragma unroll 4
-                        for (int t = 0; t < per; ++t) {
-                            const Rec<T> v = sh_rec(halo, rj[t * step]);
-                            a0 += w0[t * step] * v.u;
-                            a1 += w1[t * step] * v.w;
-                            a2 += w2[t * step] * v.t;
-                            a3 += w3[t * step] * v.p;
-                        }
-                        for (int o = L / 2; o > 0; o >>= 1) {
-                            a0 += __shfl_xor_sync(0xffffffffu, a0, o, L);
-                            a1 += __shfl_xor_sync(0xffffffffu, a1, o, L);
-                            a2 += __shfl_xor_sync(0xffffffffu, a2, o, L);
-                            a3 += __shfl_xor_sync(0xffffffffu, a3, o, L);
-                        }
-                        if (rl) {
+                    for (int t = 0; t < per; ++t) {
+                        const Rec<T> v = sh_rec(halo, rj[t * step]);
+                        a0 += w0[t * step] * v.u;
+                        a1 += w1[t * step] * v.w;
+                        a2 += w2[t * step] * v.t;
+                        a3 += w3[t * step] * v.p;
+                    }
+                    for (int o = L / 2; o > 0; o >>= 1) {
+                        a0 += __shfl_xor_sync(0xffffffffu, a0, o, L);
+                        a1 += __shfl_xor_sync(0xffffffffu, a1, o, L);
+                        a2 += __shfl_xor_sync(0xffffffffu, a2, o, L);
+                        a3 += __shfl_xor_sync(0xffffffffu, a3, o, L);
+                    }
+                    if (rl) {
 #pragma unroll
-                            for (int f = 0; f < 4; ++f) {
-                                if (f % L != ln) continue;
-                                const T acc = f == 0 ? a0 : f == 1 ? a1 : f == 2 ? a2 : a3;
-                                T b = 0;
-                                if (f == 3 && (inf & (1 << 16))) {
-                                    // pi'_z = g theta' / (c_p theta_bar (theta_bar + theta')) at the wall node
-                                    const T th = halo[(size_t)(inf & 0xffff) * 4 + 2];
-                                    b = a.gconst * th / (a.cp_tb2 + a.cp_tb * th);
-                                }
-                                if (a.own_rows) a.resg[f * a.ng + ogp[r]] = b - acc;
-                                else res[f * ci.n_rows + r] = b - acc;
+                        for (int f = 0; f < 4; ++f) {
+                            if (f % L != ln) continue;
+                            const T acc = f == 0 ? a0 : f == 1 ? a1 : f == 2 ? a2 : a3;
+                            T b = 0;
+                            if (f == 3 && (inf & (1 << 16))) {
+                                // pi'_z = g theta' / (c_p theta_bar (theta_bar + theta')) at the wall node
+                                const T th = halo[(size_t)(inf & 0xffff) * 4 + 2];
+                                b = a.gconst * th / (a.cp_tb2 + a.cp_tb * th);
                             }
+                            if (a.own_rows) a.resg[f * a.ng + ogp[r]] = b - acc;
+                            else res[f * ci.n_rows + r] = b - acc;
                         }
                     }
-                    __syncthreads();
                 }
-                if (a.own_rows && (ci.n_rows > 0 || ci.n_crows > 0)) {
-                    // ---- the band rows' residuals, formed by the CTAs owning their
-                    // wall nodes, once every CTA that forms or reads them is here
-                    if (!cta_barrier(a.arrive2, a.abort, target2, (unsigned)a.wall_ctas, a.spin_limit)) return;
-                    for (int e = threadIdx.x; e < 4 * ci.n_rows; e += blockDim.x) {
-                        const int f = e / ci.n_rows, k = e % ci.n_rows;
-                        res[e] = __ldcg(a.resg + f * a.ng + brow[k]);
-                    }
-                    __syncthreads();
-                }
-                if (ci.n_rows > 0) {
-                    // ---- ghost values from the banded inverse rows -------------------
-                    // M lanes per (ghost, field): every lane of a warp has the same
-                    // work, so no FP64 instruction runs for idle lanes
-                    const int M = lanes_for(ci.n_gc, blockDim.x, kPairLanes);
-                    const int npl = (ci.n_gc * M + 31) & ~31;
-                    for (int e = threadIdx.x; e < npl; e += blockDim.x) {
-                        const int k0 = e / M, ln = e % M;
-                        const int4 gc = gcs[k0 < ci.n_gc ? k0 : ci.n_gc - 1];   // list position, field, coefficients, count
-                        const size_t PP = ci.pair_pad;   // coefficients [entry][pair_pad]
-                        const uint16_t *cj = cidx + gc.z;
-                        const T *cv = cval + gc.z, *rf = res + gc.y * ci.n_rows;
-                        T sum = 0;
-#pragma unroll 4
-                        for (int j = ln; j < gc.w; j += M) sum += cv[j * PP] * rf[cj[j * PP]];
-                        for (int o = M / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o, M);
-                        if (k0 < ci.n_gc && ln == 0) halo[(size_t)gc.x * 4 + gc.y] = sum;
-                    }
-                    __syncthreads();
-                }
+                __syncthreads();
             }
-            if (ci.n_gh > 0 || ci.n_crows > 0) {
+            if (a.own_rows && (ci.n_rows > 0 || ci.n_crows > 0)) {
+                // ---- the band rows' residuals, formed by the CTAs owning their
+                // wall nodes, once every CTA that forms or reads them is here
+                if (!cta_barrier(a.arrive2, a.abort, target2, (unsigned)a.wall_ctas, a.spin_limit)) return;
+                for (int e = threadIdx.x; e < 4 * ci.n_rows; e += blockDim.x) {
+                    const int f = e / ci.n_rows, k = e % ci.n_rows;
+                    res[e] = __ldcg(a.resg + f * a.ng + brow[k]);
+                }
+                __syncthreads();
+            }
+            if (ci.n_rows > 0) {
+                // ---- ghost values from the banded inverse rows -------------------
+                // M lanes per (ghost, field): every lane of a warp has the same
+                // work, so no FP64 instruction runs for idle lanes
+                const int M = lanes_for(ci.n_gc, blockDim.x, kPairLanes);
+                const int npl = (ci.n_gc * M + 31) & ~31;
+                for (int e = threadIdx.x; e < npl; e += blockDim.x) {
+                    const int k0 = e / M, ln = e % M;
+                    const int4 gc = gcs[k0 < ci.n_gc ? k0 : ci.n_gc - 1];   // list position, field, coefficients, count
+                    const size_t PP = ci.pair_pad;   // coefficients [entry][pair_pad]
+                    const uint16_t *cj = cidx + gc.z;
+                    const T *cv = cval + gc.z, *rf = res + gc.y * ci.n_rows;
+                    T sum = 0;
+#pragma unroll 4
+                    for (int j = ln; j < gc.w; j += M) sum += cv[j * PP] * rf[cj[j * PP]];
+                    for (int o = M / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o, M);
+                    if (k0 < ci.n_gc && ln == 0) halo[(size_t)gc.x * 4 + gc.y] = sum;
+                }
+                __syncthreads();
+            }
+            if (ci.n_crows > 0) {
                 cp_async_wait_pending<0>();   // the rest of the list (no-op at the first stage)
                 __syncthreads();
             }
@@ -1172,7 +1034,6 @@ PArgs<T> pargs(Problem &pb, T *U, double dt, int64_t n_steps) {
     a.ring_off = ps.ring_off;
     a.cp_tb2 = (T)(pb.cp * pb.theta_bar * pb.theta_bar);
     a.cp_tb = a.cp_tb2 / (T)pb.theta_bar;
-    a.field_class = make_int4(pb.gh.field_class[0], pb.gh.field_class[1], pb.gh.field_class[2], pb.gh.field_class[3]);
     a.gconst = (T)pb.g;
     a.cp = (T)pb.cp;
     a.g_over_tb = (T)(pb.g / pb.theta_bar);
@@ -1261,133 +1122,6 @@ int allow_dynamic_smem(void *fn, int optin) {
     const int most = optin - (int)fa.sharedSizeBytes;
     RBF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     return most;
-}
-
-// Rows of the ghost values as functions of the records, [class * ng + position]:
-// (record, coefficient) with the coefficients -sum over the banded inverse row's
-// wall rows of its entry times the wall row's weight, formed in FP64.
-std::vector<std::vector<std::pair<int32_t, double>>> ghost_rows(
-    const GhostPlan &gh, int64_t ng, int npad, int64_t n_all,
-    const std::vector<std::vector<std::pair<int32_t, double>>> &band, const std::vector<int32_t> &at,
-    const std::vector<int32_t> &gidx, const std::vector<unsigned char> &gw) {
-    const float *w = reinterpret_cast<const float *>(gw.data());   // [4][ng][npad]
-    std::vector<std::vector<std::pair<int32_t, double>>> out((size_t)gh.n_class * ng);
-    std::vector<double> sum(n_all, 0.0);
-    std::vector<char> seen(n_all, 0);
-    std::vector<int32_t> used;
-    for (int f = 3; f >= 0; --f) {   // one field per class: its fields share their weights
-        const int cl = gh.field_class[f];
-        if (!out[(size_t)cl * ng].empty()) continue;
-        for (int64_t q = 0; q < ng; ++q) {
-            used.clear();
-            for (const auto &e : band[(size_t)cl * ng + q]) {
-                const int32_t r = at[e.first];
-                for (int t = 0; t < npad; ++t) {
-                    const double v = w[((size_t)f * ng + r) * npad + t];
-                    if (v == 0.0) continue;
-                    const int32_t j = gidx[(size_t)r * npad + t];
-                    if (!seen[j]) {
-                        seen[j] = 1;
-                        used.push_back(j);
-                    }
-                    sum[j] -= e.second * v;
-                }
-            }
-            auto &row = out[(size_t)cl * ng + q];
-            row.reserve(used.size());
-            for (int32_t j : used) {
-                row.emplace_back(j, sum[j]);
-                sum[j] = 0.0;
-                seen[j] = 0;
-            }
-        }
-    }
-    return out;
-}
-
-// The ghost block of an FP32 CTA (ghosts_from_records): per pair of its ghosts
-// the records they read, the coefficients (rounded once) and the pi' rows'
-// entries at the hydrostatic wall nodes.  Fills ci's section offsets.
-std::vector<unsigned char> ghost_pairs(const std::vector<int32_t> &ghosts, const GhostPlan &gh, int64_t ng, int64_t P,
-                                       const std::vector<std::vector<std::pair<int32_t, double>>> &band,
-                                       const std::vector<std::vector<std::pair<int32_t, double>>> &rows,
-                                       const std::vector<int32_t> &posv, const std::vector<int32_t> &at,
-                                       const std::vector<int32_t> &owner, const std::vector<unsigned char> &tbv,
-                                       const std::vector<int32_t> &loc, CtaInfo &ci) {
-    std::vector<int32_t> hydro;            // records of the CTA's hydrostatic wall nodes
-    std::vector<int32_t> index(ng, -1);    // their index by wall row
-    std::vector<GhostPair> pairs;
-    std::vector<uint16_t> pos;
-    std::vector<float> coef;
-    std::vector<int32_t> used, hyd;        // list positions and hydrostatic nodes of the pair
-    std::vector<char> seen(ci.n_list, 0);
-    // [class * 2 + ghost][list position], [ghost][hydrostatic node]
-    std::vector<std::vector<double>> c((size_t)gh.n_class * 2, std::vector<double>(ci.n_list, 0.0)), hb(2);
-    for (size_t k = 0; k < ghosts.size(); k += 2) {
-        used.clear();
-        hyd.clear();
-        for (int s = 0; s < 2 && k + s < ghosts.size(); ++s) {
-            const int64_t q = posv[ghosts[k + s] - P];
-            for (int cl = 0; cl < gh.n_class; ++cl)
-                for (const auto &e : rows[(size_t)cl * ng + q]) {
-                    const int32_t l = loc[e.first];
-                    seen[l] = 1;
-                    c[(size_t)cl * 2 + s][l] = e.second;
-                }
-            for (const auto &e : band[(size_t)gh.field_class[3] * ng + q]) {
-                const int32_t r = at[e.first];
-                if (!tbv[r]) continue;
-                if (index[r] < 0) {
-                    index[r] = (int32_t)hydro.size();
-                    hydro.push_back(owner[r]);
-                    hb[0].push_back(0.0);
-                    hb[1].push_back(0.0);
-                }
-                if (hb[0][index[r]] == 0.0 && hb[1][index[r]] == 0.0) hyd.push_back(index[r]);
-                hb[s][index[r]] = e.second;   // kept entries are not zero
-            }
-        }
-        for (int32_t l = 0; l < ci.n_list; ++l)
-            if (seen[l]) used.push_back(l);
-        const size_t real = used.size();
-        while (used.size() % kGhostPad) used.push_back(used[0]);   // padded with a record it reads anyway, coefficient 0
-        GhostPair g{};
-        g.pos = (int32_t)pos.size();
-        g.n_j = (int32_t)used.size();
-        for (int32_t l : used) pos.push_back((uint16_t)l);
-        g.comp = (int32_t)coef.size();
-        coef.resize(coef.size() + c.size() * used.size(), 0.f);
-        for (size_t r = 0; r < c.size(); ++r) {
-            float *to = coef.data() + g.comp + r * used.size();
-            for (size_t j = 0; j < real; ++j) {
-                to[j] = (float)c[r][used[j]];
-                c[r][used[j]] = 0.0;
-            }
-        }
-        for (int32_t l : used) seen[l] = 0;
-        g.tb = (int32_t)pos.size();
-        g.n_tb = (int32_t)hyd.size();
-        g.binv = (int32_t)coef.size();
-        for (int32_t h : hyd) pos.push_back((uint16_t)h);
-        for (auto &row : hb)
-            for (int32_t h : hyd) {
-                coef.push_back((float)row[h]);
-                row[h] = 0.0;
-            }
-        pairs.push_back(g);
-    }
-    std::vector<unsigned char> b;
-    put(b, 0, pairs.data(), pairs.size() * sizeof(GhostPair));
-    ci.o_pos = (int32_t)align16(b.size());
-    put(b, ci.o_pos, pos.data(), pos.size() * 2);
-    ci.o_comp = (int32_t)align16(b.size());
-    put(b, ci.o_comp, coef.data(), coef.size() * 4);
-    ci.n_hy = (int32_t)hydro.size();
-    ci.o_hy = (int32_t)align16(b.size());
-    put(b, ci.o_hy, hydro.data(), hydro.size() * 4);
-    ci.o_b = (int32_t)align16(b.size());
-    b.resize(align16((size_t)ci.o_b + hydro.size() * 4), 0);
-    return b;
 }
 
 }  // namespace
@@ -1634,21 +1368,6 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
             }
         }
 
-        // FP32: ghost values straight from the records, where the coefficients fit
-        const size_t list_bytes = align16((size_t)n_list * 4 * ts);
-        if (!own && !ghosts.empty()) {
-            if (ps.ghost_rows.empty()) ps.ghost_rows = ghost_rows(gh, ng, npad, pb.n_all, band, at, gidx, gwv);
-            const std::vector<unsigned char> b =
-                ghost_pairs(ghosts, gh, ng, P, band, ps.ghost_rows, posv, at, owner, tbv, loc, ci);
-            if (list_bytes + b.size() <= (size_t)smem_optin) {
-                ci.n_gh = (int32_t)ghosts.size();
-                ci.blob_off = (int64_t)blob.size();
-                ci.blob_bytes = (int32_t)b.size();
-                blob.insert(blob.end(), b.begin(), b.end());
-                smem_max = std::max(smem_max, list_bytes + b.size());
-                continue;
-            }
-        }
         // ghost block: row slots, weight sets, row info, pairs, band coefficients
         const int n_rows = (int)rows.size(), n_crows = (int)crows.size();
         ci.n_rows = n_rows;
@@ -1767,7 +1486,7 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
             ci.blob_bytes = (int32_t)b.size();
             blob.insert(blob.end(), b.begin(), b.end());
         }
-        const size_t sm = list_bytes + align16((size_t)n_rows * 4 * ts) + ci.blob_bytes;
+        const size_t sm = align16((size_t)n_list * 4 * ts) + align16((size_t)n_rows * 4 * ts) + ci.blob_bytes;
         smem_max = std::max(smem_max, sm);
     }
     if (smem_max > (size_t)smem_optin) return false;

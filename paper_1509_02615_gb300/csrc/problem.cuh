@@ -95,9 +95,6 @@ struct PersistPlan {
     DevBuf<int32_t> hlist;       // record lists of all CTAs
     DevBuf<unsigned char> cta;   // per-CTA layout records
     DevBuf<unsigned char> blob;  // per-CTA ghost-row and ghost-value data
-    // FP32: ghost values as functions of the records, per class and ghost (host;
-    // the same for every plan of the problem)
-    std::vector<std::vector<std::pair<int32_t, double>>> ghost_rows;
     DevBuf<unsigned int> arrive; // barrier arrivals, monotone across launches
     unsigned base = 0;           // its value when the next launch starts
     DevBuf<int> abort;           // set when a barrier wait gives up (sticky until rbf_sync)
