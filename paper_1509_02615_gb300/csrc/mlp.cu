@@ -32,7 +32,6 @@ constexpr int kWidth = 64;
 constexpr int kTrainRows = 32;               // rows of a training block: 31 samples and the all-zero row
 constexpr int kTrainSamples = kTrainRows - 1;
 constexpr int kTrainThreads = 320;           // 10 warps: two passes over the 592 tiles of dW1 (n = 37)
-constexpr int kMaxInputs = 240;              // widest input layer (stencils of up to 60 nodes)
 constexpr int kScaleWarps = 2048;   // warps of the scale-sum launch (256 blocks of 256 threads)
 constexpr float kClip = 4.f;   // |y| <= 4 (in output-scale units) when the correction is applied
 

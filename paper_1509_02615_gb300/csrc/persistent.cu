@@ -1129,6 +1129,7 @@ int allow_dynamic_smem(void *fn, int optin) {
 bool persistent_plan(Problem &pb, int G, int ctas) {
     PersistPlan &ps = pb.ps;
     ps.ready = false;
+    ps.net_smem = 0;
     if (pb.kind != kNS) return false;
     int dev = 0, coop = 0, smem_optin = 0;
     RBF_CUDA(cudaGetDevice(&dev));
@@ -1194,7 +1195,15 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
     }
     if (pick < 0) return false;
     threads = std::max(threads, std::min(vs[pick].maxt, 512));
+    // corrected runs (a9): the kernel with the network, the network's shared memory
+    // and the most that kernel may have
+    void *net_fn = nullptr;
+    for (const Variant &v : vs)
+        if (v.mlp && v.G == S && v.R == vs[pick].R && threads <= v.maxt && 4 * pb.n <= kMaxInputs) net_fn = v.fn;
+    const size_t net_bytes = net_fn ? mlp_layout(4 * pb.n_slots + 4, chunk, pb.n_slots).end : 0;
+    const size_t net_most = net_fn ? (size_t)allow_dynamic_smem(net_fn, smem_optin) : 0;
     smem_optin = allow_dynamic_smem(vs[pick].fn, smem_optin);
+    const size_t room = net_fn && net_most > net_bytes ? std::min(net_most - net_bytes, (size_t)smem_optin) : smem_optin;
 
     // ---- blocks -----------------------------------------------------------------
     std::vector<double> x(P), z(P);
@@ -1376,7 +1385,10 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
         rows_max = std::max(rows_max, n_rows);
         if (n_crows > 0 && n_rows == 0) return false;   // a wall node whose stencil reads no ghost
         if (n_rows > 0) ++wall_ctas;
-        if (n_rows > 0) {
+        // padded: rows and pairs at strides without bank conflicts (up to 31 more of each)
+        auto ghost_block = [&](bool padded) {
+            std::vector<unsigned char> b;
+            if (n_rows == 0) return b;
             // distinct weight sets of each formed row (fields with the same boundary operator share one)
             std::vector<std::vector<int>> setof(n_crows, std::vector<int>(4, 0));
             std::vector<std::vector<int>> sets(n_crows);
@@ -1403,9 +1415,8 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
             // each) start 32 / L banks apart
             const int L = lanes_for(std::max(n_crows, 1), threads, row_lanes(fp64));
             int RP = std::max(n_crows, 1);
-            while (RP % 32 != (32 / L) % 32) ++RP;
+            while (padded && RP % 32 != (32 / L) % 32) ++RP;
             ci.row_pad = RP;
-            std::vector<unsigned char> b;
             std::vector<uint16_t> rs((size_t)npad * RP, 0);
             std::vector<int32_t> ri(n_crows);
             for (int k = 0; k < n_crows; ++k) {
@@ -1447,7 +1458,7 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
             const int n_gc = 4 * (int)ghosts.size();   // (ghost, field) items: every field has one class
             const int Mp = lanes_for(n_gc, threads, kPairLanes);
             int PPd = std::max(n_pair, 1);
-            while (PPd % 32 != (32 / Mp) % 32) ++PPd;
+            while (padded && PPd % 32 != (32 / Mp) % 32) ++PPd;
             ci.pair_pad = PPd;
             std::vector<int32_t> gcv;
             std::vector<uint16_t> cix(maxlen * PPd, 0);
@@ -1483,11 +1494,20 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
             ci.o_cval = (int32_t)align16(b.size());
             put(b, ci.o_cval, cvl.data(), cvl.size());
             b.resize(align16(b.size()), 0);
-            ci.blob_bytes = (int32_t)b.size();
-            blob.insert(blob.end(), b.begin(), b.end());
+            return b;
+        };
+        // without the padding where it takes the room of the network, or of the plan
+        const size_t beside = align16((size_t)n_list * 4 * ts) + align16((size_t)n_rows * 4 * ts);
+        std::vector<unsigned char> b = ghost_block(true);
+        if (beside + b.size() > room) {
+            const CtaInfo ci0 = ci;
+            std::vector<unsigned char> tight = ghost_block(false);
+            if (beside + tight.size() <= room || beside + b.size() > (size_t)smem_optin) b.swap(tight);
+            else ci = ci0;
         }
-        const size_t sm = align16((size_t)n_list * 4 * ts) + align16((size_t)n_rows * 4 * ts) + ci.blob_bytes;
-        smem_max = std::max(smem_max, sm);
+        ci.blob_bytes = (int32_t)b.size();
+        blob.insert(blob.end(), b.begin(), b.end());
+        smem_max = std::max(smem_max, beside + b.size());
     }
     if (smem_max > (size_t)smem_optin) return false;
     // FP64: room for the operands' ring, where shared memory has it
@@ -1503,6 +1523,10 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
     int per_sm = 0;
     RBF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, vs[pick].fn, threads, smem_max));
     if ((int64_t)per_sm * nsm < grid) return false;
+    if (net_fn && smem_max + net_bytes <= net_most) {
+        RBF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, net_fn, threads, smem_max + net_bytes));
+        if ((int64_t)per_sm * nsm >= grid) ps.net_smem = smem_max + net_bytes;
+    }
 
     ps.G = G;
     ps.S = S;
@@ -1693,7 +1717,7 @@ void adv_persistent_run(Problem &pb, double t0, double dt, int64_t n_steps, void
 }
 
 bool persistent_mlp_ready(const Problem &pb) {
-    return pb.kind == kNS && pb.precision == 32 && pb.ps.ready && pb.diff == 1 && mlp_variant_fn(pb.ps, 32) != nullptr;
+    return pb.kind == kNS && pb.precision == 32 && pb.ps.ready && pb.diff == 1 && pb.ps.net_smem > 0;
 }
 
 void persistent_run_mlp(Problem &pb, double dt, int64_t n_steps, void *U, cudaStream_t s, const MlpView &mv) {
@@ -1702,12 +1726,6 @@ void persistent_run_mlp(Problem &pb, double dt, int64_t n_steps, void *U, cudaSt
     RBF_REQUIRE(mv.n_in == 4 * pb.n_slots + 4, "network inputs %d do not match the stencil", mv.n_in);
     if (n_steps <= 0) return;
     void *fn = mlp_variant_fn(ps, 32);
-    int smem_optin = 0, dev = 0;
-    RBF_CUDA(cudaGetDevice(&dev));
-    RBF_CUDA(cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    const size_t smem = ps.smem + mlp_layout(mv.n_in, ps.chunk, pb.n_slots).end;
-    smem_optin = allow_dynamic_smem(fn, smem_optin);
-    RBF_REQUIRE(smem <= (size_t)smem_optin, "network does not fit shared memory beside the record lists");
     PArgs<float> a = pargs<float>(pb, (float *)U, dt, n_steps);
     a.mW = reinterpret_cast<const __nv_bfloat16 *>(mv.Pb);
     a.mP = mv.P;
@@ -1719,7 +1737,7 @@ void persistent_run_mlp(Problem &pb, double dt, int64_t n_steps, void *U, cudaSt
     a.mslots = pb.n_slots;
     a.mbad = mv.bad;
     void *args[] = {&a};
-    RBF_CUDA(cudaLaunchCooperativeKernel(fn, dim3(ps.grid), dim3(ps.threads), args, smem, s));
+    RBF_CUDA(cudaLaunchCooperativeKernel(fn, dim3(ps.grid), dim3(ps.threads), args, ps.net_smem, s));
     ps.base += (unsigned)((uint64_t)ps.grid * (uint64_t)(4 * n_steps - 1));
 }
 
@@ -1753,9 +1771,6 @@ namespace rbf {
 bool persistent_tune_mlp(Problem &pb, const MlpView &mv) {
     if (pb.kind != kNS || pb.precision != 32 || !pb.S0.p) return false;
     const int nsm = sm_count();
-    int dev = 0, optin = 0;
-    RBF_CUDA(cudaGetDevice(&dev));
-    RBF_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     const size_t bytes = (size_t)pb.F * pb.n_all * sizeof(float);
     DevBuf<unsigned char> U(bytes);
     RBF_CUDA(cudaMemsetAsync(U.p, 0, bytes, pb.st));
@@ -1771,7 +1786,6 @@ bool persistent_tune_mlp(Problem &pb, const MlpView &mv) {
                 const int c = nsm / div;
                 if (c < 1 || (div > 1 && (int64_t)c * 8 > pb.n_prog)) continue;
                 if (!persistent_plan(pb, G, c) || !persistent_mlp_ready(pb)) continue;
-                if (pb.ps.smem + mlp_layout(mv.n_in, pb.ps.chunk, pb.n_slots).end > (size_t)optin) continue;
                 persistent_run_mlp(pb, 1e-3, steps, U.p, pb.st, mv);   // warm-up
                 float t = 1e30f;
                 for (int rep = 0; rep < 3; ++rep) {

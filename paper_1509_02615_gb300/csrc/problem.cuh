@@ -90,6 +90,7 @@ struct PersistPlan {
     int rows_max = 0;            // most ghost rows one CTA solves
     size_t smem = 0;
     unsigned ring_off = 0;       // FP64: where the operands' ring starts in it (0: none)
+    size_t net_smem = 0;         // FP32: a corrected run's shared memory (a9; 0: the network does not fit)
     DevBuf<unsigned char> pw;    // T [4][SLQ][grid * chunk][S][V], as Problem::pw
     DevBuf<uint16_t> lidx;       // [SLQ][grid * chunk][S][V] list position of each slot
     DevBuf<int32_t> hlist;       // record lists of all CTAs
@@ -255,6 +256,8 @@ void persistent_run(Problem &pb, double dt, int64_t n_steps, void *U, cudaStream
 bool adv_persistent_plan(Problem &pb, int threads);
 void adv_persistent_run(Problem &pb, double t0, double dt, int64_t n_steps, void *U, cudaStream_t s);
 
+constexpr int kMaxInputs = 240;   // the widest input layer of a9's network (stencils of up to 60 nodes)
+
 // a9 fused into the persistent run: the learned correction's network (BF16
 // weights, FP32 biases and scales) and its per-field strengths.
 struct MlpView {
@@ -267,7 +270,7 @@ struct MlpView {
     unsigned long long *bad;        // non-finite corrections skipped
 };
 // True if a learned run can go through the persistent kernel (FP32 problem in
-// persistent mode with a variant that holds the network).
+// persistent mode with a variant that holds the network, and room for it).
 bool persistent_mlp_ready(const Problem &pb);
 void persistent_run_mlp(Problem &pb, double dt, int64_t n_steps, void *U, cudaStream_t s, const MlpView &mv);
 // Persistent plan for corrected runs: times short corrected runs on a zero
