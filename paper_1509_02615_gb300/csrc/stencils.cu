@@ -28,6 +28,7 @@ namespace {
 
 constexpr int kMaxCand = 2048;   // candidates per window held in shared memory
 constexpr int kWarpsPerBlock = 4;
+constexpr int kMaxStencil = 128;   // largest n of a search
 
 struct Grid {
     double x0, z0, cw, ch;   // origin and cell size
@@ -383,21 +384,31 @@ knn_kernel(const double *__restrict__ x, const double *__restrict__ z, const int
     if (lane == 0) atomicCAS(status, 0, 3);
 }
 
+// First window of a search for n neighbours: about 2.5 n candidates at two nodes per cell.
+int first_window(int n) {
+    const int R0 = (int)std::ceil(std::sqrt(2.5 * n / (4.0 * 2.0)));
+    return R0 < 1 ? 1 : R0;
+}
+// Room for the candidates inside that window's radius (2 pi R0^2 on average),
+// half as many again and a margin, in whole warps.
+int ranked_room(int n) {
+    const int R0 = first_window(n);
+    return std::min(kMaxCand, ((int)(1.5 * 6.2832 * R0 * R0) + 64 + 31) / 32 * 32);
+}
+size_t ranked_smem(int n) { return (size_t)kFastWarps * ranked_room(n) * (sizeof(double) + 2 * sizeof(int)); }
+
 // Searches the stencils of every centre on a binned grid: knn_ranked_kernel,
 // then knn_kernel for the centres it listed.  `slow` takes n_centers entries;
 // counts[0] is the status and counts[1] the number listed (both cleared here).
 // Synchronises the stream.
 void search(const double *x, const double *z, int64_t n_centers, int n, const Grid &g, const int *start,
             const int *sorted, int *slow, int *counts, int32_t *idx, cudaStream_t st) {
-    // first window: about 2.5 n candidates at two nodes per cell
-    int R0 = (int)std::ceil(std::sqrt(2.5 * n / (4.0 * 2.0)));
-    R0 = R0 < 1 ? 1 : R0;
-    const int Rmax = std::max(g.ncx, g.ncz);
-    // room for the candidates inside the first window's radius (2 pi R0^2 on
-    // average), half as many again and a margin, in whole warps
-    const int cap = std::min(kMaxCand, ((int)(1.5 * 6.2832 * R0 * R0) + 64 + 31) / 32 * 32);
-    const size_t fast = (size_t)kFastWarps * cap * (sizeof(double) + 2 * sizeof(int));
-    RBF_CUDA(cudaFuncSetAttribute(knn_ranked_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fast));
+    const int R0 = first_window(n), Rmax = std::max(g.ncx, g.ncz), cap = ranked_room(n);
+    const size_t fast = ranked_smem(n);
+    // the largest search's need: the limit is the kernel's, and another thread's
+    // launch may lie between this call and the one below
+    RBF_CUDA(cudaFuncSetAttribute(knn_ranked_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)ranked_smem(kMaxStencil)));
     RBF_CUDA(cudaMemsetAsync(counts, 0, 2 * sizeof(int), st));
     knn_ranked_kernel<<<div_up(n_centers, kFastWarps), kFastWarps * 32, fast, st>>>(
         x, z, n_centers, n, g, start, sorted, R0, Rmax, cap, idx, counts, slow, counts + 1);
@@ -423,7 +434,7 @@ void search(const double *x, const double *z, int64_t n_centers, int n, const Gr
 
 void build_stencils(const double *x, const double *z, int64_t n_all, int64_t n_centers, int n,
                     double period_x, int32_t *idx, cudaStream_t st) {
-    RBF_REQUIRE(n >= 1 && n <= 128, "stencil size n=%d must be in [1, 128]", n);
+    RBF_REQUIRE(n >= 1 && n <= kMaxStencil, "stencil size n=%d must be in [1, %d]", n, kMaxStencil);
     RBF_REQUIRE(n_all >= n, "n_all=%lld smaller than the stencil size %d", (long long)n_all, n);
     RBF_REQUIRE(n_centers >= 0 && n_centers <= n_all, "n_centers=%lld out of range", (long long)n_centers);
     RBF_REQUIRE(n_all < (int64_t)1 << 31, "n_all=%lld exceeds int32 indexing", (long long)n_all);
@@ -518,7 +529,7 @@ unsigned char *static_scratch() {
 
 void build_stencils_static(const double *x, const double *z, int64_t n_all, int64_t n_centers, int n,
                            double period_x, int32_t *idx, cudaStream_t st) {
-    RBF_REQUIRE(n >= 1 && n <= 128, "stencil size n=%d must be in [1, 128]", n);
+    RBF_REQUIRE(n >= 1 && n <= kMaxStencil, "stencil size n=%d must be in [1, %d]", n, kMaxStencil);
     RBF_REQUIRE(n_all >= n, "n_all=%lld smaller than the stencil size %d", (long long)n_all, n);
     RBF_REQUIRE(n_all <= kStaticMaxNodes, "n_all=%lld exceeds the static scratch limit of %lld nodes",
                 (long long)n_all, (long long)kStaticMaxNodes);
