@@ -142,10 +142,14 @@ typedef struct rbf_ns_params {
     int32_t poly_l;     /* polynomial degree l (4)                            */
     int32_t hv_k;       /* hyperviscosity Laplacian power k (3); 0 = none     */
     int32_t hv_p;       /* PHS exponent of the Delta^k weights (>= 2k+1)      */
-    int32_t precision;  /* 64: FP64 storage and arithmetic, the stencil sums
-                           in 55-bit fixed point per stencil (closer to the
-                           exact sums than sums in FP64); 32: FP64-built
-                           weights stored in FP32, FP32 RHS and RK4           */
+    int32_t precision;  /* 64: FP64 storage and arithmetic; every stencil sum
+                           adds integer products of the full FP64 weights and
+                           values, aligned to the sum's largest product: off
+                           by less than n 2^-54 of that product and one
+                           rounding, within the bound of a sum in FP64 for any
+                           weights and values, and the same bits for every
+                           number of lanes; 32: FP64-built weights stored in
+                           FP32, FP32 RHS and RK4                             */
     int32_t threads_per_node; /* 0 = autotuned (lanes per node and, in FP32,
                                  register prefetch); else 1, 2, 4 or 8 lanes */
     int32_t storage;    /* RBF_STORE_PER_NODE (0, Sec. 3's rows) or

@@ -101,7 +101,7 @@ void choose_threads(Problem &pb, int requested) {
 
 // Algorithmic bytes of one Navier-Stokes node-RHS of the stage kernel.
 // Per-node storage: packed weights (4 operators) + index per slot (2 or 4
-// bytes), the node's own values, U_n, the RK4 accumulator read+write, the stage output,
+// bytes) + in FP64 their exponent bytes, the node's own values, U_n, the RK4 accumulator read+write, the stage output,
 // pibar and the flag byte.  Lattice storage: class nodes read a class id
 // instead of their operators, irregular nodes read both, and the class table
 // is read once per launch.
@@ -110,10 +110,11 @@ double ns_rhs_bytes(const Problem &pb) {
     const double rest = 4 * ts + 4 * ts + 8 * ts + 4 * ts + ts + 1;
     // FP32: 16-bit indices for the nodes whose neighbours are near in the order
     const double far = pb.precision == 64 || pb.pf > 0 ? 1.0 : (double)pb.n_far / (double)pb.n_prog;
-    const double ops = slots * (4 * ts + 2 + 2 * far);
+    const double q = pb.precision == 64 ? 4.0 : 0.0;
+    const double ops = slots * (4 * ts + 2 + 2 * far + q);
     if (!pb.lat.enabled) return ops + rest;
     const double cn = (double)pb.lat.class_nodes, N = (double)pb.n_prog;
-    const double table = (double)pb.lat.n_cls * pb.SLQ * pb.G * pb.V * (4 * ts + 4);   // its offsets have 4 bytes
+    const double table = (double)pb.lat.n_cls * pb.SLQ * pb.G * pb.V * (4 * ts + 4 + q);   // its offsets have 4 bytes
     return 4 + rest + (N - cn) / N * ops + table / N;
 }
 

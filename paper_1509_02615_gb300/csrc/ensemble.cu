@@ -31,6 +31,7 @@ struct BlockDesc {
     const short4 *pnear;          // FP32: indices relative to the node (nodes without kFarFlag)
     const T *wx, *wz, *wd, *wh;   // FP64: fixed-point pairs (fixdot.cuh)
     const short4 *wexp, *lexp;    // FP64: row exponents of the member's nodes, of its classes
+    const int4 *nbr, *lnbr;       // FP64: neighbours and exponent bytes of two slots, in place of pidx, of loff
     const T *pibar;
     const unsigned char *flags;
     const int32_t *lcls, *loff;   // member's lattice storage (null: per-node rows only)
@@ -185,7 +186,7 @@ __global__ void __launch_bounds__(kThreads32, 1024 / kThreads32) ens_stage_kerne
 // The FP64 form: sums in fixed point (fixdot.cuh), two threads per lane, as the
 // single-problem stage kernel has them, in blocks of kFixThreads threads.
 template <int G, bool LAT>
-__global__ void __launch_bounds__(kFixThreads, 7) ens_stage_fixed_kernel(const BlockDesc<double> *__restrict__ descs,
+__global__ void __launch_bounds__(kFixThreads, 5) ens_stage_fixed_kernel(const BlockDesc<double> *__restrict__ descs,
                                                                          EnsArgs<double> a) {
     __shared__ FixRing ring;
     const BlockDesc<double> d = descs[blockIdx.x];
@@ -198,7 +199,7 @@ __global__ void __launch_bounds__(kFixThreads, 7) ens_stage_fixed_kernel(const B
     s.step = d.n_prog * G;   // in vectors
     s.ops = s.step * d.SLQ;
     s.w = reinterpret_cast<const int4 *>(d.wx) + i * G + g;
-    s.idx = reinterpret_cast<const int2 *>(d.pidx) + i * G + g;
+    s.nbr = d.nbr + i * G + g;
     s.shift = 0;
     short4 ew;
     const int cl = (LAT && d.lcls) ? __ldg(d.lcls + i) : -1;
@@ -206,7 +207,7 @@ __global__ void __launch_bounds__(kFixThreads, 7) ens_stage_fixed_kernel(const B
         s.step = G;
         s.ops = (int64_t)d.n_cls * d.SLQ * G;
         s.w = reinterpret_cast<const int4 *>(d.lw) + (int64_t)cl * d.SLQ * G + g;
-        s.idx = reinterpret_cast<const int2 *>(d.loff) + (int64_t)cl * d.SLQ * G + g;
+        s.nbr = d.lnbr + (int64_t)cl * d.SLQ * G + g;
         s.shift = (int)i;
         ew = __ldg(d.lexp + cl);
     } else {
@@ -219,9 +220,7 @@ __global__ void __launch_bounds__(kFixThreads, 7) ens_stage_fixed_kernel(const B
     grid_dep_wait();
     grid_dep_launch();
     const double *U = a.Uin + d.rec0 * 4;   // member-local record indices from here on
-    FixHalf f;
-    fix_sums<G, LAT>(U, s, ring, fetch, f);
-    const HalfSums sums = fix_finish<G>(f, ew, h);
+    const HalfSums sums = fix_sums<G, LAT>(U, s, ring, fetch, ew);
     const Rec<double> c = load_rec(U, i);
     const double2 k = fix_tendency(sums, {a.cp, a.g_over_tb, a.theta_bar, a.dpibar, a.rd_cv}, h,
                                    make_double4(c.u, c.w, c.t, c.p), d.pibar[i], d.flags[i]);
@@ -256,6 +255,7 @@ void fill_descs(Problem &pb) {
             d.wd = pw + 2 * total;
             d.wh = pw + 3 * total;
             d.wexp = m.wexp.p;
+            d.nbr = m.nbr.p;
             d.pibar = (const T *)m.pibar.p;
             d.flags = m.flags.p;
             if (m.lat.enabled) {
@@ -263,6 +263,7 @@ void fill_descs(Problem &pb) {
                 d.loff = m.lat.loff.p;
                 d.lw = (const T *)m.lat.lw.p;
                 d.lexp = m.lat.lexp.p;
+                d.lnbr = m.lat.lnbr.p;
                 d.n_cls = m.lat.n_cls;
             }
             d.n_prog = m.n_prog;

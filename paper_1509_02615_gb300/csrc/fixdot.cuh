@@ -3,33 +3,40 @@
 // GB300's FP64 pipe takes 2 FMAs per SM and clock, its integer units 32
 // multiply-adds of 32 x 32 bits into 64 (IMAD.WIDE; both measured).  The twelve
 // sums of a node over an n-point stencil are 12 n FMAs, so the FP64 stage
-// kernels were bound by that pipe at a quarter of the memory rate.  Here each
-// factor of a sum is a fixed-point number and each product three
-// IMAD.WIDEs; sums are exact apart from the product of the two low halves:
+// kernels were bound by that pipe at a quarter of the memory rate.  Here every
+// product of a sum is a product of integers, aligned to the largest product of
+// that sum:
 //
-//   weights   w = W 2^-k, k the largest scale of the node's row of that operator
-//             with |W| <= 2^58 and sum |W| <= 2^61; W = Wh 2^28 + Wl with Wl in
-//             [-2^27, 2^27); packed as (Wh, Wl), 8 bytes like the double
-//   values    f = F 2^(ef - 1078), ef the largest biased exponent of the field
-//             in the stencil, F = Fh 2^28 + Fl with Fl in [0, 2^28), |F| < 2^56;
-//             formed from the double's bits as it is gathered
-//   sums      hh = sum Wh Fh, cr = sum Wh Fl + Wl Fh (64-bit integers: sum |Wh|
-//             <= 2^33 + 64 and at most 128 slots keep |hh| <= 2^62 and
-//             |cr| < 2^63), value (hh 2^56 + cr 2^28) 2^(ef - k - 1078)
+//   weights   w = W 2^(e - 53), 2^52 <= |W| < 2^53 (every bit of the double), in
+//             halves W = Wh 2^28 + Wl with Wl in [-2^27, 2^27), packed as
+//             (Wh, Wl), 8 bytes like the double; beside it a byte per operator and
+//             slot, q = 255 - (er - e) for the row's largest exponent er (0: no
+//             weight; weights below 2^-254 of the row's largest are cut there)
+//   values    f = M 2^(c - 1075), c the biased exponent and M the 53-bit mantissa;
+//             F = M 2^6 shifted right by E - (c + q), E the largest c + q of the
+//             sum, in halves F = Fh 2^28 + Fl with Fl in [0, 2^28); formed from the
+//             double's bits as it is gathered, per operator
+//   sums      hh = sum Wh Fh, cr = sum Wh Fl + Wl Fh (64-bit integers; at most 128
+//             products below 2^56 each keep hh in range, cr is folded into hh
+//             every sixteen slots), value (hh 2^56 + cr 2^28) 2^(E + er - 1389)
 //
-// The stencil's largest exponents come from a first pass over its records
-// (they stay in L1 or shared memory for the second), so all lanes of a node
-// work at the same exponent and their integer sums do not depend on the number
-// of lanes.  Against a double, the largest weights keep five bits more and the
-// largest values three; smaller ones are cut at that absolute place, and the
-// dropped Wl Fl is about 2^-58 of the largest product.  A plain FP64 sum rounds
-// every partial sum at 2^-53 of itself, so the fixed-point sum's error is the
-// smaller one (two to six times; tests/test_gpu_fixed_point.py measures both
-// against 113-bit sums) unless one value of a stencil exceeds the others by
-// more than 2^3 where its own weight vanishes: then the others lose what
-// exceeds that.
-// Exponents below kMinExp (values under 1e-277) count as zero; a non-finite
-// value in the stencil makes the field's sums NaN.
+// A product keeps its 106 bits down to 2^-58 of the sum's largest product and
+// the dropped Wl Fl is below 2^-55 of it, where an FP64 sum rounds every partial
+// sum at 2^-53 of itself: the error is bounded by that of the FP64 sum whatever the
+// weights and values, and measured two to eight times smaller, except where one
+// product outweighs all others together, where both round at that product's last
+// place (tests/test_gpu_fixed_point*.py, against 113-bit sums).  An alignment to
+// max |w| max |f| instead (one shift per value, exponents from the values alone)
+// is a fifth faster, but takes from every product the lead of a value that its
+// own weight does not share: a spike a thousand times its neighbours, at its own
+// node in a centred derivative, cost them 63 times an FP64 sum's error.
+//
+// The largest exponents come from a first pass over the stencil's records
+// (they stay in L1 or shared memory for the second) and its weights' bytes, and
+// the integer sums of a node's lanes are added before anything is rounded, so
+// results do not depend on the number of lanes.  Sums of non-finite values, and
+// of products so small that the result would leave the normal range, go to
+// fix_plain: FP64 FMAs from the same operands.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -41,73 +48,134 @@
 namespace rbf {
 
 constexpr int kFixZero = -4000;   // row exponent of a row of zeros
-constexpr int kMinExp = 100;
+constexpr int kFixBad = 4000;     // of a row with a weight that is not finite: its sums are NaN
 
 // ---- weights (host and device) ---------------------------------------------
-// The row exponent ew = 58 - k of a row with the given largest magnitude and
-// sum of magnitudes: |w| <= 2^ew and sum |w| <= 2^(ew + 3).
-__host__ __device__ inline int fix_exponent(double largest, double sum) {
+// The exponent er of a row with the given largest magnitude: |w| < 2^er (NaN
+// must not be lost on the way: see fix_larger).
+__host__ __device__ inline int fix_exponent(double largest) {
     if (largest == 0.0) return kFixZero;
-    int e, s;
-    frexp(largest, &e);   // largest < 2^e
-    frexp(sum, &s);
-    return e > s - 3 ? e : s - 3;
+    if (!(largest <= 1.7976931348623157e308)) return kFixBad;
+    int e;
+    frexp(largest, &e);
+    return e;
 }
-// w as (Wh, Wl) for the row exponent ew
-__host__ __device__ inline int2 fix_weight(double w, int ew) {
-    if (w == 0.0) return make_int2(0, 0);
-    const long long W = llrint(ldexp(w, 58 - ew));
+// larger of two magnitudes, or NaN if either is
+__host__ __device__ inline double fix_larger(double a, double b) { return a >= b || a != a ? a : b; }
+// w as (Wh, Wl) and its exponent byte q for the row exponent er
+__host__ __device__ inline int2 fix_weight(double w, int er, unsigned *q) {
+    *q = 0;
+    if (w == 0.0 || er == kFixBad) return make_int2(0, 0);
+    int e;
+    const double m = frexp(w, &e);
+    const int r = er - e < 254 ? er - e : 254;
+    *q = 255u - (unsigned)r;
+    const long long W = llrint(ldexp(m, 53 - (er - e - r)));
     const long long h = (W + (1LL << 27)) >> 28;
     return make_int2((int)h, (int)(W - h * (1LL << 28)));
 }
 
 // ---- sums (device) ------------------------------------------------------------
-// logical shift; amounts above 31 give 0
-__device__ __forceinline__ unsigned shr32(unsigned v, int d) {
-    unsigned r;
-    asm("shr.u32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(d));
+// arithmetic shift; amounts above 63 leave the sign
+__device__ __forceinline__ long long sar64(long long v, int d) {
+    long long r;
+    asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(d));
     return r;
 }
 __device__ __forceinline__ void mad_wide(long long &acc, int a, int b) { acc += (long long)a * b; }
 
-// One field's sums with NO operators; e20 = ef << 20.
-template <int NO>
-struct FixSums {
-    long long hh[NO], cr[NO];
-    int e20;
-    // largest: the stencil's largest high word without its sign
-    __device__ __forceinline__ void start(int largest) {
-#pragma unroll
-        for (int o = 0; o < NO; ++o) hh[o] = cr[o] = 0;
-        e20 = max(largest & 0x7ff00000, kMinExp << 20);
+// exponent byte o of a slot
+template <int O>
+__device__ __forceinline__ int fix_byte(unsigned q) {
+    return (int)__byte_perm(q, 0, 0x4440 + O);
+}
+
+// What the first pass finds of one field's values over the stencil, two 16-bit
+// numbers in a word.
+struct FixScan {
+    unsigned xz = 0, dc = 0;   // largest c + q of d/dx and d/dz; of the third operator, and largest c
+    unsigned bits = 0;         // any bit of any value but its sign
+    __device__ __forceinline__ void take(unsigned lo, int hi, unsigned qxz, unsigned qd) {
+        const unsigned a = (unsigned)hi & 0x7fffffffu, e = (a >> 20) * 0x10001u;
+        bits |= lo | a;
+        xz = __viaddmax_u16x2(e, qxz, xz);
+        dc = __viaddmax_u16x2(e, qd, dc);
     }
-    // the value (lo, hi) as F, at the field's exponent: the high 28 bits of its
-    // mantissa and the other 25 (left-aligned), shifted down by the exponents'
-    // difference in 32-bit shifts (64-bit ones cost twice the instructions)
-    __device__ __forceinline__ void split(unsigned lo, int hi, int &Fh, int &Fl) const {
-        const unsigned d = (unsigned)(e20 - (hi & 0x7ff00000)) >> 20, s = (unsigned)(hi >> 31);
-        const unsigned m = ((unsigned)hi & 0xfffffu) | 0x100000u;
-        const unsigned top = __funnelshift_r(lo, m, 25);
-        const unsigned low = shr32(__funnelshift_rc(lo << 7, top, d), 4 + max((int)d - 32, 0));
-        Fl = (int)((low ^ s) & 0xfffffffu);
-        Fh = (int)(shr32(top, d) ^ s);
+    // over the node's G slot lanes (every other lane of the warp)
+    template <int G>
+    __device__ __forceinline__ void over_lanes() {
+#pragma unroll
+        for (int k = G; k > 1; k >>= 1) {
+            bits |= __shfl_xor_sync(0xffffffffu, bits, k);
+            xz = __vmaxu2(xz, __shfl_xor_sync(0xffffffffu, xz, k));
+            dc = __vmaxu2(dc, __shfl_xor_sync(0xffffffffu, dc, k));
+        }
+    }
+    __device__ __forceinline__ int E(int o) const { return (int)(o == 0 ? xz & 0xffffu : o == 1 ? xz >> 16 : dc & 0xffffu); }
+    // whether the integer sums of operators with row exponents x, z, d hold: the
+    // values finite, every result in the normal range with 28 bits to spare below,
+    // and zeros (exponent 0, whose implicit bit is not there) shifted out
+    __device__ __forceinline__ bool holds(int x, int z, int d) const {
+        auto one = [&](int e, int er) { return er == kFixZero || (e >= 324 && e + er >= 340 && e + er <= 2356); };
+        return bits == 0 || (dc >> 16 < 2047u && one(E(0), x) && one(E(1), z) && one(E(2), d));
+    }
+};
+
+// One field's sums with three operators.
+struct FixSums {
+    long long hh[3], cr[3];
+    int E[3];
+    __device__ __forceinline__ void start(const FixScan &s) {
+#pragma unroll
+        for (int o = 0; o < 3; ++o) {
+            hh[o] = cr[o] = 0;
+            E[o] = s.bits ? s.E(o) : 0x10000;   // zeros: everything is shifted out
+        }
+    }
+    // A value (lo, hi) as F 2^4 without its shift, complemented if negative (so that
+    // after the shift the upper word is Fh and the lower one Fl 2^4), and its exponent.
+    struct Value {
+        long long Y;
+        int c;
+        __device__ __forceinline__ Value(unsigned lo, int hi) {
+            const int s = hi >> 31;
+            const unsigned T = __funnelshift_r(lo, ((unsigned)hi & 0xfffffu) | 0x100000u, 22) ^ (unsigned)s;
+            Y = (long long)((unsigned long long)T << 32 | ((lo << 10) ^ (unsigned)s));
+            c = (hi & 0x7fffffff) >> 20;
+        }
+    };
+    __device__ __forceinline__ void add(int o, const Value &v, int q, int wh, int wl) {
+        const long long F = sar64(v.Y, E[o] - v.c - q);
+        int Fh = (int)(F >> 32), Fl = (int)((unsigned)F >> 4);
         // keep the ranges from the compiler: with Fl known to be non-negative it
         // widens the products to 64 x 64 bits
         asm("" : "+r"(Fh), "+r"(Fl));
-    }
-    __device__ __forceinline__ void add(int o, int wh, int wl, int Fh, int Fl) {
         mad_wide(hh[o], wh, Fh);
         mad_wide(cr[o], wh, Fl);
         mad_wide(cr[o], wl, Fh);
     }
-    // the sum of the G lanes of a node for the row exponent ew
-    template <int G>
-    __device__ __forceinline__ double value(int o, int ew) const {
-        long long V = hh[o] * 2 + (cr[o] >> 27);
+    __device__ __forceinline__ void fold() {
 #pragma unroll
-        for (int k = G; k > 1; k >>= 1) V += __shfl_xor_sync(0xffffffffu, V, k);   // every other lane
-        const int e = (e20 >> 20) + ew - 58;   // exponent field of 2^(ef + ew - 1081)
-        const int hi = e20 == 0x7ff00000 ? 0x7ff80000 : min(max(e, 0), 2046) << 20;
+        for (int o = 0; o < 3; ++o) {
+            hh[o] += cr[o] >> 28;
+            cr[o] &= 0xfffffff;
+        }
+    }
+    // the sum of the G lanes of a node for the row exponent er, after a fold
+    template <int G>
+    __device__ __forceinline__ double value(int o, int er) const {
+        long long h = hh[o], c = cr[o];
+#pragma unroll
+        for (int k = G; k > 1; k >>= 1) {   // every other lane
+            h += __shfl_xor_sync(0xffffffffu, h, k);
+            c += __shfl_xor_sync(0xffffffffu, c, k);
+        }
+        h += c >> 28;
+        c &= 0xfffffff;
+        const int z = min(__clzll(h ^ (h >> 63)) - 1, 28);   // bits of c that fit below h
+        const long long V = (h << z) + (c >> (28 - z));
+        const int e = E[o] + er - 310 - z;   // exponent field of the power of two
+        const int hi = er == kFixBad ? 0x7ff80000 : (unsigned)(e - 1) < 2046u ? e << 20 : 0;   // zeros: 0
         return (double)V * __hiloint2double(hi, 0);
     }
 };
@@ -118,42 +186,50 @@ struct FixSums {
 // and dissipation (pi': hyperviscosity) sums of its two fields: half the
 // registers of the whole node, so that twice the warps hide the gathers.
 struct FixHalf {
-    FixSums<3> a, b;
-    __device__ __forceinline__ void slot(const int4 &r, int xh, int xl, int zh, int zl, int dh, int dl, int bh, int bl) {
-        int Fh, Fl;
-        a.split((unsigned)r.x, r.y, Fh, Fl);
-        a.add(0, xh, xl, Fh, Fl);
-        a.add(1, zh, zl, Fh, Fl);
-        a.add(2, dh, dl, Fh, Fl);
-        b.split((unsigned)r.z, r.w, Fh, Fl);
-        b.add(0, xh, xl, Fh, Fl);
-        b.add(1, zh, zl, Fh, Fl);
-        b.add(2, bh, bl, Fh, Fl);
+    FixSums a, b;
+    // sel: which byte of q is the second field's third operator (fix_third)
+    __device__ __forceinline__ void slot(const int4 &r, unsigned q, unsigned sel, int xh, int xl, int zh, int zl, int dh,
+                                         int dl, int bh, int bl) {
+        const int qx = fix_byte<0>(q), qz = fix_byte<1>(q);
+        const FixSums::Value va((unsigned)r.x, r.y);
+        a.add(0, va, qx, xh, xl);
+        a.add(1, va, qz, zh, zl);
+        a.add(2, va, fix_byte<2>(q), dh, dl);
+        const FixSums::Value vb((unsigned)r.z, r.w);
+        b.add(0, vb, qx, xh, xl);
+        b.add(1, vb, qz, zh, zl);
+        b.add(2, vb, (int)__byte_perm(q, 0, sel), bh, bl);
     }
     // two slots from one operand vector of each operator (d: third operator of
     // the first field, e: of the second)
-    __device__ __forceinline__ void slots(const int4 &r0, const int4 &r1, const int4 &x, const int4 &z, const int4 &d,
-                                          const int4 &e) {
-        slot(r0, x.x, x.y, z.x, z.y, d.x, d.y, e.x, e.y);
-        slot(r1, x.z, x.w, z.z, z.w, d.z, d.w, e.z, e.w);
+    __device__ __forceinline__ void slots(const int4 &r0, const int4 &r1, uint2 q, unsigned sel, const int4 &x,
+                                          const int4 &z, const int4 &d, const int4 &e) {
+        slot(r0, q.x, sel, x.x, x.y, z.x, z.y, d.x, d.y, e.x, e.y);
+        slot(r1, q.y, sel, x.z, x.w, z.z, z.w, d.z, d.w, e.z, e.w);
+    }
+    __device__ __forceinline__ void fold() {
+        a.fold();
+        b.fold();
     }
 };
+// selector of the second field's third operator: dissipation (w) or hyperviscosity (pi')
+__device__ __forceinline__ unsigned fix_third(int h) { return 0x4442u + (unsigned)h; }
 
-// Largest high words (signs dropped) of a half record's two fields over a stencil.
-struct FixLargest {
-    int a = 0, b = 0;
-    __device__ __forceinline__ void take(const int4 &r) {
-        a = max(a, r.y & 0x7fffffff);
-        b = max(b, r.w & 0x7fffffff);
+// The first pass over a half's two fields.
+struct FixHalfScan {
+    FixScan a, b;
+    __device__ __forceinline__ void take(const int4 &r, unsigned q, unsigned sel) {
+        const unsigned qxz = __byte_perm(q, 0, 0x4140);
+        a.take((unsigned)r.x, r.y, qxz, __byte_perm(q, 0, 0x4442));
+        b.take((unsigned)r.z, r.w, qxz, __byte_perm(q, 0, sel));
     }
-    // over the node's G slot lanes (every other lane of the warp)
     template <int G>
     __device__ __forceinline__ void over_lanes() {
-#pragma unroll
-        for (int k = G; k > 1; k >>= 1) {
-            a = max(a, __shfl_xor_sync(0xffffffffu, a, k));
-            b = max(b, __shfl_xor_sync(0xffffffffu, b, k));
-        }
+        a.template over_lanes<G>();
+        b.template over_lanes<G>();
+    }
+    __device__ __forceinline__ bool holds(short4 ew, int h) const {
+        return a.holds(ew.x, ew.y, ew.z) && b.holds(ew.x, ew.y, h ? ew.w : ew.z);
     }
 };
 
@@ -221,7 +297,7 @@ using FixRing = int4[kFixRing][4][kFixThreads / 2];
 struct FixStream {
     const int4 *w;     // the pair's first vector of operator 0
     int64_t ops;       // vectors between operators
-    const int2 *idx;   // its first two neighbour indices
+    const int4 *nbr;   // its first two neighbours' indices (x, y) and weights' exponent bytes (z, w)
     int64_t step;      // vectors between steps
     int shift;         // added to the indices
     int SLQ;           // steps
@@ -264,31 +340,89 @@ struct FixFetch {
     }
 };
 
-// The thread's part of a node's sums over the records U (two 16-byte halves
-// each); every lane of the warp takes part, with the same number of steps.
-// `fetch` has been started and its first two steps copied (constant data,
-// before the wait for the preceding kernel).
+// The thread's part of a half's sums in FP64, for what the integer sums do not
+// hold (FixScan::holds): half is the thread's half of record 0, nbr(k) the
+// neighbours of step k as in FixStream::nbr.
+template <class Nbr>
+__device__ __noinline__ HalfSums fix_plain(const int4 *half, Nbr nbr, const int4 *w, int64_t ops, int64_t step, int SLQ,
+                                           short4 ew, int h) {
+    double s[6] = {0, 0, 0, 0, 0, 0};
+    const int er[4] = {ew.x, ew.y, ew.z, h ? ew.w : ew.z};
+    for (int k = 0; k < SLQ; ++k, w += step) {
+        const int4 j = nbr(k);
+        for (int v = 0; v < 2; ++v) {
+            const int4 r = half[2 * (int64_t)(v ? j.y : j.x)];
+            const unsigned qv = (unsigned)(v ? j.w : j.z);
+            double wd[4];
+            for (int o = 0; o < 4; ++o) {
+                const int4 W = __ldg(w + (o < 3 ? o : 2 + h) * ops);
+                const long long i = (long long)(v ? W.z : W.x) * (1LL << 28) + (v ? W.w : W.y);
+                const int b = (int)(qv >> (8 * (o < 3 ? o : 2 + h)) & 255u);
+                wd[o] = er[o] == kFixBad ? __hiloint2double(0x7ff80000, 0)
+                        : b == 0         ? 0.0
+                                         : ldexp((double)i, er[o] + b - 308);
+            }
+            const double fa = __hiloint2double(r.y, r.x), fb = __hiloint2double(r.w, r.z);
+            s[0] = fma(wd[0], fa, s[0]);
+            s[1] = fma(wd[1], fa, s[1]);
+            s[2] = fma(wd[2], fa, s[2]);
+            s[3] = fma(wd[0], fb, s[3]);
+            s[4] = fma(wd[1], fb, s[4]);
+            s[5] = fma(wd[3], fb, s[5]);
+        }
+    }
+    return {s[0], s[1], s[2], s[3], s[4], s[5]};
+}
+
+// A half's sums from the integers, or over the G lanes of plain sums if any of
+// the warp's do not hold (every lane of the warp takes part).
+template <int G, class Nbr>
+__device__ __forceinline__ HalfSums fix_choose(const FixHalf &f, bool holds, const int4 *half, Nbr nbr, const int4 *w,
+                                               int64_t ops, int64_t step, int SLQ, short4 ew, int h) {
+    HalfSums s = fix_finish<G>(f, ew, h);
+    if (__all_sync(0xffffffffu, holds)) return s;
+    HalfSums p = fix_plain(half, nbr, w, ops, step, SLQ, ew, h);
+#pragma unroll
+    for (int k = G; k > 1; k >>= 1) {
+        p.ax += __shfl_xor_sync(0xffffffffu, p.ax, k);
+        p.az += __shfl_xor_sync(0xffffffffu, p.az, k);
+        p.ad += __shfl_xor_sync(0xffffffffu, p.ad, k);
+        p.bx += __shfl_xor_sync(0xffffffffu, p.bx, k);
+        p.bz += __shfl_xor_sync(0xffffffffu, p.bz, k);
+        p.bd += __shfl_xor_sync(0xffffffffu, p.bd, k);
+    }
+    return holds ? s : p;
+}
+
+// A half's sums over the records U (two 16-byte halves each); every lane of the
+// warp takes part, with the same number of steps.  `fetch` has been started
+// and its first two steps copied (constant data, before the wait for the
+// preceding kernel).
 template <int G, bool CACHED>
-__device__ __forceinline__ void fix_sums(const double *U, const FixStream &s, FixRing &ring, FixFetch<CACHED> &fetch,
-                                         FixHalf &f) {
+__device__ __forceinline__ HalfSums fix_sums(const double *U, const FixStream &s, FixRing &ring, FixFetch<CACHED> &fetch,
+                                             short4 ew) {
     const int h = threadIdx.x & 1, pair = threadIdx.x >> 1;
     const int4 *half = reinterpret_cast<const int4 *>(U) + h + 2 * (int64_t)s.shift;
-    FixLargest top;
-    const int2 *pi = s.idx;
+    const unsigned sel = fix_third(h);
+    FixHalfScan top;
+    const int4 *pn = s.nbr;
 #pragma unroll 4
-    for (int q = 0; q < s.SLQ; ++q, pi += s.step) {
-        const int2 j = __ldg(pi);
-        top.take(__ldg(half + 2 * (int64_t)j.x));
-        top.take(__ldg(half + 2 * (int64_t)j.y));
+    for (int q = 0; q < s.SLQ; ++q, pn += s.step) {
+        const int4 j = __ldg(pn);
+        top.take(__ldg(half + 2 * (int64_t)j.x), (unsigned)j.z, sel);
+        top.take(__ldg(half + 2 * (int64_t)j.y), (unsigned)j.w, sel);
     }
     top.over_lanes<G>();
+    FixHalf f;
     f.a.start(top.a);
     f.b.start(top.b);
-    pi = s.idx;
-    int2 j = __ldg(pi);
+    const bool holds = top.holds(ew, h);
+    pn = s.nbr;
+    int4 j = __ldg(pn);
     int4 n0 = __ldg(half + 2 * (int64_t)j.x), n1 = __ldg(half + 2 * (int64_t)j.y);
-    pi += s.step;
-    if (s.SLQ > 1) j = __ldg(pi);
+    uint2 e1 = make_uint2(j.z, j.w);
+    pn += s.step;
+    if (s.SLQ > 1) j = __ldg(pn);
     const int4 *v = &ring[0][0][pair];
 #pragma unroll 1
     for (int q0 = 0; q0 < s.SLQ; q0 += kFixRing) {
@@ -297,12 +431,14 @@ __device__ __forceinline__ void fix_sums(const double *U, const FixStream &s, Fi
             const int q = q0 + u;
             if (q >= s.SLQ) break;
             const int4 r0 = n0, r1 = n1;
+            const uint2 e = e1;
             if (q + 1 < s.SLQ) {   // the next step's records, and the indices of the one after
                 n0 = __ldg(half + 2 * (int64_t)j.x);
                 n1 = __ldg(half + 2 * (int64_t)j.y);
+                e1 = make_uint2(j.z, j.w);
                 if (q + 2 < s.SLQ) {
-                    pi += s.step;
-                    j = __ldg(pi);
+                    pn += s.step;
+                    j = __ldg(pn);
                 }
             }
             // step q + 2 overwrites slots that were read in step q - 2: step q - 1's
@@ -312,9 +448,15 @@ __device__ __forceinline__ void fix_sums(const double *U, const FixStream &s, Fi
             __syncwarp();   // the other thread's vectors of this step
             constexpr int kOp = kFixThreads / 2;
             const int4 *w = v + 4 * u * kOp;
-            f.slots(r0, r1, w[0], w[kOp], w[2 * kOp], w[(2 + h) * kOp]);
+            f.slots(r0, r1, e, sel, w[0], w[kOp], w[2 * kOp], w[(2 + h) * kOp]);
         }
+        if (q0 & kFixRing) f.fold();
     }
+    f.fold();
+    const int4 *nbr = s.nbr;
+    const int64_t step = s.step;
+    return fix_choose<G>(f, holds, half, [nbr, step](int k) { return __ldg(nbr + k * step); }, s.w, s.ops, s.step, s.SLQ,
+                         ew, h);
 }
 
 }  // namespace rbf

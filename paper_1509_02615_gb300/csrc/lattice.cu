@@ -157,34 +157,40 @@ void pack_lattice(Problem &pb, const std::vector<double> &comb, int nops) {
             }
         }
     }
-    L.loff.alloc(std::max<size_t>(off.size(), 1));
-    RBF_CUDA(cudaMemcpyAsync(L.loff.p, off.data(), off.size() * 4, cudaMemcpyHostToDevice, pb.st));
     L.lw.alloc(std::max<size_t>(w.size(), 1) * pb.tsize());
     std::vector<int2> fixed;
     std::vector<short4> ex;
+    std::vector<int4> nbr;
     if (pb.precision == 64) {
         // fixed point, as pack_fixed_kernel forms it for the class's first member
         fixed.resize(w.size());
         ex.resize(std::max<int32_t>(L.n_cls, 1));
+        nbr.assign(std::max<size_t>(off.size() / 2, 1), make_int4(0, 0, 0, 0));
+        for (size_t t = 0; t < off.size(); ++t) reinterpret_cast<int32_t *>(&nbr[t / 2])[t % 2] = off[t];
         for (int32_t c = 0; c < L.n_cls; ++c) {
             short e4[4];
             for (int p = 0; p < 4; ++p) {
                 const size_t at = ((size_t)p * L.n_cls + c) * per;
-                double top = 0.0, sum = 0.0;
+                double top = 0.0;
+                for (int t = 0; t < per; ++t) top = fix_larger(top, std::fabs(w[at + t]));
+                const int e = fix_exponent(top);
                 for (int t = 0; t < per; ++t) {
-                    top = std::max(top, std::fabs(w[at + t]));
-                    sum += std::fabs(w[at + t]);
+                    unsigned b = 0;
+                    fixed[at + t] = fix_weight(w[at + t], e, &b);
+                    reinterpret_cast<int32_t *>(&nbr[((size_t)c * per + t) / 2])[2 + t % 2] |= (int32_t)(b << (8 * p));
                 }
-                const int e = fix_exponent(top, sum);
-                for (int t = 0; t < per; ++t) fixed[at + t] = fix_weight(w[at + t], e);
                 e4[p] = (short)e;
             }
             ex[c] = make_short4(e4[0], e4[1], e4[2], e4[3]);
         }
         L.lexp.alloc(ex.size());
+        L.lnbr.alloc(nbr.size());
+        RBF_CUDA(cudaMemcpyAsync(L.lnbr.p, nbr.data(), L.lnbr.bytes(), cudaMemcpyHostToDevice, pb.st));
         RBF_CUDA(cudaMemcpyAsync(L.lexp.p, ex.data(), L.lexp.bytes(), cudaMemcpyHostToDevice, pb.st));
         RBF_CUDA(cudaMemcpyAsync(L.lw.p, fixed.data(), fixed.size() * sizeof(int2), cudaMemcpyHostToDevice, pb.st));
     } else {
+        L.loff.alloc(std::max<size_t>(off.size(), 1));
+        RBF_CUDA(cudaMemcpyAsync(L.loff.p, off.data(), off.size() * 4, cudaMemcpyHostToDevice, pb.st));
         std::vector<float> wf(w.begin(), w.end());
         RBF_CUDA(cudaMemcpyAsync(L.lw.p, wf.data(), wf.size() * 4, cudaMemcpyHostToDevice, pb.st));
     }

@@ -43,6 +43,7 @@ struct NSArgs {
     const short4 *pnear;          // FP32: indices relative to the node (nodes without kFarFlag)
     const T *wx, *wz, *wd, *wh;   // FP64: fixed-point pairs (fixdot.cuh), not doubles
     const short4 *wexp;           // FP64: row exponents of each node, or of each class
+    const int4 *nbr, *lnbr;       // FP64: neighbours and exponent bytes of two slots, in place of pidx, of loff
     const T *pibar;
     const unsigned char *flags;
     // split stage launches: each of the two launches takes its nodes from
@@ -239,15 +240,15 @@ __global__ void __launch_bounds__(kStageThreads<PF, LAT>, PF > 0 ? 1 : 1024 / kS
 
 // The FP64 stage (or bare right-hand side): the sums in fixed point
 // (fixdot.cuh), everything else in FP64.  On 308,097 scattered nodes with
-// n = 56 a launch took 365 us as 12 x 56 FP64 FMAs per node (0.95 of the FP64
-// pipe) and takes 173 us.  What bounds it now: the gathers through the L1 tags
-// (without the first pass 152 us, without the products 163 us, without the
-// operand stream 157 us) and, under them, 99 us of operand traffic at the copy
-// rate.  Seven blocks of 128 threads per SM (72 registers): six take 181 us,
-// eight, with spills, 181 us; one thread per node for all four fields (126
-// registers, 16 warps per SM) 225 us.
+// n = 56 a stage of a run (with its ghost kernels) took 380 us as 12 x 56 FP64
+// FMAs per node (0.95 of the FP64 pipe) and takes 224 us; with one alignment
+// per value in place of one per sum, 182 us.  What bounds it: the integer
+// pipes, some 70 instructions per slot and thread beside 18 IMAD.WIDEs, and
+// under them 110 us of operand traffic at the copy rate.  Five blocks of 128
+// threads per SM (96 registers): six, with spills, take 222 us, but the
+// right-hand side of a 125 m box 19.4 us in place of 18.6; seven 249 us.
 template <int G, bool LAT>
-__global__ void __launch_bounds__(kFixThreads, 7) ns_stage_fixed_kernel(NSArgs<double> a) {
+__global__ void __launch_bounds__(kFixThreads, 5) ns_stage_fixed_kernel(NSArgs<double> a) {
     __shared__ FixRing ring;
     const int64_t pair = (blockIdx.x * (int64_t)kFixThreads + threadIdx.x) >> 1;
     const int h = threadIdx.x & 1, g = (int)(pair % G);
@@ -266,7 +267,7 @@ __global__ void __launch_bounds__(kFixThreads, 7) ns_stage_fixed_kernel(NSArgs<d
     s.step = a.n_prog * G;   // in vectors
     s.ops = s.step * a.SLQ;
     s.w = reinterpret_cast<const int4 *>(a.wx) + i * G + g;
-    s.idx = reinterpret_cast<const int2 *>(a.pidx) + i * G + g;
+    s.nbr = a.nbr + i * G + g;
     s.shift = 0;
     short4 ew;
     const int cl = LAT ? __ldg(a.lcls + i) : -1;
@@ -274,7 +275,7 @@ __global__ void __launch_bounds__(kFixThreads, 7) ns_stage_fixed_kernel(NSArgs<d
         s.step = G;
         s.ops = (int64_t)a.n_cls * a.SLQ * G;
         s.w = reinterpret_cast<const int4 *>(a.lw) + (int64_t)cl * a.SLQ * G + g;
-        s.idx = reinterpret_cast<const int2 *>(a.loff) + (int64_t)cl * a.SLQ * G + g;
+        s.nbr = a.lnbr + (int64_t)cl * a.SLQ * G + g;
         s.shift = (int)i;
         ew = __ldg(a.lexp + cl);
     } else {
@@ -286,9 +287,7 @@ __global__ void __launch_bounds__(kFixThreads, 7) ns_stage_fixed_kernel(NSArgs<d
     fetch.copy(1);
     grid_dep_wait();     // the stage input (and its ghosts) come from earlier kernels
     grid_dep_launch();
-    FixHalf f;
-    fix_sums<G, LAT>(a.Uin, s, ring, fetch, f);
-    const HalfSums sums = fix_finish<G>(f, ew, h);
+    const HalfSums sums = fix_sums<G, LAT>(a.Uin, s, ring, fetch, ew);
     const Rec<double> c = load_rec(a.Uin, i);
     const double2 k = fix_tendency(sums, {a.cp, a.g_over_tb, a.theta_bar, a.dpibar, a.rd_cv}, h,
                                    make_double4(c.u, c.w, c.t, c.p), a.pibar[i], a.flags[i]);
@@ -463,12 +462,12 @@ __global__ void pack_kernel(const double *__restrict__ w64, const int32_t *__res
 }
 
 // FP64 operators in fixed point (fixdot.cuh): one warp per node packs its rows
-// as pack_kernel does, with (Wh, Wl) pairs in place of the values, and writes
-// the rows' exponents.
+// as pack_kernel does, with (Wh, Wl) pairs in place of the values and their
+// exponent bytes beside the indices, and writes the rows' exponents.
 __global__ void __launch_bounds__(256) pack_fixed_kernel(const double *__restrict__ w64, const int32_t *__restrict__ idx,
                                                          int64_t n_prog, int n, int nops, int first, int n_slots,
                                                          int SLQ, int G, const double *__restrict__ comb,
-                                                         int2 *__restrict__ pw, int32_t *__restrict__ pidx,
+                                                         int2 *__restrict__ pw, int4 *__restrict__ nbr,
                                                          short4 *__restrict__ wexp) {
     const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
@@ -486,23 +485,19 @@ __global__ void __launch_bounds__(256) pack_fixed_kernel(const double *__restric
             }
             return val;
         };
-        double top = 0.0, sum = 0.0;
-        for (int t = lane; t < n_slots; t += 32) {
-            const double v = fabs(weight(t));
-            top = fmax(top, v);
-            sum += v;
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            top = fmax(top, __shfl_xor_sync(0xffffffffu, top, o));
-            sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        }
-        const int e = fix_exponent(top, sum);
+        double top = 0.0;
+        for (int t = lane; t < n_slots; t += 32) top = fix_larger(top, fabs(weight(t)));
+        for (int o = 16; o > 0; o >>= 1) top = fix_larger(top, __shfl_xor_sync(0xffffffffu, top, o));
+        const int e = fix_exponent(top);
         ex[p] = (short)e;
         for (int t = lane; t < per; t += 32) {
             const int v = t % V, gq = t / V, g = gq % G, q = gq / G;
             const int64_t dst = (((int64_t)q * n_prog + i) * G + g) * V + v;
-            pw[p * total + dst] = t < n_slots ? fix_weight(weight(t), e) : make_int2(0, 0);
-            if (p == 0) pidx[dst] = t < n_slots ? idx[i * n + t + first] : (int32_t)i;
+            unsigned b = 0;
+            pw[p * total + dst] = t < n_slots ? fix_weight(weight(t), e, &b) : make_int2(0, 0);
+            int32_t *word = reinterpret_cast<int32_t *>(nbr + dst / V) + v;   // index; exponent bytes at [2]
+            word[2] = (p ? word[2] : 0) | (int32_t)(b << (8 * p));
+            if (p == 0) word[0] = t < n_slots ? idx[i * n + t + first] : (int32_t)i;
         }
     }
     if (lane == 0) wexp[i] = make_short4(ex[0], ex[1], ex[2], ex[3]);
@@ -666,10 +661,12 @@ NSArgs<T> ns_args(Problem &pb) {
     a.wd = pw + 2 * total;
     a.wh = pw + 3 * total;
     a.wexp = pb.wexp.p;
+    a.nbr = pb.nbr.p;
     a.pibar = (const T *)pb.pibar.p;
     a.flags = pb.flags.p;
     if (pb.lat.enabled) {
         a.lexp = pb.lat.lexp.p;
+        a.lnbr = pb.lat.lnbr.p;
         a.lcls = pb.lat.cls.p;
         a.loff = pb.lat.loff.p;
         a.lw = (const T *)pb.lat.lw.p;
@@ -819,7 +816,8 @@ void pack_operators(Problem &pb, bool near) {
     pb.SLQ = div_up(pb.n_slots, pb.G * pb.V);
     pb.SL = pb.SLQ * pb.V;
     const int64_t total = (int64_t)pb.SL * pb.G * pb.n_prog;
-    pb.pidx.alloc(total);
+    const bool fixed = pb.kind == kNS && pb.precision == 64;   // its indices are in pb.nbr
+    if (!fixed) pb.pidx.alloc(total);
     if (pb.kind == kAdvection) {
         pb.n_packed = pb.n_vparts + 1;
         pb.pw.alloc((size_t)pb.n_packed * total * pb.tsize());
@@ -858,9 +856,10 @@ void pack_operators(Problem &pb, bool near) {
         // the exponents do not depend on the lanes: one buffer for good, which captured
         // graphs keep reading when a persistent plan packs its own operands
         if (pb.wexp.n != (size_t)pb.n_prog) pb.wexp.alloc(pb.n_prog);
+        pb.nbr.alloc(total / pb.V);
         pack_fixed_kernel<<<div_up(pb.n_prog, 8), 256, 0, pb.st>>>(pb.w64.p, pb.idx.p, pb.n_prog, pb.n, nops, pb.diff,
                                                                    pb.n_slots, pb.SLQ, pb.G, dcomb.p, (int2 *)pb.pw.p,
-                                                                   pb.pidx.p, pb.wexp.p);
+                                                                   pb.nbr.p, pb.wexp.p);
     } else
         pack_kernel<float><<<div_up(total, 256), 256, 0, pb.st>>>(pb.w64.p, pb.idx.p, pb.n_prog, pb.n, nops, pb.diff,
                                                                   pb.n_slots, pb.SLQ, pb.G, pb.V, pb.n_packed,

@@ -238,6 +238,7 @@ struct PArgs {
     const T *pw;                    // [4][SLQ][lanes][G][V], lanes = grid * chunk (FP64: fixed-point pairs)
     const short4 *wexp;             // FP64: row exponents of each node
     const uint16_t *lidx;           // [SLQ][lanes][G][V]
+    const uint32_t *wq;             // FP64: exponent bytes, alike
     const int32_t *hlist;
     const CtaInfo *cta;
     const unsigned char *blob;
@@ -568,6 +569,7 @@ __global__ void __launch_bounds__(MAXT, 1) rk4_persistent(const __grid_constant_
     const W *wd = reinterpret_cast<const W *>(a.pw + 2 * a.total);
     const W *wh = reinterpret_cast<const W *>(a.pw + 3 * a.total);
     const L *lx = reinterpret_cast<const L *>(a.lidx);
+    const uint2 *lq = reinterpret_cast<const uint2 *>(a.wq);
     // FP64: the operands' ring behind the CTA's other shared memory
     int4 *const ring = reinterpret_cast<int4 *>(smem_raw + a.ring_off);
     FixFetch<false> fetch;
@@ -734,37 +736,46 @@ __global__ void __launch_bounds__(MAXT, 1) rk4_persistent(const __grid_constant_
                 T k[NF];
                 const Rec<T> fi = sh_rec(halo, self);
                 if constexpr (FIX) {
-                    FixLargest top;
+                    const unsigned sel = fix_third(h);
+                    FixHalfScan top;
 #pragma unroll 4
                     for (int q = 0; q < a.SLQ; ++q) {
                         const L j = __ldg(lx + off0 + q * stride);
-                        top.take(sh_half(halo, 2 * j.x + h));
-                        top.take(sh_half(halo, 2 * j.y + h));
+                        const uint2 e = __ldg(lq + off0 + q * stride);
+                        top.take(sh_half(halo, 2 * j.x + h), e.x, sel);
+                        top.take(sh_half(halo, 2 * j.y + h), e.y, sel);
                     }
                     top.over_lanes<G>();
                     FixHalf f;
                     f.a.start(top.a);
                     f.b.start(top.b);
+                    const bool holds = top.holds(ew, h);
                     int64_t off = off0;
                     if (a.ring_off) {
                         // operands two steps ahead through the pair's ring slots (fixdot.cuh)
                         const int4 *v = ring + (threadIdx.x >> 1);
                         const int np = blockDim.x >> 1;
                         L j = __ldg(lx + off);
+                        uint2 e1 = __ldg(lq + off);
 #pragma unroll 1
                         for (int q0 = 0; q0 < a.SLQ; q0 += kFixRing) {
 #pragma unroll
                             for (int u = 0; u < kFixRing; ++u) {
                                 if (q0 + u >= a.SLQ) break;
                                 const int4 r0 = sh_half(halo, 2 * j.x + h), r1 = sh_half(halo, 2 * j.y + h);
+                                const uint2 e = e1;
                                 off += stride;
-                                if (q0 + u + 1 < a.SLQ) j = __ldg(lx + off);
+                                if (q0 + u + 1 < a.SLQ) {
+                                    j = __ldg(lx + off);
+                                    e1 = __ldg(lq + off);
+                                }
                                 fetch.copy((u + 2) % kFixRing);
                                 asm volatile("cp.async.wait_group 2;" ::: "memory");
                                 __syncwarp();   // the other thread's vectors of this step
                                 const int4 *w = v + 4 * u * np;
-                                f.slots(r0, r1, w[0], w[np], w[2 * np], w[(2 + h) * np]);
+                                f.slots(r0, r1, e, sel, w[0], w[np], w[2 * np], w[(2 + h) * np]);
                             }
+                            if (q0 & kFixRing) f.fold();
                         }
                         __syncwarp();   // every slot has been read
                         fetch.start(fs, ring, np);
@@ -772,14 +783,25 @@ __global__ void __launch_bounds__(MAXT, 1) rk4_persistent(const __grid_constant_
                         fetch.copy(1);
                     } else {
                         const W *we = h ? wh : wd;
+                        for (int q0 = 0; q0 < a.SLQ; q0 += kFixRing) {
 #pragma unroll 2
-                        for (int q = 0; q < a.SLQ; ++q, off += stride) {
-                            const L j = __ldg(lx + off);
-                            f.slots(sh_half(halo, 2 * j.x + h), sh_half(halo, 2 * j.y + h), __ldg(wx + off),
-                                    __ldg(wz + off), __ldg(wd + off), __ldg(we + off));
+                            for (int q = q0; q < min(q0 + kFixRing, a.SLQ); ++q, off += stride) {
+                                const L j = __ldg(lx + off);
+                                f.slots(sh_half(halo, 2 * j.x + h), sh_half(halo, 2 * j.y + h), __ldg(lq + off), sel,
+                                        __ldg(wx + off), __ldg(wz + off), __ldg(wd + off), __ldg(we + off));
+                            }
+                            if (q0 & kFixRing) f.fold();
                         }
                     }
-                    const HalfSums sums = fix_finish<G>(f, ew, h);
+                    f.fold();
+                    const HalfSums sums =
+                        fix_choose<G>(f, holds, reinterpret_cast<const int4 *>(halo) + h,
+                                      [lx, lq, off0, stride](int k) {
+                                          const L j = __ldg(lx + off0 + k * stride);
+                                          const uint2 e = __ldg(lq + off0 + k * stride);
+                                          return make_int4(j.x, j.y, (int)e.x, (int)e.y);
+                                      },
+                                      wx + off0, a.total / V, stride, a.SLQ, ew, h);
                     const double2 kk = fix_tendency(sums, {a.cp, a.g_over_tb, a.theta_bar, a.dpibar, a.rd_cv}, h,
                                                     make_double4(fi.u, fi.w, fi.t, fi.p), pib, fl);
                     k[0] = kk.x;
@@ -1021,6 +1043,7 @@ PArgs<T> pargs(Problem &pb, T *U, double dt, int64_t n_steps) {
     a.pw = (const T *)ps.pw.p;
     a.wexp = pb.wexp.p;
     a.lidx = ps.lidx.p;
+    a.wq = ps.wq.p;
     a.hlist = ps.hlist.p;
     a.cta = (const CtaInfo *)ps.cta.p;
     a.blob = ps.blob.p;
@@ -1156,20 +1179,31 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
     const bool lat0 = pb.lat.enabled;
     DevBuf<int32_t> pidx0 = std::move(pb.pidx);
     DevBuf<unsigned char> pw0 = std::move(pb.pw);
+    DevBuf<int4> nbr0 = std::move(pb.nbr);
     pb.lat.enabled = false;
     auto restore = [&] {
         pb.pidx = std::move(pidx0);
         pb.pw = std::move(pw0);
+        pb.nbr = std::move(nbr0);
         pb.G = G0; pb.pf = pf0; pb.SLQ = SLQ0; pb.SL = SL0; pb.V = V0;
         pb.lat.enabled = lat0;
     };
     std::vector<int32_t> hp;
     std::vector<unsigned char> hw;
+    std::vector<uint32_t> hq;
     int SLQ = 0, V = 0;
     try {
         pb.G = S;
         pack_operators(pb, false);
-        hp = to_host(pb.pidx);
+        if (fp64) {
+            const std::vector<int4> nbr = to_host(pb.nbr);
+            for (const int4 &v : nbr) {
+                hp.insert(hp.end(), {v.x, v.y});
+                hq.insert(hq.end(), {(uint32_t)v.z, (uint32_t)v.w});
+            }
+        } else {
+            hp = to_host(pb.pidx);
+        }
         hw = to_host(pb.pw);
         SLQ = pb.SLQ;
         V = pb.V;
@@ -1277,6 +1311,7 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
     std::vector<unsigned char> blob;
     std::vector<uint16_t> lidx((size_t)SLQ * lanes * GV, 0);
     std::vector<unsigned char> pwp((size_t)4 * SLQ * lanes * GV * ts, 0);
+    std::vector<uint32_t> wqp(hq.empty() ? 0 : lidx.size(), 0);
     const int64_t tot_old = (int64_t)SLQ * P * GV;
     const int64_t tot_new = (int64_t)SLQ * lanes * GV;
     std::vector<int32_t> stamp(pb.n_all, -1), loc(pb.n_all, 0), wstamp(pb.n_all, -1);
@@ -1371,6 +1406,7 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
                 // a node's slots of one step are contiguous in both packings
                 const int64_t eo = ((int64_t)q * P + i) * GV, en = ((int64_t)q * lanes + p) * GV;
                 for (int s = 0; s < GV; ++s) lidx[en + s] = (uint16_t)loc[hp[eo + s]];
+                if (!hq.empty()) std::copy_n(hq.begin() + eo, GV, wqp.begin() + en);
                 for (int f = 0; f < 4; ++f)
                     memcpy(pwp.data() + ((size_t)f * tot_new + en) * ts, hw.data() + ((size_t)f * tot_old + eo) * ts,
                            (size_t)GV * ts);
@@ -1543,11 +1579,13 @@ bool persistent_plan(Problem &pb, int G, int ctas) {
     ps.ring_off = ring_off;
     ps.pw.alloc(pwp.size());
     ps.lidx.alloc(lidx.size());
+    ps.wq.alloc(wqp.size());
     ps.hlist.alloc(hlist.size());
     ps.cta.alloc(info.size() * sizeof(CtaInfo));
     ps.blob.alloc(std::max<size_t>(blob.size(), 16));
     RBF_CUDA(cudaMemcpy(ps.pw.p, pwp.data(), pwp.size(), cudaMemcpyHostToDevice));
     RBF_CUDA(cudaMemcpy(ps.lidx.p, lidx.data(), ps.lidx.bytes(), cudaMemcpyHostToDevice));
+    if (!wqp.empty()) RBF_CUDA(cudaMemcpy(ps.wq.p, wqp.data(), ps.wq.bytes(), cudaMemcpyHostToDevice));
     RBF_CUDA(cudaMemcpy(ps.hlist.p, hlist.data(), ps.hlist.bytes(), cudaMemcpyHostToDevice));
     RBF_CUDA(cudaMemcpy(ps.cta.p, info.data(), ps.cta.bytes(), cudaMemcpyHostToDevice));
     if (!blob.empty()) RBF_CUDA(cudaMemcpy(ps.blob.p, blob.data(), blob.size(), cudaMemcpyHostToDevice));

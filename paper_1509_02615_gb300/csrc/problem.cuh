@@ -93,6 +93,7 @@ struct PersistPlan {
     size_t net_smem = 0;         // FP32: a corrected run's shared memory (a9; 0: the network does not fit)
     DevBuf<unsigned char> pw;    // T [4][SLQ][grid * chunk][S][V], as Problem::pw
     DevBuf<uint16_t> lidx;       // [SLQ][grid * chunk][S][V] list position of each slot
+    DevBuf<uint32_t> wq;         // FP64: exponent bytes of each slot's weights, alike
     DevBuf<int32_t> hlist;       // record lists of all CTAs
     DevBuf<unsigned char> cta;   // per-CTA layout records
     DevBuf<unsigned char> blob;  // per-CTA ghost-row and ghost-value data
@@ -152,6 +153,8 @@ struct Problem {
     DevBuf<unsigned char> pw;     // T [n_packed][SLQ][n_prog][G][V]; NS in FP64: fixed-point
                                   // pairs int2 (fixdot.cuh) in place of the doubles
     DevBuf<short4> wexp;          // [n_prog] NS in FP64: exponents of the packed rows
+    DevBuf<int4> nbr;             // NS in FP64, in place of pidx: [SLQ][n_prog][G], the indices of two slots
+                                  // (x, y) and their weights' exponent bytes (z, w)
     DevBuf<unsigned char> pibar;  // T [n_prog]
     DevBuf<unsigned char> flags;  // [n_prog]: bit0 w Dirichlet, bit1 u Dirichlet, bit2 wall set
 
@@ -201,6 +204,7 @@ struct Problem {
         DevBuf<int32_t> loff;         // [n_cls][SLQ][G][V] relative index of each slot
         DevBuf<unsigned char> lw;     // T [4][n_cls][SLQ][G][V] packed operators (FP64: as pw)
         DevBuf<short4> lexp;          // [n_cls] FP64: exponents of the packed rows
+        DevBuf<int4> lnbr;            // FP64, in place of loff: [n_cls][SLQ][G], as nbr with relative indices
     } lat;
 
     float weight_build_ms = 0.f, ghost_setup_ms = 0.f;
