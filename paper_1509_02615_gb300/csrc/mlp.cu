@@ -31,6 +31,7 @@ namespace rbf {
 constexpr int kWidth = 64;
 constexpr int kTrainRows = 32;               // rows of a training block: 31 samples and the all-zero row
 constexpr int kTrainSamples = kTrainRows - 1;
+constexpr int kTrainSets = 608;               // most blocks of a training launch (their partials: 34 MB for n = 37)
 constexpr int kTrainThreads = 320;           // 10 warps: two passes over the 592 tiles of dW1 (n = 37)
 constexpr int kScaleWarps = 2048;   // warps of the scale-sum launch (256 blocks of 256 threads)
 constexpr float kClip = 4.f;   // |y| <= 4 (in output-scale units) when the correction is applied
@@ -299,10 +300,13 @@ __device__ __forceinline__ void rows_times(const float *A, const float *B, int b
         *reinterpret_cast<float4 *>(out + (c0 + c) * kRS + r0) = make_float4(acc[c][0], acc[c][1], acc[c][2], acc[c][3]);
 }
 
+// a block's partial: v of its first tile, then what the others add
+__device__ __forceinline__ void put(float *p, float v, bool add) { *p = add ? *p + v : v; }
+
 // G[a][b] = sum over the 32 rows of A[a][row] B[b][row] for a < na and 64
-// columns b (a weight gradient): 4 x 4 outputs per thread, interleaved so that
-// the vectors a warp reads lie in distinct banks.
-__device__ __forceinline__ void outer_sum(const float *A, int na, const float *B, float *G) {
+// columns b (a weight gradient), on top of what G holds with `add`: 4 x 4 outputs
+// per thread, interleaved so that the vectors a warp reads lie in distinct banks.
+__device__ __forceinline__ void outer_sum(const float *A, int na, const float *B, float *G, bool add) {
     const int ga = (na + 3) / 4;
     for (int e = threadIdx.x; e < ga * 16; e += blockDim.x) {
         const int tb = e & 15, ta = e >> 4;
@@ -335,7 +339,7 @@ __device__ __forceinline__ void outer_sum(const float *A, int na, const float *B
         for (int i = 0; i < 4; ++i)
             if (ta + i * ga < na)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) G[(int64_t)(ta + i * ga) * kWidth + tb + 16 * j] = acc[i][j];
+                for (int j = 0; j < 4; ++j) put(G + (int64_t)(ta + i * ga) * kWidth + tb + 16 * j, acc[i][j], add);
     }
 }
 
@@ -349,9 +353,11 @@ __device__ __forceinline__ float row_sum(const float *v) {
     return s;
 }
 
-// Fused gather + forward + backward for one block of 31 samples; the block's
-// weight gradients (X^T dH1, H1^T dH2, H2^T dY and bias sums) and loss go to
-// its own partials, which mlp_reduce_kernel sums over the blocks in block
+// Fused gather + forward + backward for tiles of 31 samples, one per block; from
+// kTrainSets blocks on a block takes every gridDim-th tile, which bounds the
+// partials (a set per tile would be 1.8 GB at a million samples).  The block's
+// weight gradients (X^T dH1, H1^T dH2, H2^T dY and bias sums) and loss go to its
+// own partials, which mlp_reduce_kernel sums over the blocks in block
 // order (so training is deterministic).  Row 31 is the all-zero feature row:
 // its output is f(0), which enters every y with the opposite sign, so its
 // output gradient is minus the sum of the others'.
@@ -375,163 +381,171 @@ __global__ void __launch_bounds__(kTrainThreads) mlp_train_kernel(TrainArgs a, O
     float *X = sf + L.X, *H1 = sf + L.H1, *H2 = sf + L.H2, *P = sf + L.P, *dH2 = sf + L.dH2, *dH1 = sf + L.dH1,
           *Y = sf + L.Y;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    // samples and features do not depend on the preceding kernel
-    if (t < kTrainRows) {
-        const int s = blockIdx.x * kTrainSamples + t;
-        int64_t k = 0, i = -1;
-        if (t < kTrainSamples && s < a.B) {
-            if (a.samples) {
-                k = a.samples[2 * (int64_t)s];
-                i = a.samples[2 * (int64_t)s + 1];
-            } else {
-                const unsigned long long h = splitmix64(a.seed ^ splitmix64((unsigned long long)a.iter * 0x100000001ull + s));
-                k = (int64_t)(h % (unsigned long long)a.n_states);
-                i = (int64_t)((h >> 32) % (unsigned long long)a.n_prog);
-            }
-        }
-        s_state[t] = state_of(k, a.n_snap) * a.n_all;
-        s_target[t] = k * a.n_prog + i;
-        s_node[t] = (int)i;
-    }
-    __syncthreads();
-    {
-        // a warp takes one slot of the 32 rows at a time (the last one: the node's own values)
-        const int i = s_node[lane];
-        const float *Uk = a.S + s_state[lane] * 4;
-        Rec<float> own = {0.f, 0.f, 0.f, 0.f};
-        if (i >= 0) own = load_rec(Uk, i);
-        const float is0 = 1.f / a.scales[0], is1 = 1.f / a.scales[1], is2 = 1.f / a.scales[2], is3 = 1.f / a.scales[3];
-#pragma unroll 4
-        for (int q = warp; q <= slots; q += kTrainThreads / 32) {
-            float f0 = 0.f, f1 = 0.f, f2 = 0.f, f3 = 0.f;
-            if (i >= 0) {
-                if (q < slots) {
-                    const Rec<float> r = load_rec(Uk, __ldg(a.idx + (int64_t)i * a.n + q + 1));
-                    f0 = (r.u - own.u) * is0;
-                    f1 = (r.w - own.w) * is1;
-                    f2 = (r.t - own.t) * is2;
-                    f3 = (r.p - own.p) * is3;
+    const int64_t tiles = (a.B + (int64_t)kTrainSamples - 1) / kTrainSamples;
+    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const bool add = tile != blockIdx.x;
+        if (add) __syncthreads();   // the rows of the tile before have been read
+        // samples and features do not depend on the preceding kernel
+        if (t < kTrainRows) {
+            const int64_t s = tile * (int64_t)kTrainSamples + t;
+            int64_t k = 0, i = -1;
+            if (t < kTrainSamples && s < a.B) {
+                if (a.samples) {
+                    k = a.samples[2 * s];
+                    i = a.samples[2 * s + 1];
                 } else {
-                    f0 = own.u / a.scales[8];
-                    f1 = own.w / a.scales[9];
-                    f2 = own.t / a.scales[10];
-                    f3 = own.p / a.scales[11];
+                    const unsigned long long h = splitmix64(a.seed ^ splitmix64((unsigned long long)a.iter * 0x100000001ull + s));
+                    k = (int64_t)(h % (unsigned long long)a.n_states);
+                    i = (int64_t)((h >> 32) % (unsigned long long)a.n_prog);
                 }
             }
-            const int c = q < slots ? q : 4 * slots, step = q < slots ? slots : 1;
-            X[c * kRS + lane] = f0;
-            X[(c + step) * kRS + lane] = f1;
-            X[(c + 2 * step) * kRS + lane] = f2;
-            X[(c + 3 * step) * kRS + lane] = f3;
+            s_state[t] = state_of(k, a.n_snap) * a.n_all;
+            s_target[t] = k * a.n_prog + i;
+            s_node[t] = (int)i;
         }
-    }
-    grid_dep_wait();     // the weights come from the preceding iteration's kernel
-    grid_dep_launch();
-    // BF16 weights, eight per load (every block of Pb starts at a multiple of 64 values)
-    const uint4 *w1 = reinterpret_cast<const uint4 *>(a.Pb + m_off.oW1), *w2 = reinterpret_cast<const uint4 *>(a.Pb + m_off.oW2);
+        __syncthreads();
+        {
+            // a warp takes one slot of the 32 rows at a time (the last one: the node's own values)
+            const int i = s_node[lane];
+            const float *Uk = a.S + s_state[lane] * 4;
+            Rec<float> own = {0.f, 0.f, 0.f, 0.f};
+            if (i >= 0) own = load_rec(Uk, i);
+            const float is0 = 1.f / a.scales[0], is1 = 1.f / a.scales[1], is2 = 1.f / a.scales[2], is3 = 1.f / a.scales[3];
 #pragma unroll 4
-    for (int e = t; e < n_in * kWidth / 8; e += kTrainThreads) put8(sf + L.W1 + 8 * e, __ldcg(w1 + e));
-#pragma unroll 2
-    for (int e = t; e < kWidth * kWidth / 8; e += kTrainThreads) {
-        float *v = sf + L.W2 + 8 * e;
-        put8(v, __ldcg(w2 + e));
-        const int m = e / (kWidth / 8), j = e % (kWidth / 8) * 8;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) sf[L.W2t + (j + q) * (kWidth + 4) + m] = v[q];
-    }
-    for (int e = t; e < kWidth * 4; e += kTrainThreads) sf[L.W3 + e] = bf(a.Pb[m_off.oW3 + e]);
-    if (t < kWidth) {
-        sf[L.b + t] = a.P[m_off.ob1 + t];
-        sf[L.b + kWidth + t] = a.P[m_off.ob2 + t];
-    }
-    if (t < 4) sf[L.b + 2 * kWidth + t] = a.P[m_off.ob3 + t];
-    __syncthreads();
-    // forward
-    rows_times(X, sf + L.W1, kWidth, n_in, P);
-    __syncthreads();
-    for (int e = t; e < kWidth * kTrainRows; e += kTrainThreads) {
-        const int j = e / kTrainRows, at = j * kRS + e % kTrainRows;
-        H1[at] = tanhf(sf[L.b + j] + (P[at] + P[kWidth * kRS + at]));
-    }
-    __syncthreads();
-    rows_times(H1, sf + L.W2, kWidth, kWidth, P);
-    __syncthreads();
-    for (int e = t; e < kWidth * kTrainRows; e += kTrainThreads) {
-        const int j = e / kTrainRows, at = j * kRS + e % kTrainRows;
-        H2[at] = tanhf(sf[L.b + kWidth + j] + (P[at] + P[kWidth * kRS + at]));
-    }
-    __syncthreads();
-    if (t < 4 * kTrainRows) {
-        const int r = t % kTrainRows, c = t / kTrainRows;
-        float y0 = 0.f, y1 = 0.f, y2 = 0.f, y3 = 0.f;
-#pragma unroll 4
-        for (int m = 0; m < kWidth; m += 4) {
-            y0 += H2[m * kRS + r] * sf[L.W3 + m * 4 + c];
-            y1 += H2[(m + 1) * kRS + r] * sf[L.W3 + m * 4 + 4 + c];
-            y2 += H2[(m + 2) * kRS + r] * sf[L.W3 + m * 4 + 8 + c];
-            y3 += H2[(m + 3) * kRS + r] * sf[L.W3 + m * 4 + 12 + c];
-        }
-        Y[r * 4 + c] = sf[L.b + 2 * kWidth + c] + ((y0 + y1) + (y2 + y3));
-    }
-    __syncthreads();
-    if (warp == 0) {
-        // loss and output gradients, one row per lane; row 31 holds f(0)
-        const bool live = s_node[lane] >= 0;
-        const float inv = 1.f / (4.f * (float)a.B);
-        const float4 y = ld4(Y + lane * 4);
-        const float yr[4] = {y.x, y.y, y.z, y.w};
-        float loss = 0.f, d[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const float f0 = __shfl_sync(0xffffffffu, yr[c], kTrainRows - 1);
-            d[c] = 0.f;
-            if (live) {
-                const float r = yr[c] - f0 - a.Tg[s_target[lane] * 4 + c] / a.scales[4 + c];
-                loss += r * r * inv;
-                d[c] = 2.f * r * inv;
+            for (int q = warp; q <= slots; q += kTrainThreads / 32) {
+                float f0 = 0.f, f1 = 0.f, f2 = 0.f, f3 = 0.f;
+                if (i >= 0) {
+                    if (q < slots) {
+                        const Rec<float> r = load_rec(Uk, __ldg(a.idx + (int64_t)i * a.n + q + 1));
+                        f0 = (r.u - own.u) * is0;
+                        f1 = (r.w - own.w) * is1;
+                        f2 = (r.t - own.t) * is2;
+                        f3 = (r.p - own.p) * is3;
+                    } else {
+                        f0 = own.u / a.scales[8];
+                        f1 = own.w / a.scales[9];
+                        f2 = own.t / a.scales[10];
+                        f3 = own.p / a.scales[11];
+                    }
+                }
+                const int c = q < slots ? q : 4 * slots, step = q < slots ? slots : 1;
+                X[c * kRS + lane] = f0;
+                X[(c + step) * kRS + lane] = f1;
+                X[(c + 2 * step) * kRS + lane] = f2;
+                X[(c + 3 * step) * kRS + lane] = f3;
             }
-            float sum = d[c];
-            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-            if (lane == kTrainRows - 1) d[c] = -sum;
-            if (lane == c) gp[m_off.ob3 + c] = sum - sum;   // the rows' gradients cancel: db3 = 0 (or NaN)
         }
-        *reinterpret_cast<float4 *>(Y + lane * 4) = make_float4(d[0], d[1], d[2], d[3]);
-        for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
-        if (lane == 0) a.Lp[blockIdx.x] = loss;
-    }
-    __syncthreads();
-    // dW3 = H2^T dY; dH2 = (dY W3^T) o (1 - h2^2)
-    for (int e = t; e < kWidth * 4; e += kTrainThreads) {
-        const int m = e >> 2, c = e & 3;
-        float s0 = 0.f, s1 = 0.f;
+        if (!add) {
+            grid_dep_wait();     // the weights come from the preceding iteration's kernel
+            grid_dep_launch();
+            // BF16 weights, eight per load (every block of Pb starts at a multiple of 64 values)
+            const uint4 *w1 = reinterpret_cast<const uint4 *>(a.Pb + m_off.oW1), *w2 = reinterpret_cast<const uint4 *>(a.Pb + m_off.oW2);
+#pragma unroll 4
+            for (int e = t; e < n_in * kWidth / 8; e += kTrainThreads) put8(sf + L.W1 + 8 * e, __ldcg(w1 + e));
+#pragma unroll 2
+            for (int e = t; e < kWidth * kWidth / 8; e += kTrainThreads) {
+                float *v = sf + L.W2 + 8 * e;
+                put8(v, __ldcg(w2 + e));
+                const int m = e / (kWidth / 8), j = e % (kWidth / 8) * 8;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) sf[L.W2t + (j + q) * (kWidth + 4) + m] = v[q];
+            }
+            for (int e = t; e < kWidth * 4; e += kTrainThreads) sf[L.W3 + e] = bf(a.Pb[m_off.oW3 + e]);
+            if (t < kWidth) {
+                sf[L.b + t] = a.P[m_off.ob1 + t];
+                sf[L.b + kWidth + t] = a.P[m_off.ob2 + t];
+            }
+            if (t < 4) sf[L.b + 2 * kWidth + t] = a.P[m_off.ob3 + t];
+        }
+        __syncthreads();
+        // forward
+        rows_times(X, sf + L.W1, kWidth, n_in, P);
+        __syncthreads();
+        for (int e = t; e < kWidth * kTrainRows; e += kTrainThreads) {
+            const int j = e / kTrainRows, at = j * kRS + e % kTrainRows;
+            H1[at] = tanhf(sf[L.b + j] + (P[at] + P[kWidth * kRS + at]));
+        }
+        __syncthreads();
+        rows_times(H1, sf + L.W2, kWidth, kWidth, P);
+        __syncthreads();
+        for (int e = t; e < kWidth * kTrainRows; e += kTrainThreads) {
+            const int j = e / kTrainRows, at = j * kRS + e % kTrainRows;
+            H2[at] = tanhf(sf[L.b + kWidth + j] + (P[at] + P[kWidth * kRS + at]));
+        }
+        __syncthreads();
+        if (t < 4 * kTrainRows) {
+            const int r = t % kTrainRows, c = t / kTrainRows;
+            float y0 = 0.f, y1 = 0.f, y2 = 0.f, y3 = 0.f;
+#pragma unroll 4
+            for (int m = 0; m < kWidth; m += 4) {
+                y0 += H2[m * kRS + r] * sf[L.W3 + m * 4 + c];
+                y1 += H2[(m + 1) * kRS + r] * sf[L.W3 + m * 4 + 4 + c];
+                y2 += H2[(m + 2) * kRS + r] * sf[L.W3 + m * 4 + 8 + c];
+                y3 += H2[(m + 3) * kRS + r] * sf[L.W3 + m * 4 + 12 + c];
+            }
+            Y[r * 4 + c] = sf[L.b + 2 * kWidth + c] + ((y0 + y1) + (y2 + y3));
+        }
+        __syncthreads();
+        if (warp == 0) {
+            // loss and output gradients, one row per lane; row 31 holds f(0)
+            const bool live = s_node[lane] >= 0;
+            const float inv = 1.f / (4.f * (float)a.B);
+            const float4 y = ld4(Y + lane * 4);
+            const float yr[4] = {y.x, y.y, y.z, y.w};
+            float loss = 0.f, d[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float f0 = __shfl_sync(0xffffffffu, yr[c], kTrainRows - 1);
+                d[c] = 0.f;
+                if (live) {
+                    const float r = yr[c] - f0 - a.Tg[s_target[lane] * 4 + c] / a.scales[4 + c];
+                    loss += r * r * inv;
+                    d[c] = 2.f * r * inv;
+                }
+                float sum = d[c];
+                for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                if (lane == kTrainRows - 1) d[c] = -sum;
+                if (lane == c) put(gp + m_off.ob3 + c, sum - sum, add);   // the rows' gradients cancel: db3 = 0 (or NaN)
+            }
+            *reinterpret_cast<float4 *>(Y + lane * 4) = make_float4(d[0], d[1], d[2], d[3]);
+            for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+            if (lane == 0) put(a.Lp + blockIdx.x, loss, add);
+        }
+        __syncthreads();
+        // dW3 = H2^T dY; dH2 = (dY W3^T) o (1 - h2^2)
+        for (int e = t; e < kWidth * 4; e += kTrainThreads) {
+            const int m = e >> 2, c = e & 3;
+            float s0 = 0.f, s1 = 0.f;
 #pragma unroll 8
-        for (int r = 0; r < kTrainRows; r += 2) {
-            s0 += H2[m * kRS + r] * Y[r * 4 + c];
-            s1 += H2[m * kRS + r + 1] * Y[r * 4 + 4 + c];
+            for (int r = 0; r < kTrainRows; r += 2) {
+                s0 += H2[m * kRS + r] * Y[r * 4 + c];
+                s1 += H2[m * kRS + r + 1] * Y[r * 4 + 4 + c];
+            }
+            put(gp + m_off.oW3 + e, s0 + s1, add);
         }
-        gp[m_off.oW3 + e] = s0 + s1;
+        for (int e = t; e < kWidth * kTrainRows; e += kTrainThreads) {
+            const int m = e / kTrainRows, r = e % kTrainRows;
+            const float4 dy = ld4(Y + r * 4), w = ld4(sf + L.W3 + m * 4);
+            const float h = H2[m * kRS + r];
+            dH2[m * kRS + r] = (dy.x * w.x + dy.y * w.y + dy.z * w.z + dy.w * w.w) * (1.f - h * h);
+        }
+        __syncthreads();
+        // dW2 = H1^T dH2, db2 = sum dH2; dH1 = (dH2 W2^T) o (1 - h1^2)
+        outer_sum(H1, kWidth, dH2, gp + m_off.oW2, add);
+        rows_times(dH2, sf + L.W2t, kWidth + 4, kWidth, P);
+        const int tail = t - (kTrainThreads - kWidth);   // the last 64 threads sum the biases
+        if (tail >= 0) put(gp + m_off.ob2 + tail, row_sum(dH2 + tail * kRS), add);
+        __syncthreads();
+        for (int e = t; e < kWidth * kTrainRows; e += kTrainThreads) {
+            const int m = e / kTrainRows, at = m * kRS + e % kTrainRows;
+            const float h = H1[at];
+            dH1[at] = (P[at] + P[kWidth * kRS + at]) * (1.f - h * h);
+        }
+        __syncthreads();
+        // dW1 = X^T dH1, db1 = sum dH1
+        outer_sum(X, n_in, dH1, gp + m_off.oW1, add);
+        if (tail >= 0) put(gp + m_off.ob1 + tail, row_sum(dH1 + tail * kRS), add);
     }
-    for (int e = t; e < kWidth * kTrainRows; e += kTrainThreads) {
-        const int m = e / kTrainRows, r = e % kTrainRows;
-        const float4 dy = ld4(Y + r * 4), w = ld4(sf + L.W3 + m * 4);
-        const float h = H2[m * kRS + r];
-        dH2[m * kRS + r] = (dy.x * w.x + dy.y * w.y + dy.z * w.z + dy.w * w.w) * (1.f - h * h);
-    }
-    __syncthreads();
-    // dW2 = H1^T dH2, db2 = sum dH2; dH1 = (dH2 W2^T) o (1 - h1^2)
-    outer_sum(H1, kWidth, dH2, gp + m_off.oW2);
-    rows_times(dH2, sf + L.W2t, kWidth + 4, kWidth, P);
-    if (t >= kTrainThreads - kWidth) gp[m_off.ob2 + t - (kTrainThreads - kWidth)] = row_sum(dH2 + (t - (kTrainThreads - kWidth)) * kRS);
-    __syncthreads();
-    for (int e = t; e < kWidth * kTrainRows; e += kTrainThreads) {
-        const int m = e / kTrainRows, at = m * kRS + e % kTrainRows;
-        const float h = H1[at];
-        dH1[at] = (P[at] + P[kWidth * kRS + at]) * (1.f - h * h);
-    }
-    __syncthreads();
-    // dW1 = X^T dH1, db1 = sum dH1
-    outer_sum(X, n_in, dH1, gp + m_off.oW1);
-    if (t >= kTrainThreads - kWidth) gp[m_off.ob1 + t - (kTrainThreads - kWidth)] = row_sum(dH1 + (t - (kTrainThreads - kWidth)) * kRS);
 }
 
 // G = sum over the blocks of their gradient partials and the iteration's loss
@@ -685,7 +699,7 @@ void mlp_launch_train(Mlp &m, Problem &pb, const float *S, const float *Tg, int6
     a.Pb = m.Pb.p;
     a.P = m.P.p;
     a.scales = m.scales.p;
-    const int nb = div_up(B, kTrainSamples);
+    const int nb = std::min(div_up(B, kTrainSamples), kTrainSets);
     if (m.Gp.n < (size_t)nb * m.n_params) m.Gp.alloc((size_t)nb * m.n_params);
     if (m.Lp.n < (size_t)nb) m.Lp.alloc(nb);
     a.Gp = m.Gp.p;
