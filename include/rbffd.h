@@ -330,7 +330,9 @@ int rbf_mlp_forward(rbf_mlp *m, const void *U, void *delta);
  * U_f += alpha[f] * dt * delta_f (alpha: host double [4], each >= 0; all
  * zero is the uncorrected solver).
  * A non-finite delta is skipped (the uncorrected step is kept) and counted
- * in *n_fallback (host, optional).  Synchronous.
+ * in *n_fallback (host, optional).  One launch of the persistent kernel if the
+ * coarse problem is in persistent mode and the network fits its shared memory,
+ * else a few kernels per step.  Synchronous.
  */
 int rbf_learned_run(rbf_mlp *m, double t0, double dt, int64_t n_steps, const double *alpha, void *U,
                     int64_t *n_fallback);
@@ -406,15 +408,16 @@ int rbf_run(rbf_problem *pb, double t0, double dt, int64_t n_steps, void *U);
  *                       every node fits one co-resident grid.
  *                       Advection problems (Sec. 6.1, RK4): every lane
  *                       keeps its packed slots in registers, each stage
- *                       gathers the stage input through L2 and the CTAs
- *                       meet at a grid barrier; results equal the graph
+ *                       gathers the stage input and the CTAs meet at a
+ *                       grid barrier; results equal the graph
  *                       mode's bit for bit with the same lanes per node.
  *   RBF_RUN_AUTO        time both on a zero state and keep the faster
  *                       (done at creation when threads_per_node is 0, and
  *                       always for advection problems).
  * lanes: lanes per node of the persistent kernel (Navier-Stokes 1, 2 or 4;
  *        advection 2, 4 or 8, which also become the lanes of the graph
- *        mode; 0 = fastest, for FP32 advection also one lane).
+ *        mode; 0 = fastest, for FP32 advection also one lane, which is
+ *        kept until the mode is set again and not taken by name).
  * ctas:  CTAs of the persistent kernel (0: fastest of 1, 1/2, 1/4, 1/8 per
  *        SM; with lanes > 0 and RBF_RUN_PERSISTENT, one per SM untimed).
  *        Advection problems take 0: their CTA count follows from the lanes
@@ -540,11 +543,14 @@ typedef struct rbf_info {
     double ghost_setup_ms;      /* GPU time of the ghost inverses           */
     double rhs_bytes_per_node;  /* algorithmic HBM bytes of one RHS stage   */
     double rhs_flops_per_node;  /* arithmetic of one RHS stage              */
-    int32_t persist_lanes;      /* persistent kernel: lanes per node (0: none) */
+    int32_t persist_lanes;      /* persistent kernel: lanes per node as asked
+                                   for (0: none); in FP64, where two threads
+                                   share a lane, 4 become 2 if a CTA's nodes
+                                   need it, with the same bits                 */
     int32_t persist_regs;       /* 1: it keeps its operands in registers    */
     int32_t persist_chunk;      /* nodes per CTA                            */
     int32_t persist_halo_max;   /* largest per-CTA record list (0 for
-                                   advection, which gathers through L2)      */
+                                   advection, which has none)               */
     int32_t persist_ctas;       /* CTAs of the persistent launch            */
     int32_t stage_split;        /* 1: split stage launches (rbf_set_stage_split) */
 } rbf_info;

@@ -367,8 +367,8 @@ __device__ __forceinline__ float row_sum(const float *v) {
 // block per SM at the default batch of 4096 (133 blocks); every product runs
 // from shared memory with 16 FMAs per two 16-byte loads.  One thread per
 // sample with the activations in registers (32 blocks of 128 threads) took
-// 207 us per launch and 217 us per iteration with its two follow-up kernels
-// at 4096 samples, n = 37; this form 21 us per iteration, reduction and Adam
+// 207 us per launch and 217 us of device time per iteration with its two
+// follow-up kernels at 4096 samples, n = 37; this form 21 us, reduction and Adam
 // included.
 __global__ void __launch_bounds__(kTrainThreads) mlp_train_kernel(TrainArgs a, Offs m_off) {
     extern __shared__ __align__(16) float sf[];

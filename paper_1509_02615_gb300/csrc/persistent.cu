@@ -22,7 +22,7 @@
 // rows.  The two steps stay apart: coefficients of the ghosts on the records
 // (products of the two, formed in FP64 and rounded once) took 770 in place of
 // 950 us for 50 steps at 400 m in FP32, but their sums do not keep the
-// residuals small, and runs in walled boxes were 1.3 to 1.7 times further from
+// residuals small, and runs in walled boxes were 1.2 to 2.1 times further from
 // FP64 (tests/test_gpu_persistent_accuracy.py).
 //
 // Learned correction (a9, MLP variants): at stage 0 of every step the CTA's
@@ -903,7 +903,7 @@ __global__ void __launch_bounds__(MAXT, 1) rk4_persistent(const __grid_constant_
 // Here each lane keeps its R packed slots (stencil index, flux weights of
 // each velocity part, hyperviscosity weight) in registers for the whole run,
 // U_n and the RK4 accumulator of its node too; a stage gathers the stage
-// input through L2, forms the tendency and the RK4 update exactly as the
+// input (ordinary loads: the barrier's acquire orders them), forms the tendency and the RK4 update exactly as the
 // stage kernel does (same slots per lane, summation order, lane reduction,
 // time factors and update), and the CTAs meet at a grid barrier.  Results
 // equal the launch-per-stage form's bit for bit with the same lanes per node.

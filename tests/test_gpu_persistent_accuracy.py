@@ -5,7 +5,7 @@ inverse and sum the stencils alike, in other orders, so their distances from the
 FP64 run differ by sampling only: over four states, some thousand nodes and
 three or more boundary classes the ratio of the two root mean squares stays
 within 15% (a form of the ghost solve that does not keep the residuals small,
-the products of the two matrices applied to the records, is at 1.3 to 1.7).
+the products of the two matrices applied to the records, is at 1.2 to 2.1).
 """
 import numpy as np
 import pytest
