@@ -34,9 +34,13 @@
 // The largest exponents come from a first pass over the stencil's records
 // (they stay in L1 or shared memory for the second) and its weights' bytes, and
 // the integer sums of a node's lanes are added before anything is rounded, so
-// results do not depend on the number of lanes.  Sums of non-finite values, and
-// of products so small that the result would leave the normal range, go to
-// fix_plain: FP64 FMAs from the same operands.
+// results do not depend on the number of lanes.  Warps with a stencil whose
+// values all lie below 2^-950 or so (the tails ahead of every front in a run from
+// rest) go to fix_low, the same sums with a look at each value's implicit bit;
+// sums of non-finite values, or that would overflow, go to fix_plain: FP64 FMAs
+// from the same operands.  (With the tails in fix_plain too, a step of the 25 m
+// bubble took 1.29 ms in its first 25 steps from rest, with fix_low 0.94, in a
+// developed flow 0.91.)
 #pragma once
 
 #include <cuda_runtime.h>
@@ -113,15 +117,22 @@ struct FixScan {
     }
     __device__ __forceinline__ int E(int o) const { return (int)(o == 0 ? xz & 0xffffu : o == 1 ? xz >> 16 : dc & 0xffffu); }
     // whether the integer sums of operators with row exponents x, z, d hold: the
-    // values finite, every result in the normal range with 28 bits to spare below,
-    // and zeros (exponent 0, whose implicit bit is not there) shifted out
+    // values finite and every result below the largest number
     __device__ __forceinline__ bool holds(int x, int z, int d) const {
-        auto one = [&](int e, int er) { return er == kFixZero || (e >= 324 && e + er >= 340 && e + er <= 2356); };
+        auto one = [&](int e, int er) { return er == kFixZero || e + er <= 2356; };
         return bits == 0 || (dc >> 16 < 2047u && one(E(0), x) && one(E(1), z) && one(E(2), d));
+    }
+    // whether they take fix_low: results below the normal range and 28 bits above it,
+    // or zeros (exponent 0, whose implicit bit is not there) not shifted out
+    __device__ __forceinline__ bool low(int x, int z, int d) const {
+        auto one = [&](int e, int er) { return er != kFixZero && (e < 324 || e + er < 340); };
+        return bits != 0 && (one(E(0), x) || one(E(1), z) || one(E(2), d));
     }
 };
 
-// One field's sums with three operators.
+// One field's sums with three operators.  LOW: for values at the low end of the
+// range too (subnormal ones have exponent 1 and no implicit bit).
+template <bool LOW>
 struct FixSums {
     long long hh[3], cr[3];
     int E[3];
@@ -129,7 +140,8 @@ struct FixSums {
 #pragma unroll
         for (int o = 0; o < 3; ++o) {
             hh[o] = cr[o] = 0;
-            E[o] = s.bits ? s.E(o) : 0x10000;   // zeros: everything is shifted out
+            // zeros: everything is shifted out; LOW: no exponent is below 1 + q
+            E[o] = s.bits ? (LOW ? max(s.E(o), 256) : s.E(o)) : 0x10000;
         }
     }
     // A value (lo, hi) as F 2^4 without its shift, complemented if negative (so that
@@ -139,9 +151,11 @@ struct FixSums {
         int c;
         __device__ __forceinline__ Value(unsigned lo, int hi) {
             const int s = hi >> 31;
-            const unsigned T = __funnelshift_r(lo, ((unsigned)hi & 0xfffffu) | 0x100000u, 22) ^ (unsigned)s;
-            Y = (long long)((unsigned long long)T << 32 | ((lo << 10) ^ (unsigned)s));
             c = (hi & 0x7fffffff) >> 20;
+            const unsigned one = LOW && c == 0 ? 0u : 0x100000u;
+            const unsigned T = __funnelshift_r(lo, ((unsigned)hi & 0xfffffu) | one, 22) ^ (unsigned)s;
+            Y = (long long)((unsigned long long)T << 32 | ((lo << 10) ^ (unsigned)s));
+            if (LOW) c = max(c, 1);
         }
     };
     __device__ __forceinline__ void add(int o, const Value &v, int q, int wh, int wl) {
@@ -174,44 +188,15 @@ struct FixSums {
         c &= 0xfffffff;
         const int z = min(__clzll(h ^ (h >> 63)) - 1, 28);   // bits of c that fit below h
         const long long V = (h << z) + (c >> (28 - z));
+        if (LOW) return er == kFixZero || E[o] == 0x10000 ? 0.0
+                        : er == kFixBad                   ? __hiloint2double(0x7ff80000, 0)
+                                                          : ldexp((double)V, E[o] + er - 1333 - z);
         const int e = E[o] + er - 310 - z;   // exponent field of the power of two
         const int hi = er == kFixBad ? 0x7ff80000 : (unsigned)(e - 1) < 2046u ? e << 20 : 0;   // zeros: 0
         return (double)V * __hiloint2double(hi, 0);
     }
 };
 
-// One half of a node's sums: two threads share a node (and, with more lanes, a
-// slot lane), h = 0 for the fields u, w and h = 1 for theta', pi'.  Each
-// gathers its 16-byte half of the neighbours' records and holds the d/dx, d/dz
-// and dissipation (pi': hyperviscosity) sums of its two fields: half the
-// registers of the whole node, so that twice the warps hide the gathers.
-struct FixHalf {
-    FixSums a, b;
-    // sel: which byte of q is the second field's third operator (fix_third)
-    __device__ __forceinline__ void slot(const int4 &r, unsigned q, unsigned sel, int xh, int xl, int zh, int zl, int dh,
-                                         int dl, int bh, int bl) {
-        const int qx = fix_byte<0>(q), qz = fix_byte<1>(q);
-        const FixSums::Value va((unsigned)r.x, r.y);
-        a.add(0, va, qx, xh, xl);
-        a.add(1, va, qz, zh, zl);
-        a.add(2, va, fix_byte<2>(q), dh, dl);
-        const FixSums::Value vb((unsigned)r.z, r.w);
-        b.add(0, vb, qx, xh, xl);
-        b.add(1, vb, qz, zh, zl);
-        b.add(2, vb, (int)__byte_perm(q, 0, sel), bh, bl);
-    }
-    // two slots from one operand vector of each operator (d: third operator of
-    // the first field, e: of the second)
-    __device__ __forceinline__ void slots(const int4 &r0, const int4 &r1, uint2 q, unsigned sel, const int4 &x,
-                                          const int4 &z, const int4 &d, const int4 &e) {
-        slot(r0, q.x, sel, x.x, x.y, z.x, z.y, d.x, d.y, e.x, e.y);
-        slot(r1, q.y, sel, x.z, x.w, z.z, z.w, d.z, d.w, e.z, e.w);
-    }
-    __device__ __forceinline__ void fold() {
-        a.fold();
-        b.fold();
-    }
-};
 // selector of the second field's third operator: dissipation (w) or hyperviscosity (pi')
 __device__ __forceinline__ unsigned fix_third(int h) { return 0x4442u + (unsigned)h; }
 
@@ -231,17 +216,58 @@ struct FixHalfScan {
     __device__ __forceinline__ bool holds(short4 ew, int h) const {
         return a.holds(ew.x, ew.y, ew.z) && b.holds(ew.x, ew.y, h ? ew.w : ew.z);
     }
+    __device__ __forceinline__ bool low(short4 ew, int h) const {
+        return a.low(ew.x, ew.y, ew.z) || b.low(ew.x, ew.y, h ? ew.w : ew.z);
+    }
 };
 
+// One half of a node's sums: two threads share a node (and, with more lanes, a
+// slot lane), h = 0 for the fields u, w and h = 1 for theta', pi'.  Each
+// gathers its 16-byte half of the neighbours' records and holds the d/dx, d/dz
+// and dissipation (pi': hyperviscosity) sums of its two fields: half the
+// registers of the whole node, so that twice the warps hide the gathers.
+template <bool LOW>
+struct FixHalf {
+    using Value = typename FixSums<LOW>::Value;
+    FixSums<LOW> a, b;
+    __device__ __forceinline__ void start(const FixHalfScan &s) {
+        a.start(s.a);
+        b.start(s.b);
+    }
+    // sel: which byte of q is the second field's third operator (fix_third)
+    __device__ __forceinline__ void slot(const int4 &r, unsigned q, unsigned sel, int xh, int xl, int zh, int zl, int dh,
+                                         int dl, int bh, int bl) {
+        const int qx = fix_byte<0>(q), qz = fix_byte<1>(q);
+        const Value va((unsigned)r.x, r.y);
+        a.add(0, va, qx, xh, xl);
+        a.add(1, va, qz, zh, zl);
+        a.add(2, va, fix_byte<2>(q), dh, dl);
+        const Value vb((unsigned)r.z, r.w);
+        b.add(0, vb, qx, xh, xl);
+        b.add(1, vb, qz, zh, zl);
+        b.add(2, vb, (int)__byte_perm(q, 0, sel), bh, bl);
+    }
+    // two slots from one operand vector of each operator (d: third operator of
+    // the first field, e: of the second)
+    __device__ __forceinline__ void slots(const int4 &r0, const int4 &r1, uint2 q, unsigned sel, const int4 &x,
+                                          const int4 &z, const int4 &d, const int4 &e) {
+        slot(r0, q.x, sel, x.x, x.y, z.x, z.y, d.x, d.y, e.x, e.y);
+        slot(r1, q.y, sel, x.z, x.w, z.z, z.w, d.z, d.w, e.z, e.w);
+    }
+    __device__ __forceinline__ void fold() {
+        a.fold();
+        b.fold();
+    }
+};
 // A half's six sums as doubles (a: first field, b: second; x, z, d).
 struct HalfSums {
     double ax, az, ad, bx, bz, bd;
 };
-template <int G>
-__device__ __forceinline__ HalfSums fix_finish(const FixHalf &f, short4 ew, int h) {
+template <int G, bool LOW>
+__device__ __forceinline__ HalfSums fix_finish(const FixHalf<LOW> &f, short4 ew, int h) {
     const int e = h ? ew.w : ew.z;
-    return {f.a.value<G>(0, ew.x), f.a.value<G>(1, ew.y), f.a.value<G>(2, ew.z),
-            f.b.value<G>(0, ew.x), f.b.value<G>(1, ew.y), f.b.value<G>(2, e)};
+    return {f.a.template value<G>(0, ew.x), f.a.template value<G>(1, ew.y), f.a.template value<G>(2, ew.z),
+            f.b.template value<G>(0, ew.x), f.b.template value<G>(1, ew.y), f.b.template value<G>(2, e)};
 }
 
 // Tendencies of Eqs. (uEq)-(piEq) of the half's two fields from its sums and
@@ -374,12 +400,31 @@ __device__ __noinline__ HalfSums fix_plain(const int4 *half, Nbr nbr, const int4
     return {s[0], s[1], s[2], s[3], s[4], s[5]};
 }
 
-// A half's sums from the integers, or over the G lanes of plain sums if any of
-// the warp's do not hold (every lane of the warp takes part).
+// A half's integer sums at the low end of the range, with the operands straight
+// from memory: every lane of the warp takes part if any needs it.
 template <int G, class Nbr>
-__device__ __forceinline__ HalfSums fix_choose(const FixHalf &f, bool holds, const int4 *half, Nbr nbr, const int4 *w,
+__device__ __noinline__ HalfSums fix_low(const FixHalfScan top, const int4 *half, Nbr nbr, const int4 *w, int64_t ops,
+                                         int64_t step, int SLQ, short4 ew, int h) {
+    asm volatile("cp.async.wait_all;" ::: "memory");   // what the ring has begun to fetch
+    FixHalf<true> f;
+    f.start(top);
+    const unsigned sel = fix_third(h);
+#pragma unroll 2
+    for (int k = 0; k < SLQ; ++k, w += step) {
+        const int4 j = nbr(k);
+        f.slots(half[2 * (int64_t)j.x], half[2 * (int64_t)j.y], make_uint2(j.z, j.w), sel, __ldg(w), __ldg(w + ops),
+                __ldg(w + 2 * ops), __ldg(w + (2 + h) * ops));
+        if ((k & 7) == 7) f.fold();
+    }
+    f.fold();
+    return fix_finish<G>(f, ew, h);
+}
+
+// s, or over the G lanes of plain sums if any of the warp's do not hold (every
+// lane of the warp takes part).
+template <int G, class Nbr>
+__device__ __forceinline__ HalfSums fix_choose(const HalfSums &s, bool holds, const int4 *half, Nbr nbr, const int4 *w,
                                                int64_t ops, int64_t step, int SLQ, short4 ew, int h) {
-    HalfSums s = fix_finish<G>(f, ew, h);
     if (__all_sync(0xffffffffu, holds)) return s;
     HalfSums p = fix_plain(half, nbr, w, ops, step, SLQ, ew, h);
 #pragma unroll
@@ -413,11 +458,16 @@ __device__ __forceinline__ HalfSums fix_sums(const double *U, const FixStream &s
         top.take(__ldg(half + 2 * (int64_t)j.y), (unsigned)j.w, sel);
     }
     top.over_lanes<G>();
-    FixHalf f;
-    f.a.start(top.a);
-    f.b.start(top.b);
     const bool holds = top.holds(ew, h);
-    pn = s.nbr;
+    const int4 *first = s.nbr;
+    const int64_t step = s.step;
+    auto nbr = [first, step](int k) { return __ldg(first + k * step); };
+    if (__any_sync(0xffffffffu, top.low(ew, h)))
+        return fix_choose<G>(fix_low<G>(top, half, nbr, s.w, s.ops, step, s.SLQ, ew, h), holds, half, nbr, s.w, s.ops, step,
+                             s.SLQ, ew, h);
+    FixHalf<false> f;
+    f.start(top);
+    pn = first;
     int4 j = __ldg(pn);
     int4 n0 = __ldg(half + 2 * (int64_t)j.x), n1 = __ldg(half + 2 * (int64_t)j.y);
     uint2 e1 = make_uint2(j.z, j.w);
@@ -453,10 +503,7 @@ __device__ __forceinline__ HalfSums fix_sums(const double *U, const FixStream &s
         if (q0 & kFixRing) f.fold();
     }
     f.fold();
-    const int4 *nbr = s.nbr;
-    const int64_t step = s.step;
-    return fix_choose<G>(f, holds, half, [nbr, step](int k) { return __ldg(nbr + k * step); }, s.w, s.ops, s.step, s.SLQ,
-                         ew, h);
+    return fix_choose<G>(fix_finish<G>(f, ew, h), holds, half, nbr, s.w, s.ops, step, s.SLQ, ew, h);
 }
 
 }  // namespace rbf

@@ -241,12 +241,13 @@ __global__ void __launch_bounds__(kStageThreads<PF, LAT>, PF > 0 ? 1 : 1024 / kS
 // The FP64 stage (or bare right-hand side): the sums in fixed point
 // (fixdot.cuh), everything else in FP64.  On 308,097 scattered nodes with
 // n = 56 a stage of a run (with its ghost kernels) took 380 us as 12 x 56 FP64
-// FMAs per node (0.95 of the FP64 pipe) and takes 224 us; with one alignment
+// FMAs per node (0.95 of the FP64 pipe) and takes 228 us; with one alignment
 // per value in place of one per sum, 182 us.  What bounds it: the integer
 // pipes, some 70 instructions per slot and thread beside 18 IMAD.WIDEs, and
-// under them 110 us of operand traffic at the copy rate.  Five blocks of 128
-// threads per SM (96 registers): six, with spills, take 222 us, but the
-// right-hand side of a 125 m box 19.4 us in place of 18.6; seven 249 us.
+// under them 109 us of operand traffic at the copy rate.  Five blocks of 128
+// threads per SM (96 registers); before fix_low was there five took 224 us, six,
+// with spills, 222 us, but the right-hand side of a 125 m box 19.4 us in place
+// of 18.6, and seven 249 us.
 template <int G, bool LAT>
 __global__ void __launch_bounds__(kFixThreads, 5) ns_stage_fixed_kernel(NSArgs<double> a) {
     __shared__ FixRing ring;

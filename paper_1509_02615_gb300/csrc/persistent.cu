@@ -746,12 +746,21 @@ __global__ void __launch_bounds__(MAXT, 1) rk4_persistent(const __grid_constant_
                         top.take(sh_half(halo, 2 * j.y + h), e.y, sel);
                     }
                     top.over_lanes<G>();
-                    FixHalf f;
-                    f.a.start(top.a);
-                    f.b.start(top.b);
                     const bool holds = top.holds(ew, h);
+                    const int4 *half = reinterpret_cast<const int4 *>(halo) + h;
+                    auto nbr = [lx, lq, off0, stride](int k) {
+                        const L j = __ldg(lx + off0 + k * stride);
+                        const uint2 e = __ldg(lq + off0 + k * stride);
+                        return make_int4(j.x, j.y, (int)e.x, (int)e.y);
+                    };
+                    const bool low = __any_sync(0xffffffffu, top.low(ew, h));
+                    HalfSums sums;
+                    FixHalf<false> f;
+                    f.start(top);
                     int64_t off = off0;
-                    if (a.ring_off) {
+                    if (low) {
+                        sums = fix_low<G>(top, half, nbr, wx + off0, a.total / V, stride, a.SLQ, ew, h);
+                    } else if (a.ring_off) {
                         // operands two steps ahead through the pair's ring slots (fixdot.cuh)
                         const int4 *v = ring + (threadIdx.x >> 1);
                         const int np = blockDim.x >> 1;
@@ -777,10 +786,6 @@ __global__ void __launch_bounds__(MAXT, 1) rk4_persistent(const __grid_constant_
                             }
                             if (q0 & kFixRing) f.fold();
                         }
-                        __syncwarp();   // every slot has been read
-                        fetch.start(fs, ring, np);
-                        fetch.copy(0);   // the next stage's first steps
-                        fetch.copy(1);
                     } else {
                         const W *we = h ? wh : wd;
                         for (int q0 = 0; q0 < a.SLQ; q0 += kFixRing) {
@@ -793,15 +798,17 @@ __global__ void __launch_bounds__(MAXT, 1) rk4_persistent(const __grid_constant_
                             if (q0 & kFixRing) f.fold();
                         }
                     }
-                    f.fold();
-                    const HalfSums sums =
-                        fix_choose<G>(f, holds, reinterpret_cast<const int4 *>(halo) + h,
-                                      [lx, lq, off0, stride](int k) {
-                                          const L j = __ldg(lx + off0 + k * stride);
-                                          const uint2 e = __ldg(lq + off0 + k * stride);
-                                          return make_int4(j.x, j.y, (int)e.x, (int)e.y);
-                                      },
-                                      wx + off0, a.total / V, stride, a.SLQ, ew, h);
+                    if (a.ring_off && !low) {
+                        __syncwarp();   // every slot has been read
+                        fetch.start(fs, ring, blockDim.x >> 1);
+                        fetch.copy(0);   // the next stage's first steps
+                        fetch.copy(1);
+                    }
+                    if (!low) {
+                        f.fold();
+                        sums = fix_finish<G>(f, ew, h);
+                    }
+                    sums = fix_choose<G>(sums, holds, half, nbr, wx + off0, a.total / V, stride, a.SLQ, ew, h);
                     const double2 kk = fix_tendency(sums, {a.cp, a.g_over_tb, a.theta_bar, a.dpibar, a.rd_cv}, h,
                                                     make_double4(fi.u, fi.w, fi.t, fi.p), pib, fl);
                     k[0] = kk.x;

@@ -114,6 +114,26 @@ def test_low_end_and_negative_zeros(lanes):
     pb.close()
 
 
+@pytest.mark.parametrize("scale", [1e-283, 1e-290, 1e-300, 1e-308, 1e-320])
+def test_whole_fields_at_the_low_end(scale):
+    nodes, prm = CASES["walls31"]()
+    rng = np.random.default_rng(10)
+    U = _smooth(nodes, rng)
+    U[1:] *= scale * 10.0 ** rng.uniform(-6, 2, (3, nodes.n_all))   # u stays in the ordinary range
+    U[1:][rng.random((3, nodes.n_all)) < 0.2] = 0.0
+    out = []
+    for lanes in (1, 2):
+        pb = rbffd.ns_problem(nodes, precision=64, threads_per_node=lanes, **prm)
+        got, Uf = _rhs(pb, U)
+        rows, idx = _rows(pb, prm["mu"])
+        ref, M, _ = _tendencies(rows, idx, nodes, Uf, LD)
+        e = np.abs(got.astype(LD) - ref).astype(float)
+        assert np.all(e <= 2.0 ** -53 * M + 4e5 * 31 * 2.0 ** -1074)
+        out.append(got)
+        pb.close()
+    assert np.array_equal(out[0], out[1])
+
+
 @pytest.mark.parametrize("lanes", [1, 2])
 def test_infinite_value_gives_what_fp64_gives(lanes):
     nodes, prm = inp.density_current_nodes(400.0), dict(n=37, l=4, mu=75.0)
