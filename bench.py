@@ -13,7 +13,7 @@ Metric: node-RHS evaluations per second (4 per node per RK4 step).  The
 headline's working set (operators, records, RK4 buffers: ~0.7 GB in FP64) is
 several times larger than L2, so steps are timed back to back without an L2
 flush, each with CUDA events on the problem's stream.  The dominant kernel is
-the FP64 stage kernel, whose stencil sums run in fixed point on the integer
+the FP64 stage kernel, whose stencil sums run as integer products on the integer
 units: its roofline is its operand traffic against HBM, with its FP64-equivalent
 rate and a DGEMM measured in the same run beside it.
 
@@ -309,7 +309,7 @@ def headline_case(torch, args, wl, world, local, p64):
             "kernel": kernel, "algorithmic_flops_per_launch": flops, "algorithmic_bytes_per_launch": bpl,
             "avg_launch_ms": avg_ms, "kernel_share_of_step": share,
             "fp64_equivalent_tflops": ach, "fp64_dgemm_tflops": p64,
-            "note": "the stencil sums are exact products of 28-bit integers on the integer units, no FP64 FMAs; the "
+            "note": "the stencil sums are integer products on the integer units, aligned per sum, no FP64 FMAs; the "
                     "DGEMM (cuBLAS via torch.matmul, 4096^3, this run) is the rate they would be bound by"}
     # end to end through the C ABI: pinned host state -> device, one RK4 step, device -> host
     Uh = rbffd.state_tensor(wl.U0, 64, device="cpu").pin_memory()
