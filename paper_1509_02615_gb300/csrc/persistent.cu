@@ -910,9 +910,10 @@ __global__ void __launch_bounds__(MAXT, 1) rk4_persistent(const __grid_constant_
 // Here each lane keeps its R packed slots (stencil index, flux weights of
 // each velocity part, hyperviscosity weight) in registers for the whole run,
 // U_n and the RK4 accumulator of its node too; a stage gathers the stage
-// input (ordinary loads: the barrier's acquire orders them), forms the tendency and the RK4 update exactly as the
-// stage kernel does (same slots per lane, summation order, lane reduction,
-// time factors and update), and the CTAs meet at a grid barrier.  Results
+// input (ordinary loads: the barrier's acquire orders them), forms the
+// tendency and the RK4 update exactly as the stage kernel does (same slots per
+// lane, summation order, lane reduction, time factors and update), and the
+// CTAs meet at a grid barrier.  Results
 // equal the launch-per-stage form's bit for bit with the same lanes per node.
 template <class T>
 struct AdvPArgs {
